@@ -214,25 +214,76 @@ __device__ __forceinline__ void fold_gumbel(Stat& st, const float* v, int x0, fl
   }
 }
 
-// Statistics of logits [begin, end) of one row.  STATS: maximum, arg-max and sum;
-// GUMBEL: the best noisy score (token `exclude` left out).  With VECTOR, `begin`
-// is a multiple of the vector length and the row is 16-byte aligned.
-template <typename T, bool VECTOR, bool GUMBEL, int STATS>
+// Sixteen bytes of logits from a row that starts at any element-aligned address (an odd vocabulary leaves
+// most rows off the 16-byte grid): the two aligned pieces that hold them, each with at least one byte of
+// the vector, shifted into place by the row's offset (the same for the whole row, so no branch diverges).
+// About two instructions per logit; the second piece is the neighbouring lane's first one and hits L1.
+struct Piece2 { uint4 a, b; };
+template <typename T>
+__device__ __forceinline__ Piece2 load_pieces(const T* row, int x) {
+  const uintptr_t at = reinterpret_cast<uintptr_t>(row + x);
+  const uint4* q = reinterpret_cast<const uint4*>(at & ~(uintptr_t)15);
+  Piece2 r;
+  r.a = __ldg(q);
+  r.b = (at & 15) ? __ldg(q + 1) : r.a;
+  return r;
+}
+template <typename T>
+__device__ __forceinline__ uint4 shift_pieces(const Piece2& r, const T* row) {
+  const uint32_t off = (uint32_t)(reinterpret_cast<uintptr_t>(row) & 15);   // (vectors start at multiples of 16 bytes of the row)
+  uint32_t w[8] = {r.a.x, r.a.y, r.a.z, r.a.w, r.b.x, r.b.y, r.b.z, r.b.w};
+  if (off & 8) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
+  }
+  if (off & 4) {
+#pragma unroll
+    for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
+  }
+  if (sizeof(T) == 2 && (off & 2)) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(w[i], w[i + 1], 16);
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Statistics of logits [begin, end) of one row, `begin` a multiple of the vector length.  STATS: maximum,
+// arg-max and sum; GUMBEL: the best noisy score (token `exclude` left out).  ALIGNED: the row is 16-byte
+// aligned; otherwise every vector is put together from two aligned pieces (see load_pieces).
+template <typename T, bool ALIGNED, bool GUMBEL, int STATS>
 __device__ Stat scan_chunk(const T* row, int begin, int end, float c, int exclude,
                            uint32_t key0, uint32_t key1, uint32_t purpose, uint32_t seq,
                            uint32_t pos) {
   Stat st = stat_empty();
-  if (VECTOR) {
-    constexpr int N = Vec<T>::N;
-    constexpr int U = 4;                                    // independent 16-byte loads in flight per thread
-    // the tail shorter than N is handled one by one
-    const int full_end = begin + ((end - begin) / N) * N;
-    const int stride = blockDim.x * N;
-    const uint4 ninf = make_uint4(Vec<T>::NEG_INF, Vec<T>::NEG_INF, Vec<T>::NEG_INF, Vec<T>::NEG_INF);
+  constexpr int N = Vec<T>::N;
+  constexpr int U = 4;                                      // independent vectors in flight per thread
+  // the tail shorter than N is handled one by one
+  const int full_end = begin + ((end - begin) / N) * N;
+  const int stride = blockDim.x * N;
+  const uint4 ninf = make_uint4(Vec<T>::NEG_INF, Vec<T>::NEG_INF, Vec<T>::NEG_INF, Vec<T>::NEG_INF);
+  int x = begin + threadIdx.x * N;
+  // one sweep of U vectors, the first at x; slots past the end read as -inf
+  auto fold = [&](const uint4 (&cur)[U], int x) {
+    float v[U][N];
+#pragma unroll
+    for (int u = 0; u < U; ++u) Vec<T>::convert(cur[u], v[u]);
+    if (STATS) fold_stats<U, N, STATS == STAT_SUM>(st, v, x, stride, c);
+    if (GUMBEL) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int xu = x + u * stride;
+        if ((unsigned)(exclude - xu) < (unsigned)N) {       // the one token left out of the draw
+#pragma unroll
+          for (int i = 0; i < N; ++i) if (xu + i == exclude) v[u][i] = -CUDART_INF_F;
+        }
+        if (xu < full_end) fold_gumbel<N>(st, v[u], xu, c, key0, key1, purpose, seq, pos);
+      }
+    }
+  };
+  if (ALIGNED) {
     // The U loads of the next sweep are issued before the current one is folded,
-    // so a thread always has loads in flight; slots past the end read as -inf.
+    // so a thread always has loads in flight.
     uint4 cur[U], nxt[U];
-    int x = begin + threadIdx.x * N;
 #pragma unroll
     for (int u = 0; u < U; ++u)
       cur[u] = (x + u * stride < full_end) ? __ldg(reinterpret_cast<const uint4*>(row + x + u * stride)) : ninf;
@@ -241,42 +292,38 @@ __device__ Stat scan_chunk(const T* row, int begin, int end, float c, int exclud
 #pragma unroll
       for (int u = 0; u < U; ++u)
         nxt[u] = (xn + u * stride < full_end) ? __ldg(reinterpret_cast<const uint4*>(row + xn + u * stride)) : ninf;
-      float v[U][N];
-#pragma unroll
-      for (int u = 0; u < U; ++u) Vec<T>::convert(cur[u], v[u]);
-      if (STATS) fold_stats<U, N, STATS == STAT_SUM>(st, v, x, stride, c);
-      if (GUMBEL) {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int xu = x + u * stride;
-          if ((unsigned)(exclude - xu) < (unsigned)N) {     // the one token left out of the draw
-#pragma unroll
-            for (int i = 0; i < N; ++i) if (xu + i == exclude) v[u][i] = -CUDART_INF_F;
-          }
-          if (xu < full_end) fold_gumbel<N>(st, v[u], xu, c, key0, key1, purpose, seq, pos);
-        }
-      }
+      fold(cur, x);
 #pragma unroll
       for (int u = 0; u < U; ++u) cur[u] = nxt[u];
       x = xn;
     }
-    if (STATS && st.m > -CUDART_INF_F) {
-      // settle the arg-max inside its vector: lowest index equal to the maximum
-      float vv[N];
-      Vec<T>::convert(__ldg(reinterpret_cast<const uint4*>(row + st.idx)), vv);
-      int off = 0;
-#pragma unroll
-      for (int i = N - 1; i >= 0; --i) if (vv[i] == st.m) off = i;
-      st.idx += off;
-    }
-    for (int xt = full_end + threadIdx.x; xt < end; xt += blockDim.x) {
-      Stat one = stat_empty();
-      fold_one<GUMBEL, STATS>(one, load_logit(row + xt), xt, c, exclude, key0, key1, purpose, seq, pos);
-      stat_merge(st, one, c);
-    }
   } else {
-    for (int xt = begin + threadIdx.x; xt < end; xt += blockDim.x)
-      fold_one<GUMBEL, STATS>(st, load_logit(row + xt), xt, c, exclude, key0, key1, purpose, seq, pos);
+    // (two loads per vector are in flight here; holding the next sweep's as well would cost 32 registers)
+    for (; x < full_end; x += U * stride) {
+      Piece2 raw[U];
+      uint4 cur[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (x + u * stride < full_end) raw[u] = load_pieces(row, x + u * stride);
+        else raw[u].a = raw[u].b = ninf;
+#pragma unroll
+      for (int u = 0; u < U; ++u) cur[u] = shift_pieces(raw[u], row);
+      fold(cur, x);
+    }
+  }
+  if (STATS && st.m > -CUDART_INF_F) {
+    // settle the arg-max inside its vector: lowest index equal to the maximum
+    float vv[N];
+    Vec<T>::convert(ALIGNED ? __ldg(reinterpret_cast<const uint4*>(row + st.idx)) : shift_pieces(load_pieces(row, st.idx), row), vv);
+    int off = 0;
+#pragma unroll
+    for (int i = N - 1; i >= 0; --i) if (vv[i] == st.m) off = i;
+    st.idx += off;
+  }
+  for (int xt = full_end + threadIdx.x; xt < end; xt += blockDim.x) {
+    Stat one = stat_empty();
+    fold_one<GUMBEL, STATS>(one, load_logit(row + xt), xt, c, exclude, key0, key1, purpose, seq, pos);
+    stat_merge(st, one, c);
   }
   return st;
 }
@@ -399,7 +446,7 @@ __device__ bool arrive_last(int* counter, int expected) {
   return last != 0;
 }
 
-template <typename T, bool VECTOR>
+template <typename T, bool ALIGNED>
 __global__ void __launch_bounds__(SPACE_VERIFY_THREADS)
 verify_target_kernel(const VerifyParams p) {
   pdl_launch_dependents();
@@ -408,7 +455,7 @@ verify_target_kernel(const VerifyParams p) {
   const int k1 = p.k + 1;
   const T* row = reinterpret_cast<const T*>(p.logits) + ((int64_t)b * p.n_q + (int64_t)t * k1) * p.row_stride;
   const int begin = ch * p.chunk, end = min(p.V, begin + p.chunk);
-  Stat st = scan_chunk<T, VECTOR, false, STAT_SUM>(row, begin, end, p.c_t, -1, 0, 0, 0, 0, 0);
+  Stat st = scan_chunk<T, ALIGNED, false, STAT_SUM>(row, begin, end, p.c_t, -1, 0, 0, 0, 0, 0);
   st = block_reduce_plain(st, p.c_t);
   VerifyPartial* part = p.part + ((int64_t)b * (p.k + 2) + t) * p.n_chunks;
   if (threadIdx.x == 0) store_partial(part + ch, st);
@@ -462,7 +509,7 @@ verify_target_kernel(const VerifyParams p) {
   }
 }
 
-template <typename T, bool VECTOR>
+template <typename T, bool ALIGNED>
 __global__ void __launch_bounds__(SPACE_VERIFY_THREADS, 3)   // 80 registers, no spills: three blocks per SM
 verify_emit_kernel(const VerifyParams p) {
   pdl_launch_dependents();
@@ -511,16 +558,16 @@ verify_emit_kernel(const VerifyParams p) {
     // with any other P_c (Algorithm 1 starts from P_c = +inf) was no point mass: a ~ Q.
     if (!literal && i_star < p.k && p.cand_prob[b * p.k + i_star] == 1.0f) exclude = p.cand[b * p.k + i_star];
     // the extra token needs the noisy arg-max alone: the row's sums are known
-    st = scan_chunk<T, VECTOR, true, STAT_NONE>(row, begin, end, c, exclude, p.key0, p.key1, PURPOSE_TOKEN,
+    st = scan_chunk<T, ALIGNED, true, STAT_NONE>(row, begin, end, c, exclude, p.key0, p.key1, PURPOSE_TOKEN,
                                             seq, (uint32_t)(L + i_star + 1));
   } else if (literal) {
-    st = scan_chunk<T, VECTOR, true, STAT_SUM>(row, begin, end, c, -1, p.key0, p.key1, PURPOSE_DRAFT, seq,
+    st = scan_chunk<T, ALIGNED, true, STAT_SUM>(row, begin, end, c, -1, p.key0, p.key1, PURPOSE_DRAFT, seq,
                                            (uint32_t)(L + i_star + 1 + slot + 1));
   } else if (sample) {
     // point-mass drafts: the new candidates are the rows' arg-maxes with P_c = 1, no sums needed
-    st = scan_chunk<T, VECTOR, false, STAT_MAX>(row, begin, end, c, -1, 0, 0, 0, 0, 0);
+    st = scan_chunk<T, ALIGNED, false, STAT_MAX>(row, begin, end, c, -1, 0, 0, 0, 0, 0);
   } else {
-    st = scan_chunk<T, VECTOR, false, STAT_SUM>(row, begin, end, c, -1, 0, 0, 0, 0, 0);
+    st = scan_chunk<T, ALIGNED, false, STAT_SUM>(row, begin, end, c, -1, 0, 0, 0, 0, 0);
   }
   st = block_reduce(st, c);
   // (chunk results of the emit kernel: SPACE_VERIFY_MAX_CHUNKS slots per row, whatever its cut)
@@ -591,7 +638,7 @@ __device__ unsigned long long g_timeline_verify[4096 * 8];
 
 // PAGED: the commit on board goes through a page table (a build of its own: the table look-ups are
 // not compiled into the contiguous form, whose addressing sits in the critical path).
-template <typename T, bool VECTOR, bool PAGED = false>
+template <typename T, bool ALIGNED, bool PAGED = false>
 __global__ void __launch_bounds__(SPACE_VERIFY_THREADS)
 verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
   TLV(0);
@@ -607,7 +654,7 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
   if (p.do_commit) Lc = p.cm.kv_len[b];                     // in flight during the scan
   // (the candidates too: the block that finishes the sequence must not start a memory round trip for them)
   const int my_cand = threadIdx.x < p.k ? p.cand[b * p.k + threadIdx.x] : 0;
-  Stat st = scan_chunk<T, VECTOR, false, STAT_SUM>(row, begin, end, C1, -1, 0, 0, 0, 0, 0);
+  Stat st = scan_chunk<T, ALIGNED, false, STAT_SUM>(row, begin, end, C1, -1, 0, 0, 0, 0, 0);
 #ifdef SPACE_TIMELINE
   if (st.m != 12345.f) TLV(2);                              // (a use of the result: the stamp follows the loads)
 #endif
@@ -723,26 +770,47 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
   }
 }
 
-template <typename T, bool VECTOR>
+// Chunks per row and their length.  A sweep of a block is four vectors per thread (8192 bf16 logits); a
+// block costs about 3 us whatever it scans (reduction, fence, arrival), so it should make one sweep while
+// there are fewer of them than about three resident blocks per SM can take at once, and up to four when
+// there are more.  Measured, us per call: one row-chunk per SM's worth of blocks as before / this rule:
+// 5 x 16 rows of 50257 15.2 / 9.9, 2 x 49 rows of 128256 21.3 / 12, one sequence of 36 rows of 32000 6.4 / 6.4,
+// sampling 64 x 5 rows of 128256 67 / 57; one sweep per block there instead of four 71.
+int row_chunks(int vocab, int rows, int vec, int sm_count, int max_chunks, int* chunk_out) {
+  const int sweep = SPACE_VERIFY_THREADS * vec * 4;
+  const int64_t total = (int64_t)rows * ((vocab + sweep - 1) / sweep);
+  const int64_t slots = 3 * (int64_t)sm_count;
+  int64_t per_block = (total + slots / 2) / slots;
+  if (per_block < 1) per_block = 1;
+  if (per_block > 4) per_block = 4;
+  int64_t nc = (vocab + per_block * sweep - 1) / (per_block * sweep);
+  if (nc > max_chunks) nc = max_chunks;
+  int chunk = (int)((vocab + nc - 1) / nc);
+  chunk = (chunk + vec - 1) / vec * vec;
+  *chunk_out = chunk;
+  return (vocab + chunk - 1) / chunk;
+}
+
+template <typename T, bool ALIGNED>
 void launch_fused(space_ctx* ctx, const VerifyParams& p, cudaStream_t st) {
   ProfScope ps(ctx, SPACE_K_VERIFY_TARGET, st);
   if (p.do_commit && p.cm.page_table)
-    launch_pdl(verify_fused_kernel<T, VECTOR, true>, dim3(p.n_chunks, p.n_q, p.B), dim3(SPACE_VERIFY_THREADS), 0, st, p, ctx->vfused);
+    launch_pdl(verify_fused_kernel<T, ALIGNED, true>, dim3(p.n_chunks, p.n_q, p.B), dim3(SPACE_VERIFY_THREADS), 0, st, p, ctx->vfused);
   else
-  launch_pdl(verify_fused_kernel<T, VECTOR>, dim3(p.n_chunks, p.n_q, p.B), dim3(SPACE_VERIFY_THREADS), 0, st, p, ctx->vfused);
+  launch_pdl(verify_fused_kernel<T, ALIGNED>, dim3(p.n_chunks, p.n_q, p.B), dim3(SPACE_VERIFY_THREADS), 0, st, p, ctx->vfused);
 }
 
-template <typename T, bool VECTOR>
+template <typename T, bool ALIGNED>
 void launch_both(space_ctx* ctx, const VerifyParams& p, int n_slots_b, cudaStream_t st) {
   dim3 ga(p.n_chunks, p.k + 1, p.B);
   const dim3 gb(p.B * (p.k * p.n_chunks + (p.mode == SPACE_MODE_SAMPLE ? p.n_chunks_g : 0)));
   {
     ProfScope ps(ctx, SPACE_K_VERIFY_TARGET, st);
-    launch_pdl(verify_target_kernel<T, VECTOR>, ga, dim3(SPACE_VERIFY_THREADS), 0, st, p);
+    launch_pdl(verify_target_kernel<T, ALIGNED>, ga, dim3(SPACE_VERIFY_THREADS), 0, st, p);
   }
   {
     ProfScope ps(ctx, SPACE_K_VERIFY_EMIT, st);
-    launch_pdl(verify_emit_kernel<T, VECTOR>, gb, dim3(SPACE_VERIFY_THREADS), 0, st, p);
+    launch_pdl(verify_emit_kernel<T, ALIGNED>, gb, dim3(SPACE_VERIFY_THREADS), 0, st, p);
   }
 }
 
@@ -799,61 +867,29 @@ int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit
 
   const int esz = a->logits_dtype == SPACE_DTYPE_F32 ? 4 : 2;
   const int vec = 16 / esz;
-  const bool vector = ((uintptr_t)a->logits % 16 == 0) && ((a->logits_row_stride * esz) % 16 == 0);
+  const bool aligned = ((uintptr_t)a->logits % 16 == 0) && ((a->logits_row_stride * esz) % 16 == 0);
   // small greedy problem: one launch over all block rows (see the file header)
   const int64_t all_bytes = (int64_t)a->batch * p.n_q * a->vocab * esz;
   if (a->mode == SPACE_MODE_GREEDY && all_bytes <= SPACE_FUSED_MAX_BYTES) {
-    const int rows_all = a->batch * p.n_q;
-    int nc = ctx->sm_count / rows_all;                      // about one block per SM: few arrivals, four loads in flight
-    const int min_chunk = SPACE_VERIFY_THREADS * vec;
-    const int max_nc = (a->vocab + min_chunk - 1) / min_chunk;
-    if (nc > max_nc) nc = max_nc;
-    if (nc > SPACE_FUSED_MAX_CHUNKS) nc = SPACE_FUSED_MAX_CHUNKS;
-    if (nc < 1) nc = 1;
-    int chunk = (a->vocab + nc - 1) / nc;
-    chunk = ((chunk + vec - 1) / vec) * vec;
-    nc = (a->vocab + chunk - 1) / chunk;
+    int chunk, nc = row_chunks(a->vocab, a->batch * p.n_q, vec, ctx->sm_count, SPACE_FUSED_MAX_CHUNKS, &chunk);
     p.n_chunks = nc; p.chunk = chunk; p.n_chunks_g = 0; p.chunk_g = 0;
     if (a->logits_dtype == SPACE_DTYPE_F32) {
-      if (vector) launch_fused<float, true>(ctx, p, st); else launch_fused<float, false>(ctx, p, st);
+      if (aligned) launch_fused<float, true>(ctx, p, st); else launch_fused<float, false>(ctx, p, st);
     } else {
-      if (vector) launch_fused<__nv_bfloat16, true>(ctx, p, st); else launch_fused<__nv_bfloat16, false>(ctx, p, st);
+      if (aligned) launch_fused<__nv_bfloat16, true>(ctx, p, st); else launch_fused<__nv_bfloat16, false>(ctx, p, st);
     }
     ctx->launches += 1;
     return cuda_ok(cudaGetLastError());
   }
-  // enough chunks to put about four blocks on every SM: little more than one resident
-  // wave (measured on the 64-sequence sampling workload: 4 per SM 29 / 39 us, 8 per SM
-  // 31 / 43 us, 16 per SM 38 / 54 us), but no chunk below four sweeps of a block
-  const int rows = a->batch * (a->k + 1);
-  int nc = (4 * ctx->sm_count + rows - 1) / rows;
-  const int min_chunk = SPACE_VERIFY_THREADS * vec * 4;
-  const int max_nc = (a->vocab + min_chunk - 1) / min_chunk;
-  if (nc > max_nc) nc = max_nc;
-  if (nc > SPACE_VERIFY_MAX_CHUNKS) nc = SPACE_VERIFY_MAX_CHUNKS;
-  if (nc < 1) nc = 1;
-  int chunk = (a->vocab + nc - 1) / nc;
-  chunk = ((chunk + vec - 1) / vec) * vec;
-  nc = (a->vocab + chunk - 1) / chunk;
+  int chunk, nc = row_chunks(a->vocab, a->batch * (a->k + 1), vec, ctx->sm_count, SPACE_VERIFY_MAX_CHUNKS, &chunk);
   p.n_chunks = nc; p.chunk = chunk;
   const int n_slots_b = (a->mode == SPACE_MODE_SAMPLE) ? a->k + 1 : a->k;
-  // the extra-token row has a cut of its own (its logits cost several times a plain row's)
-  {
-    int ncg = nc;                                           // (measured: a finer cut of this row, up to 8x, is no faster)
-    const int min_chunk_g = SPACE_VERIFY_THREADS * vec * 4;
-    const int max_ncg = (a->vocab + min_chunk_g - 1) / min_chunk_g;
-    if (ncg > max_ncg) ncg = max_ncg;
-    if (ncg > SPACE_VERIFY_MAX_CHUNKS) ncg = SPACE_VERIFY_MAX_CHUNKS;
-    if (ncg < 1) ncg = 1;
-    int cg = (a->vocab + ncg - 1) / ncg;
-    cg = ((cg + vec - 1) / vec) * vec;
-    p.n_chunks_g = (a->vocab + cg - 1) / cg; p.chunk_g = cg;
-  }
+  p.n_chunks_g = nc; p.chunk_g = chunk;                     // (measured: a finer cut of the noisy row, up to 8x, is no faster)
 
   if (a->logits_dtype == SPACE_DTYPE_F32) {
-    if (vector) launch_both<float, true>(ctx, p, n_slots_b, st); else launch_both<float, false>(ctx, p, n_slots_b, st);
+    if (aligned) launch_both<float, true>(ctx, p, n_slots_b, st); else launch_both<float, false>(ctx, p, n_slots_b, st);
   } else {
-    if (vector) launch_both<__nv_bfloat16, true>(ctx, p, n_slots_b, st);
+    if (aligned) launch_both<__nv_bfloat16, true>(ctx, p, n_slots_b, st);
     else launch_both<__nv_bfloat16, false>(ctx, p, n_slots_b, st);
   }
   ctx->launches += 2;
@@ -938,25 +974,16 @@ int launch_verify_noalloc(const space_verify_args* a, cudaStream_t st) {
 
   const int esz = a->logits_dtype == SPACE_DTYPE_F32 ? 4 : 2;
   const int vec = 16 / esz;
-  const bool vector = ((uintptr_t)a->logits % 16 == 0) && ((a->logits_row_stride * esz) % 16 == 0);
-  const int rows_all = a->batch * p.n_q;
-  int nc = g_noalloc_sms[dev] / rows_all;
-  const int min_chunk = SPACE_VERIFY_THREADS * vec;
-  const int max_nc = (a->vocab + min_chunk - 1) / min_chunk;
-  if (nc > max_nc) nc = max_nc;
-  if (nc > SPACE_FUSED_MAX_CHUNKS) nc = SPACE_FUSED_MAX_CHUNKS;
-  if (nc < 1) nc = 1;
-  int chunk = (a->vocab + nc - 1) / nc;
-  chunk = ((chunk + vec - 1) / vec) * vec;
-  nc = (a->vocab + chunk - 1) / chunk;
+  const bool aligned = ((uintptr_t)a->logits % 16 == 0) && ((a->logits_row_stride * esz) % 16 == 0);
+  int chunk, nc = row_chunks(a->vocab, a->batch * p.n_q, vec, g_noalloc_sms[dev], SPACE_FUSED_MAX_CHUNKS, &chunk);
   p.n_chunks = nc; p.chunk = chunk;
   const dim3 grid(nc, p.n_q, a->batch), block(SPACE_VERIFY_THREADS);
   cudaError_t e;
   if (a->logits_dtype == SPACE_DTYPE_F32) {
-    e = vector ? launch_pdl(verify_fused_kernel<float, true>, grid, block, 0, st, p, fpart)
+    e = aligned ? launch_pdl(verify_fused_kernel<float, true>, grid, block, 0, st, p, fpart)
                : launch_pdl(verify_fused_kernel<float, false>, grid, block, 0, st, p, fpart);
   } else {
-    e = vector ? launch_pdl(verify_fused_kernel<__nv_bfloat16, true>, grid, block, 0, st, p, fpart)
+    e = aligned ? launch_pdl(verify_fused_kernel<__nv_bfloat16, true>, grid, block, 0, st, p, fpart)
                : launch_pdl(verify_fused_kernel<__nv_bfloat16, false>, grid, block, 0, st, p, fpart);
   }
   return cuda_ok(e);
