@@ -214,39 +214,6 @@ __device__ __forceinline__ void fold_gumbel(Stat& st, const float* v, int x0, fl
   }
 }
 
-// Sixteen bytes of logits from a row that starts at any element-aligned address (an odd vocabulary leaves
-// most rows off the 16-byte grid): the two aligned pieces that hold them, each with at least one byte of
-// the vector, shifted into place by the row's offset (the same for the whole row, so no branch diverges).
-// About two instructions per logit; the second piece is the neighbouring lane's first one and hits L1.
-struct Piece2 { uint4 a, b; };
-template <typename T>
-__device__ __forceinline__ Piece2 load_pieces(const T* row, int x) {
-  const uintptr_t at = reinterpret_cast<uintptr_t>(row + x);
-  const uint4* q = reinterpret_cast<const uint4*>(at & ~(uintptr_t)15);
-  Piece2 r;
-  r.a = __ldg(q);
-  r.b = (at & 15) ? __ldg(q + 1) : r.a;
-  return r;
-}
-template <typename T>
-__device__ __forceinline__ uint4 shift_pieces(const Piece2& r, const T* row) {
-  const uint32_t off = (uint32_t)(reinterpret_cast<uintptr_t>(row) & 15);   // (vectors start at multiples of 16 bytes of the row)
-  uint32_t w[8] = {r.a.x, r.a.y, r.a.z, r.a.w, r.b.x, r.b.y, r.b.z, r.b.w};
-  if (off & 8) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) w[i] = w[i + 2];
-  }
-  if (off & 4) {
-#pragma unroll
-    for (int i = 0; i < 5; ++i) w[i] = w[i + 1];
-  }
-  if (sizeof(T) == 2 && (off & 2)) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(w[i], w[i + 1], 16);
-  }
-  return make_uint4(w[0], w[1], w[2], w[3]);
-}
-
 // Statistics of logits [begin, end) of one row, `begin` a multiple of the vector length.  STATS: maximum,
 // arg-max and sum; GUMBEL: the best noisy score (token `exclude` left out).  ALIGNED: the row is 16-byte
 // aligned; otherwise every vector is put together from two aligned pieces (see load_pieces).
@@ -770,27 +737,6 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
   }
 }
 
-// Chunks per row and their length.  A sweep of a block is four vectors per thread (8192 bf16 logits); a
-// block costs about 3 us whatever it scans (reduction, fence, arrival), so it should make one sweep while
-// there are fewer of them than about three resident blocks per SM can take at once, and up to four when
-// there are more.  Measured, us per call: one row-chunk per SM's worth of blocks as before / this rule:
-// 5 x 16 rows of 50257 15.2 / 9.9, 2 x 49 rows of 128256 21.3 / 12, one sequence of 36 rows of 32000 6.4 / 6.4,
-// sampling 64 x 5 rows of 128256 67 / 57; one sweep per block there instead of four 71.
-int row_chunks(int vocab, int rows, int vec, int sm_count, int max_chunks, int* chunk_out) {
-  const int sweep = SPACE_VERIFY_THREADS * vec * 4;
-  const int64_t total = (int64_t)rows * ((vocab + sweep - 1) / sweep);
-  const int64_t slots = 3 * (int64_t)sm_count;
-  int64_t per_block = (total + slots / 2) / slots;
-  if (per_block < 1) per_block = 1;
-  if (per_block > 4) per_block = 4;
-  int64_t nc = (vocab + per_block * sweep - 1) / (per_block * sweep);
-  if (nc > max_chunks) nc = max_chunks;
-  int chunk = (int)((vocab + nc - 1) / nc);
-  chunk = (chunk + vec - 1) / vec * vec;
-  *chunk_out = chunk;
-  return (vocab + chunk - 1) / chunk;
-}
-
 template <typename T, bool ALIGNED>
 void launch_fused(space_ctx* ctx, const VerifyParams& p, cudaStream_t st) {
   ProfScope ps(ctx, SPACE_K_VERIFY_TARGET, st);
@@ -833,10 +779,8 @@ extern "C" int space_debug_timeline_read_verify(unsigned long long* host_dst, in
 
 int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit_args* cm, cudaStream_t st) {
   if (a->mode == SPACE_MODE_SAMPLE && a->top_k > 0) {
-    // filtered target distributions: kernels of their own (verify_filter.cu); the commit follows as its own launch
-    const int rc = launch_verify_filtered(ctx, a, st);
-    if (rc != SPACE_OK || !cm) return rc;
-    return launch_commit(ctx, cm, st);
+    // filtered target distributions: kernels of their own (verify_filter.cu), which carry the commit too
+    return launch_verify_filtered(ctx, a, cm, st);
   }
   if (cm && cm->page_table) {
     // paged cache: only the single-launch greedy form carries the commit through a page table; the

@@ -8,18 +8,27 @@
 // the extra token from row i* (Gumbel arg-max over the kept tokens, Philox noise keyed by the token as
 // in verify.cu) and emits the tokens.  Phase 1 does the same for the k mask rows of group i* and
 // writes the next candidates (their arg-maxes with P_c = 1, or samples from the filtered rows with
-// their probabilities when candidates are sampled).
+// their probabilities when candidates are sampled); with a commit on board its blocks also move the
+// accepted cache rows.  A small batch goes through one launch instead (PHASE_BOTH): every block row is
+// searched, and the last block runs both halves on the rows it needs.
 //
 // SPACE_RESAMPLE_RESIDUAL_DRAFT keeps sampled candidates lossless (Sec. 3.2 claims an unchanged output
 // distribution): phase 1 also writes every candidate's filtered distribution D as a list of top_k
 // (token, probability) pairs, and phase 0 of the next step, after rejecting candidate i, draws the extra
 // token from norm(max(0, Q - D_i)) -- one warp, its 32 lanes holding Q's kept tokens and D_i's entries.
 //
-// Top-k selection: every warp keeps a sorted list of at most 32 (logit, token) keys, one per lane, and
-// a threshold (its last key); a logit above the threshold is inserted with one ballot and one shuffle.
+// Top-k selection, per block and segment (a few sweeps of 256 threads x four 16-byte vectors): one pass
+// keeps every thread's maximum; the maxima of 128 groups of two threads are ranked against each other; the
+// top_k-th of them is a bound tau that at least top_k logits reach and, for rows in no particular order,
+// only about top_k do (128 groups of which top_k hold a larger logit: 10 for top_k = 10, 37 for 32).  Only
+// groups whose maximum reaches tau can hold such a logit, so at most top_k groups' worth are collected
+// whatever the row looks like; their threads read their vectors again.  The collected keys are ranked
+// together with the list of the segments before by counting.
+// (Inserting logit by logit into warp lists, with a ballot and shuffles each, took 47 us per launch on
+// 24 x 3 rows of 128256 logits and 65 us on ten rows of 32000 with top_k = 32.)
 // Keys are 64-bit words whose unsigned order is "larger logit, then lower token", so exact ties go to
-// the lower token everywhere.  Warp lists meet in shared memory, block lists in a scratch array, and an
-// arrival counter picks the block that finishes a sequence.
+// the lower token everywhere.  Block lists go to a scratch array, and an arrival counter picks the block
+// that finishes a sequence; it merges the lists of a row with one warp, a list per lane.
 #include "common.cuh"
 #include <math_constants.h>
 
@@ -28,6 +37,15 @@ namespace {
 constexpr int FILT_THREADS = 256;
 constexpr int FILT_MAX_CHUNKS = 16;
 constexpr int FILT_MAX_K = 32;
+constexpr int FILT_GROUP = 2;                            // threads per group whose maximum is ranked
+constexpr int FILT_GROUPS = FILT_THREADS / FILT_GROUP;
+constexpr int FILT_U = 4;                                // vectors per thread and sweep
+constexpr int FILT_BUF = 4096;                           // keys a segment may collect
+// A call with at most this many block rows and bytes of logits takes one launch over all block rows (measured,
+// us, two launches / one: 2 MB 22 / 18, 12 MB 28 / 21, 18 MB 36 / 34, 41 MB 39 / 52).
+constexpr int FILT_BOTH_ROWS = 256;
+constexpr int64_t FILT_BOTH_BYTES = 16ll << 20;
+enum { PHASE_TARGETS = 0, PHASE_MASKS = 1, PHASE_BOTH = 2 };
 
 struct FiltParams {
   int B, k, V, n_q, n_chunks, chunk, top_k, phase;
@@ -41,14 +59,16 @@ struct FiltParams {
   const int32_t* draft_tok; const float* draft_prob;      // [B, k, list_stride] or NULL (no lists)
   int32_t* next_draft_tok; float* next_draft_prob;        // [B, k, list_stride]
   int list_stride;
-  unsigned long long* part;            // [B][k+1][FILT_MAX_CHUNKS][32]
+  unsigned long long* part;            // [B][rows of the phase][FILT_MAX_CHUNKS][32]
   int* counter;                        // [B], self-resetting
+  int do_commit;                       // phase 1 / one launch: the accepted cache rows move as well
+  CommitParams cm;
 };
 
 __device__ __forceinline__ float fexp2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
 __device__ __forceinline__ unsigned long long make_key(float v, int idx) {
-  uint32_t u = __float_as_uint(v);
+  uint32_t u = __float_as_uint(v + 0.f);                  // (-0 counts as 0)
   u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
   return ((unsigned long long)u << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)idx);
 }
@@ -58,19 +78,15 @@ __device__ __forceinline__ void split_key(unsigned long long key, float& v, int&
   v = __uint_as_float(u);
   idx = (int)(0xFFFFFFFFu - (uint32_t)key);
 }
-__device__ __forceinline__ unsigned long long shfl64(unsigned long long x, int src) {
-  const uint32_t lo = __shfl_sync(0xFFFFFFFFu, (uint32_t)x, src), hi = __shfl_sync(0xFFFFFFFFu, (uint32_t)(x >> 32), src);
+__device__ __forceinline__ unsigned long long shfl_xor64(unsigned long long x, int o) {
+  const uint32_t lo = __shfl_xor_sync(0xFFFFFFFFu, (uint32_t)x, o), hi = __shfl_xor_sync(0xFFFFFFFFu, (uint32_t)(x >> 32), o);
   return ((unsigned long long)hi << 32) | lo;
 }
-// The warp's list: lane j < K holds the j-th largest key seen so far (0 = empty), lanes >= K hold 0.
-// Inserts x (the same value in every lane) if it beats the K-th key.
-__device__ __forceinline__ void list_insert(unsigned long long& mine, unsigned long long x, int K, int lane) {
-  const int pos = __popc(__ballot_sync(0xFFFFFFFFu, mine > x));
-  const uint32_t lo = __shfl_up_sync(0xFFFFFFFFu, (uint32_t)mine, 1), hi = __shfl_up_sync(0xFFFFFFFFu, (uint32_t)(mine >> 32), 1);
-  if (pos < K) {
-    if (lane == pos) mine = x;
-    else if (lane > pos && lane < K) mine = ((unsigned long long)hi << 32) | lo;
-  }
+// Largest key over the warp, in every lane (keys are distinct, or 0 = none).
+__device__ __forceinline__ unsigned long long warp_max64(unsigned long long x) {
+  const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(x >> 32));
+  const uint32_t lo = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(x >> 32) == hi ? (uint32_t)x : 0u);
+  return ((unsigned long long)hi << 32) | lo;
 }
 
 __device__ __forceinline__ float ld_logit(const float* p) { return *p; }
@@ -86,116 +102,213 @@ __device__ __forceinline__ void unpack16(const uint4& v, float (&f)[8], const __
   for (int i = 0; i < 4; ++i) { f[2 * i] = __uint_as_float(w[i] << 16); f[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u); }
 }
 
-// VECTOR: the row and the chunk start are 16-byte aligned (the launcher checks): every lane fetches four
-// 16-byte pieces per sweep, all in flight together, instead of one logit at a time.
-template <typename T, bool VECTOR>
+struct FiltShared {
+  unsigned long long group_max[FILT_GROUPS];
+  unsigned long long run[2][FILT_MAX_K];                  // sorted top_k so far (two copies: one is read, one written)
+  unsigned long long tau;
+  int count, last, bits, i_star;
+  int ok[SPACE_MAX_K + 1];
+  unsigned long long buf[FILT_BUF];    // collected keys of a segment, later the chunk lists of the rows the last block works on
+};
+static_assert(FILT_BUF >= FILT_MAX_K * FILT_GROUP * FILT_U * 8, "one sweep's keys of the longest list must fit");
+static_assert(FILT_BUF >= (SPACE_MAX_K + 1) * FILT_MAX_CHUNKS * FILT_MAX_K, "the chunk lists of k+1 rows must fit");
+
+// The N logits at x of a row whose chunk ends at `end` (-inf past it).
+template <typename T, bool ALIGNED, int N>
+__device__ __forceinline__ void whole_vector(const Piece2& raw, const T* row, int x, int end, float (&f)[N]) {
+  if (x + N <= end) unpack16(ALIGNED ? raw.a : shift_pieces(raw, row), f, (const T*)nullptr);
+  else
+#pragma unroll
+    for (int i = 0; i < N; ++i) f[i] = x + i < end ? ld_logit(row + x + i) : -CUDART_INF_F;
+}
+template <typename T, bool ALIGNED>
+__device__ __forceinline__ Piece2 request_vector(const T* row, int x, int end) {
+  Piece2 raw;
+  raw.a = raw.b = make_uint4(0, 0, 0, 0);
+  if (x + 16 / (int)sizeof(T) <= end) {
+    if (ALIGNED) raw.a = __ldg(reinterpret_cast<const uint4*>(row + x));
+    else raw = load_pieces(row, x);
+  }
+  return raw;
+}
+
+// Top K of logits [begin, end) of a row as a sorted list in sh.run[returned copy].  ALIGNED: the row is
+// 16-byte aligned (else see load_pieces).
+template <typename T, bool ALIGNED>
+__device__ int chunk_top_k(const T* row, int begin, int end, int K, FiltShared& sh) {
+  constexpr int N = 16 / (int)sizeof(T), U = FILT_U;
+  constexpr int stride = FILT_THREADS * N;
+  const int tid = threadIdx.x;
+  // sweeps per segment: as many as the buffer can hold the collected keys of (K groups' worth)
+  const int sweeps = max(1, FILT_BUF / (K * FILT_GROUP * U * N));
+  int cur = 0;
+  if (tid < FILT_MAX_K) sh.run[0][tid] = 0ull;
+  for (int s0 = begin; s0 < end; s0 += sweeps * U * stride) {
+    const int s1 = min(end, s0 + sweeps * U * stride);
+    // ---- this thread's largest logit of the segment: value and the vector that has it first
+    float m = -CUDART_INF_F;
+    int at = -1;
+    for (int x = s0 + tid * N; x < s1; x += U * stride) {
+      Piece2 raw[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) raw[u] = request_vector<T, ALIGNED>(row, x + u * stride, s1);
+      float vm[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        float a[N];
+        whole_vector<T, ALIGNED, N>(raw[u], row, x + u * stride, s1, a);
+#pragma unroll
+        for (int w = N / 2; w > 0; w >>= 1)
+#pragma unroll
+          for (int i = 0; i < w; ++i) a[i] = fmaxf(a[i], a[i + w]);
+        vm[u] = a[0];
+      }
+      float sm = vm[0];
+#pragma unroll
+      for (int u = 1; u < U; ++u) sm = fmaxf(sm, vm[u]);
+      if (sm > m || at < 0) {
+        m = sm;
+#pragma unroll
+        for (int u = U - 1; u >= 0; --u) if (vm[u] == sm) at = x + u * stride;
+      }
+    }
+    unsigned long long mine = 0ull;                       // (0: no logit)
+    if (at >= 0) {
+      float f[N];
+      whole_vector<T, ALIGNED, N>(request_vector<T, ALIGNED>(row, at, s1), row, at, s1, f);
+      int off = 0;
+#pragma unroll
+      for (int i = N - 1; i >= 0; --i) if (f[i] == m) off = i;
+      mine = make_key(m, at + off);
+    }
+    unsigned long long g = mine;
+#pragma unroll
+    for (int o = 1; o < FILT_GROUP; o <<= 1) { const unsigned long long other = shfl_xor64(g, o); g = other > g ? other : g; }
+    if ((tid & (FILT_GROUP - 1)) == 0) sh.group_max[tid / FILT_GROUP] = g;
+    if (tid == 0) { sh.count = 0; sh.tau = 1ull; }        // fewer than K groups with a logit: take them all
+    // (the K-th key of the list so far: a later segment's logit counts only if it is larger)
+    const unsigned long long kth = s0 == begin ? 0ull : sh.run[cur][K - 1];
+    if (!__syncthreads_or(mine > kth)) continue;
+    // ---- tau: the K-th largest group maximum
+    if (tid < FILT_GROUPS) {
+      const unsigned long long x = sh.group_max[tid];
+      int above = 0;
+#pragma unroll 16
+      for (int j = 0; j < FILT_GROUPS; ++j) above += sh.group_max[j] > x;
+      if (x != 0ull && above == K - 1) sh.tau = x;
+    }
+    __syncthreads();
+    const unsigned long long tau = sh.tau > kth ? sh.tau : kth;
+    // ---- collect the logits that reach it: the few threads that hold one look at their vectors again (L1, L2)
+    if (mine >= tau) {
+      float tv; int ti;
+      split_key(tau, tv, ti);
+      for (int x = s0 + tid * N; x < s1; x += U * stride) {
+        Piece2 raw[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) raw[u] = request_vector<T, ALIGNED>(row, x + u * stride, s1);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          float f[N];
+          whole_vector<T, ALIGNED, N>(raw[u], row, x + u * stride, s1, f);
+#pragma unroll
+          for (int i = 0; i < N; ++i) {
+            const int xi = x + u * stride + i;
+            if (!(f[i] < tv) && xi < s1) {
+              const unsigned long long key = make_key(f[i], xi);
+              if (key >= tau) sh.buf[atomicAdd(&sh.count, 1)] = key;
+            }
+          }
+        }
+      }
+    }
+    if (tid < FILT_MAX_K) sh.run[cur ^ 1][tid] = 0ull;
+    __syncthreads();
+    // ---- rank them together with the list so far
+    const int n = sh.count, total = n + (s0 == begin ? 0 : K);
+    for (int i = tid; i < total; i += FILT_THREADS) {
+      const unsigned long long x = i < n ? sh.buf[i] : sh.run[cur][i - n];
+      int rank = 0;
+      for (int j = 0; j < n; ++j) rank += sh.buf[j] > x;
+      if (s0 != begin)
+        for (int j = 0; j < K; ++j) rank += sh.run[cur][j] > x;
+      if (x != 0ull && rank < K) sh.run[cur ^ 1][rank] = x;
+    }
+    cur ^= 1;
+    __syncthreads();
+  }
+  return cur;
+}
+
+// Sorted top K of a row from its chunks' sorted lists in shared memory (lists[c * 32 + j]), lane j
+// holding the j-th largest: every lane stands for one list, K rounds of a warp-wide maximum.
+__device__ __forceinline__ unsigned long long merge_lists(const unsigned long long* lists, int n_chunks, int K, int lane) {
+  unsigned long long mine = 0ull;
+  int at = 0;
+  unsigned long long head = lane < n_chunks ? lists[lane * FILT_MAX_K] : 0ull;
+  for (int j = 0; j < K; ++j) {
+    const unsigned long long best = warp_max64(head);
+    if (best == 0ull) break;                                // (the same in every lane)
+    if (lane == j) mine = best;
+    if (head == best) { ++at; head = at < K ? lists[lane * FILT_MAX_K + at] : 0ull; }
+  }
+  return mine;
+}
+
+template <typename T, bool ALIGNED>
 __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltParams p) {
+  __shared__ FiltShared sh;
   pdl_launch_dependents();
   pdl_wait();
   const int b = blockIdx.z, r = blockIdx.y, ch = blockIdx.x;
   const int k1 = p.k + 1, K = p.top_k;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_rows = p.phase == 0 ? k1 : p.k;
-  const int i_star0 = p.phase == 0 ? 0 : max(0, min(p.n_accept[b], p.k));
-  const int brow = p.phase == 0 ? r * k1 : i_star0 * k1 + r + 1;          // target row r, or mask row (i*, r+1)
+  const int n_rows = gridDim.y;
+  const int i_star0 = p.phase == PHASE_MASKS ? max(0, min(p.n_accept[b], p.k)) : 0;
+  // target row r, mask row (i*, r+1), or block row r
+  const int brow = p.phase == PHASE_TARGETS ? r * k1 : p.phase == PHASE_MASKS ? i_star0 * k1 + r + 1 : r;
   const T* row = reinterpret_cast<const T*>(p.logits) + ((int64_t)b * p.n_q + brow) * p.row_stride;
   const int begin = ch * p.chunk, end = min(p.V, begin + p.chunk);
-
-  // ---- this warp's top-K of its share of the chunk ------------------------------------
-  unsigned long long mine = 0ull;
-  int scalar_from = begin;                                  // what the one-by-one loop below still has to look at
-  if (VECTOR) {
-    constexpr int N = 16 / (int)sizeof(T), U = 4;
-    const int full_end = begin + ((end - begin) / N) * N;
-    constexpr int stride = FILT_THREADS * N;
-    unsigned long long tau = 0ull;                          // the warp's K-th key so far (0: fewer than K keys)
-    for (int xw = begin + warp * 32 * N; xw < full_end; xw += U * stride) {   // (the same trip count in every lane)
-      uint4 v[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int x = xw + lane * N + u * stride;
-        v[u] = x < full_end ? __ldg(reinterpret_cast<const uint4*>(row + x)) : make_uint4(0, 0, 0, 0);
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int x = xw + lane * N + u * stride;
-        float f[N];
-        unpack16(v[u], f, (const T*)nullptr);
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-          const unsigned long long key = x < full_end ? make_key(f[i], x + i) : 0ull;
-          unsigned pass = __ballot_sync(0xFFFFFFFFu, key > tau);
-          while (pass) {
-            const int src = __ffs(pass) - 1;
-            pass &= pass - 1;
-            list_insert(mine, shfl64(key, src), K, lane);
-            tau = shfl64(mine, K - 1);
-          }
-        }
-      }
-    }
-    scalar_from = full_end;                                 // (fewer than N logits, looked at by every warp: keys are unique, a
-  }                                                         //  second look at one changes nothing -- but only warp 0 does it)
-  for (int x0 = scalar_from + (VECTOR ? 0 : warp * 32); x0 < end && (!VECTOR || warp == 0); x0 += VECTOR ? 32 : FILT_THREADS) {
-    const int x = x0 + lane;
-    const unsigned long long key = x < end ? make_key(ld_logit(row + x), x) : 0ull;
-    const unsigned long long tau = shfl64(mine, K - 1);
-    unsigned pass = __ballot_sync(0xFFFFFFFFu, key > tau);
-    while (pass) {
-      const int src = __ffs(pass) - 1;
-      pass &= pass - 1;
-      list_insert(mine, shfl64(key, src), K, lane);
-    }
+  int Lc = 0;
+  if (p.do_commit) {                                        // (phase 1: i* is known, every block moves its slice)
+    Lc = p.cm.kv_len[b];
+    if (p.phase == PHASE_MASKS && commit_fits(p.cm, Lc))
+      commit_rows_any(p.cm, b, Lc, i_star0, r * p.n_chunks + ch, n_rows * p.n_chunks, threadIdx.x, FILT_THREADS);
   }
-  // ---- block list: warp 0 merges the eight warp lists ----------------------------------
-  __shared__ unsigned long long sh_list[FILT_THREADS / 32][32];
-  sh_list[warp][lane] = mine;
-  __syncthreads();
-  unsigned long long* part = p.part + (((int64_t)b * k1 + r) * FILT_MAX_CHUNKS) * 32;
+  const int cur = chunk_top_k<T, ALIGNED>(row, begin, end, K, sh);
+  unsigned long long* part = p.part + (int64_t)b * n_rows * FILT_MAX_CHUNKS * FILT_MAX_K;
+  // ---- the chunk's list, then arrival: the last block of the sequence finishes it (warp 0 publishes and counts)
   if (warp == 0) {
-    for (int w = 1; w < FILT_THREADS / 32; ++w) {
-      const unsigned long long other = sh_list[w][lane];
-      for (int j = 0; j < K; ++j) {
-        const unsigned long long x = shfl64(other, j);
-        if (x == 0ull) break;                               // (uniform: x is the same in every lane)
-        list_insert(mine, x, K, lane);
-      }
+    if (lane < K) __stcg(part + ((int64_t)r * FILT_MAX_CHUNKS + ch) * FILT_MAX_K + lane, sh.run[cur][lane]);
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) {
+      const int prev = atomicAdd(p.counter + b, 1);
+      sh.last = prev == n_rows * p.n_chunks - 1;
+      if (sh.last) p.counter[b] = 0;
+      sh.bits = 0;
     }
-    *reinterpret_cast<volatile unsigned long long*>(part + ch * 32 + lane) = mine;
   }
-  // ---- arrival: the last block of the sequence finishes it -------------------------------
-  __shared__ int sh_last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int prev = atomicAdd(p.counter + b, 1);
-    sh_last = prev == n_rows * p.n_chunks - 1;
-    if (sh_last) p.counter[b] = 0;
-  }
-  __syncthreads();
-  if (!sh_last) return;
+  __syncthreads();                                          // (also: every thread's read of the old length precedes the arrival)
+  if (!sh.last) return;
   __threadfence();
 
-  // ---- last block: warp w builds the filtered distribution of row w ----------------------
-  __shared__ int sh_ok[SPACE_MAX_K + 1];
-  __shared__ int sh_bits;
-  if (threadIdx.x == 0) sh_bits = 0;
   const bool with_lists = p.resample == SPACE_RESAMPLE_RESIDUAL_DRAFT;
   const bool literal = p.resample == SPACE_RESAMPLE_PAPER_LITERAL || with_lists;   // candidates are sampled
   const uint32_t seq = p.seq_id ? p.seq_id[b] : (uint32_t)b;
   const int L = p.kv_len ? p.kv_len[b] : 0;
   float z = 0.f, q = 0.f; int idx = -1; bool keep = false;
-  if (warp < n_rows) {
-    unsigned long long lst = 0ull;
-    const unsigned long long* pr = p.part + (((int64_t)b * k1 + warp) * FILT_MAX_CHUNKS) * 32;
-    for (int c = 0; c < p.n_chunks; ++c) {
-      const unsigned long long other = __ldcg(pr + c * 32 + lane);
-      for (int j = 0; j < K; ++j) {
-        const unsigned long long x = shfl64(other, j);
-        if (x == 0ull) break;
-        list_insert(lst, x, K, lane);
-      }
+  // ---- filtered distribution of row list_row(w) by warp w < count
+  auto build = [&](int count, int first, int step) {
+    for (int i = threadIdx.x; i < count * p.n_chunks * FILT_MAX_K; i += FILT_THREADS) {
+      const int j = i % FILT_MAX_K, c = (i / FILT_MAX_K) % p.n_chunks, w = i / (FILT_MAX_K * p.n_chunks);
+      if (j < K) sh.buf[(w * FILT_MAX_CHUNKS + c) * FILT_MAX_K + j] =
+          __ldcg(part + ((int64_t)(first + w * step) * FILT_MAX_CHUNKS + c) * FILT_MAX_K + j);
     }
+    __syncthreads();
+    z = 0.f; q = 0.f; idx = -1; keep = false;
+    if (warp >= count) return;
+    const unsigned long long lst = merge_lists(sh.buf + warp * FILT_MAX_CHUNKS * FILT_MAX_K, p.n_chunks, K, lane);
     const bool valid = lst != 0ull;
     if (valid) split_key(lst, z, idx);
     // temperature, then softmax over the top-k, then the shortest prefix that reaches top_p
@@ -219,10 +332,11 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) ksum += __shfl_xor_sync(0xFFFFFFFFu, ksum, o);
     q = keep ? pj / ksum : 0.f;
-  }
-  __syncthreads();                                          // sh_bits is zero for everyone
+  };
 
-  if (p.phase == 0) {
+  int i_star = i_star0;
+  if (p.phase != PHASE_MASKS) {
+    build(k1, 0, p.phase == PHASE_BOTH ? k1 : 1);
     // acceptance test of candidate c_{t+1} against the filtered law of target row t (warp t)
     if (warp < p.k) {
       const int c = p.cand[b * p.k + warp];
@@ -230,15 +344,14 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
       const unsigned hit = __ballot_sync(0xFFFFFFFFu, keep && idx == c);
       const float qc = hit ? __shfl_sync(0xFFFFFFFFu, q, __ffs(hit) - 1) : 0.f;
       if (lane == 0) {
-        if (!in_range) atomicOr(&sh_bits, SPACE_ST_BAD_CANDIDATE);
+        if (!in_range) atomicOr(&sh.bits, SPACE_ST_BAD_CANDIDATE);
         const Philox4 w = philox4x32_10(0u, PURPOSE_ACCEPT, seq, (uint32_t)(L + warp + 1), p.key0, p.key1);
         const float pc = p.cand_prob[b * p.k + warp];
-        sh_ok[warp] = in_range && pc > 0.f && uniform_open(w.x) * pc <= qc;   // r <= Q'/P_c  <=>  r P_c <= Q'
+        sh.ok[warp] = in_range && pc > 0.f && uniform_open(w.x) * pc <= qc;   // r <= Q'/P_c  <=>  r P_c <= Q'
       }
     }
     __syncthreads();
-    int i_star = 0;
-    while (i_star < p.k && sh_ok[i_star]) ++i_star;
+    while (i_star < p.k && sh.ok[i_star]) ++i_star;
     if (warp == i_star) {
       // extra token: Gumbel arg-max over the kept tokens of row i*, the rejected point-mass candidate left out
       int exclude = -1;
@@ -289,10 +402,20 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
         p.n_accept[b] = i_star;
         p.n_out[b] = n_out;
         p.finished[b] = (uint8_t)(eos_mask != 0);
-        if (p.status && sh_bits) atomicOr(p.status + b, sh_bits);
+        if (p.status && sh.bits) atomicOr(p.status + b, sh.bits);
       }
     }
-  } else if (warp < p.k) {
+  }
+  if (p.phase == PHASE_TARGETS) return;
+  // (one launch: the whole move falls to this block, i* has only just become known)
+  if (p.do_commit && p.phase == PHASE_BOTH && commit_fits(p.cm, Lc))
+    commit_rows_any(p.cm, b, Lc, i_star, 0, 1, threadIdx.x, FILT_THREADS);
+  __syncthreads();                                          // the list buffer is free again
+  if (p.phase == PHASE_BOTH) build(p.k, i_star * k1 + 1, 1);
+  else build(p.k, 0, 1);
+  // every thread of the sequence's blocks has read the old length by now
+  if (p.do_commit && threadIdx.x == 0) commit_tables(p.cm, b, Lc, i_star, commit_fits(p.cm, Lc));
+  if (warp < p.k) {
     // next candidate o = warp + 1 from mask row (i*, o)
     int tok; float pr;
     if (!literal) {                                         // point-mass draft: the row's arg-max, P_c = 1
@@ -300,7 +423,7 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
     } else {
       float sc = -CUDART_INF_F;
       if (keep) {
-        const Philox4 ph = philox4x32_10((uint32_t)(idx >> 2), PURPOSE_DRAFT, seq, (uint32_t)(L + i_star0 + 1 + warp + 1),
+        const Philox4 ph = philox4x32_10((uint32_t)(idx >> 2), PURPOSE_DRAFT, seq, (uint32_t)(L + i_star + 1 + warp + 1),
                                          p.key0, p.key1);
         const uint32_t w4[4] = {ph.x, ph.y, ph.z, ph.w};
         sc = fmaf(z, p.c_t, gumbel2_from_uniform(uniform_open(w4[idx & 3])));
@@ -325,11 +448,14 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
 
 }  // namespace
 
+// lists of the k+1 target rows of every sequence, or of all block rows of a small batch
 size_t verify_filter_scratch_bytes(int max_batch, int k_max) {
-  return (size_t)max_batch * (k_max + 1) * FILT_MAX_CHUNKS * 32 * sizeof(unsigned long long);
+  const int rows = max_batch * (k_max + 1);
+  return (size_t)(rows > FILT_BOTH_ROWS ? rows : FILT_BOTH_ROWS) * FILT_MAX_CHUNKS * FILT_MAX_K * sizeof(unsigned long long);
 }
 
-int launch_verify_filtered(space_ctx* ctx, const space_verify_args* a, cudaStream_t st) {
+// cm != nullptr: the commit rides along
+int launch_verify_filtered(space_ctx* ctx, const space_verify_args* a, const space_commit_args* cm, cudaStream_t st) {
   if (a->top_k < 1 || a->top_k > FILT_MAX_K || !(a->top_p > 0.f) || a->top_p > 1.f) return SPACE_E_INVALID_ARG;
   FiltParams p;
   memset(&p, 0, sizeof(p));
@@ -345,30 +471,30 @@ int launch_verify_filtered(space_ctx* ctx, const space_verify_args* a, cudaStrea
   p.draft_tok = a->draft_tok; p.draft_prob = a->draft_prob;
   p.next_draft_tok = a->next_draft_tok; p.next_draft_prob = a->next_draft_prob; p.list_stride = a->top_k;
   p.part = reinterpret_cast<unsigned long long*>(ctx->vtopk);
-  // about two blocks per SM over the (k+1) rows of every sequence, at least 8192 logits per block
-  const int rows = a->batch * (a->k + 1);
-  int nc = (2 * ctx->sm_count + rows - 1) / rows;   // (4, 8, 16 per SM measured slower: every block starts from an empty list)
-  const int max_nc = (a->vocab + 8191) / 8192;
-  if (nc > max_nc) nc = max_nc;
-  if (nc > FILT_MAX_CHUNKS) nc = FILT_MAX_CHUNKS;
-  if (nc < 1) nc = 1;
-  p.chunk = (((a->vocab + nc - 1) / nc + 7) / 8) * 8;       // chunk starts stay 16-byte aligned
-  p.n_chunks = (a->vocab + p.chunk - 1) / p.chunk;
   const int esz = a->logits_dtype == SPACE_DTYPE_F32 ? 4 : 2;
-  const bool vector = ((uintptr_t)a->logits % 16 == 0) && ((a->logits_row_stride * esz) % 16 == 0);
-  for (int phase = 0; phase < 2; ++phase) {
+  const bool aligned = ((uintptr_t)a->logits % 16 == 0) && ((a->logits_row_stride * esz) % 16 == 0);
+  if (cm) fill_commit_params(ctx, cm, &p.cm);
+  const bool both = (int64_t)a->batch * p.n_q <= FILT_BOTH_ROWS && (int64_t)a->batch * p.n_q * a->vocab * esz <= FILT_BOTH_BYTES;
+  // the commit rides along, except where one block would have more than 32 KB of rows to move (a launch of
+  // its own, about 2 us, is faster then)
+  const bool carry = cm && !(both && (int64_t)a->k * p.cm.H_kv * p.cm.d * 4 > (32 << 10));
+  for (int phase = both ? PHASE_BOTH : PHASE_TARGETS; phase <= (both ? PHASE_BOTH : PHASE_MASKS); ++phase) {
     p.phase = phase;
-    p.counter = ctx->counters + (phase == 0 ? 0 : ctx->cfg.max_batch);
-    const dim3 grid(p.n_chunks, phase == 0 ? a->k + 1 : a->k, a->batch);
-    ProfScope ps(ctx, phase == 0 ? SPACE_K_VERIFY_TARGET : SPACE_K_VERIFY_EMIT, st);
+    p.do_commit = carry && phase != PHASE_TARGETS;
+    p.counter = ctx->counters + (phase == PHASE_MASKS ? ctx->cfg.max_batch : 0);
+    const int rows = phase == PHASE_TARGETS ? a->k + 1 : phase == PHASE_MASKS ? a->k : p.n_q;
+    p.n_chunks = row_chunks(a->vocab, a->batch * rows, 16 / esz, ctx->sm_count, FILT_MAX_CHUNKS, &p.chunk);
+    const dim3 grid(p.n_chunks, rows, a->batch);
+    ProfScope ps(ctx, phase == PHASE_MASKS ? SPACE_K_VERIFY_EMIT : SPACE_K_VERIFY_TARGET, st);
     if (a->logits_dtype == SPACE_DTYPE_F32) {
-      if (vector) launch_pdl(verify_filter_kernel<float, true>, grid, dim3(FILT_THREADS), 0, st, p);
+      if (aligned) launch_pdl(verify_filter_kernel<float, true>, grid, dim3(FILT_THREADS), 0, st, p);
       else launch_pdl(verify_filter_kernel<float, false>, grid, dim3(FILT_THREADS), 0, st, p);
     } else {
-      if (vector) launch_pdl(verify_filter_kernel<__nv_bfloat16, true>, grid, dim3(FILT_THREADS), 0, st, p);
+      if (aligned) launch_pdl(verify_filter_kernel<__nv_bfloat16, true>, grid, dim3(FILT_THREADS), 0, st, p);
       else launch_pdl(verify_filter_kernel<__nv_bfloat16, false>, grid, dim3(FILT_THREADS), 0, st, p);
     }
+    ctx->launches += 1;
   }
-  ctx->launches += 2;
+  if (cm && !carry) return launch_commit(ctx, cm, st);
   return cuda_ok(cudaGetLastError());
 }
