@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
     // nothing was issued; fall through to the teardown
   } else if (warp == WARP_K || warp == WARP_V) {
     // ================= K / V producers ====================================
-    if (lane == 0) {
+    if (elect_one()) {
       const bool is_k = warp == WARP_K;
       const int n_st = is_k ? S::K_STAGES : S::V_STAGES;
       const int b_full = is_k ? B_KFULL : B_VFULL, b_empty = is_k ? B_KEMPTY : B_VEMPTY;
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
     }
   } else if (warp == WARP_MMA) {
     // ================= S issuer ============================================
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t IDESC_QK = instr_desc(TILE_N, 0);
       uint32_t gt = 0, seg = 0;
       bool ok = true;
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
     // ================= O issuer ============================================
     // A thread of its own: the S products of later tiles need not queue behind
     // the sixteen instructions of an O product or wait for its operands.
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t IDESC_PV = instr_desc(DH, 1);
       uint32_t g = 0;
       bool ok = true;

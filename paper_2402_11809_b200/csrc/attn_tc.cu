@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     // nothing was issued; fall through to the teardown
   } else if (warp == WARP_K || warp == WARP_V) {
     // ================= K / V producers ====================================
-    if (lane == 0) {
+    if (elect_one()) {
       const bool is_k = warp == WARP_K;
       const int n_st = is_k ? S::K_STAGES : S::V_STAGES;
       const int b_full = is_k ? B_KFULL : B_VFULL, b_empty = is_k ? B_KEMPTY : B_VEMPTY;
@@ -691,7 +691,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     }
   } else if (warp == WARP_MMA) {
     // ================= S^T issuer ==========================================
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc_qk = instr_desc_rt(n_pad, 0, 0);   // A = K tile (K-major), B = Q (K-major)
       // descriptors of the first stage of every operand; a later stage or k-step
       // only adds to the 14-bit address field (16-byte units, no carry possible)
@@ -742,7 +742,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     // ================= O^T issuer ===========================================
     // A thread of its own: the S^T products of the next tile need not queue
     // behind the sixteen instructions of this one.
-    if (lane == 0) {
+    if (elect_one()) {
       // B = [P_hi | P_lo]: the two 64-column blocks lie one leading-dimension stride
       // apart, so a single product of N = 128 gives O_hi^T in columns 0..63 and
       // O_lo^T in columns 64..127 (an instruction costs the same at every N here);

@@ -29,6 +29,19 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
+// True in one lane of the (converged) warp.  The roles that issue tensor-core products and TMA requests pick
+// their thread with this, not with a comparison of the lane number: the compiler knows that one thread is left
+// then and keeps the descriptors in uniform registers.  Picked by lane number every operand of every
+// instruction is moved there first; measured, cycles per M = 128, K = 16 product in a row, by lane / elected:
+// both operands in shared memory N = 32 108 / 59, N = 64 108 / 75, N = 128 108 / 107, N = 224 155 / 155
+// (43 + N/2), first operand in TMEM N = 128 108 / 74 (10 + N/2).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.b32 %0, 1, 0, q;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
