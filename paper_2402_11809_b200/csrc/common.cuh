@@ -148,6 +148,7 @@ struct space_ctx {
   char* vtopk;             // filtered sampling: top-k lists per (sequence, row, chunk)
   int32_t* scratch_status; // [max_batch] used when the caller passes no status array
   char* lm_part;           // output-projection statistics [256 block rows][sm_count] x 16 bytes
+  char* lm_gather;         // gathered mask rows of the projection's second phase
   int* lm_counter;         // {arrival counter, first timeout site}
   // staging for space_step_host
   char* stage;
@@ -282,6 +283,7 @@ int launch_verify_noalloc(const space_verify_args* a, cudaStream_t st);
 int launch_commit(space_ctx* ctx, const space_commit_args* a, cudaStream_t st);
 int launch_lmhead_verify(space_ctx* ctx, const space_lmhead_args* a, cudaStream_t st);
 size_t lmhead_partial_bytes(int sm_count);
+size_t lmhead_gather_bytes();
 int launch_attn_simt(space_ctx* ctx, const space_attn_args* a, const uint64_t* mask_rows,
                      cudaStream_t st);
 int launch_attn_tensor(space_ctx* ctx, const space_attn_args* a, const uint64_t* mask_rows,

@@ -40,8 +40,13 @@ constexpr int LM_M = 128;                   // block rows per accumulator (MMA M
 constexpr int LM_MAX_BOX = 256;             // vocabulary rows per box (MMA N), at most
 constexpr int LM_KB = 64;                   // hidden elements per slice (128 bytes: one swizzle row)
 constexpr int LM_MAX_STAGES = 10;
+constexpr int LM_L2_AHEAD = 8;              // slices of W a block asks L2 for before its dependency wait (4: half the gain)
 constexpr float LM_NEG = -3.0e38f;          // "no logit yet": finite, so that differences never give NaN
 constexpr int LM_MAX_N = 256;               // block rows of the whole batch, padded to 16
+// Which block rows a launch projects: all of them, the target rows of every sequence (row b(k+1)+t), or
+// the mask rows of every sequence's group i* (row bk+o-1; i* is the launch before's result).
+enum { LM_ALL = 0, LM_TARGETS = 1, LM_MASKS = 2 };
+constexpr int64_t LM_GATHER_ELEMS = 128 * 8192;   // mask rows gathered for the second phase
 constexpr uint64_t LM_WAIT_NS = 1000000000ull;
 constexpr float LOG2E = 1.4426950408889634f;
 
@@ -51,7 +56,8 @@ struct LmNoisy { float gs, gz; int gidx, pad; };   // best noisy score of a rang
 struct LmParams {
   CUtensorMap tm_w, tm_wt, tm_h;   // W in boxes of n_box rows, W in boxes of tail_rows rows, hidden rows
   int B, k, V, D, n_q;
-  int n_rows;                 // B * n_q
+  int phase;                  // LM_*
+  int n_rows;                 // rows of the launch (B * n_q when it takes all)
   int n_pad;                  // n_rows rounded up to 16: rows of the hidden-state tile
   int n_mt;                   // accumulators of 128 block rows (1 or 2)
   int stages;
@@ -107,16 +113,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
       : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-
-// Statistics of a set of logits: (m, s, i) = (max, sum of exp(z - m), lowest arg-max);
-// the empty set is (LM_NEG, 0, INT_MAX).  fold: union of two sets.  One of the two
-// exponentials is exp(0), so a single ex2 serves.
-__device__ __forceinline__ void stat_fold(float& m, float& s, int& i, float m2, float s2, int i2) {
-  if (m2 > m || (m2 == m && i2 < i)) i = i2;
-  const float e = fast_exp2(-fabsf(m - m2) * LOG2E);
-  s = (m >= m2) ? fmaf(s2, e, s) : fmaf(s, e, s2);
-  m = fmaxf(m, m2);
-}
 
 // (maximum, lowest token) of a row as one 64-bit key whose unsigned order is "larger logit
 // first, then lower token": the ranges of all thread blocks combine with one atomicMax each.
@@ -220,17 +216,29 @@ __device__ __forceinline__ void fold16_noisy(float& m, float& s, int& idx, RowNo
   }
 }
 
-// Per-row constants of the sampling mode: block row `row` of the batch is row i = row mod n_q of
-// sequence b; target rows (i = t(k+1)) score candidate c_{t+1} and draw the extra token of the
+// Row `row` of a launch: target row t (o = 0) or mask row (t, o) of sequence b.  False: padding.
+__device__ __forceinline__ bool row_place(const LmParams& p, int row, int& b, int& t, int& o) {
+  if (row >= p.n_rows) return false;
+  const int k1 = p.k + 1;
+  if (p.phase == LM_ALL) {
+    b = row / p.n_q;
+    const int i = row - b * p.n_q;
+    t = i / k1; o = i - t * k1;
+    return true;
+  }
+  if (p.phase == LM_TARGETS) { b = row / k1; t = row - b * k1; o = 0; return true; }
+  b = row / p.k; o = row - b * p.k + 1; t = p.n_accept[b];
+  return true;
+}
+
+// Per-row constants of the sampling mode; target rows score candidate c_{t+1} and draw the extra token of the
 // case i* = t at position L+t+1; mask rows (t, o) draw candidate o of that case at position
 // L+t+1+o when candidates are sampled (Algorithm 1 as printed).
 __device__ __forceinline__ void row_noisy_init(RowNoisy& r, const LmParams& p, int row) {
   r.gs = -CUDART_INF_F; r.gz = 0.f; r.gidx = 0x7FFFFFFF; r.zc = LM_NEG;
   r.cand_tok = -1; r.exclude = -1; r.purpose = 0; r.seq = 0; r.pos = 0; r.noisy = false;
-  if (row >= p.n_rows) return;
-  const int k1 = p.k + 1;
-  const int b = row / p.n_q, i = row - b * p.n_q;
-  const int t = i / k1, o = i - t * k1;
+  int b, t, o;
+  if (!row_place(p, row, b, t, o)) return;
   const bool literal = p.resample == SPACE_RESAMPLE_PAPER_LITERAL;
   r.seq = p.seq_id ? p.seq_id[b] : p.seq_base + (uint32_t)b;
   const int L = p.kv_len ? p.kv_len[b] : 0;
@@ -245,15 +253,6 @@ __device__ __forceinline__ void row_noisy_init(RowNoisy& r, const LmParams& p, i
   }
 }
 
-// (max, lowest arg-max) over the warp, result in every lane
-__device__ __forceinline__ void warp_max_idx(float& m, int& idx) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    const float om = __shfl_xor_sync(0xFFFFFFFFu, m, off);
-    const int oi = __shfl_xor_sync(0xFFFFFFFFu, idx, off);
-    if (om > m || (om == m && oi < idx)) { m = om; idx = oi; }
-  }
-}
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, off);
@@ -318,6 +317,15 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.tm_wt) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.tm_h) : "memory");
   }
+  if (warp == 0 && lane == 0) {
+    // With a programmatic launch the block is resident before its dependency wait returns: ask L2 for its
+    // first slices of W meanwhile (a request to the point of coherence, so whatever the kernel before still
+    // writes is what the loads will see).  57.2 -> 55.8 us per call on V = 32000, D = 4096, 36 rows.
+    const int first = (int)(((long long)p.V * blockIdx.x) / gridDim.x) & ~15;
+    const uint64_t pol = l2_evict_first_policy();
+    for (int kb = 0; kb < min(LM_L2_AHEAD, (p.D + LM_KB - 1) / LM_KB); ++kb)
+      tma_prefetch_l2_4d(&p.tm_w, kb * LM_KB, first, 0, 0, pol);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -337,33 +345,29 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
 
   if (warp == 0) {
     // ================= producer ==============================================
-    if (lane == 0) {
-      const int ipb = (KB + kbs - 1) / kbs;                // stages per box
-      const uint32_t n_it = (uint32_t)(nb * ipb);
+    if (elect_one()) {
       bool ok = !*abort_flag;
-      // stage `it`: the W tiles and the hidden tiles of its slices
-      auto issue = [&](uint32_t it) {
-        const int box = (int)it / ipb, kb0 = ((int)it - box * ipb) * kbs;
-        const int s = it % S;
-        const int nk = min(kbs, KB - kb0);
+      // (the ring's place is kept as a stage and a phase bit: divisions by the run-time stage count took
+      // longer than the requests they were for, on the one thread every stage waits for)
+      uint32_t it = 0, s = 0, empty_phase = 1;               // the first pass over the ring finds it free
+      for (int box = 0; box < nb && ok; ++box) {
         const int row0 = r0 + box * p.n_box;
-        const bool tail = r1 - row0 <= p.tail_rows;        // the remaining rows fit the small box
-        const uint32_t st_base = sm_base + (uint32_t)s * L.stage_bytes;
+        const bool tail = r1 - row0 <= p.tail_rows;          // the remaining rows fit the small box
         const CUtensorMap* tm = tail ? &p.tm_wt : &p.tm_w;
-        const uint32_t w_bytes = (uint32_t)(tail ? p.tail_rows : p.n_box) * LM_KB * 2;
-        mbar_expect_tx(LBAR(B_FULL + s), (uint32_t)nk * (w_bytes + L.a_bytes));
-        for (int j = 0; j < nk; ++j)
-          tma_load_4d(st_base + L.b_in_stage + (uint32_t)j * L.b_bytes, tm, LBAR(B_FULL + s), (kb0 + j) * LM_KB, row0, 0, 0);
-        for (int j = 0; j < nk; ++j)
-          tma_load_4d(st_base + (uint32_t)j * L.a_bytes, &p.tm_h, LBAR(B_FULL + s), (kb0 + j) * LM_KB, 0, 0, 0);
-      };
-      // (requesting the first stages' W tiles before the dependency wait, so that they stream under the
-      // previous kernel's tail, measured 0.8 us slower per step in graph replay and was left out)
-      uint32_t it = 0;
-      for (; it < n_it && ok; ++it) {
-        if (it >= (uint32_t)S) ok = mbar_wait(LBAR(B_EMPTY + it % S), ((it / S) - 1) & 1, abort_flag, p.err, 1);
-        if (!ok) break;
-        issue(it);
+        const uint32_t slice_bytes = (uint32_t)(tail ? p.tail_rows : p.n_box) * LM_KB * 2 + L.a_bytes;
+        for (int kb0 = 0; kb0 < KB; kb0 += kbs, ++it) {
+          // stage `it`: the W tiles and the hidden tiles of its slices
+          if (it >= (uint32_t)S) ok = mbar_wait(LBAR(B_EMPTY + s), empty_phase, abort_flag, p.err, 1);
+          if (!ok) break;
+          const int nk = min(kbs, KB - kb0);
+          const uint32_t st_base = sm_base + s * L.stage_bytes;
+          mbar_expect_tx(LBAR(B_FULL + s), (uint32_t)nk * slice_bytes);
+          for (int j = 0; j < nk; ++j)
+            tma_load_4d(st_base + L.b_in_stage + (uint32_t)j * L.b_bytes, tm, LBAR(B_FULL + s), (kb0 + j) * LM_KB, row0, 0, 0);
+          for (int j = 0; j < nk; ++j)
+            tma_load_4d(st_base + (uint32_t)j * L.a_bytes, &p.tm_h, LBAR(B_FULL + s), (kb0 + j) * LM_KB, 0, 0, 0);
+          if (++s == (uint32_t)S) { s = 0; empty_phase ^= 1; }
+        }
       }
       if (!ok) {
         // copies already requested still land: wait for them (bounded) before the block exits
@@ -373,24 +377,24 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
     }
   } else if (warp == 1) {
     // ================= MMA issuer =============================================
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t desc0 = smem_desc_k128(sm_base);
-      uint32_t it = 0;
+      uint32_t s = 0, full_phase = 0;
+      int buf = 0;
       bool ok = !*abort_flag;
       for (int box = 0; box < nb && ok; ++box) {
-        const int buf = box % n_bufs;
         const int row0 = r0 + box * p.n_box;
         const uint32_t idesc = instr_desc((r1 - row0 <= p.tail_rows) ? p.tail_rows : p.n_box);
-        if (box >= n_bufs) ok = mbar_wait(LBAR(B_ACCEMPTY + buf), ((box / n_bufs) - 1) & 1, abort_flag, p.err, 2);
+        // (the buffer's user before this one: box - n_bufs)
+        if (box >= n_bufs) ok = mbar_wait(LBAR(B_ACCEMPTY + buf), (n_bufs == 2 ? (box >> 1) - 1 : box - 1) & 1, abort_flag, p.err, 2);
         if (!ok) break;
         tc_fence_after();
-        for (int kb0 = 0; kb0 < KB; kb0 += kbs, ++it) {
-          const int s = it % S;
+        for (int kb0 = 0; kb0 < KB; kb0 += kbs) {
           const int nk = min(kbs, KB - kb0);
-          ok = mbar_wait(LBAR(B_FULL + s), (it / S) & 1, abort_flag, p.err, 3);
+          ok = mbar_wait(LBAR(B_FULL + s), full_phase, abort_flag, p.err, 3);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t st_off = (uint32_t)s * L.stage_bytes;
+          const uint32_t st_off = s * L.stage_bytes;
           for (int j = 0; j < nk; ++j) {
             const uint64_t wd = desc0 + (uint64_t)((st_off + L.b_in_stage + (uint32_t)j * L.b_bytes) >> 4);
             for (int mt = 0; mt < p.n_mt; ++mt) {
@@ -403,8 +407,10 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
             }
           }
           tc_commit(LBAR(B_EMPTY + s));
+          if (++s == (uint32_t)S) { s = 0; full_phase ^= 1; }
         }
         if (ok) tc_commit(LBAR(B_ACCFULL + buf));
+        buf = n_bufs == 2 ? buf ^ 1 : 0;
       }
     }
   } else {
@@ -423,8 +429,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
     const bool warp_a = quarter * 32 < p.n_rows, warp_b = p.n_mt == 2 && LM_M + quarter * 32 < p.n_rows;
     bool ok = true;
     for (int box = 0; box < nb; ++box) {
-      const int buf = box % n_bufs;
-      ok = ok && mbar_wait(LBAR(B_ACCFULL + buf), (box / n_bufs) & 1, abort_flag, p.err, 4, true);
+      const int buf = n_bufs == 2 ? box & 1 : 0;
+      ok = ok && mbar_wait(LBAR(B_ACCFULL + buf), (n_bufs == 2 ? box >> 1 : box) & 1, abort_flag, p.err, 4, true);
       ok = __all_sync(0xFFFFFFFFu, ok);
       if (!ok) break;
       tc_fence_after();
@@ -491,6 +497,10 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       // only the k mask rows of group i* of every sequence need their sums, so only those rows'
       // per-range partials are read, all of them at once over the 128 threads.
       const int k1 = p.k + 1;
+      // the launch's rows of target t and of mask row (i*, j+1) of sequence b
+      const bool with_targets = p.phase != LM_MASKS, with_masks = p.phase != LM_TARGETS;
+      auto target_row = [&](int b, int t) { return p.phase == LM_ALL ? b * p.n_q + t * k1 : b * k1 + t; };
+      auto mask_row = [&](int b, int i_star, int j) { return p.phase == LM_ALL ? b * p.n_q + i_star * k1 + j + 1 : b * p.k + j; };
       float* row_m = row_s;                                // [n_rows] maxima (row_s is reused: sums come later)
       int* istar = reinterpret_cast<int*>(smem_raw);       // [B] (the pipeline stages are idle now)
       float* terms = reinterpret_cast<float*>(smem_raw) + LM_MAX_N;   // [B * k][G] scaled sums of the ranges
@@ -522,7 +532,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
               if (at < total) {
                 const int g = at % G, bj = at / G;
                 const int b = bj / p.k, jj = bj - b * p.k;
-                const int row = b * p.n_q + (mask_rows ? istar[b] * k1 + jj + 1 : jj * k1);
+                const int row = mask_rows ? mask_row(b, istar[b], jj) : target_row(b, jj);
                 mx[u] = row_m[row];
                 v[u] = __ldcg(reinterpret_cast<const int4*>(p.part + (size_t)row * G + g));
               }
@@ -560,9 +570,9 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           gz_out = gz;
           return gi;
         };
+        if (with_targets) {
         sum_rows(false);                                   // target rows t = 0..k-1 of every sequence
         for (int b = ew; b < p.B; b += 4) {
-          const int* ri = row_i + b * p.n_q;
           const int t = lane;
           const int cv = (t < p.k) ? cand_s[b * p.k + t] : -1;
           const bool in_range = cv >= 0 && cv < p.V;
@@ -571,7 +581,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           const uint32_t seq = p.seq_id ? p.seq_id[b] : p.seq_base + (uint32_t)b;
           const int Lb = p.kv_len ? p.kv_len[b] : 0;
           if (t < p.k && in_range) {
-            const int row = b * p.n_q + t * k1;
+            const int row = target_row(b, t);
             const float zc = __ldcg(p.zc + row);
             const float q = fast_exp2((zc - row_m[row]) * cT) / tsum[b * p.k + t];
             const Philox4 w = philox4x32_10(0u, PURPOSE_ACCEPT, seq, (uint32_t)(Lb + t + 1), p.key0, p.key1);
@@ -581,7 +591,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           const unsigned acc_mask = __ballot_sync(0xFFFFFFFFu, okc);
           const int i_star = __ffs(~acc_mask) - 1;          // first candidate that is not accepted (k when all are)
           float gz_unused;
-          const int bonus = best_noisy(b * p.n_q + i_star * k1, gz_unused);   // a: the draw of the case i* (row i*)
+          const int bonus = best_noisy(target_row(b, i_star), gz_unused);   // a: the draw of the case i* (row i*)
           const int j = lane;
           const int c_j = __shfl_sync(0xFFFFFFFFu, cv, min(j, p.k - 1));
           const int tok = (j < i_star) ? c_j : (j == i_star ? bonus : -1);
@@ -589,10 +599,6 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           const unsigned eos_mask = __ballot_sync(0xFFFFFFFFu, is_eos && j < k1);
           const int n_out = eos_mask ? __ffs(eos_mask) - 1 : i_star + 1;
           if (j < k1) p.out_tokens[b * k1 + j] = (j < n_out) ? tok : -1;
-          if (j < p.k && !literal) {                        // point-mass drafts: arg-max of mask row (i*, j+1), P_c = 1
-            p.next_cand[b * p.k + j] = ri[i_star * k1 + j + 1];
-            p.next_cand_prob[b * p.k + j] = 1.f;
-          }
           if (j == 0) {
             istar[b] = i_star;
             p.n_accept[b] = i_star;
@@ -601,13 +607,22 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
             if (p.status && bad) atomicOr(p.status + b, SPACE_ST_BAD_CANDIDATE);
           }
         }
+        } else {
+          for (int b = et; b < p.B; b += 128) istar[b] = p.n_accept[b];
+        }
         epi_sync();
-        if (literal) {
+        if (with_masks && !literal) {                      // point-mass drafts: arg-max of mask row (i*, j+1), P_c = 1
+          for (int bj = et; bj < p.B * p.k; bj += 128) {
+            const int b = bj / p.k, j = bj - b * p.k;
+            p.next_cand[bj] = row_i[mask_row(b, istar[b], j)];
+            p.next_cand_prob[bj] = 1.f;
+          }
+        } else if (with_masks) {
           // candidates sampled from the mask rows of group i*, with their probabilities
           sum_rows(true);
           for (int bj = ew; bj < p.B * p.k; bj += 4) {
             const int b = bj / p.k, jj = bj - b * p.k;
-            const int row = b * p.n_q + istar[b] * k1 + jj + 1;
+            const int row = mask_row(b, istar[b], jj);
             float gz;
             const int tok = best_noisy(row, gz);
             if (lane == 0) {
@@ -618,22 +633,20 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         }
       } else {
       // acceptance scan and emitted tokens: one warp per sequence
-      for (int b = ew; b < p.B; b += 4) {
-        const int* ri = row_i + b * p.n_q;
+      for (int b = ew; b < p.B && with_targets; b += 4) {
         const int cv = (lane < p.k) ? cand_s[b * p.k + lane] : -1;
         const bool in_range = cv >= 0 && cv < p.V;
         const unsigned bad = __ballot_sync(0xFFFFFFFFu, lane < p.k && !in_range);
-        const bool match = lane < p.k && in_range && cv == ri[lane * k1];
+        const bool match = lane < p.k && in_range && cv == row_i[target_row(b, lane)];
         const unsigned acc_mask = __ballot_sync(0xFFFFFFFFu, match);
         const int i_star = __ffs(~acc_mask) - 1;            // first candidate that does not match (k when all do)
         const int j = lane;
         const int c_j = __shfl_sync(0xFFFFFFFFu, cv, min(j, p.k - 1));
-        const int tok = (j < i_star) ? c_j : (j == i_star ? ri[i_star * k1] : -1);
+        const int tok = (j < i_star) ? c_j : (j == i_star ? row_i[target_row(b, i_star)] : -1);
         const bool is_eos = p.eos_id >= 0 && j <= i_star && tok == p.eos_id;
         const unsigned eos_mask = __ballot_sync(0xFFFFFFFFu, is_eos && j < k1);
         const int n_out = eos_mask ? __ffs(eos_mask) - 1 : i_star + 1;
         if (j < k1) p.out_tokens[b * k1 + j] = (j < n_out) ? tok : -1;
-        if (j < p.k) p.next_cand[b * p.k + j] = ri[i_star * k1 + j + 1];  // mask row (i*, j+1)
         if (j == 0) {
           istar[b] = i_star;
           p.n_accept[b] = i_star;
@@ -642,9 +655,10 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           if (p.status && bad) atomicOr(p.status + b, SPACE_ST_BAD_CANDIDATE);
         }
       }
+      if (!with_targets) for (int b = et; b < p.B; b += 128) istar[b] = p.n_accept[b];
       epi_sync();
       // sums of the mask rows of group i*: (sequence, mask row, range) triples spread over the threads
-      const int total = p.B * p.k * G;
+      const int total = with_masks ? p.B * p.k * G : 0;
       for (int i0 = et; i0 < total; i0 += 128 * 8) {
         int4 v[8]; float mx[8];
 #pragma unroll
@@ -654,7 +668,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           if (at < total) {
             const int g = at % G, bj = at / G;
             const int b = bj / p.k, jj = bj - b * p.k;
-            const int row = b * p.n_q + istar[b] * k1 + jj + 1;
+            const int row = mask_row(b, istar[b], jj);
             mx[u] = row_m[row];
             v[u] = __ldcg(reinterpret_cast<const int4*>(p.part + (size_t)row * G + g));
           }
@@ -667,11 +681,15 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       }
       epi_sync();
       // fixed summation order: the result does not depend on which block came last or on timing
-      for (int bj = ew; bj < p.B * p.k; bj += 4) {
+      for (int bj = ew; bj < p.B * p.k && with_masks; bj += 4) {
         float sv = 0.f;
         for (int g = lane; g < G; g += 32) sv += terms[bj * G + g];
         sv = warp_sum(sv);
-        if (lane == 0) p.next_cand_prob[bj] = 1.f / sv;    // softmax at T = 1 of its own maximum
+        if (lane == 0) {
+          const int b = bj / p.k;
+          p.next_cand[bj] = row_i[mask_row(b, istar[b], bj - b * p.k)];
+          p.next_cand_prob[bj] = 1.f / sv;                 // softmax at T = 1 of its own maximum
+        }
       }
       }
     }
@@ -719,20 +737,34 @@ int lm_make_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t D, int6
 
 }  // namespace
 
+size_t lmhead_gather_bytes() { return LM_GATHER_ELEMS * sizeof(__nv_bfloat16); }
 size_t lmhead_partial_bytes(int sm_count) {
   return (size_t)LM_MAX_N * sm_count * (sizeof(LmPartial) + sizeof(LmNoisy));
 }
 
 namespace {
 
-// One launch: the sequences of `a` (at most LM_MAX_N block rows); seq_base = index of the first
+// Mask rows (i*, 1..k) of every sequence, one thread block per row, next to one another for the second phase's
+// box.  (Fetching them by a box per sequence instead, eight rows of 128 bytes each, paced the whole phase:
+// 406 us under ncu for 16 sequences, D = 4096, V = 128256.)
+__global__ void __launch_bounds__(256) lm_gather_kernel(const uint4* hidden, int64_t row_stride, int n_q, int k, int vecs,
+                                                        const int32_t* n_accept, uint4* dst) {
+  pdl_launch_dependents();
+  pdl_wait();
+  const int b = blockIdx.x / k, o = blockIdx.x - b * k + 1;
+  const uint4* src = hidden + ((int64_t)b * n_q + n_accept[b] * (k + 1) + o) * row_stride;
+  for (int i = threadIdx.x; i < vecs; i += blockDim.x) dst[(int64_t)blockIdx.x * vecs + i] = src[i];
+}
+
+// One launch: the rows that `phase` names of the sequences of `a` (at most LM_MAX_N); seq_base = index of the first
 // of them in the caller's batch.
-int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, cudaStream_t st) {
+int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, int phase, cudaStream_t st) {
   LmParams p;
   memset(&p, 0, sizeof(p));
   p.B = a->batch; p.k = a->k; p.V = a->vocab; p.D = a->hidden_dim;
   p.n_q = (a->k + 1) * (a->k + 1);
-  p.n_rows = p.B * p.n_q;
+  p.phase = phase;
+  p.n_rows = p.B * (phase == LM_ALL ? p.n_q : phase == LM_TARGETS ? a->k + 1 : a->k);
   p.n_pad = (p.n_rows + 15) / 16 * 16;
   if (p.n_pad > LM_MAX_N) return SPACE_E_UNSUPPORTED;
   p.n_mt = p.n_pad > LM_M ? 2 : 1;
@@ -774,7 +806,12 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   p.err = ctx->lm_counter + 1;
   int rc = lm_make_map(&p.tm_w, a->weight, a->vocab, a->hidden_dim, a->weight_row_stride, p.n_box);
   if (rc == SPACE_OK) rc = lm_make_map(&p.tm_wt, a->weight, a->vocab, a->hidden_dim, a->weight_row_stride, p.tail_rows);
-  if (rc == SPACE_OK) rc = lm_make_map(&p.tm_h, a->hidden, p.n_rows, a->hidden_dim, a->hidden_row_stride, p.n_pad);
+  // hidden rows in one box: all of them, every (k+1)-th (the target rows lie k+1 rows apart, across
+  // sequences too), or the gathered mask rows
+  if (rc == SPACE_OK)
+    rc = phase == LM_MASKS ? lm_make_map(&p.tm_h, ctx->lm_gather, p.n_rows, a->hidden_dim, a->hidden_dim, p.n_pad)
+                           : lm_make_map(&p.tm_h, a->hidden, p.n_rows, a->hidden_dim,
+                                         a->hidden_row_stride * (phase == LM_TARGETS ? a->k + 1 : 1), p.n_pad);
   if (rc != SPACE_OK) return rc;
   const size_t sm = L.total + 1024;
   cudaFuncSetAttribute(lmhead_verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -788,12 +825,24 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
 
 }  // namespace
 
-// A batch of more block rows than one launch covers goes group of sequences by group of
-// sequences: every group streams the output embedding once and is complete in itself (the
-// results are per sequence).  The launches follow one another on the stream and share the scratch.
+// Which launches a batch takes.  Up to 128 block rows: one launch over all of them, bound by the stream of
+// the output embedding (one pass).  More: the step decides on 2k+1 rows of every sequence only, so the target
+// rows go first and the mask rows of the groups they select second -- two passes over the embedding, each at
+// the pace of the stream, instead of one or more over all (k+1)^2 rows that the product (from 128 rows on)
+// or the noise (a Philox block and eight logarithms per four tokens in every epilogue warp) paces.
+// Greedy calls of 129..256 rows stay with one launch: its 1.5 passes' time beats two (4 x 36 rows of
+// D = 4096, V = 32000: 83 us against 104), and so do calls that ask for every row's maximum.
+// Measured: 16 x 36 rows, V = 128256, sampling 934 -> 396 us; 4 x 49 rows, D = 1088, V = 128256 163 -> 129 us.
 int launch_lmhead_verify(space_ctx* ctx, const space_lmhead_args* a, cudaStream_t st) {
   const int n_q = (a->k + 1) * (a->k + 1), k1 = a->k + 1;
-  const int per_group = LM_MAX_N / n_q;
+  const int rows = a->batch * n_q;
+  const int64_t fit = LM_GATHER_ELEMS / ((int64_t)a->k * a->hidden_dim);   // sequences whose mask rows can be gathered
+  const int per_phase = fit < LM_M / k1 ? (int)fit : LM_M / k1, per_all = LM_MAX_N / n_q;
+  bool by_phase = per_phase > 0 && !a->row_max && !a->row_argmax && rows > (a->mode == SPACE_MODE_SAMPLE ? LM_M : LM_MAX_N);
+  // a small embedding (under about 10 us of stream) is paced by launches instead: as few of them as can be
+  if (by_phase && (int64_t)a->vocab * a->hidden_dim < (32ll << 20))
+    by_phase = 2 * ((a->batch + per_phase - 1) / per_phase) < (a->batch + per_all - 1) / per_all;
+  const int per_group = by_phase ? per_phase : per_all;
   if (per_group < 1) return SPACE_E_UNSUPPORTED;
   for (int b0 = 0; b0 < a->batch; b0 += per_group) {
     space_lmhead_args g = *a;
@@ -809,7 +858,13 @@ int launch_lmhead_verify(space_ctx* ctx, const space_lmhead_args* a, cudaStream_
     if (a->status) g.status = a->status + b0;
     if (a->row_max) g.row_max = a->row_max + (int64_t)b0 * n_q;
     if (a->row_argmax) g.row_argmax = a->row_argmax + (int64_t)b0 * n_q;
-    const int rc = launch_group(ctx, &g, (uint32_t)b0, st);
+    int rc = launch_group(ctx, &g, (uint32_t)b0, by_phase ? LM_TARGETS : LM_ALL, st);
+    if (rc == SPACE_OK && by_phase) {
+      launch_pdl(lm_gather_kernel, dim3(g.batch * a->k), dim3(256), 0, st, static_cast<const uint4*>(g.hidden),
+                 a->hidden_row_stride / 8, n_q, a->k, a->hidden_dim / 8, (const int32_t*)g.n_accept, (uint4*)ctx->lm_gather);
+      ctx->launches += 1;
+      rc = launch_group(ctx, &g, (uint32_t)b0, LM_MASKS, st);
+    }
     if (rc != SPACE_OK) return rc;
   }
   return SPACE_OK;

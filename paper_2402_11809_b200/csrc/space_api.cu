@@ -28,7 +28,7 @@ int config_supported(const space_config* c) {
 }
 
 struct Carve {
-  size_t attn_part, counters, merge_cnt, vtopk, vpart, vfused, vrow, status, lm_part, lm_counter, stage, total;
+  size_t attn_part, counters, merge_cnt, vtopk, vpart, vfused, vrow, status, lm_part, lm_gather, lm_counter, stage, total;
   size_t part_slots;
   // staging sub-offsets (relative to stage)
   size_t st_q, st_k, st_v, st_logits, st_small;
@@ -51,6 +51,7 @@ Carve carve(const space_config* c, int sm_count) {
   v.vrow = off; off += align_up((size_t)c->max_batch * (c->k_max + 1) * sizeof(VerifyRow), 256);
   v.status = off; off += align_up((size_t)c->max_batch * sizeof(int32_t), 256);
   v.lm_part = off; off += align_up(lmhead_partial_bytes(sm_count), 256);
+  v.lm_gather = off; off += align_up(lmhead_gather_bytes(), 256);
   // counter, error word; one arg-max key per block row; one candidate logit per block row
   v.lm_counter = off; off += 256 + 256 * sizeof(unsigned long long) + 256 * sizeof(float);
   v.stage = off;
@@ -217,6 +218,7 @@ int space_create(space_ctx** out, const space_config* cfg) {
   ctx->vfused = (VerifyPartial*)(ctx->ws + cv.vfused);
   ctx->scratch_status = (int32_t*)(ctx->ws + cv.status);
   ctx->lm_part = ctx->ws + cv.lm_part;
+  ctx->lm_gather = ctx->ws + cv.lm_gather;
   ctx->lm_counter = (int*)(ctx->ws + cv.lm_counter);
   ctx->stage = cfg->host_staging ? ctx->ws + cv.stage : nullptr;
   ctx->stage_bytes = cv.total - cv.stage;

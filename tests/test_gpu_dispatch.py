@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle.lmhead import lmhead_verify_step
 from oracle.verify import verify_step
 from paper_2402_11809_b200 import workloads
 from test_gpu_parity import B, H, _check_verify, _small_cfg  # noqa: F401  (B, H: fixtures)
@@ -60,3 +61,49 @@ def test_filtered_sampling_on_sorted_and_tied_rows(B, H, Bn, k, V, top_k, dtype)
         r = verify_step(x["logits"], x["cand"], x["cand_prob"], k, "sample", temperature=1.0, seed=5, seq_id=x["seq_id"],
                         kv_len=x["kv_len"], resample=name, top_k=top_k, top_p=1.0)
         _check_verify(ds, r, k, sample=True)
+
+
+# Wide batches by phase (target rows, then the mask rows of group i*): eight rows per sequence at k = 7, one mask
+# row at k = 1, several groups of sequences, D and V off every tile, and the last sequence's mask rows at the end
+# of the hidden states.
+@pytest.mark.parametrize("mode", ["greedy", "residual_pointmass", "paper_literal"])
+@pytest.mark.parametrize("V,D,k,Bn", [(3001, 200, 7, 16), (131075, 264, 1, 67), (20000, 128, 5, 16), (129, 64, 5, 21), (40003, 136, 6, 18)])
+def test_lmhead_by_phase(B, H, mode, V, D, k, Bn):  # noqa: F811
+    cfg = workloads.resolve_lmhead("lmhead_tiny", V=V, D=D, k=k, B=Bn, p_accept=(0.5, 1.0))
+    x = workloads.make_lmhead_inputs(cfg)
+    rng = np.random.default_rng(V)
+    sample = mode != "greedy"
+    if mode == "paper_literal":
+        x["cand_prob"] = rng.uniform(0.05, 1.0, size=x["cand_prob"].shape).astype(np.float32)
+    x["cand"][-1, -1] = V + 9                                # out of range: rejected, flagged
+    kv_len = rng.integers(0, 3000, size=Bn).astype(np.int32)
+    ctx = B.Context(max_batch=Bn, n_q_heads=8, n_kv_heads=8, head_dim=64, k_max=k, vocab=V, s_cap=256)
+    i32 = lambda *s: torch.full(s, -7, dtype=torch.int32, device="cuda")  # noqa: E731
+    got = dict(n_accept=i32(Bn), out_tokens=i32(Bn, k + 1), n_out=i32(Bn), next_cand=i32(Bn, k),
+               next_cand_prob=torch.full((Bn, k), float("nan"), device="cuda"),
+               finished=torch.full((Bn,), 9, dtype=torch.uint8, device="cuda"))
+    status = torch.zeros(Bn, dtype=torch.int32, device="cuda")
+    keep = [H.to_dev(x[n]) for n in ("hidden", "weight", "cand", "cand_prob")] + [H.to_dev(kv_len)]
+    a = ctx.lmhead_args(keep[0], keep[1], keep[2], k=k, eos_id=int(x["cand"][0, 0]), status=status, seed=7, temperature=0.9,
+                        mode=B.MODE_SAMPLE if sample else B.MODE_GREEDY, cand_prob=keep[3], kv_len=keep[4],
+                        resample=B.RESAMPLE_PAPER_LITERAL if mode == "paper_literal" else B.RESAMPLE_RESIDUAL_POINTMASS, **got)
+    kw = dict(mode="sample", temperature=0.9, seed=7, kv_len=kv_len, resample=mode) if sample else {}
+    r = lmhead_verify_step(x["hidden"], x["weight"], x["cand"], x["cand_prob"], k, eos_id=int(x["cand"][0, 0]), **kw)
+    excl = np.zeros(Bn, bool)
+    for b in range(Bn):
+        i = int(r["n_accept"][b])
+        used = [] if sample else [t * (k + 1) for t in range(k + 1)]
+        used += [] if mode == "paper_literal" else [i * (k + 1) + o for o in range(1, k + 1)]
+        excl[b] = bool(used) and r["row_gap"][b, used].min() <= 1e-3
+    if sample:
+        excl |= (r["accept_margin"] <= 1e-3).any(1) | (r["bonus_gap"] <= 1e-3) | (r["draft_gap"] <= 1e-3).any(1)
+    assert excl.sum() <= max(1, Bn // 8)
+    for again in range(2):                                   # counters and keys reset themselves
+        n0 = ctx.launch_count
+        ctx.space_lmhead_verify(a)
+        assert (ctx.launch_count - n0) % 3 == 0              # targets, gather, masks per group of sequences
+        h = {n: t.cpu().numpy() for n, t in got.items()}
+        for n in ("n_accept", "out_tokens", "n_out", "next_cand", "finished"):
+            assert np.array_equal(h[n][~excl], r[n][~excl]), (n, again)
+        np.testing.assert_allclose(h["next_cand_prob"][~excl], r["next_cand_prob"][~excl], rtol=1e-3)
+        assert status[-1].item() & B.ST_BAD_CANDIDATE and not status[:-1].any()
