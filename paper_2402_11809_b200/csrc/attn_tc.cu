@@ -46,6 +46,8 @@ constexpr int TILE_N = 128;            // keys per tile
 constexpr int SHARE_COST = 4;          // fixed cost of a share (query load, first tile, last product, epilogue) in tiles; swept 2..8
 constexpr int ROWS = 128;              // MMA M
 constexpr int THREADS = 384;            // K, MMA, V, Q warps + 8 softmax warps
+constexpr int CLUSTER_SLACK = 10;
+constexpr int MAX_CLUSTER = 16;         // blocks per cluster (more than 8 need the opt-in)
 constexpr uint64_t WAIT_NS = 1000000000ull;   // one second per wait
 
 struct AttnParams {
@@ -55,7 +57,7 @@ struct AttnParams {
   int n_pad;                           // rows_per_mb * G rounded up to 16: N of the MMAs
   int n_groups;                        // thread-block groups (grid = n_groups * n_mblocks)
   int out_dtype;
-  int spec;                            // one sequence: every group requests its first K tile before the length is read
+  int pieces;                          // > 0: the grid is cut into clusters of pieces * n_mblocks blocks, one per (sequence, head)
   int64_t s_cap;                       // rows a sequence may hold (paged: pages_per_seq * SPACE_PAGE_SIZE)
   // Paged cache (page_table != nullptr): tm_k / tm_v describe a pool [n_pages][H_kv][TILE_N][d]; tile t
   // of sequence b is the whole page page_table[b * pages_per_seq + t].  No tile is shifted back then:
@@ -67,9 +69,10 @@ struct AttnParams {
   void* out; float* lse; int32_t* status;
   float* part;                         // [slots][ROWS*(DH+2)]
   int* err;                            // one word: first timeout site
-  int2* desc;                          // [B*H_kv*n_mblocks] {first partial slot, number of partials} of each cut
+  int2* desc;                          // [B*H_kv*n_mblocks] {first partial slot, number of partials} of each cut (read by the merge kernel)
   int* owner;                          // [grid] (sequence, kv head) whose last piece this thread block computed, or -1
   int merge_by_owner;                  // the merge grid is indexed by attention thread block, not by (sequence, head)
+  int* arrived;                        // [B*H_kv*n_mblocks] pieces of a cut whose partial is stored (self-resetting)
   // Eq. 5 per (query column, block key), worked out by the host once per call: bit q of
   // visq[mb][j] says that query column q of query-row block mb (block row mb * rows_per_mb + q / G,
   // any of its G heads) sees block key j
@@ -108,7 +111,7 @@ __device__ unsigned long long g_timeline_merge[4096 * 4];
 #else
 #define TL(i) do { } while (0)
 #define TLM(i) do { } while (0)
-#endif   // slot: partial slot; dfirst/dn: cut (aligned mode)
+#endif
 
 // PTX helpers: tc_common.cuh.  Every wait of this kernel is bounded by WAIT_NS.
 using namespace tc;
@@ -143,9 +146,8 @@ __device__ __forceinline__ void even_cut(int T, int n_keys, int a, int piece, in
 struct Partition {
   const int* seq_len;    // [B]   verified length, or -1 for a sequence that does not fit
   const int* prefix;     // [B+1] flat offset of sequence b
-  // aligned mode: {b, h, t0, n, T, L, first slot of the cut, pieces in the cut, step, early requests
-  // serve the first share, head stride from share to share, slot (slots per head when the stride is
-  // not 0), number of shares}
+  // aligned and clustered mode: {b, h, t0, n, T, L, first slot of the cut, pieces in the cut, step, the
+  // early requests serve the share, slot, number of shares (0 or 1)}
   const int* seg0;
   int B, H_kv, n_q, group, ngroups;
   long long cur, end;
@@ -163,7 +165,7 @@ struct Partition {
     group = group_; ngroups = n_groups;
     aligned = agroups >= 0;
     if (aligned) {
-      cur = 0; end = seg0_[12];
+      cur = 0; end = seg0_[11];
       return;
     }
     const long long W = pf[B_];
@@ -174,19 +176,12 @@ struct Partition {
   }
   __device__ bool next(Seg& s) {
     if (aligned) {
-      // the shares were worked out once per thread block during the set-up: one, or (one
-      // sequence, groups left over after every head got its pieces) the last tile of several heads
+      // the share was worked out once per thread block during the set-up
       if (cur >= end) return false;
       const int4 u = reinterpret_cast<const int4*>(seg0)[0], v = reinterpret_cast<const int4*>(seg0)[1];
       s.b = u.x; s.h = u.y; s.t0 = u.z; s.n = u.w; s.T = v.x; s.L = v.y; s.dfirst = v.z; s.dn = v.w;
       s.step = seg0[8];
-      s.slot = seg0[11];
-      const int hstep = seg0[10];
-      if (hstep > 0) {
-        s.h = u.y + (int)cur * hstep;
-        s.dfirst = s.h * seg0[11];
-        s.slot = s.dfirst + seg0[11] - 1;
-      }
+      s.slot = seg0[10];
       ++cur;
       return true;
     }
@@ -346,6 +341,64 @@ __device__ __noinline__ void piece_rescale(uint32_t taddr, const float* fq) {
   tmem_wait_st();
 }
 
+// Shared memory of another block of the cluster.
+__device__ __forceinline__ uint32_t map_cluster(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t a) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
+}
+
+// Query row r of the row block that starts at block row i0, columns 4 c4 .. of (sequence b, kv head h).
+template <int DH>
+__device__ __forceinline__ void store_out(const AttnParams& p, int b, int h, int i0, int r, int c4, const float4& v) {
+  const int gsh = __ffs(p.G) - 1;                           // G is a power of two
+  const int ri = i0 + (r >> gsh), hq = h * p.G + (r & (p.G - 1));
+  const size_t off = (((size_t)b * p.n_q + ri) * p.H_q + hq) * DH + c4 * 4;
+  if (p.out_dtype == SPACE_DTYPE_F32) {
+    *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + off) = v;
+  } else {
+    const __nv_bfloat162 x = __floats2bfloat162_rn(v.x, v.y), y = __floats2bfloat162_rn(v.z, v.w);
+    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + off) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&x), *reinterpret_cast<const uint32_t*>(&y));
+  }
+}
+
+// Four output elements of one query row from the partials of a cut: running reference, denominator and
+// accumulator.
+struct MergeAcc {
+  float mx, den;
+  float4 a;
+  __device__ __forceinline__ void clear() { mx = -CUDART_INF_F; den = 0.f; a = make_float4(0.f, 0.f, 0.f, 0.f); }
+  __device__ __forceinline__ void add(float m, float l, const float4& o) {
+    const float mn = fmaxf(mx, m);
+    if (mn > -CUDART_INF_F) {
+      const float e0 = fast_exp2(mx - mn), e1 = fast_exp2(m - mn);
+      den = den * e0 + l * e1;
+      a.x = a.x * e0 + o.x * e1; a.y = a.y * e0 + o.y * e1;
+      a.z = a.z * e0 + o.z * e1; a.w = a.w * e0 + o.w * e1;
+    }
+    mx = mn;
+  }
+  template <int DH>
+  __device__ __forceinline__ void store(const AttnParams& p, int b, int h, int i0, int r, int c4) const {
+    const float rd = 1.f / den;
+    const int gsh = __ffs(p.G) - 1;
+    const int ri = i0 + (r >> gsh), hq = h * p.G + (r & (p.G - 1));
+    store_out<DH>(p, b, h, i0, r, c4, make_float4(a.x * rd, a.y * rd, a.z * rd, a.w * rd));
+    if (p.lse && c4 == 0) p.lse[((size_t)b * p.H_q + hq) * p.n_q + ri] = (mx + log2f(den)) * 0.6931471805599453f;
+  }
+};
+
 // Warp roles
 constexpr int WARP_K = 0, WARP_MMA = 1, WARP_V = 2, WARP_PV = 3, WARP_SOFTMAX0 = 4;
 constexpr int L2_AHEAD_TILES = 1;      // tiles per operand a block asks L2 for before its dependency wait (more of them
@@ -416,12 +469,11 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     const int j = threadIdx.x - WARP_SOFTMAX0 * 32;
     visq[j] = p.visq[mb][j];
   }
-  // single-sequence partition (explained where the tables are built, below)
-  const int sp_base = max(p.n_groups / p.H_kv, 1), sp_extra = p.n_groups - sp_base * p.H_kv;
-  const bool sp_helper = group >= sp_base * p.H_kv;
-  const int sp_h = sp_helper ? group - sp_base * p.H_kv : group / sp_base;
-  const int sp_piece = sp_helper ? 0 : group - sp_h * sp_base;
-  const bool early = p.spec && !sp_helper;                 // this group requests Q and its first K tile at once
+  // Clustered cut (explained below): this block's piece of (sequence, head) `pair`
+  const int cl_pair = p.pieces ? group / p.pieces : 0, cl_piece = p.pieces ? group - cl_pair * p.pieces : 0;
+  const bool cl_mine = p.pieces && cl_pair < p.B * p.H_kv;
+  const int cl_b = cl_pair / p.H_kv, cl_h = cl_pair - cl_b * p.H_kv;
+  const bool early = cl_mine;                              // this block requests Q and its first K tile at once
   if (warp == WARP_K && lane == 0)
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.tm_k) : "memory");
   if (warp == WARP_V && lane == 0)
@@ -429,7 +481,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   if (warp == WARP_MMA && lane == 0)
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.tm_q) : "memory");
   if (early && !PAGED && lane == 0 && (warp == WARP_K || warp == WARP_V)) {
-    // A regular group's tiles (sp_piece, sp_piece + sp_base, ...) of head sp_h do not depend on the
+    // A piece's tiles (cl_piece, cl_piece + pieces, ...) do not depend on the
     // length, so L2 is asked for them now, while the kernel before this one may still be running:
     // with a programmatic launch this block is resident long before its dependency wait returns,
     // and the tile loads after the wait then find their lines in L2 instead of paying the DRAM
@@ -437,12 +489,12 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     // kernel still writes is what the loads will see.  The length is read here as a hint for how
     // many tiles are worth asking for (a stale value costs or saves a request, never an error).
     const uint64_t pol = l2_evict_first_policy();
-    const int Lh = *reinterpret_cast<const volatile int*>(p.kv_len);
+    const int Lh = *reinterpret_cast<const volatile int*>(p.kv_len + cl_b);
     const int Th = (Lh >= 0 && (int64_t)Lh + p.n_q <= p.s_cap) ? (Lh + p.n_q) / TILE_N : 0;   // whole tiles
     const CUtensorMap* tm = warp == WARP_K ? &p.tm_k : &p.tm_v;
-    for (int j = 0, t = sp_piece; j < L2_AHEAD_TILES && t < Th; ++j, t += sp_base) {
+    for (int j = 0, t = cl_piece; j < L2_AHEAD_TILES && t < Th; ++j, t += p.pieces) {
 #pragma unroll
-      for (int hf = 0; hf < S::HALVES; ++hf) tma_prefetch_l2_4d(tm, hf * 64, t * TILE_N, sp_h, 0, pol);
+      for (int hf = 0; hf < S::HALVES; ++hf) tma_prefetch_l2_4d(tm, hf * 64, t * TILE_N, cl_h, cl_b, pol);
     }
   }
   // barriers and the TMEM allocation are visible to every warp before the first
@@ -453,86 +505,63 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   if (threadIdx.x == 0) TL(1);
   pdl_wait();                                              // global memory from here on
   if (threadIdx.x == 0) TL(2);
-  const bool single = p.B == 1;
-  // One sequence, no more kv heads than groups: every head gets `base` groups (piece i of a head
-  // takes tiles i, i + base, ...: its first tile does not depend on the length), and the groups
-  // left over are helpers that each take the last tile of some heads -- the one with the block's
-  // own keys, whose Eq. 5 mask makes it the slowest -- so that no regular piece carries it on top
-  // of its share of the full tiles.
+  // Clustered cut, for at most one (sequence, kv head) per cluster of blocks: cluster c takes pair c, and
+  // piece i of it tiles i, i + pieces, ...  So which pair and which first tile a block works on does not
+  // depend on the lengths (it requests its query rows and its first K tile before it has read any), there
+  // are no tables to build, and the pieces' partials meet in shared memory of the cluster.  Very unequal or
+  // very long sequences are cut over the whole grid instead, as larger batches are.
   if (early && warp == WARP_K && lane == 0 && !*abort_flag) {
-    // Which head and which first tile a regular group works on does not depend on the length,
-    // so its query rows and its first K tile are requested before the length is even read (one
-    // memory round trip earlier).  Should the length turn out too short for that tile, the S^T
-    // issuer lets both buffers go unused.
+    // Should the length turn out too short for the requested tile, or the cut not be taken, the S^T issuer
+    // lets both buffers go unused.
     mbar_expect_tx(BAR(B_QFULL), (uint32_t)n_pad * DH * 2);
 #pragma unroll
     for (int hf = 0; hf < S::HALVES; ++hf)
-      tma_load_4d(sm_base + S::Q_OFF + hf * (n_pad * 128), &p.tm_q, BAR(B_QFULL), hf * 64, sp_h * p.G, i0, 0);
+      tma_load_4d(sm_base + S::Q_OFF + hf * (n_pad * 128), &p.tm_q, BAR(B_QFULL), hf * 64, cl_h * p.G, i0, cl_b);
     mbar_expect_tx(BAR(B_KFULL), S::TILE_BYTES);
 #pragma unroll
     for (int hf = 0; hf < S::HALVES; ++hf)
       tma_load_4d_hint(sm_base + S::K_OFF + hf * (TILE_N * 128), &p.tm_k, BAR(B_KFULL), hf * 64,
-                       PAGED ? 0 : sp_piece * TILE_N, sp_h, PAGED ? page_of(p, 0, sp_piece, false) : 0,
+                       PAGED ? 0 : cl_piece * TILE_N, cl_h, PAGED ? page_of(p, cl_b, cl_piece, false) : cl_b,
                        l2_evict_first_policy());
     TL(3);
   }
-  if (single) {
-    // One sequence (the usual decoding case): the tables have a closed form, so every
-    // thread works them out for itself from the one length (identical values, each
-    // thread reads back what it wrote) and no warp has to hand them over.
-    const int L0 = p.kv_len[0];
-    const bool okL = L0 >= 0 && (int64_t)L0 + p.n_q <= p.s_cap;
-    if (!okL && blockIdx.x == 0 && threadIdx.x == 0 && p.status) atomicOr(p.status, SPACE_ST_CAPACITY);
-    const int L = okL ? L0 : -1;
-    const int T = okL ? (L + p.n_q + TILE_N - 1) / TILE_N : 0;
-    if (threadIdx.x == 0 && L0 != 0x7FFFFFFF) TL(14);
-    seq_len[0] = L; prefix[0] = 0; prefix[1] = okL ? (T + SHARE_COST) * p.H_kv : 0;
-    int ag = -1, spec_ok = 0;
-    const int W = T * p.H_kv;
-    const bool cut_aligned = W > 0 && W < 8 * p.n_groups && p.H_kv <= p.n_groups;
-    const bool helpers = cut_aligned && sp_extra > 0 && T > sp_base;   // the last tile goes to a helper group
-    if (p.spec && sp_helper && helpers) {
-      // A helper knows its first share as soon as it has the length: the last tile of head sp_h.
-      // Its query rows and that tile are requested here, ahead of the tables and the producer's
-      // own start-up, which would come a microsecond later.
-      spec_ok = 1;
-      if (warp == WARP_K && lane == 0 && !*abort_flag) {
-        const int n_keys = L + p.n_q;
-        const int kt = PAGED ? 0 : ((T * TILE_N <= n_keys) ? (T - 1) * TILE_N : n_keys - TILE_N);
-        const int kb = PAGED ? page_of(p, 0, T - 1) : 0;
-        mbar_expect_tx(BAR(B_QFULL), (uint32_t)n_pad * DH * 2);
-#pragma unroll
-        for (int hf = 0; hf < S::HALVES; ++hf)
-          tma_load_4d(sm_base + S::Q_OFF + hf * (n_pad * 128), &p.tm_q, BAR(B_QFULL), hf * 64, sp_h * p.G, i0, 0);
-        mbar_expect_tx(BAR(B_KFULL), S::TILE_BYTES);
-#pragma unroll
-        for (int hf = 0; hf < S::HALVES; ++hf)
-          tma_load_4d_hint(sm_base + S::K_OFF + hf * (TILE_N * 128), &p.tm_k, BAR(B_KFULL), hf * 64, kt, sp_h, kb,
-                           l2_evict_first_policy());
-        TL(3);
+  bool clustered = false;
+  int cl_n = 0;                                            // pieces of this block's pair that have tiles
+  if (p.pieces) {
+    // every warp works the same things out for itself: nothing has to be handed over
+    auto tiles_of = [&](int L) { return (L >= 0 && (int64_t)L + p.n_q <= p.s_cap) ? (L + p.n_q + TILE_N - 1) / TILE_N : 0; };
+    const int L0 = cl_mine ? p.kv_len[cl_b] : -1;
+    int Tmax, W;
+    if (p.B == 1) {
+      Tmax = W = tiles_of(p.kv_len[0]);
+    } else {
+      Tmax = W = 0;
+      for (int b0 = 0; b0 < p.B; b0 += 32) {
+        const int T = b0 + lane < p.B ? tiles_of(p.kv_len[b0 + lane]) : 0;
+        Tmax = max(Tmax, __reduce_max_sync(0xFFFFFFFFu, T));
+        W += __reduce_add_sync(0xFFFFFFFFu, T);
       }
     }
-    if (cut_aligned) {
-      ag = p.n_groups;
-      const int Treg = helpers ? T - 1 : T;                // tiles cut among the regular pieces
-      const int dn = helpers ? sp_base + 1 : min(sp_base, T);
-      if (!sp_helper) {
-        const int n_mine = sp_piece < Treg ? (Treg - sp_piece + sp_base - 1) / sp_base : 0;
-        spec_ok = (n_mine > 0 && (sp_piece + 1) * TILE_N <= L + p.n_q) ? 1 : 0;   // the requested tile is this share's first
-        if (PAGED && spec_ok && warp == WARP_K && lane == 0) (void)page_of(p, 0, sp_piece);   // flags a bad entry
-        reinterpret_cast<int4*>(seg0)[0] = make_int4(0, sp_h, sp_piece, n_mine);
-        reinterpret_cast<int4*>(seg0)[1] = make_int4(T, L, sp_h * (sp_base + 1), dn);
-        seg0[8] = sp_base; seg0[10] = 0; seg0[11] = sp_h * (sp_base + 1) + sp_piece; seg0[12] = n_mine > 0 ? 1 : 0;
-      } else {
-        // helper e: the last tile of heads e, e + extra, e + 2 extra, ...
-        reinterpret_cast<int4*>(seg0)[0] = make_int4(0, sp_h, T - 1, 1);
-        reinterpret_cast<int4*>(seg0)[1] = make_int4(T, L, 0, dn);
-        seg0[8] = 1; seg0[10] = sp_extra; seg0[11] = sp_base + 1;
-        seg0[12] = helpers ? (p.H_kv - sp_h + sp_extra - 1) / sp_extra : 0;
-      }
+    // tiles of the longest piece against an even share of all tiles and what the cut over the grid costs on
+    // top: starting more than one share per block and the merge in global memory, about ten tiles' time
+    clustered = (Tmax + p.pieces - 1) / p.pieces <= (W * p.H_kv + p.n_groups - 1) / p.n_groups + CLUSTER_SLACK;
+    if (threadIdx.x == 0 && W != 0x7FFFFFFF) TL(14);
+    if (clustered) {
+      const int T = tiles_of(L0), L = T ? L0 : -1;
+      if (cl_mine && !T && cl_piece == 0 && cl_h == 0 && mb == 0 && threadIdx.x == 0 && p.status)
+        atomicOr(p.status + cl_b, SPACE_ST_CAPACITY);
+      const int n_mine = cl_piece < T ? (T - cl_piece + p.pieces - 1) / p.pieces : 0;
+      cl_n = min(p.pieces, T);
+      const int spec_ok = (n_mine > 0 && (PAGED || (cl_piece + 1) * TILE_N <= L + p.n_q)) ? 1 : 0;   // the requested tile is the first
+      if (PAGED && spec_ok && warp == WARP_K && lane == 0) (void)page_of(p, cl_b, cl_piece);   // flags a bad entry
+      // (identical values by every thread, each reads back what it wrote)
+      reinterpret_cast<int4*>(seg0)[0] = make_int4(cl_b, cl_h, cl_piece, n_mine);
+      reinterpret_cast<int4*>(seg0)[1] = make_int4(T, L, 0, cl_n);
+      reinterpret_cast<int4*>(seg0)[2] = make_int4(p.pieces, spec_ok, 0, n_mine > 0 ? 1 : 0);
+      *agroups = 0;
     }
-    seg0[9] = spec_ok;
-    *agroups = ag;
+  }
+  if (clustered) {
   } else if (warp == WARP_SOFTMAX0) {
     // per-sequence tile counts and their running sum, 32 sequences per round
     int carry = 0, nvalid = 0;
@@ -560,7 +589,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     // aligned mode when a group would get fewer than 8 tiles: groups per (sequence,
     // head) a_b = floor(groups * T_b / W), at least 1 tile each; fall back to the flat
     // cut if that needs more groups than there are
-    if (lane == 0) { seg0[8] = 1; seg0[9] = 0; seg0[10] = 0; seg0[11] = group; seg0[12] = 0; }   // no share yet
+    if (lane == 0) { seg0[8] = 1; seg0[9] = 0; seg0[10] = group; seg0[11] = 0; }   // no share yet
     __syncwarp();
     const int Wv = carry;                                  // list entries (tiles + share costs)
     const int W = Wv - SHARE_COST * p.H_kv * nvalid;       // real tiles
@@ -591,7 +620,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           even_cut(T, L + p.n_q, a, piece, t0, t1);
           reinterpret_cast<int4*>(seg0)[0] = make_int4(b, h, t0, t1 - t0);
           reinterpret_cast<int4*>(seg0)[1] = make_int4(T, L, first + h * a, a);
-          seg0[12] = 1;
+          seg0[11] = 1;
         }
         acarry += __shfl_sync(0xFFFFFFFFu, incl, 31);
       }
@@ -602,7 +631,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       *agroups = acarry;
     }
   }
-  if (!single) __syncthreads();                            // the tables of warp 4 reach every warp
+  if (!clustered) __syncthreads();                         // the tables of warp 4 reach every warp
   const uint32_t tmem = *tmem_slot;
   // TMEM columns: S^T buffers at 0 and 128 (n_pad <= 128 columns each), [O_hi^T | O_lo^T] at 256
   // (64 columns each)
@@ -623,12 +652,12 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       const int b_full = is_k ? B_KFULL : B_VFULL, b_empty = is_k ? B_KEMPTY : B_VEMPTY;
       const uint32_t ring = sm_base + (is_k ? S::K_OFF : S::V_OFF);
       const CUtensorMap* tm = is_k ? &p.tm_k : &p.tm_v;
-      // Early requests (one sequence): when this share's first tile is the requested one, the K
+      // Early requests: when this share's first tile is the requested one, the K
       // producer skips the query rows and that tile; when it is not, the two buffers are given
       // back by the S^T issuer and the rings start one slot further.
       if (is_k) TL(15);
       const uint64_t kv_policy = l2_evict_first_policy();
-      bool pre = p.spec && is_k && seg0[9] != 0;           // Q and the first K tile of the first share are on their way
+      bool pre = is_k && seg0[9] != 0;           // Q and the first K tile of the first share are on their way
       const uint32_t koff = (early && is_k && !pre) ? 1u : 0u;
       uint32_t gt = 0, seg = koff;
       bool ok = true;
@@ -710,7 +739,6 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       }
       while (ok && part.next(sg)) {
         const uint32_t qb = seg % S::Q_BUFS, use = seg / S::Q_BUFS;
-        if (gt == 0) TL(12);
         ok = mbar_wait(BAR(B_QFULL + qb), use & 1, abort_flag, p.err, 6);
         const uint64_t qd = qdesc0 + (uint64_t)((qb * S::Q_BYTES) >> 4);
         const int n = sg.n;
@@ -1044,24 +1072,25 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       const bool whole = sg.n == sg.T;
       const int item = sg.b * p.H_kv + sg.h;
       float* pslot = p.part + ((size_t)sg.slot * p.n_mblocks + mb) * (ROWS * (DH + 2));
+      // How this (sequence, head) was cut, {first partial slot, number of partials}: read by the merge kernel
+      // (every piece writes the same pair)
+      int2 cut_d = make_int2(sg.slot, 1);
       if (sidx == 0 && ok) {
-        // how this (sequence, head) was cut, read by attn_merge_kernel (every group of
-        // the cut writes the same pair)
-        // {first partial slot, number of partials}
-        int2 d = make_int2(sg.slot, 1);
         if (sg.dfirst >= 0) {
-          d = make_int2(sg.dfirst, sg.dn);
+          cut_d = make_int2(sg.dfirst, sg.dn);
         } else if (!whole) {
           const long long W = prefix[p.B];
           const long long NG = W < p.n_groups ? W : p.n_groups;
-          const long long f0 = (long long)prefix[sg.b] + (long long)sg.h * (sg.T + SHARE_COST);
-          const int g0 = group_of(f0 + SHARE_COST, W, NG);  // group of the first tile
-          d.x = item + g0;
-          d.y = group_of(f0 + SHARE_COST + sg.T - 1, W, NG) - g0 + 1;
+          const long long f0 = (long long)prefix[sg.b] + (long long)sg.h * (sg.T + SHARE_COST) + SHARE_COST;
+          const int g0 = group_of(f0, W, NG);               // group of the first tile
+          cut_d = make_int2(item + g0, group_of(f0 + sg.T - 1, W, NG) - g0 + 1);
         }
-        p.desc[(size_t)item * p.n_mblocks + mb] = d;
+        if (!p.pieces) p.desc[(size_t)item * p.n_mblocks + mb] = cut_d;
         if (!whole && sg.tile_at(sg.n - 1) == sg.T - 1) own = item;   // the piece with the pair's last tile; at most one per block
       }
+      // Where a piece's partial goes: shared memory of the cluster (the P buffer is idle now), or its slot
+      // in global memory.
+      const bool to_smem = clustered && !whole;
       if (sidx < m_valid && ok) {                           // per-row scalars
         const int q = sidx;
         if (whole) {
@@ -1069,6 +1098,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
             const int i = i0 + q / p.G, hq = sg.h * p.G + q % p.G;
             p.lse[((size_t)sg.b * p.H_q + hq) * p.n_q + i] = (mref[q] + log2f(fq[q])) * 0.6931471805599453f;
           }
+        } else if (to_smem) {
+          xq[q] = mref[q];                                  // (the sums stay in fq)
         } else {
           pslot[ROWS * DH + q] = mref[q];
           pslot[ROWS * DH + ROWS + q] = fq[q];
@@ -1111,6 +1142,11 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
               if (q0 + e < m_valid && d_ok)
                 reinterpret_cast<__nv_bfloat16*>(p.out)[off[e]] = __float2bfloat16_rn(__uint_as_float(o[e]) * rr[e]);
           }
+        } else if (to_smem) {
+          float* dst = reinterpret_cast<float*>(sm + S::P_OFF) + q0 * DH + kl;
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            if (q0 + e < m_valid && d_ok) dst[e * DH] = __uint_as_float(o[e]);
         } else {
           float* dst = pslot + (size_t)q0 * DH + kl;
 #pragma unroll
@@ -1121,10 +1157,114 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       tc_fence_before();
       soft_sync();                                          // scratch, fq and mref are reused by the next share
       if (sidx == 0) TL(11);
+      if (p.pieces && !whole && !to_smem) {
+        // ---- clusters were launched, but the lengths are too unequal for them: the piece that finds all the
+        // others stored combines them.  (No merge kernel follows such a launch.  As the rule for larger
+        // batches this was slower, 137 against 130 us on sixteen ragged sequences: every piece waits for its
+        // fence and its atomic.)
+        int* flag = reinterpret_cast<int*>(xq);
+        if (sidx == 0) {
+          int* arrived = p.arrived + (size_t)item * p.n_mblocks + mb;
+          __threadfence();                                  // (the barrier above ordered every thread's stores before this)
+          const int last = atomicAdd(arrived, 1) == cut_d.y - 1;
+          if (last) { *arrived = 0; __threadfence(); }      // ready for the next launch
+          flag[0] = last; flag[1] = cut_d.x; flag[2] = cut_d.y;
+        }
+        soft_sync();
+        const bool last = flag[0] != 0;
+        const int d0 = flag[1], dn = flag[2];
+        if (last && ok) {
+          const size_t slot_floats = (size_t)ROWS * (DH + 2), gstride = (size_t)p.n_mblocks * slot_floats;
+          const float* ps = p.part + ((size_t)d0 * p.n_mblocks + mb) * slot_floats;
+          // rows in batches whose weights exp2(m - M) / sum fit the P buffer (idle now): dn floats per row
+          float* wgt = reinterpret_cast<float*>(sm + S::P_OFF);
+          const int rows_at_once = min(m_valid, 2 * S::P_PART / 4 / dn);
+          for (int r0 = 0; r0 < m_valid; r0 += rows_at_once) {
+            const int nr = min(rows_at_once, m_valid - r0);
+            soft_sync();
+            for (int rr = warp - WARP_SOFTMAX0; rr < nr; rr += 8) {
+              const float* pr = ps + ROWS * DH + r0 + rr;
+              float M = -CUDART_INF_F, den = 0.f;
+              for (int x = lane; x < dn; x += 32) M = fmaxf(M, __ldcg(pr + (size_t)x * gstride));
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
+              for (int x = lane; x < dn; x += 32) {
+                const float e = fast_exp2(__ldcg(pr + (size_t)x * gstride) - M);
+                wgt[rr * dn + x] = e;
+                den = fmaf(__ldcg(pr + (size_t)x * gstride + ROWS), e, den);
+              }
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xFFFFFFFFu, den, o);
+              const float rd = 1.f / den;
+              for (int x = lane; x < dn; x += 32) wgt[rr * dn + x] *= rd;
+              if (p.lse && lane == 0) {
+                const int q = r0 + rr;
+                p.lse[((size_t)sg.b * p.H_q + sg.h * p.G + q % p.G) * p.n_q + i0 + q / p.G] = (M + log2f(den)) * 0.6931471805599453f;
+              }
+            }
+            soft_sync();
+            for (int idx = sidx; idx < nr * (DH / 4); idx += 256) {
+              const int rr = idx / (DH / 4), c4 = idx % (DH / 4);
+              float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+              const float* po = ps + (size_t)(r0 + rr) * DH + c4 * 4;
+              for (int x0 = 0; x0 < dn; x0 += 16) {         // all loads of a batch are issued before any is used
+                float4 ov[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                  ov[j] = x0 + j < dn ? __ldcg(reinterpret_cast<const float4*>(po + (size_t)(x0 + j) * gstride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                  const float w = x0 + j < dn ? wgt[rr * dn + x0 + j] : 0.f;
+                  a.x = fmaf(ov[j].x, w, a.x); a.y = fmaf(ov[j].y, w, a.y);
+                  a.z = fmaf(ov[j].z, w, a.z); a.w = fmaf(ov[j].w, w, a.w);
+                }
+              }
+              store_out<DH>(p, sg.b, sg.h, i0, r0 + rr, c4, a);
+            }
+          }
+        }
+        soft_sync();                                        // flag lies in the scratch of the next share
+      }
     }
-    if (sidx == 0) p.owner[blockIdx.x] = own;
+    if (!p.pieces && sidx == 0) p.owner[blockIdx.x] = own;
   }
-
+  if (clustered && cl_n > 1) {
+    // ---- the pieces of this cluster's pair meet: every block combines its part of the rows from all pieces'
+    // shared memory.  (A block of the cluster without a tile takes part too.  Every wait above is bounded, so
+    // every block arrives here.)
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const uint32_t mine = sm_base;
+    const int stride = p.pieces * THREADS;
+    for (int idx = cl_piece * THREADS + (int)threadIdx.x; idx < m_valid * (DH / 4) && !*abort_flag; idx += stride) {
+      const int r = idx / (DH / 4), c4 = idx % (DH / 4);
+      MergeAcc acc;
+      acc.clear();
+      for (int x0 = 0; x0 < cl_n; x0 += 4) {
+        float ms[4], ls[4];
+        float4 ov[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (x0 + j < cl_n) {
+            const uint32_t rk = (uint32_t)((x0 + j) * p.n_mblocks + mb);
+            ms[j] = ld_cluster(map_cluster(mine + S::XQ_OFF + r * 4, rk));
+            ls[j] = ld_cluster(map_cluster(mine + S::FQ_OFF + r * 4, rk));
+            ov[j] = ld_cluster4(map_cluster(mine + S::P_OFF + (r * DH + c4 * 4) * 4, rk));
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (x0 + j < cl_n) acc.add(ms[j], ls[j], ov[j]);
+      }
+      acc.template store<DH>(p, cl_b, cl_h, i0, r, c4);
+    }
+    // No block leaves while another may still read its shared memory: this half says that this block has read
+    // (relaxed: nothing is handed over, so it need not wait for the output's stores), the other half is at the exit.
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 0) TL(12);
   // ---- teardown -----------------------------------------------------------
   tc_fence_before();
   __syncthreads();
@@ -1134,6 +1274,10 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   }
   if (threadIdx.x == 0 && *abort_flag && p.status) {
     for (int b = 0; b < p.B; ++b) atomicOr(p.status + b, SPACE_ST_TIMEOUT);
+  }
+  if (clustered && cl_n > 1) {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   }
   if (threadIdx.x == 32) TL(13);                          // after the TMEM release
 }
@@ -1173,8 +1317,8 @@ __global__ void __launch_bounds__(128) attn_merge_kernel(const AttnParams p) {
   const size_t slot_floats = (size_t)ROWS * (DH + 2);
   const float* ps = p.part + ((size_t)d.x * p.n_mblocks + mb) * slot_floats;
   const size_t gstride = (size_t)p.n_mblocks * slot_floats;
-  float mx = -CUDART_INF_F, den = 0.f;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  MergeAcc acc;
+  acc.clear();
   // batches of eight partials: all loads of a batch are issued before any is used
   for (int x0 = 0; x0 < n; x0 += 8) {
     float ms[8], ls[8];
@@ -1190,32 +1334,10 @@ __global__ void __launch_bounds__(128) attn_merge_kernel(const AttnParams p) {
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      if (x0 + j < n) {
-        const float mn = fmaxf(mx, ms[j]);
-        if (mn > -CUDART_INF_F) {
-          const float e0 = fast_exp2(mx - mn), e1 = fast_exp2(ms[j] - mn);
-          den = den * e0 + ls[j] * e1;
-          acc.x = acc.x * e0 + ov[j].x * e1; acc.y = acc.y * e0 + ov[j].y * e1;
-          acc.z = acc.z * e0 + ov[j].z * e1; acc.w = acc.w * e0 + ov[j].w * e1;
-        }
-        mx = mn;
-      }
+      if (x0 + j < n) acc.add(ms[j], ls[j], ov[j]);
     }
   }
-  const float rd = 1.f / den;
-  const int ri = i0 + r / p.G, hq = h * p.G + r % p.G;
-  const size_t off = (((size_t)b * p.n_q + ri) * p.H_q + hq) * DH + c4 * 4;
-  if (p.out_dtype == SPACE_DTYPE_F32) {
-    *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + off) =
-        make_float4(acc.x * rd, acc.y * rd, acc.z * rd, acc.w * rd);
-  } else {
-    const __nv_bfloat162 a = __floats2bfloat162_rn(acc.x * rd, acc.y * rd);
-    const __nv_bfloat162 b2 = __floats2bfloat162_rn(acc.z * rd, acc.w * rd);
-    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + off) =
-        make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b2));
-  }
-  if (p.lse && c4 == 0)
-    p.lse[((size_t)b * p.H_q + hq) * p.n_q + ri] = (mx + log2f(den)) * 0.6931471805599453f;
+  acc.template store<DH>(p, b, h, i0, r, c4);
   TLM(3);
 }
 
@@ -1265,19 +1387,39 @@ size_t smem_bytes(int max_batch) {
   return Smem<DH>::TABLE_OFF + (size_t)(2 * max_batch + 1) * sizeof(int);
 }
 
+// Launch with clusters of `size` blocks (1: none).  max_clusters != nullptr: no launch, the largest number of
+// such clusters that can be resident instead.
 template <int DH, bool PAGED>
-cudaError_t launch_main(const AttnParams& p, int n_ctas, int max_batch, cudaStream_t st) {
-  const size_t sm = smem_bytes<DH>(max_batch);
-  // the shared-memory limit of the kernel is raised once per device (to the most any batch needs)
+cudaError_t launch_main(const AttnParams& p, int n_ctas, int max_batch, int size, cudaStream_t st, int* max_clusters = nullptr) {
+  // the kernel's limits are raised once per device (to the most any batch needs)
   static unsigned long long done_mask = 0;                 // (one per instantiation)
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 64 || !((done_mask >> dev) & 1ull)) {
     cudaFuncSetAttribute(attn_tc_kernel<DH, PAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem_bytes<DH>(128));
+    cudaFuncSetAttribute(attn_tc_kernel<DH, PAGED>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (dev < 64) done_mask |= 1ull << dev;
   }
-  return launch_pdl(attn_tc_kernel<DH, PAGED>, dim3(n_ctas), dim3(THREADS), sm, st, p, max_batch);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_ctas); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = smem_bytes<DH>(max_batch); cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = size; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = size > 1 ? 2 : 1;
+  if (max_clusters) {
+    cfg.attrs = attr + 1; cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(max_clusters, attn_tc_kernel<DH, PAGED>, &cfg);
+  }
+  return cudaLaunchKernelEx(&cfg, attn_tc_kernel<DH, PAGED>, p, max_batch);
+}
+
+template <int DH>
+cudaError_t launch_form(const AttnParams& p, int n_ctas, int max_batch, int size, cudaStream_t st, int* max_clusters = nullptr) {
+  return p.page_table ? launch_main<DH, true>(p, n_ctas, max_batch, size, st, max_clusters)
+                      : launch_main<DH, false>(p, n_ctas, max_batch, size, st, max_clusters);
 }
 
 }  // namespace
@@ -1329,10 +1471,10 @@ int launch_attn_tensor(space_ctx* ctx, const space_attn_args* a, const uint64_t*
   p.scale_log2 = a->scale * 1.4426950408889634f;
   p.kv_len = a->kv_len; p.out = a->out; p.lse = a->lse; p.status = a->status;
   p.part = ctx->attn_part; p.err = ctx->counters + 3 * cfg.max_batch;
+  p.arrived = ctx->arrived;
   p.desc = reinterpret_cast<int2*>(ctx->merge_cnt);
   p.owner = ctx->merge_cnt + (size_t)cfg.max_batch * cfg.n_kv_heads * 8 * 2;
   p.merge_by_owner = (a->batch * p.H_kv * p.n_mblocks > pl.n_ctas) ? 1 : 0;
-  p.spec = (a->batch == 1 && p.H_kv <= p.n_groups) ? 1 : 0;
   if (p.n_mblocks > 2) return SPACE_E_UNSUPPORTED;         // (cannot happen: at most 64 block rows, at least 32 per block)
   if (ctx->visq_k != a->k || ctx->visq_variant != a->mask_variant) {
     memset(ctx->visq, 0, sizeof(ctx->visq));
@@ -1373,23 +1515,40 @@ int launch_attn_tensor(space_ctx* ctx, const space_attn_args* a, const uint64_t*
   memcpy(&p.tm_k, ctx->tm_k, sizeof(CUtensorMap));
   memcpy(&p.tm_v, ctx->tm_v, sizeof(CUtensorMap));
 
-  const int m_valid_max = p.rows_per_mb * p.G;
-  const dim3 mgrid(p.merge_by_owner ? pl.n_ctas : a->batch * p.H_kv * p.n_mblocks, (m_valid_max * (DH / 4) + 127) / 128);
+  // Clustered cut when every (sequence, kv head) gets a cluster of its own: as many pieces as there are SMs
+  // for (and tiles a sequence may have), in clusters that fit next to one another.  The grid fills the chip
+  // all the same: the kernel falls back to a cut over all of it when the lengths are too unequal.
+  const int pairs = a->batch * p.H_kv;
+  const int64_t cap_tiles = (p.s_cap + TILE_N - 1) / TILE_N;
+  int n_ctas = pl.n_ctas, size = 1;
+  for (int c = cap_tiles < MAX_CLUSTER / p.n_mblocks ? (int)cap_tiles : MAX_CLUSTER / p.n_mblocks; c >= 1; --c) {
+    const int sz = c * p.n_mblocks;
+    if (pairs * sz > ctx->sm_count) continue;
+    int& fit = ctx->cluster_fit[sz];                        // clusters of sz blocks that fit (asked once)
+    if (sz == 1) fit = ctx->sm_count;
+    if (fit == 0 && (DH == 128 ? launch_form<128>(p, ctx->sm_count / sz * sz, cfg.max_batch, sz, st, &fit)
+                               : launch_form<64>(p, ctx->sm_count / sz * sz, cfg.max_batch, sz, st, &fit)) != cudaSuccess) {
+      cudaGetLastError();
+      fit = -1;
+    }
+    if (fit < pairs) continue;
+    p.pieces = c; size = sz; n_ctas = fit * sz;
+    break;
+  }
+  p.n_groups = n_ctas / p.n_mblocks;
   {
     ProfScope ps(ctx, SPACE_K_ATTN, st);
-    if (a->page_table) {
-      if (DH == 128) launch_main<128, true>(p, pl.n_ctas, cfg.max_batch, st);
-      else launch_main<64, true>(p, pl.n_ctas, cfg.max_batch, st);
-    } else {
-      if (DH == 128) launch_main<128, false>(p, pl.n_ctas, cfg.max_batch, st);
-      else launch_main<64, false>(p, pl.n_ctas, cfg.max_batch, st);
-    }
+    if (DH == 128) launch_form<128>(p, n_ctas, cfg.max_batch, size, st);
+    else launch_form<64>(p, n_ctas, cfg.max_batch, size, st);
   }
-  {
+  if (!p.pieces) {
+    const int m_valid_max = p.rows_per_mb * p.G;
+    const dim3 mgrid(p.merge_by_owner ? n_ctas : a->batch * p.H_kv * p.n_mblocks, (m_valid_max * (DH / 4) + 127) / 128);
     ProfScope ps(ctx, SPACE_K_MERGE, st);
     if (DH == 128) launch_pdl(attn_merge_kernel<128>, mgrid, dim3(128), 0, st, p);
     else launch_pdl(attn_merge_kernel<64>, mgrid, dim3(128), 0, st, p);
+    ctx->launches += 1;
   }
-  ctx->launches += 2;
+  ctx->launches += 1;
   return cuda_ok(cudaGetLastError());
 }

@@ -141,7 +141,8 @@ struct space_ctx {
   float* attn_part;        // split partials
   size_t attn_part_slots;
   int* counters;           // [4][max_batch] self-resetting arrival counters
-  int* merge_cnt;          // attention split arrivals, one per (sequence, kv head, row block)
+  int* merge_cnt;          // attention, row kernel: cut descriptors, one per (sequence, kv head, row block), and owners
+  int* arrived;            // attention: pieces of a cut that are stored, one per (sequence, kv head, row block)
   VerifyPartial* vpart;    // [max_batch][k_max+2][SPACE_VERIFY_MAX_CHUNKS]
   VerifyRow* vrow;         // [max_batch][k_max+1]
   VerifyPartial* vfused;   // [max_batch][SPACE_MAX_ROWS][16] single-launch greedy path
@@ -163,6 +164,7 @@ struct space_ctx {
   // cached block layout (Eq. 5 mask rows) and the attention kernel's visibility words, per (k, mask variant)
   int lay_k, lay_variant;                // lay_k = 0: nothing cached
   uint64_t lay_mask[SPACE_MAX_ROWS];
+  int cluster_fit[17];                   // transposed attention kernel: resident clusters of that many blocks (0: not asked yet)
   int visq_k, visq_variant;
   uint64_t visq[2][SPACE_MAX_ROWS];
   // cached TMA descriptors

@@ -28,7 +28,7 @@ int config_supported(const space_config* c) {
 }
 
 struct Carve {
-  size_t attn_part, counters, merge_cnt, vtopk, vpart, vfused, vrow, status, lm_part, lm_gather, lm_counter, stage, total;
+  size_t attn_part, counters, merge_cnt, arrived, vtopk, vpart, vfused, vrow, status, lm_part, lm_gather, lm_counter, stage, total;
   size_t part_slots;
   // staging sub-offsets (relative to stage)
   size_t st_q, st_k, st_v, st_logits, st_small;
@@ -43,6 +43,8 @@ Carve carve(const space_config* c, int sm_count) {
   v.merge_cnt = off;
   // up to 8 row blocks, one {first, count} pair each; then one word per thread block of the attention grid
   off += align_up((size_t)c->max_batch * c->n_kv_heads * 8 * sizeof(int2) + (size_t)(sm_count + 8) * sizeof(int), 256);
+  // pieces of a cut that are stored, per (sequence, kv head, row block)
+  v.arrived = off; off += align_up((size_t)c->max_batch * c->n_kv_heads * 8 * sizeof(int), 256);
   v.vtopk = off; off += align_up(verify_filter_scratch_bytes(c->max_batch, c->k_max), 256);
   v.vpart = off;
   off += align_up((size_t)c->max_batch * (c->k_max + 2) * SPACE_VERIFY_MAX_CHUNKS * sizeof(VerifyPartial), 256);
@@ -212,6 +214,7 @@ int space_create(space_ctx** out, const space_config* cfg) {
   ctx->attn_part_slots = cv.part_slots;
   ctx->counters = (int*)(ctx->ws + cv.counters);
   ctx->merge_cnt = (int*)(ctx->ws + cv.merge_cnt);
+  ctx->arrived = (int*)(ctx->ws + cv.arrived);
   ctx->vpart = (VerifyPartial*)(ctx->ws + cv.vpart);
   ctx->vtopk = ctx->ws + cv.vtopk;
   ctx->vrow = (VerifyRow*)(ctx->ws + cv.vrow);

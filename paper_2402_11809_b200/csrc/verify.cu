@@ -625,16 +625,9 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
 #ifdef SPACE_TIMELINE
   if (st.m != 12345.f) TLV(2);                              // (a use of the result: the stamp follows the loads)
 #endif
-  // KV commit on board: which candidates are accepted is known only to the last block, at the very
-  // end, so every block moves its slice of ALL k candidate rows now, while the logits stream.
-  // Rows L+1 .. L+i* end up exactly as the plain commit leaves them; rows L+i*+1 .. L+k, which lie
-  // beyond the new length and held mask-token rows nobody reads again, receive the rejected
-  // candidates' rows instead.
-  if (p.do_commit && commit_fits(p.cm, Lc))
-    commit_rows_impl<PAGED>(p.cm, b, Lc, p.k, row_i * p.n_chunks + ch, p.n_q * p.n_chunks, threadIdx.x, blockDim.x);
   // ---- block result and arrival: two block barriers in all.  Every warp reduces its own
   // (maximum, arg-max, sum); eight lanes of warp 0 combine the warps, and lane 0 publishes the
-  // chunk's result, fences it and counts the block in.
+  // chunk's result and counts the block in (one 16-byte store, one release-acquire atomic).
   constexpr int NW = SPACE_VERIFY_THREADS / 32;
   __shared__ float wm[NW], ws[NW];
   __shared__ int wi[NW];
@@ -647,7 +640,7 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
     sv = warp_sum(sv);
     if (lane == 0) { wm[warp] = m; wi[warp] = idx; ws[warp] = sv; }
   }
-  __syncthreads();
+  __syncthreads();                                          // (also: every thread's read of the old length precedes the arrival)
   VerifyPartial* pb = fpart + (int64_t)b * SPACE_MAX_ROWS * SPACE_FUSED_MAX_CHUNKS;
   if (warp == 0) {
     float m = lane < NW ? wm[lane] : -CUDART_INF_F;
@@ -657,83 +650,77 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
     float sv = (lane < NW && own > -CUDART_INF_F) ? ws[lane] * fast_exp2((own - m) * C1) : 0.f;
     sv = warp_sum(sv, NW);
     if (lane == 0) {
-      Stat r = stat_empty();
-      r.m = m; r.idx = idx; r.s = sv;
-      store_partial(pb + row_i * p.n_chunks + ch, r);
-      __threadfence();
-      const int prev = atomicAdd(p.counter_a + b, 1);
+      __stcg(reinterpret_cast<float4*>(pb + row_i * p.n_chunks + ch), make_float4(m, sv, 0.f, __int_as_float(idx)));
+      int prev;
+      asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(prev) : "l"(p.counter_a + b) : "memory");
       const int last = prev == p.n_q * p.n_chunks - 1;
       if (last) p.counter_a[b] = 0;                         // ready for the next launch
       sh_last = last;
     }
+  } else if (p.do_commit && commit_fits(p.cm, Lc)) {
+    // KV commit on board: which candidates are accepted is known only to the last block, at the very
+    // end, so every block moves its slice of ALL k candidate rows (warp 0 has the arrival to make, whose
+    // release would wait for its stores).  Rows L+1 .. L+i* end up exactly as the plain commit leaves
+    // them; rows L+i*+1 .. L+k, which lie beyond the new length and held mask-token rows nobody reads
+    // again, receive the rejected candidates' rows instead.
+    commit_rows_impl<PAGED>(p.cm, b, Lc, p.k, row_i * p.n_chunks + ch, p.n_q * p.n_chunks, threadIdx.x - 32, SPACE_VERIFY_THREADS - 32);
   }
-  __syncthreads();                                          // (also: every thread's read of the old length precedes the arrival)
+  __syncthreads();
   TLV(3);
   if (!sh_last) return;
-  // (No fence on this side: every chunk result was fenced by its writer before that block's count, the
-  // counts are ordered in L2, and the loads below go to L2 -- after the barrier that followed lane 0's own
-  // count.  A fence here would also wait for this thread's row stores of the commit.)
+  // (No fence here: every chunk result was released by its writer before that block's count, the acquire was
+  // lane 0's, and the loads below go to L2 after the barrier that followed it.)
 
   // ---- last block of sequence b -------------------------------------------
   __shared__ float row_s[SPACE_MAX_ROWS];
   __shared__ int row_idx[SPACE_MAX_ROWS];
-  __shared__ int sh_cand[SPACE_MAX_K];
-  if (threadIdx.x < p.k) sh_cand[threadIdx.x] = my_cand;
   // two rows per warp at a time: lanes 0..15 and 16..31 each fetch and reduce one row's chunk results
   // (all fetches of a warp are in flight together)
   constexpr int RPW = (SPACE_MAX_ROWS + 2 * NW - 1) / (2 * NW);   // row pairs per warp at most
-  float pm[RPW], ps[RPW]; int pi[RPW];
+  float4 pr[RPW];
   const int cl = lane & 15;
 #pragma unroll
   for (int it = 0; it < RPW; ++it) {
     const int r = (warp + it * NW) * 2 + (lane >> 4);
-    pm[it] = -CUDART_INF_F; ps[it] = 0.f; pi[it] = 0x7FFFFFFF;
-    if (r < p.n_q && cl < p.n_chunks) {
-      const VerifyPartial* q = pb + r * p.n_chunks + cl;
-      pm[it] = __ldcg(&q->m); ps[it] = __ldcg(&q->s); pi[it] = __ldcg(&q->idx);
-    }
+    pr[it] = make_float4(-CUDART_INF_F, 0.f, 0.f, __int_as_float(0x7FFFFFFF));
+    if (r < p.n_q && cl < p.n_chunks) pr[it] = __ldcg(reinterpret_cast<const float4*>(pb + r * p.n_chunks + cl));
   }
 #pragma unroll
   for (int it = 0; it < RPW; ++it) {
     const int r = (warp + it * NW) * 2 + (lane >> 4);
-    float bm = pm[it]; int bi = pi[it];
+    float bm = pr[it].x; int bi = __float_as_int(pr[it].w);
     warp_max_idx(bm, bi, 16);
-    float sv = (pm[it] > -CUDART_INF_F) ? ps[it] * fast_exp2((pm[it] - bm) * C1) : 0.f;
+    float sv = (pr[it].x > -CUDART_INF_F) ? pr[it].y * fast_exp2((pr[it].x - bm) * C1) : 0.f;
     sv = warp_sum(sv, 16);
     if (cl == 0 && r < p.n_q) { row_s[r] = sv; row_idx[r] = bi; }
   }
   __syncthreads();
   TLV(4);
-  if (threadIdx.x >= 32) return;
-  // acceptance: longest prefix of candidates equal to the arg-max chain
-  int i_star = 0, bits = 0;
-  for (int t = 0; t < p.k; ++t) {
-    const int c = sh_cand[t];
-    if (c < 0 || c >= p.V) bits |= SPACE_ST_BAD_CANDIDATE;
-  }
-  while (i_star < p.k && sh_cand[i_star] >= 0 && sh_cand[i_star] < p.V &&
-         sh_cand[i_star] == row_idx[i_star * k1]) ++i_star;
+  if (warp != 0) return;
+  // acceptance: longest prefix of candidates equal to the arg-max chain (lane t holds candidate c_{t+1})
   const int j = lane;
-  if (j < k1) {
-    int tok = (j < i_star) ? sh_cand[j] : (j == i_star ? row_idx[i_star * k1] : -1);
-    const bool is_eos = p.eos_id >= 0 && j <= i_star && tok == p.eos_id;
-    const unsigned eos_mask = __ballot_sync((1u << k1) - 1u, is_eos);
-    const int n_out = eos_mask ? __ffs(eos_mask) - 1 : i_star + 1;
-    p.out_tokens[b * k1 + j] = (j < n_out) ? tok : -1;
-    if (j < p.k) {                                          // next candidate j+1 from mask row (i*, j+1)
-      const int mr = i_star * k1 + j + 1;
-      p.next_cand[b * p.k + j] = row_idx[mr];
-      p.next_cand_prob[b * p.k + j] = 1.f / row_s[mr];      // softmax at T = 1 of its own maximum
-    }
-    if (j == 0) {
-      p.n_accept[b] = i_star;
-      p.n_out[b] = n_out;
-      p.finished[b] = (uint8_t)(eos_mask != 0);
-      if (p.status && bits) atomicOr(p.status + b, bits);
-      // new length and index tables; every block of the sequence read the old length before it arrived
-      if (p.do_commit) commit_tables(p.cm, b, Lc, i_star, commit_fits(p.cm, Lc));
-      TLV(5);
-    }
+  const bool is_cand = j < p.k, in_range = my_cand >= 0 && my_cand < p.V;
+  const int arg = j < k1 ? row_idx[j * k1] : -1;
+  const unsigned bad = __ballot_sync(0xFFFFFFFFu, is_cand && !in_range);
+  const unsigned match = __ballot_sync(0xFFFFFFFFu, is_cand && in_range && my_cand == arg);
+  const int i_star = __ffs(~match) - 1;                     // the first that does not match (k when all do)
+  const int tok = j < i_star ? my_cand : (j == i_star ? arg : -1);
+  const unsigned eos_mask = __ballot_sync(0xFFFFFFFFu, p.eos_id >= 0 && j <= i_star && tok == p.eos_id);
+  const int n_out = eos_mask ? __ffs(eos_mask) - 1 : i_star + 1;
+  if (j < k1) p.out_tokens[b * k1 + j] = (j < n_out) ? tok : -1;
+  if (is_cand) {                                            // next candidate j+1 from mask row (i*, j+1)
+    const int mr = i_star * k1 + j + 1;
+    p.next_cand[b * p.k + j] = row_idx[mr];
+    p.next_cand_prob[b * p.k + j] = 1.f / row_s[mr];        // softmax at T = 1 of its own maximum
+  }
+  if (j == 0) {
+    p.n_accept[b] = i_star;
+    p.n_out[b] = n_out;
+    p.finished[b] = (uint8_t)(eos_mask != 0);
+    if (p.status && bad) atomicOr(p.status + b, SPACE_ST_BAD_CANDIDATE);
+    // new length and index tables; every block of the sequence read the old length before it arrived
+    if (p.do_commit) commit_tables(p.cm, b, Lc, i_star, commit_fits(p.cm, Lc));
+    TLV(5);
   }
 }
 

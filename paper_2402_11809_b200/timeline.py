@@ -4,7 +4,7 @@ The kernels carry optional %globaltimer stamps (compiled in with -DSPACE_TIMELIN
 csrc/verify.cu).  This module builds a second copy of the library with them, libspace_timeline.so, next to
 the regular one, replays a graph of eight steps of a single-sequence workload and prints, in microseconds
 after the attention kernel's dependency wait of the last step: when the attention blocks pass their stages
-(regular groups and helper groups apart), when the merge and verify blocks become resident, when their
+when the merge and verify blocks become resident, when their
 dependency waits return and when they finish.  What a kernel boundary costs and where a launch spends its
 time cannot be seen from outside the kernels: a profiler serialises the launches.
 
@@ -47,11 +47,9 @@ def main(argv):
     B.lib = lib
     name = argv[1] if len(argv) > 1 else "llama7b"
     cfg = workloads.resolve(name)
-    if cfg["B"] != 1:
-        raise SystemExit("the trace is laid out for one sequence (regular and helper groups)")
     k = cfg["k"]
     sets = [workloads.make_step_inputs(cfg, set_index=i) for i in range(8)]
-    ctx = B.Context(device=0, max_batch=1, n_q_heads=cfg["H_q"], n_kv_heads=cfg["H_kv"], head_dim=cfg["d"],
+    ctx = B.Context(device=0, max_batch=cfg["B"], n_q_heads=cfg["H_q"], n_kv_heads=cfg["H_kv"], head_dim=cfg["d"],
                     k_max=k, vocab=cfg["V"], s_cap=sets[0]["s_cap"])
     ds = [H.DeviceStep(cfg, x) for x in sets]
 
@@ -83,27 +81,26 @@ def main(argv):
     V = read(lib.space_debug_timeline_read_verify, 4096, 8)
     t0 = A[:, 2][A[:, 2] > 0].min()                          # the attention's dependency wait returns
     us = lambda x: (np.asarray(x) - t0) / 1e3
-    n_reg = (148 // cfg["H_kv"]) * cfg["H_kv"]
-    names = {3: "first request", 12: "S^T issuer at its first wait", 4: "first K tile in use", 5: "first S^T ready",
+    names = {3: "first request", 4: "first K tile in use", 5: "first S^T ready",
              6: "first P ready", 8: "last S^T ready", 9: "last P ready", 10: "last O^T done", 11: "partial stored",
+             14: "length read", 12: "pieces combined",
              13: "exit"}
     print(f"{name}: one step of a graph of eight, microseconds after the attention's dependency wait returned")
-    for cls, sel in (("regular groups", np.arange(148) < n_reg), ("helper groups", np.arange(148) >= n_reg)):
-        if not sel.any():
-            continue
-        print(f"  attention, {cls} ({int(sel.sum())} blocks): median / max")
-        for i, nm in names.items():
-            v = us(A[sel, i][A[sel, i] > 0])
-            if len(v):
-                print(f"    {nm:30s} {np.median(v):6.2f} / {v.max():6.2f}")
+    last = A[:, 2] >= t0                                     # blocks of the last launch (the grid may be smaller than the chip)
+    print(f"  attention ({int(last.sum())} blocks): median / max")
+    for i, nm in names.items():
+        v = us(A[last, i][A[last, i] > t0])
+        if len(v):
+            print(f"    {nm:30s} {np.median(v):6.2f} / {v.max():6.2f}")
     # the stamps of the last launch of each kernel: its dependency wait returned after the attention's (t0);
     # a point a block did not pass in that launch still holds an older stamp and is left out
     M, V = M[M[:, 1] > t0], V[V[:, 1] > t0]
     after = lambda T, col: T[:, col][T[:, col] > T[:, 1].min()]
-    print(f"  attention: last block out {us(A[:, 13]).max():.2f}")
-    print(f"  merge ({len(M)} blocks): resident {us(M[:, 0]).min():.2f} .. {us(M[:, 0]).max():.2f}; wait returned "
-          f"{us(M[:, 1]).min():.2f}; descriptor in registers {us(after(M, 2)).min():.2f} .. {us(after(M, 2)).max():.2f}; "
-          f"output stored {us(after(M, 3)).min():.2f} .. {us(after(M, 3)).max():.2f}")
+    print(f"  attention: last block out {us(A[last, 13]).max():.2f}")
+    if len(M):                                               # (a clustered cut has no merge kernel)
+        print(f"  merge ({len(M)} blocks): resident {us(M[:, 0]).min():.2f} .. {us(M[:, 0]).max():.2f}; wait returned "
+              f"{us(M[:, 1]).min():.2f}; descriptor in registers {us(after(M, 2)).min():.2f} .. {us(after(M, 2)).max():.2f}; "
+              f"output stored {us(after(M, 3)).min():.2f} .. {us(after(M, 3)).max():.2f}")
     fin = V[V[:, 5] > V[:, 1].min()]
     print(f"  verify + commit ({len(V)} blocks): resident {us(V[:, 0]).min():.2f} .. {us(V[:, 0]).max():.2f}; wait returned "
           f"{us(V[:, 1]).min():.2f}; logits in registers {us(V[:, 2]).min():.2f} .. {us(V[:, 2]).max():.2f}; counted in "
