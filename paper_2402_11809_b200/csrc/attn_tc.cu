@@ -772,11 +772,11 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     // behind the sixteen instructions of this one.
     if (elect_one()) {
       // B = [P_hi | P_lo]: the two 64-column blocks lie one leading-dimension stride
-      // apart, so a single product of N = 128 gives O_hi^T in columns 0..63 and
-      // O_lo^T in columns 64..127 (an instruction costs the same at every N here);
+      // apart, so a single product gives O_hi^T in columns 0..63 and O_lo^T from
+      // column 64 on (it costs 43 + N/2 cycles, two products of half the width 43 more);
       // the epilogue adds the two.  Columns past the padded query rows hold whatever
       // the shared memory held; they only reach output columns nobody reads.
-      const uint32_t idesc_pv = instr_desc_rt(128, 1, 1);   // A = V^T (d contiguous), B = P^T (queries contiguous)
+      const uint32_t idesc_pv = instr_desc_rt(64 + n_pad, 1, 1);   // A = V^T (d contiguous), B = P^T (queries contiguous)
       // V^T and P^T: 64-wide blocks TILE_N*128 bytes apart, 8-key groups 1024 bytes apart
       static_assert(S::P_PART == TILE_N * 128, "P_lo must follow P_hi at the block stride");
       const uint64_t vdesc0 = smem_desc(sm_base + S::V_OFF, TILE_N * 128, 1024);

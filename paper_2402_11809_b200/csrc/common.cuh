@@ -100,6 +100,20 @@ __device__ __forceinline__ uint4 shift_pieces(const Piece2& r, const T* row) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// Asks L2 for a chunk's first sweep of logits, for the time before a kernel's dependency wait: with a programmatic
+// launch the blocks are resident while the kernel before them still runs.  Only a request to the point of
+// coherence: whatever is still being written is what the loads after the wait will see.  (One sequence of 36
+// rows of 32000 behind its attention: step 20.6 -> 19.9 us; eight steps for two sequences 199 -> 192 us.)
+template <typename T>
+__device__ __forceinline__ void prefetch_chunk(const T* row, int begin, int end) {
+  constexpr int N = 16 / (int)sizeof(T);
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int x = begin + (u * SPACE_VERIFY_THREADS + (int)threadIdx.x) * N;
+    if ((threadIdx.x & 7) == 0 && x < end) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + x));   // (a 128-byte line)
+  }
+}
+
 // Chunks per row and their length.  A sweep of a block is four vectors per thread (8192 bf16 logits); a
 // block costs about 3 us whatever it scans (reduction, fence, arrival), so it should make one sweep while
 // there are fewer of them than about three resident blocks per SM can take at once, and up to four when

@@ -54,33 +54,50 @@ __global__ void __launch_bounds__(64) decode_begin_kernel(const DecodeParams p) 
   write_block_rows(p, b, last, p.s.kv_len[b]);
 }
 
+// Everything the step needs is fetched at once (one memory round trip: the sequence's numbers by every thread,
+// its tokens and candidates by the lanes of either warp), then only stored.
 __global__ void __launch_bounds__(64) decode_advance_kernel(const DecodeParams p) {
   pdl_launch_dependents();
   pdl_wait();
-  const int b = blockIdx.x;
-  if (p.s.finished[b]) return;                              // latched: the step's results are dropped
-  const int k = p.s.k;
+  const int b = blockIdx.x, k = p.s.k, lane = threadIdx.x & 31;
+  const bool was_finished = p.s.finished[b] != 0;
   const int have = p.s.n_tokens[b];
   int n = p.n_out[b];
+  const bool step_done = p.step_finished[b] != 0;
+  const int L = p.kv_len_next[b], old_last = p.s.last_token[b];
+  const int tok = lane <= k ? p.out_tokens[b * (k + 1) + lane] : 0;
+  const int cand = lane < k ? p.next_cand[b * k + lane] : 0;
+  const float prob = lane < k ? p.next_cand_prob[b * k + lane] : 0.f;
   n = max(0, min(n, k + 1));
+  const int last_out = __shfl_sync(0xFFFFFFFFu, tok, max(n - 1, 0));
+  __syncthreads();                                          // every thread has read the old state
+  if (was_finished) return;                                 // latched: the step's results are dropped
   const int room = p.s.max_tokens - have;
   const bool full = n >= room;                              // the output buffer ends the sequence too
   const int n_take = min(n, room);
-  if (threadIdx.x < n_take) p.s.tokens[(int64_t)b * p.s.max_tokens + have + threadIdx.x] = p.out_tokens[b * (k + 1) + threadIdx.x];
-  const bool done = p.step_finished[b] != 0 || full;
-  const int last = n > 0 ? p.out_tokens[b * (k + 1) + n - 1] : p.s.last_token[b];
-  const int L = p.kv_len_next[b];
-  if (!done && threadIdx.x < k) {                           // the candidates of the next step
-    p.s.cand[b * k + threadIdx.x] = p.next_cand[b * k + threadIdx.x];
-    p.s.cand_prob[b * k + threadIdx.x] = p.next_cand_prob[b * k + threadIdx.x];
-  }
-  __syncthreads();                                          // every thread has read the old state
+  const bool done = step_done || full;
+  const int last = n > 0 ? last_out : old_last;
+  if ((int)threadIdx.x < n_take) p.s.tokens[(int64_t)b * p.s.max_tokens + have + threadIdx.x] = tok;
   if (threadIdx.x == 0) {
     p.s.n_tokens[b] = have + n_take;
     if (done) p.s.finished[b] = 1;
     else { p.s.last_token[b] = last; p.s.kv_len[b] = L; }
   }
-  if (!done) write_block_rows(p, b, last, L);
+  if (done) return;
+  if ((int)threadIdx.x < k) {                               // the candidates of the next step
+    p.s.cand[b * k + threadIdx.x] = cand;
+    p.s.cand_prob[b * k + threadIdx.x] = prob;
+  }
+  // block rows of the next step (see write_block_rows; candidate g lies in lane g - 1)
+  const int k1 = k + 1;
+  for (int i0 = 0; i0 < p.n_q; i0 += 64) {
+    const int i = i0 + threadIdx.x, g = i / k1, o = i - g * k1;
+    const int c = __shfl_sync(0xFFFFFFFFu, cand, (g - 1) & 31);
+    if (i < p.n_q) {
+      p.s.block_tokens[b * p.n_q + i] = o != 0 ? p.s.mask_token_id : (g == 0 ? last : c);
+      p.s.block_pos[b * p.n_q + i] = L + p.relpos[i];
+    }
+  }
 }
 
 int fill(space_ctx* ctx, const space_decode_state* s, DecodeParams* p) {

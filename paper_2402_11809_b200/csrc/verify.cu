@@ -417,11 +417,12 @@ template <typename T, bool ALIGNED>
 __global__ void __launch_bounds__(SPACE_VERIFY_THREADS)
 verify_target_kernel(const VerifyParams p) {
   pdl_launch_dependents();
-  pdl_wait();
   const int b = blockIdx.z, t = blockIdx.y, ch = blockIdx.x;
   const int k1 = p.k + 1;
   const T* row = reinterpret_cast<const T*>(p.logits) + ((int64_t)b * p.n_q + (int64_t)t * k1) * p.row_stride;
   const int begin = ch * p.chunk, end = min(p.V, begin + p.chunk);
+  prefetch_chunk<T>(row, begin, end);
+  pdl_wait();
   Stat st = scan_chunk<T, ALIGNED, false, STAT_SUM>(row, begin, end, p.c_t, -1, 0, 0, 0, 0, 0);
   st = block_reduce_plain(st, p.c_t);
   VerifyPartial* part = p.part + ((int64_t)b * (p.k + 2) + t) * p.n_chunks;
@@ -615,6 +616,7 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
   constexpr float C1 = 1.4426950408889634f;                 // T = 1
   const T* row = reinterpret_cast<const T*>(p.logits) + ((int64_t)b * p.n_q + row_i) * p.row_stride;
   const int begin = ch * p.chunk, end = min(p.V, begin + p.chunk);
+  prefetch_chunk<T>(row, begin, end);
   pdl_wait();
   TLV(1);
   int Lc = 0;

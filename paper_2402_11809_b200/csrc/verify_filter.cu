@@ -259,16 +259,19 @@ template <typename T, bool ALIGNED>
 __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltParams p) {
   __shared__ FiltShared sh;
   pdl_launch_dependents();
-  pdl_wait();
   const int b = blockIdx.z, r = blockIdx.y, ch = blockIdx.x;
   const int k1 = p.k + 1, K = p.top_k;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_rows = gridDim.y;
+  const int begin = ch * p.chunk, end = min(p.V, begin + p.chunk);
+  if (p.phase != PHASE_MASKS)                              // (which mask rows are read is not known yet)
+    prefetch_chunk<T>(reinterpret_cast<const T*>(p.logits) + ((int64_t)b * p.n_q + (p.phase == PHASE_TARGETS ? r * k1 : r)) * p.row_stride,
+                      begin, end);
+  pdl_wait();
   const int i_star0 = p.phase == PHASE_MASKS ? max(0, min(p.n_accept[b], p.k)) : 0;
   // target row r, mask row (i*, r+1), or block row r
   const int brow = p.phase == PHASE_TARGETS ? r * k1 : p.phase == PHASE_MASKS ? i_star0 * k1 + r + 1 : r;
   const T* row = reinterpret_cast<const T*>(p.logits) + ((int64_t)b * p.n_q + brow) * p.row_stride;
-  const int begin = ch * p.chunk, end = min(p.V, begin + p.chunk);
   int Lc = 0;
   if (p.do_commit) {                                        // (phase 1: i* is known, every block moves its slice)
     Lc = p.cm.kv_len[b];
