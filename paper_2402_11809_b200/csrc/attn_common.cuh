@@ -1,0 +1,247 @@
+// What the two tensor-core attention kernels (attn_tc.cu, attn_rows.cu) share: how partial results of a
+// (sequence, kv head, query-row block) that was cut over several thread blocks are combined, either in the
+// shared memory of a cluster or, from global memory, by the block that stored the last of them.  `P` is a
+// kernel's parameter struct (G, H_q, n_q, n_mblocks, out_dtype, out, lse, part).
+#pragma once
+#include "common.cuh"
+#include "tc_common.cuh"
+#include <math_constants.h>
+
+namespace attn {
+
+constexpr int ROWS = 128;              // query rows of a partial's slot in global memory
+constexpr int MAX_CLUSTER = 16;        // blocks per cluster (more than 8 need the opt-in)
+// The clustered cut is taken while its longest piece has at most this many tiles more than an even share of
+// all tiles: that is about what the cut over the grid costs on top (starting more than one share per block,
+// the merge in global memory).
+constexpr int CLUSTER_SLACK = 10;
+
+// Shared memory of another block of the cluster.
+__device__ __forceinline__ uint32_t map_cluster(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t a) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
+}
+
+// Query row r of the row block that starts at block row i0, columns 4 c4 .. of (sequence b, kv head h).
+template <int DH, class P>
+__device__ __forceinline__ void store_out(const P& p, int b, int h, int i0, int r, int c4, const float4& v) {
+  const int gsh = __ffs(p.G) - 1;                           // G is a power of two
+  const int ri = i0 + (r >> gsh), hq = h * p.G + (r & (p.G - 1));
+  const size_t off = (((size_t)b * p.n_q + ri) * p.H_q + hq) * DH + c4 * 4;
+  if (p.out_dtype == SPACE_DTYPE_F32) {
+    *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + off) = v;
+  } else {
+    const __nv_bfloat162 x = __floats2bfloat162_rn(v.x, v.y), y = __floats2bfloat162_rn(v.z, v.w);
+    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + off) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&x), *reinterpret_cast<const uint32_t*>(&y));
+  }
+}
+template <class P>
+__device__ __forceinline__ void store_lse(const P& p, int b, int h, int i0, int r, float v) {
+  const int gsh = __ffs(p.G) - 1;
+  p.lse[((size_t)b * p.H_q + h * p.G + (r & (p.G - 1))) * p.n_q + i0 + (r >> gsh)] = v;
+}
+
+// Four output elements of one query row from the partials of a cut: running reference, denominator and
+// accumulator.
+struct MergeAcc {
+  float mx, den;
+  float4 a;
+  __device__ __forceinline__ void clear() { mx = -CUDART_INF_F; den = 0.f; a = make_float4(0.f, 0.f, 0.f, 0.f); }
+  __device__ __forceinline__ void add(float m, float l, const float4& o) {
+    const float mn = fmaxf(mx, m);
+    if (mn > -CUDART_INF_F) {
+      const float e0 = tc::fast_exp2(mx - mn), e1 = tc::fast_exp2(m - mn);
+      den = den * e0 + l * e1;
+      a.x = a.x * e0 + o.x * e1; a.y = a.y * e0 + o.y * e1;
+      a.z = a.z * e0 + o.z * e1; a.w = a.w * e0 + o.w * e1;
+    }
+    mx = mn;
+  }
+  template <int DH, class P>
+  __device__ __forceinline__ void store(const P& p, int b, int h, int i0, int r, int c4) const {
+    const float rd = 1.f / den;
+    store_out<DH>(p, b, h, i0, r, c4, make_float4(a.x * rd, a.y * rd, a.z * rd, a.w * rd));
+    if (p.lse && c4 == 0) store_lse(p, b, h, i0, r, (mx + log2f(den)) * 0.6931471805599453f);
+  }
+};
+
+// The pieces of a cluster's pair meet: every block combines its part of the rows from all pieces' shared
+// memory (o_at / m_at / l_at: addresses of the accumulators, references and sums, the same in every block).
+// All threads of the cluster's blocks take part, those of a piece without tiles too; every wait before this
+// is bounded, so all of them arrive.  cluster_leave() must follow before the block exits.
+template <int DH, class P>
+__device__ __forceinline__ void cluster_merge(const P& p, int b, int h, int i0, int m_valid, int piece, int pieces, int n,
+                                              int mb, uint32_t o_at, uint32_t m_at, uint32_t l_at, volatile int* abort_flag) {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  const int stride = pieces * (int)blockDim.x;
+  for (int idx = piece * (int)blockDim.x + (int)threadIdx.x; idx < m_valid * (DH / 4) && !*abort_flag; idx += stride) {
+    const int r = idx / (DH / 4), c4 = idx % (DH / 4);
+    MergeAcc acc;
+    acc.clear();
+    for (int x0 = 0; x0 < n; x0 += 4) {                     // all loads of a batch are issued before any is used
+      float ms[4], ls[4];
+      float4 ov[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (x0 + j < n) {
+          const uint32_t rank = (uint32_t)((x0 + j) * p.n_mblocks + mb);
+          ms[j] = ld_cluster(map_cluster(m_at + r * 4, rank));
+          ls[j] = ld_cluster(map_cluster(l_at + r * 4, rank));
+          ov[j] = ld_cluster4(map_cluster(o_at + (r * DH + c4 * 4) * 4, rank));
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (x0 + j < n) acc.add(ms[j], ls[j], ov[j]);
+    }
+    acc.template store<DH>(p, b, h, i0, r, c4);
+  }
+  // No block leaves while another may still read its shared memory: this half says that this block has read
+  // (relaxed: nothing is handed over, so it need not wait for the output's stores).
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_leave() {
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+}
+
+// Clusters were launched, but the lengths are too unequal for them: the piece that finds all the others stored
+// combines them from global memory (no merge kernel follows such a launch).  As the rule for larger batches
+// this was slower, 137 against 130 us on sixteen ragged sequences: every piece waits for its fence and its
+// atomic.  Called by `nt` threads (tid 0 .. nt-1, whole warps) that `sync` synchronises, after all of them have
+// stored their piece; cut: {first slot, pieces}, read from thread 0.  buf: buf_floats floats of shared memory.
+template <int DH, class P, class Sync>
+__device__ __forceinline__ void merge_if_last(const P& p, int b, int h, int i0, int m_valid, int mb, int2 cut, int* arrived,
+                                              float* buf, int buf_floats, int tid, int nt, Sync sync) {
+  int* flag = reinterpret_cast<int*>(buf);
+  if (tid == 0) {
+    __threadfence();                                        // (the barrier before ordered every thread's stores before this)
+    const int last = atomicAdd(arrived, 1) == cut.y - 1;
+    if (last) { *arrived = 0; __threadfence(); }            // ready for the next launch
+    flag[0] = last; flag[1] = cut.x; flag[2] = cut.y;
+  }
+  sync();
+  const bool last = flag[0] != 0;
+  const int d0 = flag[1], n = flag[2];
+  sync();                                                   // (the flags' place is used below)
+  if (!last) return;
+  const size_t slot_floats = (size_t)ROWS * (DH + 2), gstride = (size_t)p.n_mblocks * slot_floats;
+  const float* ps = p.part + ((size_t)d0 * p.n_mblocks + mb) * slot_floats;
+  const int warp = tid >> 5, lane = tid & 31;
+  // rows in batches whose weights exp2(m - M) / sum fit the buffer: n floats per row
+  const int at_once = min(m_valid, buf_floats / n);
+  for (int r0 = 0; r0 < m_valid; r0 += at_once) {
+    const int nr = min(at_once, m_valid - r0);
+    for (int rr = warp; rr < nr; rr += nt >> 5) {
+      const float* pr = ps + ROWS * DH + r0 + rr;
+      float M = -CUDART_INF_F, den = 0.f;
+      for (int x = lane; x < n; x += 32) M = fmaxf(M, __ldcg(pr + (size_t)x * gstride));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
+      for (int x = lane; x < n; x += 32) {
+        const float e = tc::fast_exp2(__ldcg(pr + (size_t)x * gstride) - M);
+        buf[rr * n + x] = e;
+        den = fmaf(__ldcg(pr + (size_t)x * gstride + ROWS), e, den);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xFFFFFFFFu, den, o);
+      const float rd = 1.f / den;
+      for (int x = lane; x < n; x += 32) buf[rr * n + x] *= rd;
+      if (p.lse && lane == 0) store_lse(p, b, h, i0, r0 + rr, (M + log2f(den)) * 0.6931471805599453f);
+    }
+    sync();
+    for (int idx = tid; idx < nr * (DH / 4); idx += nt) {
+      const int rr = idx / (DH / 4), c4 = idx % (DH / 4);
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+      const float* po = ps + (size_t)(r0 + rr) * DH + c4 * 4;
+      for (int x0 = 0; x0 < n; x0 += 16) {                  // all loads of a batch are issued before any is used
+        float4 ov[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          ov[j] = x0 + j < n ? __ldcg(reinterpret_cast<const float4*>(po + (size_t)(x0 + j) * gstride)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const float w = x0 + j < n ? buf[rr * n + x0 + j] : 0.f;
+          a.x = fmaf(ov[j].x, w, a.x); a.y = fmaf(ov[j].y, w, a.y);
+          a.z = fmaf(ov[j].z, w, a.z); a.w = fmaf(ov[j].w, w, a.w);
+        }
+      }
+      store_out<DH>(p, b, h, i0, r0 + rr, c4, a);
+    }
+    sync();
+  }
+}
+
+// Whether the clustered cut serves these lengths (all lanes of a warp call this; every warp gets the same
+// answer): the longest piece in tiles against an even share.  tiles_of(L): tiles of a sequence of length L.
+template <class P, class F>
+__device__ __forceinline__ bool cluster_fits(const P& p, int lane, F tiles_of) {
+  int Tmax = 0, W = 0;
+  if (p.B == 1) {
+    Tmax = W = tiles_of(p.kv_len[0]);
+  } else {
+    for (int b0 = 0; b0 < p.B; b0 += 32) {
+      const int T = b0 + lane < p.B ? tiles_of(p.kv_len[b0 + lane]) : 0;
+      Tmax = max(Tmax, __reduce_max_sync(0xFFFFFFFFu, T));
+      W += __reduce_add_sync(0xFFFFFFFFu, T);
+    }
+  }
+  return (Tmax + p.pieces - 1) / p.pieces <= (W * p.H_kv + p.n_groups - 1) / p.n_groups + CLUSTER_SLACK;
+}
+
+// Host side: launch with programmatic serialization and, when size > 1, clusters of `size` blocks; with
+// max_clusters, no launch but the number of such clusters that can be resident.
+template <typename K, typename... Args>
+static inline cudaError_t launch_clusters(K kernel, int n_ctas, int threads, size_t smem, int size, cudaStream_t st,
+                                          int* max_clusters, const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_ctas); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = size; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  if (max_clusters) {
+    cfg.attrs = attr + 1; cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(max_clusters, kernel, &cfg);
+  }
+  cfg.attrs = attr; cfg.numAttrs = size > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// The clustered cut of `pairs` (sequence, kv head) pairs: as many pieces as there are SMs for (and tiles a
+// sequence may have), in clusters of pieces * n_mblocks blocks that fit next to one another.  fit[size]:
+// clusters of that size that can be resident, 0 = not asked yet (ask(size) tells).  Returns the pieces (0: more
+// pairs than fit) and the number of clusters that fill the chip.
+template <typename Ask>
+static inline int plan_clusters(int pairs, int n_mblocks, int64_t cap_tiles, int sm_count, int* fit, Ask ask, int* n_clusters) {
+  for (int c = cap_tiles < MAX_CLUSTER / n_mblocks ? (int)cap_tiles : MAX_CLUSTER / n_mblocks; c >= 1; --c) {
+    const int size = c * n_mblocks;
+    if (pairs * size > sm_count) continue;
+    if (fit[size] == 0) {
+      if (size == 1) fit[size] = sm_count;
+      else if (ask(size, &fit[size]) != cudaSuccess || fit[size] == 0) { cudaGetLastError(); fit[size] = -1; }
+    }
+    if (fit[size] < pairs) continue;
+    *n_clusters = fit[size];
+    return c;
+  }
+  return 0;
+}
+
+}  // namespace attn

@@ -14,13 +14,13 @@
 // and the block drains and exits.
 #include "common.cuh"
 #include "tc_common.cuh"
+#include "attn_common.cuh"
 #include <cuda.h>
 #include <math_constants.h>
 
 namespace {
 
 constexpr int TILE_N = 128;            // keys per tile
-constexpr int ROWS = 128;              // MMA M
 constexpr int THREADS = 384;            // K (+Q), S-issuer, V, O-issuer warps + 8 softmax warps
 constexpr uint64_t WAIT_NS = 1000000000ull;   // one second per wait
 constexpr float RESCALE_THRESHOLD = 8.f;
@@ -33,6 +33,7 @@ struct AttnParams {
   int B, n_q, H_q, H_kv, G;
   int n_mblocks, rows_per_mb;          // query-row blocks per kv head; block rows i per block
   int n_groups;                        // thread-block groups (grid = n_groups * n_mblocks)
+  int pieces;                          // > 0: the grid is cut into clusters of pieces * n_mblocks blocks, one per (sequence, head)
   int out_dtype;
   int64_t s_cap;                       // rows a sequence may hold (paged: pages_per_seq * SPACE_PAGE_SIZE)
   // Paged cache (page_table != nullptr): tm_k / tm_v describe a pool [n_pages][H_kv][TILE_N][d] and tile t
@@ -47,22 +48,26 @@ struct AttnParams {
   int2* desc;                          // [B*H_kv*n_mblocks] {first group, number of groups} of each cut
   int* owner;                          // [grid] (sequence, kv head) whose last piece this thread block computed, or -1
   int merge_by_owner;                  // the merge grid is indexed by attention thread block, not by (sequence, head)
+  int* arrived;                        // [B*H_kv*n_mblocks] pieces of a cut whose partial is stored (self-resetting)
   uint64_t mask[SPACE_MAX_ROWS];
 };
 
-struct Seg { int b, h, t0, t1, T, L; };
+// One share: tiles t0, t0 + step, ... (n of them) of the T tiles of (sequence b, kv head h).
+struct Seg { int b, h, t0, n, step, T, L; };
 
 // Page of tile t of sequence b (paged cache).  An entry outside the pool is flagged and answered
 // with a page past the pool's end: the TMA load then fills the tile with zeros.
-__device__ __forceinline__ int page_of(const AttnParams& p, int b, int t) {
+// (flag = false: a request made before the length is known, for a tile the sequence may not have.)
+__device__ __forceinline__ int page_of(const AttnParams& p, int b, int t, bool flag = true) {
   const int pg = t < p.pages_per_seq ? p.page_table[(int64_t)b * p.pages_per_seq + t] : -1;
   if (pg >= 0 && pg < p.n_pages) return pg;
-  if (p.status) atomicOr(p.status + b, SPACE_ST_BAD_PAGE);
+  if (flag && p.status) atomicOr(p.status + b, SPACE_ST_BAD_PAGE);
   return p.n_pages;
 }
 
 // PTX helpers: tc_common.cuh.  Every wait of this kernel is bounded by WAIT_NS.
 using namespace tc;
+using namespace attn;
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site) {
   return mbar_wait_bounded(bar, parity, abort_flag, err, site, WAIT_NS, 0);
 }
@@ -112,10 +117,12 @@ struct Partition {
   int B, H_kv, n_q;
   long long cur, end;
   int b;
+  const int* one;        // clustered cut: {b, h, t0, n, T, L, step}, this block's only share
+  __device__ void init_one(const int* share) { one = share; cur = 0; end = share[3] > 0 ? 1 : 0; }
   // Only min(n_groups, W) groups take part, so every taking-part group owns at
   // least one tile and the groups of one (sequence, head) are consecutive.
   __device__ void init(const int* sl, const int* pf, int B_, int H, int nq, int group, int n_groups) {
-    seq_len = sl; prefix = pf; B = B_; H_kv = H; n_q = nq; b = 0;
+    seq_len = sl; prefix = pf; B = B_; H_kv = H; n_q = nq; b = 0; one = nullptr;
     const long long W = pf[B_];
     const long long NG = W < n_groups ? W : n_groups;
     if (group >= NG) { cur = end = 0; return; }
@@ -123,6 +130,13 @@ struct Partition {
     end = muldiv(W, group + 1, NG);
   }
   __device__ bool next(Seg& s) {
+    if (one) {
+      if (cur >= end) return false;
+      ++cur;
+      const int4 u = reinterpret_cast<const int4*>(one)[0], v = reinterpret_cast<const int4*>(one)[1];
+      s.b = u.x; s.h = u.y; s.t0 = u.z; s.n = u.w; s.T = v.x; s.L = v.y; s.step = v.z;
+      return true;
+    }
     // The list holds T + SHARE_COST entries per (sequence, head); the first
     // SHARE_COST stand for the fixed cost of starting a share there, so that
     // equal list shares are shares of about equal time.
@@ -139,7 +153,7 @@ struct Partition {
       cur += n;
       const int t0 = max(r0 - SHARE_COST, 0), t1 = max(r0 + (int)n - SHARE_COST, 0);
       if (t1 <= t0) continue;                               // only cost entries here: no tiles
-      s.b = b; s.h = h; s.t0 = t0; s.t1 = t1; s.T = T; s.L = L;
+      s.b = b; s.h = h; s.t0 = t0; s.n = t1 - t0; s.step = 1; s.T = T; s.L = L;
       return true;
     }
   }
@@ -167,10 +181,15 @@ struct Smem {
   // q_full, q_empty, k_full[], k_empty[], v_full[], v_empty[], s_full[3], p_ready[3], pv_done[3], drain
   static constexpr int N_BARS = 2 + 2 * K_STAGES + 2 * V_STAGES + 3 * S_BUFS + 1;
   static constexpr int MISC_OFF = BAR_OFF + (N_BARS * 8 + 15) / 16 * 16;   // tmem base, abort flag
-  static constexpr int XMAX_OFF = MISC_OFF + 32;             // [2 parities][2 halves][ROWS] float
+  static constexpr int SEG0_OFF = MISC_OFF + 16;             // the only share of a clustered cut (8 ints)
+  static constexpr int XMAX_OFF = MISC_OFF + 48;             // [2 parities][2 halves][ROWS] float
   static constexpr int XSUM_OFF = XMAX_OFF + 2 * 2 * ROWS * 4;   // [2 halves][ROWS] float
   static constexpr int EPI_PITCH = 36;                       // floats per staged row: 32 columns + 4 (16-byte aligned, conflict-free)
   static constexpr int EPI_OFF = XSUM_OFF + 2 * ROWS * 4;    // [8 warps][32 rows][EPI_PITCH] float: epilogue transpose
+  // a piece's partial for the cluster, in the slot format of global memory: over the K (and V) stages, all
+  // consumed by then
+  static constexpr int PART_OFF = K_OFF;
+  static_assert(PART_OFF + ROWS * (DH + 2) * 4 <= BAR_OFF, "a partial must fit the K and V stages");
   static constexpr int TABLE_OFF = EPI_OFF + 8 * 32 * EPI_PITCH * 4;   // seq_len[max_batch], prefix[max_batch+1]
 };
 
@@ -202,6 +221,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
   float* xsum = reinterpret_cast<float*>(sm + S::XSUM_OFF);
   int* seq_len = reinterpret_cast<int*>(sm + S::TABLE_OFF);
   int* prefix = seq_len + max_batch;
+  int* seg0 = reinterpret_cast<int*>(sm + S::SEG0_OFF);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int group = blockIdx.x / p.n_mblocks, mb = blockIdx.x % p.n_mblocks;
@@ -228,7 +248,61 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (warp == WARP_MMA) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (warp == WARP_K && lane == 0)
+    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.tm_k) : "memory");
+  if (warp == WARP_V && lane == 0)
+    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.tm_v) : "memory");
+  if (warp == WARP_MMA && lane == 0)
+    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.tm_q) : "memory");
+  // Clustered cut (see attn_tc.cu): piece cl_piece of pair cl_pair, tiles cl_piece, cl_piece + pieces, ...
+  const int cl_pair = p.pieces ? group / p.pieces : 0, cl_piece = p.pieces ? group - cl_pair * p.pieces : 0;
+  const bool cl_mine = p.pieces && cl_pair < p.B * p.H_kv;
+  const int cl_b = cl_pair / p.H_kv, cl_h = cl_pair - cl_b * p.H_kv;
+  // barriers and the TMEM allocation are visible to every warp before the first global access (with a
+  // programmatic launch this part runs under the previous kernel)
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
   pdl_wait();                                              // global memory from here on
+  if (cl_mine && warp == WARP_K && lane == 0 && !*abort_flag) {
+    // the query rows and the first K tile, before any length is read (should the length turn out too short for
+    // that tile, or the cut not be taken, the S issuer lets both buffers go unused)
+    mbar_expect_tx(BAR(B_QFULL), S::Q_BYTES);
+#pragma unroll
+    for (int hf = 0; hf < S::HALVES; ++hf)
+      tma_load_4d(sm_base + S::Q_OFF + hf * (ROWS * 128), &p.tm_q, BAR(B_QFULL), hf * 64, cl_h * p.G, i0, cl_b);
+    mbar_expect_tx(BAR(B_KFULL), S::TILE_BYTES);
+#pragma unroll
+    for (int hf = 0; hf < S::HALVES; ++hf)
+      tma_load_4d(sm_base + S::K_OFF + hf * (TILE_N * 128), &p.tm_k, BAR(B_KFULL), hf * 64,
+                  p.page_table ? 0 : cl_piece * TILE_N, cl_h, p.page_table ? page_of(p, cl_b, cl_piece, false) : cl_b);
+  }
+  bool clustered = false, spec_ok = false;                 // spec_ok: the early requests serve this block's share
+  int cl_n = 0;                                            // pieces of this block's pair that have tiles
+  if (p.pieces) {
+    // every warp works the same things out for itself: nothing has to be handed over
+    auto tiles_of = [&](int L) { return (L >= 0 && (int64_t)L + p.n_q <= p.s_cap) ? (L + p.n_q + TILE_N - 1) / TILE_N : 0; };
+    const int L0 = cl_mine ? p.kv_len[cl_b] : -1;
+    clustered = cluster_fits(p, lane, tiles_of);
+    if (clustered) {
+      const int T = tiles_of(L0), L = T ? L0 : -1;
+      if (cl_mine && !T && cl_piece == 0 && cl_h == 0 && mb == 0 && threadIdx.x == 0 && p.status)
+        atomicOr(p.status + cl_b, SPACE_ST_CAPACITY);
+      const int n_mine = cl_piece < T ? (T - cl_piece + p.pieces - 1) / p.pieces : 0;
+      cl_n = min(p.pieces, T);
+      spec_ok = n_mine > 0 && (p.page_table || (cl_piece + 1) * TILE_N <= L + p.n_q);
+      if (p.page_table && spec_ok && warp == WARP_K && lane == 0) (void)page_of(p, cl_b, cl_piece);   // flags a bad entry
+      // (identical values by every thread, each reads back what it wrote)
+      reinterpret_cast<int4*>(seg0)[0] = make_int4(cl_b, cl_h, cl_piece, n_mine);
+      reinterpret_cast<int4*>(seg0)[1] = make_int4(T, L, p.pieces, 0);
+    }
+  }
+  if (!clustered) {
   if (warp == WARP_SOFTMAX0) {
     // per-sequence tile counts and their running sum, 32 sequences per round
     int carry = 0;
@@ -253,25 +327,14 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
     }
     if (lane == 0) prefix[p.B] = carry;
   }
-  if (warp == WARP_MMA) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  __syncthreads();                                          // the tables reach every warp
   }
-  if (warp == WARP_K && lane == 0)
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.tm_k) : "memory");
-  if (warp == WARP_V && lane == 0)
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.tm_v) : "memory");
-  if (warp == WARP_MMA && lane == 0)
-    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.tm_q) : "memory");
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const uint32_t TM_S0 = tmem, TM_O = tmem + S::S_BUFS * TILE_N;   // S buffers at columns 0, 128, 256; O at 384
 
   Partition part;
-  part.init(seq_len, prefix, p.B, p.H_kv, p.n_q, group, p.n_groups);
+  if (clustered) part.init_one(seg0);
+  else part.init(seq_len, prefix, p.B, p.H_kv, p.n_q, group, p.n_groups);
   Seg sg;
   const bool dead = *abort_flag != 0;
 
@@ -285,23 +348,28 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
       const int b_full = is_k ? B_KFULL : B_VFULL, b_empty = is_k ? B_KEMPTY : B_VEMPTY;
       const uint32_t ring = sm_base + (is_k ? S::K_OFF : S::V_OFF);
       const CUtensorMap* tm = is_k ? &p.tm_k : &p.tm_v;
-      uint32_t gt = 0, seg = 0;
+      // gt counts the ring's tiles; early requests that serve no share take the first place of either buffer
+      bool pre = is_k && spec_ok;                           // Q and the first K tile of the share are on their way
+      uint32_t gt = cl_mine && is_k && !spec_ok ? 1u : 0u, seg = gt;
       bool ok = true;
       while (ok && part.next(sg)) {
         const int n_keys = sg.L + p.n_q;
         if (is_k) {
           // the K producer also loads this share's query rows, once the last S
           // product of the share before has read the buffer
-          if (seg > 0) ok = mbar_wait(BAR(B_QEMPTY), (seg - 1) & 1, abort_flag, p.err, 3);
-          if (!ok) break;
-          mbar_expect_tx(BAR(B_QFULL), S::Q_BYTES);
+          if (!pre) {
+            if (seg > 0) ok = mbar_wait(BAR(B_QEMPTY), (seg - 1) & 1, abort_flag, p.err, 3);
+            if (!ok) break;
+            mbar_expect_tx(BAR(B_QFULL), S::Q_BYTES);
 #pragma unroll
-          for (int hf = 0; hf < S::HALVES; ++hf)
-            tma_load_4d(sm_base + S::Q_OFF + hf * (ROWS * 128), &p.tm_q, BAR(B_QFULL), hf * 64,
-                        sg.h * p.G, i0, sg.b);
+            for (int hf = 0; hf < S::HALVES; ++hf)
+              tma_load_4d(sm_base + S::Q_OFF + hf * (ROWS * 128), &p.tm_q, BAR(B_QFULL), hf * 64,
+                          sg.h * p.G, i0, sg.b);
+          }
           ++seg;
         }
-        for (int t = sg.t0; t < sg.t1 && ok; ++t, ++gt) {
+        for (int j = 0, t = sg.t0; j < sg.n && ok; ++j, t += sg.step, ++gt) {
+          if (pre) { pre = false; continue; }
           const int s = gt % n_st;
           if (gt >= (uint32_t)n_st)
             ok = mbar_wait(BAR(b_empty + s), ((gt / n_st) - 1) & 1, abort_flag, p.err, is_k ? 1 : 2);
@@ -327,15 +395,23 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
     // ================= S issuer ============================================
     if (elect_one()) {
       constexpr uint32_t IDESC_QK = instr_desc(TILE_N, 0);
-      uint32_t gt = 0, seg = 0;
+      uint32_t gt = 0, seg = 0, koff = 0;
       bool ok = true;
+      if (cl_mine && !spec_ok) {
+        // the early requests serve no share: once they have landed their buffers go back unused
+        ok = mbar_wait(BAR(B_QFULL), 0, abort_flag, p.err, 15);
+        if (ok) ok = mbar_wait(BAR(B_KFULL), 0, abort_flag, p.err, 16);
+        mbar_arrive(BAR(B_QEMPTY));
+        mbar_arrive(BAR(B_KEMPTY));
+        seg = 1; koff = 1;
+      }
       while (ok && part.next(sg)) {
         ok = mbar_wait(BAR(B_QFULL), seg & 1, abort_flag, p.err, 6);
-        const int n = sg.t1 - sg.t0;
+        const int n = sg.n;
         for (int j = 0; j < n && ok; ++j, ++gt) {
-          const int s = gt % S::K_STAGES;
+          const int s = (gt + koff) % S::K_STAGES;
           const uint32_t buf = gt % NS;
-          ok = mbar_wait(BAR(B_KFULL + s), (gt / S::K_STAGES) & 1, abort_flag, p.err, 7);
+          ok = mbar_wait(BAR(B_KFULL + s), ((gt + koff) / S::K_STAGES) & 1, abort_flag, p.err, 7);
           // S buffer `buf` held the P of tile gt - 3, read by that tile's O product
           if (ok && gt >= NS) ok = mbar_wait(BAR(B_PVDONE + buf), ((gt / NS) - 1) & 1, abort_flag, p.err, 8);
           if (!ok) break;
@@ -364,7 +440,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
       uint32_t g = 0;
       bool ok = true;
       while (ok && part.next(sg)) {
-        for (int t = sg.t0; t < sg.t1 && ok; ++t, ++g) {
+        for (int j = 0; j < sg.n && ok; ++j, ++g) {
           // O += (P_hi + P_lo) V; the first product of a share overwrites O
           const int s = g % S::V_STAGES;
           const uint32_t buf = g % NS;
@@ -381,7 +457,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
               // V tile is MN-major: 64-wide d blocks TILE_N*128 bytes apart, 8-key groups 1024 bytes apart
               const uint64_t bd = smem_desc(vsm + kk * 2048, TILE_N * 128, 1024);
               mma_ts(TM_O, ptm + part_i * (TILE_N / 2) + kk * 8, bd, IDESC_PV,
-                     (t == sg.t0 && kk == 0 && part_i == 0) ? 0u : 1u);
+                     (j == 0 && kk == 0 && part_i == 0) ? 0u : 1u);
             }
           }
           tc_commit(BAR(B_VEMPTY + s));
@@ -418,7 +494,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
     while (part.next(sg)) {
       const int n_keys = sg.L + p.n_q;
       float m_ref = -CUDART_INF_F, l_sum = 0.f;
-      for (int t = sg.t0; t < sg.t1; ++t, ++gt) {
+      for (int jt = 0, t = sg.t0; jt < sg.n; ++jt, t += sg.step, ++gt) {
         const uint32_t buf = gt % NS;
         ok &= mbar_wait(BAR(B_SFULL + buf), (gt / NS) & 1, abort_flag, p.err, 9);
         tc_fence_after();
@@ -468,7 +544,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
         tmax = fmaxf(tmax, xm[(half ^ 1) * ROWS + m]);
         tmax *= c;                                         // c > 0
         if (!(tmax > -CUDART_INF_F)) tmax = -CUDART_INF_F; // also catches NaN
-        const bool first = (t == sg.t0);
+        const bool first = (jt == 0);
         const bool need = !first && (tmax > m_ref + RESCALE_THRESHOLD);
         if (first) m_ref = tmax;
         if (__any_sync(0xFFFFFFFFu, need)) {
@@ -542,25 +618,28 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
       xsum[half * ROWS + m] = l_sum;
       pair_sync(quarter);
       const float l_tot = l_sum + xsum[(half ^ 1) * ROWS + m];
-      const bool whole = (sg.t0 == 0 && sg.t1 == sg.T);
+      const bool whole = sg.n == sg.T, to_smem = clustered && !whole;
       const int hq = sg.h * p.G + g;
       const int item = sg.b * p.H_kv + sg.h;
-      float* pslot = p.part + ((size_t)(item + group) * p.n_mblocks + mb) * (ROWS * (DH + 2));
+      float* pslot = to_smem ? reinterpret_cast<float*>(sm + S::PART_OFF)
+                             : p.part + ((size_t)(item + group) * p.n_mblocks + mb) * (ROWS * (DH + 2));
       const float inv = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
-      if (sidx == 0 && ok) {
-        // how this (sequence, head) was cut: first group and number of groups,
-        // read by attn_rows_merge_kernel (every group of the cut writes the same pair)
-        int2 d = make_int2(group, 1);
+      // how this (sequence, head) was cut, {first group, number of groups}: read by attn_rows_merge_kernel (every
+      // group of the cut writes the same pair)
+      int2 cut_d = make_int2(group, 1);
+      if (sidx == 0 && ok && !clustered) {
         if (!whole) {
           const long long W = prefix[p.B];
           const long long NG = W < p.n_groups ? W : p.n_groups;
           const long long f0 = (long long)prefix[sg.b] + (long long)sg.h * (sg.T + SHARE_COST) + SHARE_COST;
-          d.x = group_of(f0, W, NG);                        // group of the first tile
-          d.y = group_of(f0 + sg.T - 1, W, NG) - d.x + 1;
+          cut_d.x = group_of(f0, W, NG);                    // group of the first tile
+          cut_d.y = group_of(f0 + sg.T - 1, W, NG) - cut_d.x + 1;
         }
-        p.desc[(size_t)item * p.n_mblocks + mb] = d;
-        if (sg.t0 > 0 && sg.t1 == sg.T) own = item;        // at most one per block: only its first share can start late
+        if (!p.pieces) p.desc[(size_t)item * p.n_mblocks + mb] = cut_d;
+        if (sg.t0 > 0 && sg.t0 + sg.n == sg.T) own = item; // at most one per block: only its first share can start late
       }
+      // A partial goes to the cluster's shared memory over the K stages: every softmax thread is past the last O
+      // product by now, so all products of this block (its only share) have read them.
       // O leaves TMEM with one row per lane; written like that, a store instruction
       // would touch 32 different lines.  Each warp turns its 32 x 32 block through
       // shared memory so that eight lanes write 128 contiguous bytes of one row.
@@ -611,8 +690,20 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
           pslot[ROWS * DH + ROWS + m] = l_tot;
         }
       }
+      if (p.pieces && !clustered && !whole) {
+        auto sync = [&] { asm volatile("bar.sync 5, %0;" ::"r"(n_soft) : "memory"); };
+        sync();                                             // every thread's stores, and the staging is idle
+        cut_d.x += item;                                    // slots are numbered by item + group
+        merge_if_last<DH>(p, sg.b, sg.h, i0, m_valid, mb, cut_d, p.arrived + (size_t)item * p.n_mblocks + mb,
+                          reinterpret_cast<float*>(sm + S::EPI_OFF), 8 * 32 * S::EPI_PITCH, sidx, n_soft, sync);
+      }
     }
-    if (sidx == 0) p.owner[blockIdx.x] = own;
+    if (!p.pieces && sidx == 0) p.owner[blockIdx.x] = own;
+  }
+  if (clustered && cl_n > 1) {
+    const uint32_t at = sm_base + S::PART_OFF;
+    cluster_merge<DH>(p, cl_b, cl_h, i0, m_valid, cl_piece, p.pieces, cl_n, mb, at, at + ROWS * DH * 4, at + (ROWS * DH + ROWS) * 4,
+                      abort_flag);
   }
 
   // ---- teardown -----------------------------------------------------------
@@ -625,6 +716,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
   if (threadIdx.x == 0 && *abort_flag && p.status) {
     for (int b = 0; b < p.B; ++b) atomicOr(p.status + b, SPACE_ST_TIMEOUT);
   }
+  if (clustered && cl_n > 1) cluster_leave();
 }
 
 // Combine the partials of every (sequence, kv head, query-row block) that was
@@ -659,35 +751,13 @@ __global__ void __launch_bounds__(128) attn_rows_merge_kernel(const AttnParams p
   const size_t slot_floats = (size_t)ROWS * (DH + 2);
   const float* ps = p.part + ((size_t)(item + d.x) * p.n_mblocks + mb) * slot_floats;
   const size_t gstride = (size_t)p.n_mblocks * slot_floats;
-  float mx = -CUDART_INF_F, den = 0.f;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  MergeAcc acc;
+  acc.clear();
 #pragma unroll 8
-  for (int x = 0; x < n; ++x, ps += gstride) {
-    const float ms = __ldcg(ps + ROWS * DH + r), ls = __ldcg(ps + ROWS * DH + ROWS + r);
-    const float4 ov = __ldcg(reinterpret_cast<const float4*>(ps + (size_t)r * DH) + c4);
-    const float mn = fmaxf(mx, ms);
-    if (mn > -CUDART_INF_F) {
-      const float e0 = fast_exp2(mx - mn), e1 = fast_exp2(ms - mn);
-      den = den * e0 + ls * e1;
-      acc.x = acc.x * e0 + ov.x * e1; acc.y = acc.y * e0 + ov.y * e1;
-      acc.z = acc.z * e0 + ov.z * e1; acc.w = acc.w * e0 + ov.w * e1;
-    }
-    mx = mn;
-  }
-  const float rd = 1.f / den;
-  const int ri = i0 + r / p.G, hq = h * p.G + r % p.G;
-  const size_t off = (((size_t)b * p.n_q + ri) * p.H_q + hq) * DH + c4 * 4;
-  if (p.out_dtype == SPACE_DTYPE_F32) {
-    *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + off) =
-        make_float4(acc.x * rd, acc.y * rd, acc.z * rd, acc.w * rd);
-  } else {
-    const __nv_bfloat162 a = __floats2bfloat162_rn(acc.x * rd, acc.y * rd);
-    const __nv_bfloat162 b2 = __floats2bfloat162_rn(acc.z * rd, acc.w * rd);
-    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + off) =
-        make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b2));
-  }
-  if (p.lse && c4 == 0)
-    p.lse[((size_t)b * p.H_q + hq) * p.n_q + ri] = (mx + log2f(den)) * 0.6931471805599453f;
+  for (int x = 0; x < n; ++x, ps += gstride)
+    acc.add(__ldcg(ps + ROWS * DH + r), __ldcg(ps + ROWS * DH + ROWS + r),
+            __ldcg(reinterpret_cast<const float4*>(ps + (size_t)r * DH) + c4));
+  acc.template store<DH>(p, b, h, i0, r, c4);
 }
 
 // ------------------------------------------------------------------ host side
@@ -736,6 +806,24 @@ size_t smem_bytes(int max_batch) {
   return Smem<DH>::TABLE_OFF + (size_t)(2 * max_batch + 2) * sizeof(int);
 }
 
+template <int DH>
+cudaError_t launch_dim(const AttnParams& p, int n_ctas, int max_batch, int size, cudaStream_t st, int* max_clusters) {
+  // the kernel's limits are raised once per device (to the most any batch needs)
+  static unsigned long long done_mask = 0;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev >= 64 || !((done_mask >> dev) & 1ull)) {
+    cudaFuncSetAttribute(attn_rows_kernel<DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<DH>(128));
+    cudaFuncSetAttribute(attn_rows_kernel<DH>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (dev < 64) done_mask |= 1ull << dev;
+  }
+  return launch_clusters(attn_rows_kernel<DH>, n_ctas, THREADS, smem_bytes<DH>(max_batch), size, st, max_clusters, p, max_batch);
+}
+cudaError_t launch_main(int DH, const AttnParams& p, int n_ctas, int max_batch, int size, cudaStream_t st, int* max_clusters) {
+  return DH == 128 ? launch_dim<128>(p, n_ctas, max_batch, size, st, max_clusters)
+                   : launch_dim<64>(p, n_ctas, max_batch, size, st, max_clusters);
+}
+
 }  // namespace
 
 int launch_attn_rows(space_ctx* ctx, const space_attn_args* a, const uint64_t* mask_rows,
@@ -759,6 +847,7 @@ int launch_attn_rows(space_ctx* ctx, const space_attn_args* a, const uint64_t* m
   p.desc = reinterpret_cast<int2*>(ctx->merge_cnt);
   p.owner = ctx->merge_cnt + (size_t)cfg.max_batch * cfg.n_kv_heads * 8 * 2;
   p.merge_by_owner = (a->batch * p.H_kv * p.n_mblocks > pl.n_ctas) ? 1 : 0;
+  p.arrived = ctx->arrived;
   for (int i = 0; i < SPACE_MAX_ROWS; ++i) p.mask[i] = mask_rows[i];
 
   // TMA descriptors, rebuilt only when a base pointer or a stride changes
@@ -785,31 +874,24 @@ int launch_attn_rows(space_ctx* ctx, const space_attn_args* a, const uint64_t* m
   memcpy(&p.tm_k, ctx->tm_k, sizeof(CUtensorMap));
   memcpy(&p.tm_v, ctx->tm_v, sizeof(CUtensorMap));
 
-  const int m_valid_max = p.rows_per_mb * p.G;
-  const dim3 mgrid(p.merge_by_owner ? pl.n_ctas : a->batch * p.H_kv * p.n_mblocks, (m_valid_max * (DH / 4) + 127) / 128);
-  if (DH == 128) {
-    const size_t sm = smem_bytes<128>(cfg.max_batch);
-    cudaFuncSetAttribute(attn_rows_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    {
-      ProfScope ps(ctx, SPACE_K_ATTN, st);
-      launch_pdl(attn_rows_kernel<128>, dim3(pl.n_ctas), dim3(THREADS), sm, st, p, cfg.max_batch);
-    }
-    {
-      ProfScope ps(ctx, SPACE_K_MERGE, st);
-      launch_pdl(attn_rows_merge_kernel<128>, mgrid, dim3(128), 0, st, p);
-    }
-  } else {
-    const size_t sm = smem_bytes<64>(cfg.max_batch);
-    cudaFuncSetAttribute(attn_rows_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    {
-      ProfScope ps(ctx, SPACE_K_ATTN, st);
-      launch_pdl(attn_rows_kernel<64>, dim3(pl.n_ctas), dim3(THREADS), sm, st, p, cfg.max_batch);
-    }
-    {
-      ProfScope ps(ctx, SPACE_K_MERGE, st);
-      launch_pdl(attn_rows_merge_kernel<64>, mgrid, dim3(128), 0, st, p);
-    }
+  int n_ctas = pl.n_ctas, size = 1, n_clusters = 0;
+  p.pieces = plan_clusters(a->batch * p.H_kv, p.n_mblocks, (p.s_cap + TILE_N - 1) / TILE_N, ctx->sm_count, ctx->cluster_fit[1],
+                           [&](int sz, int* fit) { return launch_main(DH, p, ctx->sm_count / sz * sz, cfg.max_batch, sz, st, fit); },
+                           &n_clusters);
+  if (p.pieces) { size = p.pieces * p.n_mblocks; n_ctas = n_clusters * size; }
+  p.n_groups = n_ctas / p.n_mblocks;
+  {
+    ProfScope ps(ctx, SPACE_K_ATTN, st);
+    launch_main(DH, p, n_ctas, cfg.max_batch, size, st, nullptr);
+    ctx->launches += 1;
   }
-  ctx->launches += 2;
+  if (!p.pieces) {
+    const int m_valid_max = p.rows_per_mb * p.G;
+    const dim3 mgrid(p.merge_by_owner ? n_ctas : a->batch * p.H_kv * p.n_mblocks, (m_valid_max * (DH / 4) + 127) / 128);
+    ProfScope ps(ctx, SPACE_K_MERGE, st);
+    if (DH == 128) launch_pdl(attn_rows_merge_kernel<128>, mgrid, dim3(128), 0, st, p);
+    else launch_pdl(attn_rows_merge_kernel<64>, mgrid, dim3(128), 0, st, p);
+    ctx->launches += 1;
+  }
   return cuda_ok(cudaGetLastError());
 }

@@ -37,6 +37,7 @@
 // keys and the Eq. 5 mask.
 #include "common.cuh"
 #include "tc_common.cuh"
+#include "attn_common.cuh"
 #include <cuda.h>
 #include <math_constants.h>
 
@@ -44,10 +45,7 @@ namespace {
 
 constexpr int TILE_N = 128;            // keys per tile
 constexpr int SHARE_COST = 4;          // fixed cost of a share (query load, first tile, last product, epilogue) in tiles; swept 2..8
-constexpr int ROWS = 128;              // MMA M
 constexpr int THREADS = 384;            // K, MMA, V, Q warps + 8 softmax warps
-constexpr int CLUSTER_SLACK = 10;
-constexpr int MAX_CLUSTER = 16;         // blocks per cluster (more than 8 need the opt-in)
 constexpr uint64_t WAIT_NS = 1000000000ull;   // one second per wait
 
 struct AttnParams {
@@ -115,6 +113,7 @@ __device__ unsigned long long g_timeline_merge[4096 * 4];
 
 // PTX helpers: tc_common.cuh.  Every wait of this kernel is bounded by WAIT_NS.
 using namespace tc;
+using namespace attn;
 __device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site) {
   return mbar_wait_bounded(bar, parity, abort_flag, err, site, WAIT_NS, 64);   // sleeps between polls
 }
@@ -341,64 +340,6 @@ __device__ __noinline__ void piece_rescale(uint32_t taddr, const float* fq) {
   tmem_wait_st();
 }
 
-// Shared memory of another block of the cluster.
-__device__ __forceinline__ uint32_t map_cluster(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ float ld_cluster(uint32_t a) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
-  return v;
-}
-__device__ __forceinline__ float4 ld_cluster4(uint32_t a) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
-  return v;
-}
-
-// Query row r of the row block that starts at block row i0, columns 4 c4 .. of (sequence b, kv head h).
-template <int DH>
-__device__ __forceinline__ void store_out(const AttnParams& p, int b, int h, int i0, int r, int c4, const float4& v) {
-  const int gsh = __ffs(p.G) - 1;                           // G is a power of two
-  const int ri = i0 + (r >> gsh), hq = h * p.G + (r & (p.G - 1));
-  const size_t off = (((size_t)b * p.n_q + ri) * p.H_q + hq) * DH + c4 * 4;
-  if (p.out_dtype == SPACE_DTYPE_F32) {
-    *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + off) = v;
-  } else {
-    const __nv_bfloat162 x = __floats2bfloat162_rn(v.x, v.y), y = __floats2bfloat162_rn(v.z, v.w);
-    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + off) =
-        make_uint2(*reinterpret_cast<const uint32_t*>(&x), *reinterpret_cast<const uint32_t*>(&y));
-  }
-}
-
-// Four output elements of one query row from the partials of a cut: running reference, denominator and
-// accumulator.
-struct MergeAcc {
-  float mx, den;
-  float4 a;
-  __device__ __forceinline__ void clear() { mx = -CUDART_INF_F; den = 0.f; a = make_float4(0.f, 0.f, 0.f, 0.f); }
-  __device__ __forceinline__ void add(float m, float l, const float4& o) {
-    const float mn = fmaxf(mx, m);
-    if (mn > -CUDART_INF_F) {
-      const float e0 = fast_exp2(mx - mn), e1 = fast_exp2(m - mn);
-      den = den * e0 + l * e1;
-      a.x = a.x * e0 + o.x * e1; a.y = a.y * e0 + o.y * e1;
-      a.z = a.z * e0 + o.z * e1; a.w = a.w * e0 + o.w * e1;
-    }
-    mx = mn;
-  }
-  template <int DH>
-  __device__ __forceinline__ void store(const AttnParams& p, int b, int h, int i0, int r, int c4) const {
-    const float rd = 1.f / den;
-    const int gsh = __ffs(p.G) - 1;
-    const int ri = i0 + (r >> gsh), hq = h * p.G + (r & (p.G - 1));
-    store_out<DH>(p, b, h, i0, r, c4, make_float4(a.x * rd, a.y * rd, a.z * rd, a.w * rd));
-    if (p.lse && c4 == 0) p.lse[((size_t)b * p.H_q + hq) * p.n_q + ri] = (mx + log2f(den)) * 0.6931471805599453f;
-  }
-};
-
 // Warp roles
 constexpr int WARP_K = 0, WARP_MMA = 1, WARP_V = 2, WARP_PV = 3, WARP_SOFTMAX0 = 4;
 constexpr int L2_AHEAD_TILES = 1;      // tiles per operand a block asks L2 for before its dependency wait (more of them
@@ -531,21 +472,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     // every warp works the same things out for itself: nothing has to be handed over
     auto tiles_of = [&](int L) { return (L >= 0 && (int64_t)L + p.n_q <= p.s_cap) ? (L + p.n_q + TILE_N - 1) / TILE_N : 0; };
     const int L0 = cl_mine ? p.kv_len[cl_b] : -1;
-    int Tmax, W;
-    if (p.B == 1) {
-      Tmax = W = tiles_of(p.kv_len[0]);
-    } else {
-      Tmax = W = 0;
-      for (int b0 = 0; b0 < p.B; b0 += 32) {
-        const int T = b0 + lane < p.B ? tiles_of(p.kv_len[b0 + lane]) : 0;
-        Tmax = max(Tmax, __reduce_max_sync(0xFFFFFFFFu, T));
-        W += __reduce_add_sync(0xFFFFFFFFu, T);
-      }
-    }
-    // tiles of the longest piece against an even share of all tiles and what the cut over the grid costs on
-    // top: starting more than one share per block and the merge in global memory, about ten tiles' time
-    clustered = (Tmax + p.pieces - 1) / p.pieces <= (W * p.H_kv + p.n_groups - 1) / p.n_groups + CLUSTER_SLACK;
-    if (threadIdx.x == 0 && W != 0x7FFFFFFF) TL(14);
+    clustered = cluster_fits(p, lane, tiles_of);
+    if (threadIdx.x == 0 && L0 != 0x7FFFFFFF) TL(14);
     if (clustered) {
       const int T = tiles_of(L0), L = T ? L0 : -1;
       if (cl_mine && !T && cl_piece == 0 && cl_h == 0 && mb == 0 && threadIdx.x == 0 && p.status)
@@ -1157,113 +1085,15 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       tc_fence_before();
       soft_sync();                                          // scratch, fq and mref are reused by the next share
       if (sidx == 0) TL(11);
-      if (p.pieces && !whole && !to_smem) {
-        // ---- clusters were launched, but the lengths are too unequal for them: the piece that finds all the
-        // others stored combines them.  (No merge kernel follows such a launch.  As the rule for larger
-        // batches this was slower, 137 against 130 us on sixteen ragged sequences: every piece waits for its
-        // fence and its atomic.)
-        int* flag = reinterpret_cast<int*>(xq);
-        if (sidx == 0) {
-          int* arrived = p.arrived + (size_t)item * p.n_mblocks + mb;
-          __threadfence();                                  // (the barrier above ordered every thread's stores before this)
-          const int last = atomicAdd(arrived, 1) == cut_d.y - 1;
-          if (last) { *arrived = 0; __threadfence(); }      // ready for the next launch
-          flag[0] = last; flag[1] = cut_d.x; flag[2] = cut_d.y;
-        }
-        soft_sync();
-        const bool last = flag[0] != 0;
-        const int d0 = flag[1], dn = flag[2];
-        if (last && ok) {
-          const size_t slot_floats = (size_t)ROWS * (DH + 2), gstride = (size_t)p.n_mblocks * slot_floats;
-          const float* ps = p.part + ((size_t)d0 * p.n_mblocks + mb) * slot_floats;
-          // rows in batches whose weights exp2(m - M) / sum fit the P buffer (idle now): dn floats per row
-          float* wgt = reinterpret_cast<float*>(sm + S::P_OFF);
-          const int rows_at_once = min(m_valid, 2 * S::P_PART / 4 / dn);
-          for (int r0 = 0; r0 < m_valid; r0 += rows_at_once) {
-            const int nr = min(rows_at_once, m_valid - r0);
-            soft_sync();
-            for (int rr = warp - WARP_SOFTMAX0; rr < nr; rr += 8) {
-              const float* pr = ps + ROWS * DH + r0 + rr;
-              float M = -CUDART_INF_F, den = 0.f;
-              for (int x = lane; x < dn; x += 32) M = fmaxf(M, __ldcg(pr + (size_t)x * gstride));
-#pragma unroll
-              for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
-              for (int x = lane; x < dn; x += 32) {
-                const float e = fast_exp2(__ldcg(pr + (size_t)x * gstride) - M);
-                wgt[rr * dn + x] = e;
-                den = fmaf(__ldcg(pr + (size_t)x * gstride + ROWS), e, den);
-              }
-#pragma unroll
-              for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xFFFFFFFFu, den, o);
-              const float rd = 1.f / den;
-              for (int x = lane; x < dn; x += 32) wgt[rr * dn + x] *= rd;
-              if (p.lse && lane == 0) {
-                const int q = r0 + rr;
-                p.lse[((size_t)sg.b * p.H_q + sg.h * p.G + q % p.G) * p.n_q + i0 + q / p.G] = (M + log2f(den)) * 0.6931471805599453f;
-              }
-            }
-            soft_sync();
-            for (int idx = sidx; idx < nr * (DH / 4); idx += 256) {
-              const int rr = idx / (DH / 4), c4 = idx % (DH / 4);
-              float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-              const float* po = ps + (size_t)(r0 + rr) * DH + c4 * 4;
-              for (int x0 = 0; x0 < dn; x0 += 16) {         // all loads of a batch are issued before any is used
-                float4 ov[16];
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                  ov[j] = x0 + j < dn ? __ldcg(reinterpret_cast<const float4*>(po + (size_t)(x0 + j) * gstride)) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                  const float w = x0 + j < dn ? wgt[rr * dn + x0 + j] : 0.f;
-                  a.x = fmaf(ov[j].x, w, a.x); a.y = fmaf(ov[j].y, w, a.y);
-                  a.z = fmaf(ov[j].z, w, a.z); a.w = fmaf(ov[j].w, w, a.w);
-                }
-              }
-              store_out<DH>(p, sg.b, sg.h, i0, r0 + rr, c4, a);
-            }
-          }
-        }
-        soft_sync();                                        // flag lies in the scratch of the next share
-      }
+      if (p.pieces && !whole && !to_smem)                   // (the P buffer is idle)
+        merge_if_last<DH>(p, sg.b, sg.h, i0, m_valid, mb, cut_d, p.arrived + (size_t)item * p.n_mblocks + mb,
+                          reinterpret_cast<float*>(sm + S::P_OFF), 2 * S::P_PART / 4, sidx, 256, [] { soft_sync(); });
     }
     if (!p.pieces && sidx == 0) p.owner[blockIdx.x] = own;
   }
-  if (clustered && cl_n > 1) {
-    // ---- the pieces of this cluster's pair meet: every block combines its part of the rows from all pieces'
-    // shared memory.  (A block of the cluster without a tile takes part too.  Every wait above is bounded, so
-    // every block arrives here.)
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    const uint32_t mine = sm_base;
-    const int stride = p.pieces * THREADS;
-    for (int idx = cl_piece * THREADS + (int)threadIdx.x; idx < m_valid * (DH / 4) && !*abort_flag; idx += stride) {
-      const int r = idx / (DH / 4), c4 = idx % (DH / 4);
-      MergeAcc acc;
-      acc.clear();
-      for (int x0 = 0; x0 < cl_n; x0 += 4) {
-        float ms[4], ls[4];
-        float4 ov[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (x0 + j < cl_n) {
-            const uint32_t rk = (uint32_t)((x0 + j) * p.n_mblocks + mb);
-            ms[j] = ld_cluster(map_cluster(mine + S::XQ_OFF + r * 4, rk));
-            ls[j] = ld_cluster(map_cluster(mine + S::FQ_OFF + r * 4, rk));
-            ov[j] = ld_cluster4(map_cluster(mine + S::P_OFF + (r * DH + c4 * 4) * 4, rk));
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (x0 + j < cl_n) acc.add(ms[j], ls[j], ov[j]);
-      }
-      acc.template store<DH>(p, cl_b, cl_h, i0, r, c4);
-    }
-    // No block leaves while another may still read its shared memory: this half says that this block has read
-    // (relaxed: nothing is handed over, so it need not wait for the output's stores), the other half is at the exit.
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-  }
+  if (clustered && cl_n > 1)
+    cluster_merge<DH>(p, cl_b, cl_h, i0, m_valid, cl_piece, p.pieces, cl_n, mb, sm_base + S::P_OFF, sm_base + S::XQ_OFF,
+                      sm_base + S::FQ_OFF, abort_flag);
   if (threadIdx.x == 0) TL(12);
   // ---- teardown -----------------------------------------------------------
   tc_fence_before();
@@ -1275,10 +1105,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   if (threadIdx.x == 0 && *abort_flag && p.status) {
     for (int b = 0; b < p.B; ++b) atomicOr(p.status + b, SPACE_ST_TIMEOUT);
   }
-  if (clustered && cl_n > 1) {
-    __syncwarp();
-    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-  }
+  if (clustered && cl_n > 1) cluster_leave();
   if (threadIdx.x == 32) TL(13);                          // after the TMEM release
 }
 
@@ -1387,10 +1214,8 @@ size_t smem_bytes(int max_batch) {
   return Smem<DH>::TABLE_OFF + (size_t)(2 * max_batch + 1) * sizeof(int);
 }
 
-// Launch with clusters of `size` blocks (1: none).  max_clusters != nullptr: no launch, the largest number of
-// such clusters that can be resident instead.
 template <int DH, bool PAGED>
-cudaError_t launch_main(const AttnParams& p, int n_ctas, int max_batch, int size, cudaStream_t st, int* max_clusters = nullptr) {
+cudaError_t launch_main(const AttnParams& p, int n_ctas, int max_batch, int size, cudaStream_t st, int* max_clusters) {
   // the kernel's limits are raised once per device (to the most any batch needs)
   static unsigned long long done_mask = 0;                 // (one per instantiation)
   int dev = 0;
@@ -1401,19 +1226,7 @@ cudaError_t launch_main(const AttnParams& p, int n_ctas, int max_batch, int size
     cudaFuncSetAttribute(attn_tc_kernel<DH, PAGED>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (dev < 64) done_mask |= 1ull << dev;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_ctas); cfg.blockDim = dim3(THREADS); cfg.dynamicSmemBytes = smem_bytes<DH>(max_batch); cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = size; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = size > 1 ? 2 : 1;
-  if (max_clusters) {
-    cfg.attrs = attr + 1; cfg.numAttrs = 1;
-    return cudaOccupancyMaxActiveClusters(max_clusters, attn_tc_kernel<DH, PAGED>, &cfg);
-  }
-  return cudaLaunchKernelEx(&cfg, attn_tc_kernel<DH, PAGED>, p, max_batch);
+  return launch_clusters(attn_tc_kernel<DH, PAGED>, n_ctas, THREADS, smem_bytes<DH>(max_batch), size, st, max_clusters, p, max_batch);
 }
 
 template <int DH>
@@ -1515,26 +1328,16 @@ int launch_attn_tensor(space_ctx* ctx, const space_attn_args* a, const uint64_t*
   memcpy(&p.tm_k, ctx->tm_k, sizeof(CUtensorMap));
   memcpy(&p.tm_v, ctx->tm_v, sizeof(CUtensorMap));
 
-  // Clustered cut when every (sequence, kv head) gets a cluster of its own: as many pieces as there are SMs
-  // for (and tiles a sequence may have), in clusters that fit next to one another.  The grid fills the chip
+  // Clustered cut when every (sequence, kv head) gets a cluster of its own.  The grid fills the chip
   // all the same: the kernel falls back to a cut over all of it when the lengths are too unequal.
-  const int pairs = a->batch * p.H_kv;
-  const int64_t cap_tiles = (p.s_cap + TILE_N - 1) / TILE_N;
-  int n_ctas = pl.n_ctas, size = 1;
-  for (int c = cap_tiles < MAX_CLUSTER / p.n_mblocks ? (int)cap_tiles : MAX_CLUSTER / p.n_mblocks; c >= 1; --c) {
-    const int sz = c * p.n_mblocks;
-    if (pairs * sz > ctx->sm_count) continue;
-    int& fit = ctx->cluster_fit[sz];                        // clusters of sz blocks that fit (asked once)
-    if (sz == 1) fit = ctx->sm_count;
-    if (fit == 0 && (DH == 128 ? launch_form<128>(p, ctx->sm_count / sz * sz, cfg.max_batch, sz, st, &fit)
-                               : launch_form<64>(p, ctx->sm_count / sz * sz, cfg.max_batch, sz, st, &fit)) != cudaSuccess) {
-      cudaGetLastError();
-      fit = -1;
-    }
-    if (fit < pairs) continue;
-    p.pieces = c; size = sz; n_ctas = fit * sz;
-    break;
-  }
+  int n_ctas = pl.n_ctas, size = 1, n_clusters = 0;
+  auto ask = [&](int sz, int* fit) {
+    const int n = ctx->sm_count / sz * sz;
+    return DH == 128 ? launch_form<128>(p, n, cfg.max_batch, sz, st, fit) : launch_form<64>(p, n, cfg.max_batch, sz, st, fit);
+  };
+  p.pieces = plan_clusters(a->batch * p.H_kv, p.n_mblocks, (p.s_cap + TILE_N - 1) / TILE_N, ctx->sm_count, ctx->cluster_fit[0],
+                           ask, &n_clusters);
+  if (p.pieces) { size = p.pieces * p.n_mblocks; n_ctas = n_clusters * size; }
   p.n_groups = n_ctas / p.n_mblocks;
   {
     ProfScope ps(ctx, SPACE_K_ATTN, st);

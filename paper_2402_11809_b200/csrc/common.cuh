@@ -178,7 +178,7 @@ struct space_ctx {
   // cached block layout (Eq. 5 mask rows) and the attention kernel's visibility words, per (k, mask variant)
   int lay_k, lay_variant;                // lay_k = 0: nothing cached
   uint64_t lay_mask[SPACE_MAX_ROWS];
-  int cluster_fit[17];                   // transposed attention kernel: resident clusters of that many blocks (0: not asked yet)
+  int cluster_fit[2][17];                // transposed and row attention kernel: resident clusters of that many blocks (0: not asked yet)
   int visq_k, visq_variant;
   uint64_t visq[2][SPACE_MAX_ROWS];
   // cached TMA descriptors
