@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle.attention import attention_step
 from oracle.lmhead import lmhead_verify_step
 from oracle.verify import verify_step
 from paper_2402_11809_b200 import workloads
@@ -107,3 +108,61 @@ def test_lmhead_by_phase(B, H, mode, V, D, k, Bn):  # noqa: F811
             assert np.array_equal(h[n][~excl], r[n][~excl]), (n, again)
         np.testing.assert_allclose(h["next_cand_prob"][~excl], r["next_cand_prob"][~excl], rtol=1e-3)
         assert status[-1].item() & B.ST_BAD_CANDIDATE and not status[:-1].any()
+
+
+# Attention over at most one (sequence, kv head) per cluster: fewer tiles than pieces, first tiles that lie past the
+# end or are the last, partial one, two query-row blocks per pair, lengths too unequal for the clustered cut (a long
+# sequence next to short ones, at both kernels), and a sequence that does not fit.
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("k,d,H_q,H_kv,lens", [
+    (5, 128, 2, 2, (1, 90, 91, 92, 93, 700)), (2, 64, 4, 4, (0, 119, 120, 247, 1500)), (7, 128, 4, 2, (250, 300)),
+    (4, 64, 8, 8, (1000,)), (3, 128, 2, 2, (9000, 40, 7)), (1, 64, 1, 1, (12000,)), (6, 64, 32, 4, (700, 905)),
+    (4, 128, 16, 4, (30, 1500)), (4, 64, 8, 2, (9000, 5)), (6, 128, 16, 2, (2000,)),
+])
+def test_attention_clustered_cut(B, H, k, d, H_q, H_kv, lens, paged):  # noqa: F811
+    cfg = _small_cfg(k, (min(lens), max(lens)), d=d, H_q=H_q, H_kv=H_kv, Bn=len(lens), V=64, seed=k)
+    x = workloads.make_step_inputs(cfg, poison_tail=True)
+    x["kv_len"][:] = lens
+    rng = np.random.default_rng(1)
+    for b, L in enumerate(lens):                             # keys for these lengths, the rest as poisoned as it was
+        for name in ("k_cache", "v_cache"):
+            x[name][b] = 0x7FC0
+            x[name][b, :, : L + x["n_q"]] = workloads.f32_to_bf16_bits(rng.standard_normal((H_kv, L + x["n_q"], d), dtype=np.float32))
+    y = workloads.to_pages(x) if paged else x
+    y["kv_len"] = x["kv_len"].copy()
+    if len(lens) > 2:
+        y["kv_len"][1] = y["s_cap"]                          # does not fit: flagged, left alone
+    ctx = H.make_context(cfg, y)
+    ds = H.DeviceStep(cfg, y)
+    for again in range(2):                                   # arrival counters reset themselves
+        ds.out.fill_(float("nan"))
+        ds.status.zero_()
+        ds.attn(ctx)
+        torch.cuda.synchronize()
+        got, st = ds.out.cpu().numpy().astype(np.float64), ds.status.cpu().numpy()
+        for b, L in enumerate(lens):
+            if y["kv_len"][b] != L:
+                assert st[b] == B.ST_CAPACITY and np.isnan(got[b]).all()
+                continue
+            assert st[b] == 0
+            ref, lse = attention_step(x["q"][b:b + 1], x["k_cache"][b:b + 1], x["v_cache"][b:b + 1], x["kv_len"][b:b + 1], k, x["scale"])
+            H.check_attention(got[b:b + 1], ref, f"sequence {b} of length {L}")
+            np.testing.assert_allclose(ds.lse[b].cpu().numpy(), lse[0], rtol=0, atol=2e-3)
+
+
+# A page's tail rows are cleared while the V ring is several rounds in (head size 64: four V stages, three S buffers).
+@pytest.mark.parametrize("d", [64, 128])
+def test_rows_kernel_long_paged_shares(B, H, d):  # noqa: F811
+    k, H_q, H_kv = 4, 8, 2
+    cfg = _small_cfg(k, (2300, 2350), d=d, H_q=H_q, H_kv=H_kv, Bn=80, V=64, seed=3)     # more pairs than blocks: long shares
+    x = workloads.to_pages(workloads.make_step_inputs(cfg))
+    ctx = H.make_context(cfg, x)
+    ds = H.DeviceStep(cfg, x)
+    ds.attn(ctx)
+    torch.cuda.synchronize()
+    assert not ds.status.any()
+    assert torch.isfinite(ds.out).all()
+    c = workloads.make_step_inputs(cfg)
+    for b in (0, 41, 79):
+        ref, _ = attention_step(c["q"][b:b + 1], c["k_cache"][b:b + 1], c["v_cache"][b:b + 1], c["kv_len"][b:b + 1], k, c["scale"])
+        H.check_attention(ds.out[b:b + 1].cpu().numpy().astype(np.float64), ref, f"sequence {b}")
