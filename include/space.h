@@ -251,8 +251,9 @@ typedef struct {
   float*    next_cand_prob;    /* host [B, k]                                  */
   uint8_t*  finished;          /* host [B]                                     */
   int32_t*  status;            /* host [B]                                     */
-  int64_t*  h2d_bytes;         /* host, optional: bytes copied to the device   */
-  int64_t*  d2h_bytes;         /* host, optional: bytes copied back            */
+  int64_t*  h2d_bytes;         /* host, optional: bytes of input the device is handed (all rows of logits, though
+                                  from pinned buffers only those the step decides on travel) */
+  int64_t*  d2h_bytes;         /* host, optional: bytes handed back            */
   int32_t   cache_resident;    /* 0: upload rows 0 .. kv_len+n_q-1 of every sequence's K and V.
                                   1: the KV cache is the decoder's state and already sits in the context's
                                   staging copy from an earlier call (rows 0 .. kv_len-1 of every sequence,
@@ -345,9 +346,11 @@ int space_lmhead_verify(space_ctx* ctx, const space_lmhead_args* args, void* str
 int space_kv_commit(space_ctx* ctx, const space_commit_args* args, void* stream);
 
 /* The three stages from host buffers; synchronises `stream` before returning.
- * (The logits go up and the attention output comes down on a second stream of the
- * context, ordered against `stream` by events, so that both copies overlap the kernels;
- * when the call returns everything it enqueued on either stream has finished.)
+ * (The logits go up, or are verified, on a second stream of the context, ordered against
+ * `stream` by events, beside the attention; when the call returns everything it enqueued on
+ * either stream has finished.  With cache_resident and pinned, 16-byte aligned q, caches,
+ * logits and out, kernels move the pieces, the attention stores its output into host memory and
+ * verification reads the rows of logits it needs where they lie.)
  * Needs cfg.host_staging.  Only sequence prefixes in use are copied (with
  * cache_resident: only the block's rows, see the field).  The call stages the
  * small per-sequence arrays in a pinned buffer of the context: one call at a

@@ -161,7 +161,7 @@ struct space_ctx {
   VerifyRow* vrow;         // [max_batch][k_max+1]
   VerifyPartial* vfused;   // [max_batch][SPACE_MAX_ROWS][16] single-launch greedy path
   char* vtopk;             // filtered sampling: top-k lists per (sequence, row, chunk)
-  int32_t* scratch_status; // [max_batch] used when the caller passes no status array
+  int32_t* vstatus;        // [max_batch] status bits of a verification that runs beside the attention (space_step_host)
   char* lm_part;           // output-projection statistics [256 block rows][sm_count] x 16 bytes
   char* lm_gather;         // gathered mask rows of the projection's second phase
   int* lm_counter;         // {arrival counter, first timeout site}
@@ -289,9 +289,30 @@ __device__ __forceinline__ void commit_tables(const CommitParams& p, int b, int 
   }
 }
 
+// ---- space_step_host: transfers by kernels over the device mapping of pinned host memory (host_copy.cu) ----
+struct HostCopyParams {
+  int B, H_kv;
+  int row_vecs, run_vecs;              // 16-byte pieces per cache row, and per run of rows moved
+  int small_words;                     // 4-byte words of the small arrays
+  int64_t s_cap, q_vecs;
+  const uint4* h_q; uint4* d_q;
+  uint4* h_k; uint4* h_v; uint4* d_k; uint4* d_v;      // [B, H_kv, s_cap, d] on both sides
+  int32_t* h_small; int32_t* d_small; int32_t* d_status;
+  // way down: the commit's part
+  int k, speculative;                  // speculative: all k candidate rows move, as in the single-launch verify
+  const int32_t* n_accept; int32_t* d_vstatus;         // the verification's status bits (cleared for the next call)
+  int32_t* h_status; int32_t* h_len_out;
+  int32_t len[128];                    // first row moved of every sequence, -1: none (it does not fit)
+  int32_t old_len[128];
+};
+int launch_host_upload(space_ctx* ctx, const HostCopyParams& p, cudaStream_t st);
+int launch_host_download(space_ctx* ctx, const HostCopyParams& p, cudaStream_t st);
+
 // ---- per-stage launchers (defined next to their kernels) -------------------
 // cm != nullptr: the verify kernels also carry out the commit described by cm (one launch less)
-int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit_args* cm, cudaStream_t st);
+// mapped: the logits lie in host memory (read where they are, by the launches that read only the rows they need)
+int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit_args* cm, cudaStream_t st, bool mapped = false);
+bool verify_is_fused(const space_verify_args* a);   // whether a call on device logits takes one launch
 int launch_verify_filtered(space_ctx* ctx, const space_verify_args* a, const space_commit_args* cm, cudaStream_t st);
 size_t verify_filter_scratch_bytes(int max_batch, int k_max);
 void fill_commit_params(const space_ctx* ctx, const space_commit_args* a, CommitParams* p);

@@ -2,6 +2,7 @@
 // exported entry points declared in include/space.h.
 #include "common.cuh"
 #include "tc_common.cuh"
+#include <cstddef>
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -80,6 +81,20 @@ int device_sm_count(int device, int* sms) {
   if (prop.major != 10) return SPACE_E_NO_DEVICE;
   *sms = prop.multiProcessorCount;
   return SPACE_OK;
+}
+
+// The device's view of pinned host memory [p, p + n), or NULL where the kernels cannot use it (pageable,
+// not mapped, not 16-byte aligned).
+void* device_view(const void* p, size_t n) {
+  cudaPointerAttributes first, last;
+  if (((uintptr_t)p & 15u) || n == 0) return nullptr;
+  if (cudaPointerGetAttributes(&first, p) != cudaSuccess || first.type != cudaMemoryTypeHost || !first.devicePointer ||
+      cudaPointerGetAttributes(&last, (const char*)p + n - 1) != cudaSuccess || last.type != cudaMemoryTypeHost ||
+      (char*)last.devicePointer - (char*)first.devicePointer != (ptrdiff_t)(n - 1)) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return first.devicePointer;
 }
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
@@ -219,7 +234,7 @@ int space_create(space_ctx** out, const space_config* cfg) {
   ctx->vtopk = ctx->ws + cv.vtopk;
   ctx->vrow = (VerifyRow*)(ctx->ws + cv.vrow);
   ctx->vfused = (VerifyPartial*)(ctx->ws + cv.vfused);
-  ctx->scratch_status = (int32_t*)(ctx->ws + cv.status);
+  ctx->vstatus = (int32_t*)(ctx->ws + cv.status);
   ctx->lm_part = ctx->ws + cv.lm_part;
   ctx->lm_gather = ctx->ws + cv.lm_gather;
   ctx->lm_counter = (int*)(ctx->ws + cv.lm_counter);
@@ -410,45 +425,25 @@ int space_step_host(space_ctx* ctx, const space_host_step_args* a, void* stream)
   int32_t* d_kvlen_out = (int32_t*)(d_small + 10 * slot);
 
   int64_t h2d = 0, d2h = 0;
-  auto up = [&](void* dst, const void* src, size_t n) {
-    h2d += (int64_t)n;
-    return cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, st) == cudaSuccess;
-  };
   bool ok = true;
   const size_t row_b = (size_t)d * 2, head_pitch = (size_t)c.s_cap * row_b;
   const size_t seq_b = (size_t)c.n_kv_heads * head_pitch;
   const int esz = a->logits_dtype == SPACE_DTYPE_F32 ? 4 : 2;
-  // Two streams: what attention needs (q, the K/V rows, the lengths) goes up first on `st`; the logits
-  // follow on the second stream while attention already runs; the attention output comes down on the
-  // second stream while verification runs.  Events order the two; the call ends with everything done.
-  cudaStream_t sb = ctx->aux_stream;
-  ok = ok && up(d_q, a->q, (size_t)B * n_q * c.n_q_heads * d * 2);
+  const size_t q_bytes = (size_t)B * n_q * c.n_q_heads * d * 2, out_bytes = 2 * q_bytes;
+  const size_t cache_bytes = (size_t)B * seq_b, logit_bytes = (size_t)B * n_q * a->vocab * esz;
   // the small per-sequence arrays travel as one block each way through a pinned mirror of their slots
   char* hsm = ctx->host_small;
   memcpy(hsm, a->kv_len, (size_t)B * 4);
   memcpy(hsm + slot, a->cand, (size_t)B * k * 4);
   memcpy(hsm + 2 * slot, a->cand_prob, (size_t)B * k * 4);
-  ok = ok && cudaMemcpyAsync(d_small, hsm, 3 * slot, cudaMemcpyHostToDevice, st) == cudaSuccess;
-  h2d += (int64_t)B * 4 * (1 + 2 * k);
-  for (int b = 0; b < B && ok; ++b) {
-    const int64_t L = a->kv_len[b];
-    if (L < 0 || L + n_q > c.s_cap) continue;            // flagged by the kernels
-    // everything in use, or (cache kept from an earlier call) the block's own rows only
-    const size_t first = a->cache_resident ? (size_t)L * row_b : 0;
-    const size_t w = (size_t)(L + n_q) * row_b - first;
-    ok = ok && cudaMemcpy2DAsync(d_k + b * seq_b + first, head_pitch, (const char*)a->k_cache + b * seq_b + first,
-                                 head_pitch, w, c.n_kv_heads, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    ok = ok && cudaMemcpy2DAsync(d_v + b * seq_b + first, head_pitch, (const char*)a->v_cache + b * seq_b + first,
-                                 head_pitch, w, c.n_kv_heads, cudaMemcpyHostToDevice, st) == cudaSuccess;
-    h2d += 2 * (int64_t)w * c.n_kv_heads;
+  auto fits = [&](int b) { return a->kv_len[b] >= 0 && (int64_t)a->kv_len[b] + n_q <= c.s_cap; };   // (else flagged by the kernels)
+  for (int b = 0; b < B; ++b) {
+    if (!fits(b)) continue;
+    h2d += 2 * (int64_t)((a->cache_resident ? 0 : a->kv_len[b]) + n_q) * (int64_t)row_b * c.n_kv_heads;
+    d2h += 2 * (int64_t)k1 * (int64_t)row_b * c.n_kv_heads;
   }
-  ok = ok && cudaMemsetAsync(d_status, 0, (size_t)B * 4, st) == cudaSuccess;
-  ok = ok && cudaEventRecord(ctx->aux_ev[0], st) == cudaSuccess;          // attention's inputs are on their way
-  ok = ok && cudaStreamWaitEvent(sb, ctx->aux_ev[0], 0) == cudaSuccess;
-  h2d += (int64_t)((size_t)B * n_q * a->vocab * esz);
-  ok = ok && cudaMemcpyAsync(d_logits, a->logits, (size_t)B * n_q * a->vocab * esz, cudaMemcpyHostToDevice, sb) == cudaSuccess;
-  ok = ok && cudaEventRecord(ctx->aux_ev[1], sb) == cudaSuccess;          // logits uploaded
-  if (!ok) { cudaGetLastError(); return SPACE_E_CUDA; }
+  h2d += (int64_t)q_bytes + (int64_t)B * 4 * (1 + 2 * k) + (int64_t)logit_bytes;
+  d2h += (int64_t)out_bytes + (int64_t)B * (4 + k1 * 4 + 4 + k * 4 + k * 4 + 1 + 4 + 4);
 
   space_attn_args at{};
   at.batch = B; at.k = k; at.mask_variant = a->mask_variant; at.out_dtype = SPACE_DTYPE_F32;
@@ -456,42 +451,100 @@ int space_step_host(space_ctx* ctx, const space_host_step_args* a, void* stream)
   at.q = d_q; at.k_cache = d_k; at.v_cache = d_v;
   at.kv_stride_b = (int64_t)c.n_kv_heads * c.s_cap * d; at.kv_stride_h = c.s_cap * d; at.kv_stride_s = d;
   at.kv_len = d_kvlen; at.out = d_out; at.lse = nullptr; at.status = d_status;
-  int rc = space_attn_step(ctx, &at, stream);
-  if (rc != SPACE_OK) return rc;
-  // the attention output leaves on the second stream, under the verification kernels
-  ok = ok && cudaEventRecord(ctx->aux_ev[2], st) == cudaSuccess;
-  ok = ok && cudaStreamWaitEvent(sb, ctx->aux_ev[2], 0) == cudaSuccess;
-  d2h += (int64_t)((size_t)B * n_q * c.n_q_heads * d * 4);
-  ok = ok && cudaMemcpyAsync(a->out, d_out, (size_t)B * n_q * c.n_q_heads * d * 4, cudaMemcpyDeviceToHost, sb) == cudaSuccess;
-  ok = ok && cudaEventRecord(ctx->aux_ev[3], sb) == cudaSuccess;
-  ok = ok && cudaStreamWaitEvent(st, ctx->aux_ev[1], 0) == cudaSuccess;   // verification needs the logits
-  if (!ok) { cudaGetLastError(); return SPACE_E_CUDA; }
   space_verify_args ve{};
   ve.batch = B; ve.k = k; ve.vocab = a->vocab; ve.logits_dtype = a->logits_dtype; ve.mode = a->mode;
   ve.resample = a->resample; ve.eos_id = a->eos_id; ve.temperature = a->temperature; ve.seed = a->seed;
   ve.logits = d_logits; ve.logits_row_stride = a->vocab; ve.cand = d_cand; ve.cand_prob = d_cprob;
   ve.seq_id = nullptr; ve.kv_len = d_kvlen; ve.n_accept = d_nacc; ve.out_tokens = d_tok; ve.n_out = d_nout;
   ve.next_cand = d_ncand; ve.next_cand_prob = d_nprob; ve.finished = d_fin; ve.status = d_status;
-  space_commit_args cm{};
-  cm.batch = B; cm.k = k; cm.k_cache = d_k; cm.v_cache = d_v;
-  cm.kv_stride_b = at.kv_stride_b; cm.kv_stride_h = at.kv_stride_h; cm.kv_stride_s = at.kv_stride_s;
-  cm.n_accept = d_nacc; cm.kv_len = d_kvlen; cm.kv_len_out = d_kvlen_out; cm.status = d_status;
-  rc = space_verify_commit(ctx, &ve, &cm, stream);
+  int rc = check_verify_args(ctx, &ve);
   if (rc != SPACE_OK) return rc;
 
-  ok = ok && cudaMemcpyAsync(hsm + 3 * slot, d_small + 3 * slot, 8 * slot, cudaMemcpyDeviceToHost, st) == cudaSuccess;
-  d2h += (int64_t)B * (4 + k1 * 4 + 4 + k * 4 + k * 4 + 1 + 4 + 4);
-  for (int b = 0; b < B && ok; ++b) {                    // rows L .. L+k: the compacted rows
-    const int64_t L = a->kv_len[b];
-    if (L < 0 || L + n_q > c.s_cap) continue;
-    const size_t offb = b * seq_b + (size_t)L * row_b, w = (size_t)k1 * row_b;
-    ok = ok && cudaMemcpy2DAsync((char*)a->k_cache + offb, head_pitch, d_k + offb, head_pitch, w, c.n_kv_heads,
-                                 cudaMemcpyDeviceToHost, st) == cudaSuccess;
-    ok = ok && cudaMemcpy2DAsync((char*)a->v_cache + offb, head_pitch, d_v + offb, head_pitch, w, c.n_kv_heads,
-                                 cudaMemcpyDeviceToHost, st) == cudaSuccess;
-    d2h += 2 * (int64_t)w * c.n_kv_heads;
+  // Two streams beside one another, ordered by events: what the attention needs and the attention on `st`, the
+  // logits (and what is made of them) on the second.  The call ends with everything done.
+  cudaStream_t sb = ctx->aux_stream;
+  void *v_q, *v_k, *v_v, *v_logits, *v_out, *v_small;
+  if (a->cache_resident && (v_small = device_view(hsm, 11 * slot)) && (v_q = device_view(a->q, q_bytes)) &&
+      (v_k = device_view(a->k_cache, cache_bytes)) && (v_v = device_view(a->v_cache, cache_bytes)) &&
+      (v_logits = device_view(a->logits, logit_bytes)) && (v_out = device_view(a->out, out_bytes))) {
+    // ---- pinned buffers and a resident cache: kernels reach into host memory (host_copy.cu).  One moves q, the
+    // block's K/V rows and the small arrays up; the attention stores its output where it is wanted; verification
+    // reads the 2k+1 rows of logits that it needs over PCIe beside the attention, instead of having all (k+1)^2
+    // copied (one 7B-shaped sequence: 0.7 of 2.3 MB); one kernel commits and brings the rows and results back.
+    HostCopyParams hc;
+    memset(&hc, 0, offsetof(HostCopyParams, len));
+    hc.B = B; hc.H_kv = c.n_kv_heads; hc.row_vecs = d / 8; hc.run_vecs = n_q * (d / 8);
+    hc.small_words = (int)(3 * slot / 4); hc.s_cap = c.s_cap; hc.q_vecs = (int64_t)(q_bytes / 16);
+    hc.h_q = (const uint4*)v_q; hc.d_q = (uint4*)d_q;
+    hc.h_k = (uint4*)v_k; hc.h_v = (uint4*)v_v; hc.d_k = (uint4*)d_k; hc.d_v = (uint4*)d_v;
+    hc.h_small = (int32_t*)v_small; hc.d_small = (int32_t*)d_small; hc.d_status = d_status;
+    for (int b = 0; b < B; ++b) { hc.len[b] = fits(b) ? a->kv_len[b] : -1; hc.old_len[b] = a->kv_len[b]; }
+    ok = launch_host_upload(ctx, hc, st) == SPACE_OK;
+    // (the verification reads over PCIe after the upload, which the attention waits for)
+    ok = ok && cudaEventRecord(ctx->aux_ev[0], st) == cudaSuccess;
+    ok = ok && cudaStreamWaitEvent(sb, ctx->aux_ev[0], 0) == cudaSuccess;
+    ve.logits = v_logits; ve.status = ctx->vstatus;
+    ok = ok && launch_verify(ctx, &ve, nullptr, sb, true) == SPACE_OK;
+    ok = ok && cudaEventRecord(ctx->aux_ev[1], sb) == cudaSuccess;
+    if (!ok) { cudaGetLastError(); return SPACE_E_CUDA; }
+    at.out = v_out;
+    rc = space_attn_step(ctx, &at, stream);
+    if (rc != SPACE_OK) return rc;
+    ok = ok && cudaStreamWaitEvent(st, ctx->aux_ev[1], 0) == cudaSuccess;
+    // rows L .. L+k (the compacted ones) and the results
+    hc.run_vecs = k1 * (d / 8); hc.small_words = (int)(6 * slot / 4);
+    hc.h_small = (int32_t*)v_small + 3 * slot / 4; hc.d_small = (int32_t*)(d_small + 3 * slot);
+    hc.k = k; hc.speculative = verify_is_fused(&ve); hc.n_accept = d_nacc; hc.d_vstatus = ctx->vstatus;
+    hc.h_status = (int32_t*)v_small + 9 * slot / 4; hc.h_len_out = (int32_t*)v_small + 10 * slot / 4;
+    ok = ok && launch_host_download(ctx, hc, st) == SPACE_OK;
+  } else {
+    // ---- any host memory: copies.  What the attention needs goes up first; the logits follow on the second
+    // stream while the attention already runs; its output comes down there while verification runs.
+    auto up = [&](void* dst, const void* src, size_t n) {
+      return cudaMemcpyAsync(dst, src, n, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    };
+    ok = up(d_q, a->q, q_bytes) && up(d_small, hsm, 3 * slot);
+    for (int b = 0; b < B && ok; ++b) {
+      if (!fits(b)) continue;
+      // everything in use, or (cache kept from an earlier call) the block's own rows only
+      const size_t first = a->cache_resident ? (size_t)a->kv_len[b] * row_b : 0;
+      const size_t w = (size_t)(a->kv_len[b] + n_q) * row_b - first;
+      ok = ok && cudaMemcpy2DAsync(d_k + b * seq_b + first, head_pitch, (const char*)a->k_cache + b * seq_b + first,
+                                   head_pitch, w, c.n_kv_heads, cudaMemcpyHostToDevice, st) == cudaSuccess;
+      ok = ok && cudaMemcpy2DAsync(d_v + b * seq_b + first, head_pitch, (const char*)a->v_cache + b * seq_b + first,
+                                   head_pitch, w, c.n_kv_heads, cudaMemcpyHostToDevice, st) == cudaSuccess;
+    }
+    ok = ok && cudaMemsetAsync(d_status, 0, (size_t)B * 4, st) == cudaSuccess;
+    ok = ok && cudaEventRecord(ctx->aux_ev[0], st) == cudaSuccess;          // attention's inputs are on their way
+    ok = ok && cudaStreamWaitEvent(sb, ctx->aux_ev[0], 0) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(d_logits, a->logits, logit_bytes, cudaMemcpyHostToDevice, sb) == cudaSuccess;
+    ok = ok && cudaEventRecord(ctx->aux_ev[1], sb) == cudaSuccess;          // logits uploaded
+    if (!ok) { cudaGetLastError(); return SPACE_E_CUDA; }
+    rc = space_attn_step(ctx, &at, stream);
+    if (rc != SPACE_OK) return rc;
+    ok = ok && cudaEventRecord(ctx->aux_ev[2], st) == cudaSuccess;
+    ok = ok && cudaStreamWaitEvent(sb, ctx->aux_ev[2], 0) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(a->out, d_out, out_bytes, cudaMemcpyDeviceToHost, sb) == cudaSuccess;
+    ok = ok && cudaEventRecord(ctx->aux_ev[3], sb) == cudaSuccess;
+    ok = ok && cudaStreamWaitEvent(st, ctx->aux_ev[1], 0) == cudaSuccess;   // verification needs the logits
+    if (!ok) { cudaGetLastError(); return SPACE_E_CUDA; }
+    space_commit_args cm{};
+    cm.batch = B; cm.k = k; cm.k_cache = d_k; cm.v_cache = d_v;
+    cm.kv_stride_b = at.kv_stride_b; cm.kv_stride_h = at.kv_stride_h; cm.kv_stride_s = at.kv_stride_s;
+    cm.n_accept = d_nacc; cm.kv_len = d_kvlen; cm.kv_len_out = d_kvlen_out; cm.status = d_status;
+    rc = space_verify_commit(ctx, &ve, &cm, stream);
+    if (rc != SPACE_OK) return rc;
+    ok = ok && cudaMemcpyAsync(hsm + 3 * slot, d_small + 3 * slot, 8 * slot, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    for (int b = 0; b < B && ok; ++b) {                    // rows L .. L+k: the compacted rows
+      if (!fits(b)) continue;
+      const size_t offb = b * seq_b + (size_t)a->kv_len[b] * row_b, w = (size_t)k1 * row_b;
+      ok = ok && cudaMemcpy2DAsync((char*)a->k_cache + offb, head_pitch, d_k + offb, head_pitch, w, c.n_kv_heads,
+                                   cudaMemcpyDeviceToHost, st) == cudaSuccess;
+      ok = ok && cudaMemcpy2DAsync((char*)a->v_cache + offb, head_pitch, d_v + offb, head_pitch, w, c.n_kv_heads,
+                                   cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    }
+    ok = ok && cudaStreamWaitEvent(st, ctx->aux_ev[3], 0) == cudaSuccess;   // ... and the output has arrived
   }
-  ok = ok && cudaStreamWaitEvent(st, ctx->aux_ev[3], 0) == cudaSuccess;   // ... and the output has arrived
   if (!ok) { cudaGetLastError(); return SPACE_E_CUDA; }
   if (cudaStreamSynchronize(st) != cudaSuccess) return SPACE_E_CUDA;
   memcpy(a->n_accept, hsm + 3 * slot, (size_t)B * 4);

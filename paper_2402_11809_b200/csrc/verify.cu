@@ -52,6 +52,7 @@ struct VerifyParams {
   VerifyRow* rows;           // [B][k+1]
   int* counter_a;            // [B]
   int* counter_b;            // [B]
+  int mapped;                // the logits lie in host memory (nothing is asked of L2 ahead of time)
   int do_commit;             // the kernels also move the accepted cache rows (space_verify_commit)
   CommitParams cm;
 };
@@ -421,7 +422,7 @@ verify_target_kernel(const VerifyParams p) {
   const int k1 = p.k + 1;
   const T* row = reinterpret_cast<const T*>(p.logits) + ((int64_t)b * p.n_q + (int64_t)t * k1) * p.row_stride;
   const int begin = ch * p.chunk, end = min(p.V, begin + p.chunk);
-  prefetch_chunk<T>(row, begin, end);
+  if (!p.mapped) prefetch_chunk<T>(row, begin, end);
   pdl_wait();
   Stat st = scan_chunk<T, ALIGNED, false, STAT_SUM>(row, begin, end, p.c_t, -1, 0, 0, 0, 0, 0);
   st = block_reduce_plain(st, p.c_t);
@@ -616,7 +617,7 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
   constexpr float C1 = 1.4426950408889634f;                 // T = 1
   const T* row = reinterpret_cast<const T*>(p.logits) + ((int64_t)b * p.n_q + row_i) * p.row_stride;
   const int begin = ch * p.chunk, end = min(p.V, begin + p.chunk);
-  prefetch_chunk<T>(row, begin, end);
+  if (!p.mapped) prefetch_chunk<T>(row, begin, end);
   pdl_wait();
   TLV(1);
   int Lc = 0;
@@ -766,7 +767,12 @@ extern "C" int space_debug_timeline_read_verify(unsigned long long* host_dst, in
 }
 #endif
 
-int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit_args* cm, cudaStream_t st) {
+bool verify_is_fused(const space_verify_args* a) {
+  const int64_t rows = (int64_t)a->batch * (a->k + 1) * (a->k + 1);
+  return a->mode == SPACE_MODE_GREEDY && rows * a->vocab * (a->logits_dtype == SPACE_DTYPE_F32 ? 4 : 2) <= SPACE_FUSED_MAX_BYTES;
+}
+
+int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit_args* cm, cudaStream_t st, bool mapped) {
   if (a->mode == SPACE_MODE_SAMPLE && a->top_k > 0) {
     // filtered target distributions: kernels of their own (verify_filter.cu), which carry the commit too
     return launch_verify_filtered(ctx, a, cm, st);
@@ -774,14 +780,14 @@ int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit
   if (cm && cm->page_table) {
     // paged cache: only the single-launch greedy form carries the commit through a page table; the
     // two-launch form is followed by the commit kernel
-    const int64_t all_b = (int64_t)a->batch * (a->k + 1) * (a->k + 1) * a->vocab * (a->logits_dtype == SPACE_DTYPE_F32 ? 4 : 2);
-    if (!(a->mode == SPACE_MODE_GREEDY && all_b <= SPACE_FUSED_MAX_BYTES)) {
+    if (!verify_is_fused(a)) {
       const int rc = launch_verify(ctx, a, nullptr, st);
       if (rc != SPACE_OK) return rc;
       return launch_commit(ctx, cm, st);
     }
   }
   VerifyParams p;
+  p.mapped = mapped;
   p.do_commit = cm != nullptr;
   if (cm) fill_commit_params(ctx, cm, &p.cm); else memset(&p.cm, 0, sizeof(p.cm));
   p.B = a->batch; p.k = a->k; p.V = a->vocab; p.n_q = (a->k + 1) * (a->k + 1);
@@ -802,8 +808,9 @@ int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit
   const int vec = 16 / esz;
   const bool aligned = ((uintptr_t)a->logits % 16 == 0) && ((a->logits_row_stride * esz) % 16 == 0);
   // small greedy problem: one launch over all block rows (see the file header)
-  const int64_t all_bytes = (int64_t)a->batch * p.n_q * a->vocab * esz;
-  if (a->mode == SPACE_MODE_GREEDY && all_bytes <= SPACE_FUSED_MAX_BYTES) {
+  // (over PCIe, at about 46 GB/s, the rows that only the single launch reads must not cost more than a second launch)
+  const int64_t spare_bytes = (int64_t)a->batch * (p.n_q - 2 * a->k - 1) * a->vocab * esz;
+  if (verify_is_fused(a) && (!mapped || spare_bytes <= 512 << 10)) {
     int chunk, nc = row_chunks(a->vocab, a->batch * p.n_q, vec, ctx->sm_count, SPACE_FUSED_MAX_CHUNKS, &chunk);
     p.n_chunks = nc; p.chunk = chunk; p.n_chunks_g = 0; p.chunk_g = 0;
     if (a->logits_dtype == SPACE_DTYPE_F32) {
@@ -902,7 +909,7 @@ int launch_verify_noalloc(const space_verify_args* a, cudaStream_t st) {
   p.status = a->status;
   p.part = nullptr; p.rows = nullptr;
   p.counter_a = reinterpret_cast<int*>(base); p.counter_b = nullptr;
-  p.do_commit = 0; memset(&p.cm, 0, sizeof(p.cm));
+  p.mapped = 0; p.do_commit = 0; memset(&p.cm, 0, sizeof(p.cm));
   VerifyPartial* fpart = reinterpret_cast<VerifyPartial*>(base + SPACE_NOALLOC_COUNTER_BYTES);
 
   const int esz = a->logits_dtype == SPACE_DTYPE_F32 ? 4 : 2;

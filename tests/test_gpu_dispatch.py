@@ -166,3 +166,45 @@ def test_rows_kernel_long_paged_shares(B, H, d):  # noqa: F811
     for b in (0, 41, 79):
         ref, _ = attention_step(c["q"][b:b + 1], c["k_cache"][b:b + 1], c["v_cache"][b:b + 1], c["kv_len"][b:b + 1], k, c["scale"])
         H.check_attention(ds.out[b:b + 1].cpu().numpy().astype(np.float64), ref, f"sequence {b}")
+
+
+# space_step_host reaches into pinned buffers by kernels and copies pageable or misaligned ones; one sequence does
+# not fit its cache and is left alone.  V = 40001: the verification takes two launches over PCIe.
+@pytest.mark.parametrize("V", [501, 40001])
+@pytest.mark.parametrize("where", ["pinned", "pageable", "misaligned"])
+def test_host_step_transfers(B, H, where, V):  # noqa: F811
+    k, Bn, H_q, H_kv, d = 3, 3, 4, 2, 64
+    cfg = workloads.resolve("tiny", B=Bn, H_q=H_q, H_kv=H_kv, d=d, L=(20, 140), k=k, V=V, logits_dtype="bf16", seed=5)
+    x = workloads.make_step_inputs(cfg)
+    n_q, cap = x["n_q"], x["s_cap"]
+    x["kv_len"][1] = cap - n_q + 1                           # one row too many
+    ctx = B.Context(max_batch=Bn, n_q_heads=H_q, n_kv_heads=H_kv, head_dim=d, k_max=k, vocab=V, host_staging=1, s_cap=cap)
+
+    def host(a):
+        a = a.view(np.int16) if a.dtype == np.uint16 else a
+        flat = torch.zeros(a.size + 1, dtype=torch.from_numpy(a).dtype, pin_memory=where != "pageable")
+        t = flat[1:] if where == "misaligned" else flat[:-1]
+        return t.view(a.shape).copy_(torch.from_numpy(a))
+
+    z = lambda *s, dt=torch.int32: torch.zeros(s, dtype=dt)  # noqa: E731
+    r = verify_step(x["logits"], x["cand"], x["cand_prob"], k, "greedy")
+    for resident in (0, 1, 1):
+        h = {n: host(x[n]) for n in ("q", "k_cache", "v_cache", "logits", "cand", "cand_prob", "kv_len")}
+        h.update(out=host(np.zeros((Bn, n_q, H_q, d), np.float32)), n_accept=z(Bn), out_tokens=z(Bn, k + 1), n_out=z(Bn),
+                 next_cand=z(Bn, k), next_cand_prob=z(Bn, k, dt=torch.float32), finished=z(Bn, dt=torch.uint8), status=z(Bn))
+        ctx.space_step_host(B.HostStepArgs(batch=Bn, k=k, vocab=V, logits_dtype=B.DTYPE_BF16, mode=B.MODE_GREEDY, eos_id=-1,
+                                           scale=x["scale"], temperature=1.0, cache_resident=resident,
+                                           **{n: t.data_ptr() for n, t in h.items()}))
+        assert h["status"].tolist() == [0, B.ST_CAPACITY, 0]
+        for n in ("n_accept", "out_tokens", "n_out", "next_cand"):
+            assert np.array_equal(h[n].numpy(), r[n]), (n, resident)
+        for b in (0, 2):
+            L, na = int(x["kv_len"][b]), int(r["n_accept"][b])
+            ref, _ = attention_step(x["q"][b:b + 1], x["k_cache"][b:b + 1], x["v_cache"][b:b + 1], x["kv_len"][b:b + 1], k, x["scale"])
+            H.check_attention(h["out"][b:b + 1].numpy().astype(np.float64), ref, where)
+            assert int(h["kv_len"][b]) == L + na + 1
+            for name in ("k_cache", "v_cache"):
+                got = h[name].numpy().view(np.uint16)[b]
+                for g in range(na + 1):
+                    assert np.array_equal(got[:, L + g], x[name][b][:, L + g * (k + 1)])
+        assert np.array_equal(h["k_cache"].numpy().view(np.uint16)[1], x["k_cache"][1])
