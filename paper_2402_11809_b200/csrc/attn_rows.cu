@@ -68,8 +68,11 @@ __device__ __forceinline__ int page_of(const AttnParams& p, int b, int t, bool f
 // PTX helpers: tc_common.cuh.  Every wait of this kernel is bounded by WAIT_NS.
 using namespace tc;
 using namespace attn;
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site) {
+__device__ __noinline__ bool mbar_wait_long(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site) {
   return mbar_wait_bounded(bar, parity, abort_flag, err, site, WAIT_NS, 0);
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site) {
+  return mbar_try(bar, parity) || mbar_wait_long(bar, parity, abort_flag, err, site);   // (see mbar_wait_bounded)
 }
 __device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity) { mbar_drain_bounded(bar, parity, WAIT_NS); }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {

@@ -114,8 +114,11 @@ __device__ unsigned long long g_timeline_merge[4096 * 4];
 // PTX helpers: tc_common.cuh.  Every wait of this kernel is bounded by WAIT_NS.
 using namespace tc;
 using namespace attn;
-__device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site) {
+__device__ __noinline__ bool mbar_wait_long(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site) {
   return mbar_wait_bounded(bar, parity, abort_flag, err, site, WAIT_NS, 64);   // sleeps between polls
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site) {
+  return mbar_try(bar, parity) || mbar_wait_long(bar, parity, abort_flag, err, site);   // (see mbar_wait_bounded)
 }
 __device__ __noinline__ void mbar_drain(uint32_t bar, uint32_t parity) { mbar_drain_bounded(bar, parity, WAIT_NS); }
 

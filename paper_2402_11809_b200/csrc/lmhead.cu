@@ -85,9 +85,13 @@ struct LmParams {
 // PTX helpers: tc_common.cuh.  Every wait of this kernel is bounded by LM_WAIT_NS.
 // `backoff`: sleep between polls (the epilogue warps, which wait for a whole group of products).
 using namespace tc;
-__device__ __noinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site,
-                                          bool backoff = false) {
+__device__ __noinline__ bool mbar_wait_long(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site,
+                                            bool backoff) {
   return mbar_wait_bounded(bar, parity, abort_flag, err, site, LM_WAIT_NS, backoff ? 128u : 0u);
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int site,
+                                          bool backoff = false) {
+  return mbar_try(bar, parity) || mbar_wait_long(bar, parity, abort_flag, err, site, backoff);   // (see mbar_wait_bounded)
 }
 __device__ __noinline__ void mbar_drain(uint32_t bar, uint32_t parity) { mbar_drain_bounded(bar, parity, LM_WAIT_NS); }
 // Shared-memory matrix descriptor: K-major rows of 128 bytes, 128-byte swizzle

@@ -53,7 +53,9 @@ __device__ __forceinline__ uint64_t global_ns() {
 // before; the first expiry sets the block's abort flag and records `site` in *err (first one wins).
 // Once the flag is set every later wait returns at once, so the block drains instead of blocking.
 // sleep_ns > 0: sleep between polls (leaves the issue slots to the working warps).
-// (Inlined here; a kernel that wants one out-of-line copy wraps it in a __noinline__ function.)
+// (Inlined here; the kernels keep one out-of-line copy and try the barrier once before they call it: a wait
+// that has nothing to wait for takes 65 cycles that way instead of 166, and a role's loop has two or three of
+// them per tile.)
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, volatile int* abort_flag,
                                                int* err, int site, uint64_t limit_ns, uint32_t sleep_ns) {
   if (*abort_flag) return mbar_try(bar, parity);            // draining: never block
