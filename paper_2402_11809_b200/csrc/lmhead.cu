@@ -779,14 +779,16 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   const int max_len = (a->vocab + grid - 1) / grid + 15;   // the longest vocabulary range (boundaries are multiples of 16)
   p.n_box = max_len >= LM_MAX_BOX ? LM_MAX_BOX : (max_len + 15) / 16 * 16;
   p.tail_rows = (((max_len - 1) % p.n_box) + 1 + 15) / 16 * 16;
-  // Slices per stage and stages: two slices when that leaves at least three stages (measured 1..4
-  // slices on V = 32000, D = 4096: within 3 %), else one; as many stages as fit, at most LM_MAX_STAGES.
+  // Slices per stage: one (finer hand-over, more W in flight: with 144 block rows of V = 32000 two would leave
+  // two stages, 84 us instead of 69), except where a slice's products take less time than its hand-over, that is
+  // with few tokens per thread block (us for one / two / four: 64 rows of V = 2091 30 / 24 / 22, 25 rows of
+  // V = 5000 26 / 22 / 19, V = 12000 28 / 26 / -).  As many stages as fit, at most LM_MAX_STAGES.
   const size_t budget = 220 * 1024;
   int stages = 0;
-  for (p.kbs = 2; p.kbs >= 1; --p.kbs) {
+  for (p.kbs = p.n_box <= 128 ? 4 : 1; p.kbs >= 1; p.kbs /= 2) {
     stages = LM_MAX_STAGES;
     while (stages > 1 && LmSmem(p.n_pad, p.n_box, stages, p.kbs).total + 1024 > budget) --stages;
-    if (stages >= (p.kbs == 2 ? 3 : 2)) break;
+    if (stages >= (p.kbs > 1 ? 3 : 2)) break;
   }
   if (stages < 2) return SPACE_E_UNSUPPORTED;
   p.stages = stages;
