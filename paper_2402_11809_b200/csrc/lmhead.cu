@@ -23,8 +23,8 @@
 // whose box holds only the rows a range's tail can have, so a range reads at
 // most 15 rows of its neighbour.
 //
-// Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2..5 epilogue (one TMEM
-// lane quarter each).  With at most 128 block rows two accumulators alternate
+// Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2..9 epilogue (two per TMEM
+// lane quarter).  With at most 128 block rows two accumulators alternate
 // between boxes so that the epilogue of one box runs under the products of the
 // next.  Every wait is bounded; an expired wait sets SPACE_ST_TIMEOUT, the block
 // drains and exits.
@@ -35,7 +35,9 @@
 
 namespace {
 
-constexpr int LM_THREADS = 192;
+constexpr int LM_EPI = 8;                   // epilogue warps: two per TMEM lane quarter
+constexpr int LM_EPI_T = 32 * LM_EPI;
+constexpr int LM_THREADS = 64 + LM_EPI_T;
 constexpr int LM_M = 128;                   // block rows per accumulator (MMA M)
 constexpr int LM_MAX_BOX = 256;             // vocabulary rows per box (MMA N), at most
 constexpr int LM_KB = 64;                   // hidden elements per slice (128 bytes: one swizzle row)
@@ -116,7 +118,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(LM_EPI_T) : "memory"); }
 
 // (maximum, lowest token) of a row as one 64-bit key whose unsigned order is "larger logit
 // first, then lower token": the ranges of all thread blocks combine with one atomicMax each.
@@ -307,7 +309,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
   if (threadIdx.x == 0) {
     *abort_flag = (sm_base & 1023u) ? 1 : 0;               // swizzled tiles need a 1024-byte aligned base
     for (int s = 0; s < S; ++s) { mbar_init(LBAR(B_FULL + s), 1); mbar_init(LBAR(B_EMPTY + s), 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(LBAR(B_ACCFULL + a), 1); mbar_init(LBAR(B_ACCEMPTY + a), 4); }
+    for (int a = 0; a < 2; ++a) { mbar_init(LBAR(B_ACCFULL + a), 1); mbar_init(LBAR(B_ACCEMPTY + a), LM_EPI); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -421,16 +423,20 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
     // ================= epilogue ================================================
     const int quarter = warp & 3;                          // TMEM lanes 32*quarter .. +31
     const int ew = warp - 2;
-    const int row_a = quarter * 32 + lane;                 // this thread's block rows: row_a and row_a + 128
+    // The two warps of a lane quarter: with two accumulators each has one of them; with one accumulator they
+    // take its column groups in turn and meet at the end (a warp alone was what a sampling call waited for).
+    const int half = ew >> 2;
+    const bool split = p.n_mt == 1;
+    const int row = quarter * 32 + lane + (split ? 0 : half * LM_M);   // this thread's block row
     // the candidates are an input: fetched now, so that the last block's scan does not wait for them
-    for (int t = threadIdx.x - 64; t < p.B * p.k; t += 128) cand_s[t] = p.cand[t];
-    float m0 = LM_NEG, s0 = 0.f, m1 = LM_NEG, s1 = 0.f;
-    int i0 = 0x7FFFFFFF, i1 = 0x7FFFFFFF;
+    for (int t = threadIdx.x - 64; t < p.B * p.k; t += LM_EPI_T) cand_s[t] = p.cand[t];
+    float m0 = LM_NEG, s0 = 0.f;
+    int i0 = 0x7FFFFFFF;
     const bool sample = p.mode == SPACE_MODE_SAMPLE;
-    RowNoisy n0, n1;
-    if (sample) { row_noisy_init(n0, p, row_a); row_noisy_init(n1, p, p.n_mt == 2 ? LM_M + row_a : p.n_rows); }
+    RowNoisy n0;
+    if (sample) row_noisy_init(n0, p, row);
     // a warp whose 32 lanes hold no block row only takes part in the hand-shakes
-    const bool warp_a = quarter * 32 < p.n_rows, warp_b = p.n_mt == 2 && LM_M + quarter * 32 < p.n_rows;
+    const bool has_rows = row - lane < p.n_rows;
     bool ok = true;
     for (int box = 0; box < nb; ++box) {
       const int buf = n_bufs == 2 ? box & 1 : 0;
@@ -440,9 +446,9 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       tc_fence_after();
       const int row0 = r0 + box * p.n_box;
       const int n_valid = min(r1 - row0, (r1 - row0 <= p.tail_rows) ? p.tail_rows : p.n_box);
-      const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * p.n_mt * LM_MAX_BOX);
-      if (warp_a) {
-        for (int c0 = 0; c0 < n_valid; c0 += 16) {
+      const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((split ? buf : half) * LM_MAX_BOX);
+      if (has_rows) {
+        for (int c0 = split ? 16 * half : 0; c0 < n_valid; c0 += split ? 32 : 16) {
           uint32_t v[16];
           tmem_ld16(acc + (uint32_t)c0, v);
           tmem_wait_ld();
@@ -450,56 +456,59 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           else fold16(m0, s0, i0, v, row0 + c0, n_valid - c0);
         }
       }
-      if (warp_b) {
-        for (int c0 = 0; c0 < n_valid; c0 += 16) {
-          uint32_t v[16];
-          tmem_ld16(acc + (uint32_t)(LM_MAX_BOX + c0), v);
-          tmem_wait_ld();
-          if (sample) fold16_noisy(m1, s1, i1, n1, v, row0 + c0, n_valid - c0, p.c_t, p.key0, p.key1);
-          else fold16(m1, s1, i1, v, row0 + c0, n_valid - c0);
-        }
-      }
       // this accumulator buffer may be overwritten by the products of the next box that uses it
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(LBAR(B_ACCEMPTY + buf));
     }
+    if (split) {
+      // the second half's columns join the first's (the pipeline stages are idle: every product is done)
+      float* x = reinterpret_cast<float*>(smem_raw) + quarter * 32 + lane;   // [7][LM_M]
+      if (half == 1 && has_rows) {
+        x[0] = m0; x[LM_M] = s0; x[2 * LM_M] = __int_as_float(i0);
+        if (sample) { x[3 * LM_M] = n0.gs; x[4 * LM_M] = n0.gz; x[5 * LM_M] = __int_as_float(n0.gidx); x[6 * LM_M] = n0.zc; }
+      }
+      epi_sync();
+      if (half == 0 && has_rows) {
+        const float m2 = x[0], s2 = x[LM_M], c = sample ? p.c_t : LOG2E;
+        const int i2 = __float_as_int(x[2 * LM_M]);
+        if (m2 > m0 || (m2 == m0 && i2 < i0)) i0 = i2;
+        const float e = fast_exp2(-fabsf(m0 - m2) * c);     // (one of the two exponentials is exp(0))
+        s0 = (m0 >= m2) ? fmaf(s2, e, s0) : fmaf(s0, e, s2);
+        m0 = fmaxf(m0, m2);
+        if (sample) {
+          const float g2 = x[3 * LM_M];
+          const int gi2 = __float_as_int(x[5 * LM_M]);
+          if (g2 > n0.gs || (g2 == n0.gs && gi2 < n0.gidx)) { n0.gs = g2; n0.gz = x[4 * LM_M]; n0.gidx = gi2; }
+          n0.zc = fmaxf(n0.zc, x[6 * LM_M]);
+        }
+      }
+    }
     // publish this block's statistics of every block row
-    if (row_a < p.n_rows) {
+    if (row < p.n_rows && !(split && half == 1)) {
       LmPartial out; out.m = m0; out.s = s0; out.idx = i0; out.pad = 0;
-      *reinterpret_cast<int4*>(p.part + (size_t)row_a * G + c) = *reinterpret_cast<const int4*>(&out);
-      atomicMax(p.keys + row_a, argmax_key(m0, i0));
+      *reinterpret_cast<int4*>(p.part + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&out);
+      atomicMax(p.keys + row, argmax_key(m0, i0));
       if (sample) {
         LmNoisy g; g.gs = n0.gs; g.gz = n0.gz; g.gidx = n0.gidx; g.pad = 0;
-        *reinterpret_cast<int4*>(p.gpart + (size_t)row_a * G + c) = *reinterpret_cast<const int4*>(&g);
-        if ((unsigned)(n0.cand_tok - r0) < (unsigned)(r1 - r0)) p.zc[row_a] = n0.zc;   // this block owns the candidate's token
+        *reinterpret_cast<int4*>(p.gpart + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&g);
+        if ((unsigned)(n0.cand_tok - r0) < (unsigned)(r1 - r0)) p.zc[row] = n0.zc;   // this block owns the candidate's token
       }
     }
-    if (p.n_mt == 2 && LM_M + row_a < p.n_rows) {
-      LmPartial out; out.m = m1; out.s = s1; out.idx = i1; out.pad = 0;
-      *reinterpret_cast<int4*>(p.part + (size_t)(LM_M + row_a) * G + c) = *reinterpret_cast<const int4*>(&out);
-      atomicMax(p.keys + LM_M + row_a, argmax_key(m1, i1));
-      if (sample) {
-        LmNoisy g; g.gs = n1.gs; g.gz = n1.gz; g.gidx = n1.gidx; g.pad = 0;
-        *reinterpret_cast<int4*>(p.gpart + (size_t)(LM_M + row_a) * G + c) = *reinterpret_cast<const int4*>(&g);
-        if ((unsigned)(n1.cand_tok - r0) < (unsigned)(r1 - r0)) p.zc[LM_M + row_a] = n1.zc;
-      }
-    }
-    __threadfence();
     epi_sync();
-    const int et = threadIdx.x - 64;                       // 0..127
+    const int et = threadIdx.x - 64;                       // 0 .. LM_EPI_T-1
     if (et == 0) {
+      __threadfence();                                      // (the barrier ordered every thread's stores before this)
       const int prev = atomicAdd(p.counter, 1);
       const int last = prev == G - 1;
-      if (last) *p.counter = 0;                            // ready for the next launch
+      if (last) { *p.counter = 0; __threadfence(); }       // ready for the next launch
       *last_flag = last;
     }
     epi_sync();
     if (*last_flag) {
-      __threadfence();
       // ---- last thread block.  Every row's (maximum, arg-max) is already combined in its key;
       // only the k mask rows of group i* of every sequence need their sums, so only those rows'
-      // per-range partials are read, all of them at once over the 128 threads.
+      // per-range partials are read, all of them at once over the threads.
       const int k1 = p.k + 1;
       // the launch's rows of target t and of mask row (i*, j+1) of sequence b
       const bool with_targets = p.phase != LM_MASKS, with_masks = p.phase != LM_TARGETS;
@@ -508,7 +517,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       float* row_m = row_s;                                // [n_rows] maxima (row_s is reused: sums come later)
       int* istar = reinterpret_cast<int*>(smem_raw);       // [B] (the pipeline stages are idle now)
       float* terms = reinterpret_cast<float*>(smem_raw) + LM_MAX_N;   // [B * k][G] scaled sums of the ranges
-      for (int r = et; r < p.n_rows; r += 128) {
+      for (int r = et; r < p.n_rows; r += LM_EPI_T) {
         const unsigned long long key = atomicExch(p.keys + r, 0ull);      // read, and ready for the next launch
         float m; int idx;
         argmax_unkey(key, m, idx);
@@ -527,11 +536,11 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         const bool literal = p.resample == SPACE_RESAMPLE_PAPER_LITERAL;
         auto sum_rows = [&](bool mask_rows) {
           const int total = p.B * p.k * G;
-          for (int i0 = et; i0 < total; i0 += 128 * 8) {
+          for (int i0 = et; i0 < total; i0 += LM_EPI_T * 8) {
             int4 v[8]; float mx[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-              const int at = i0 + u * 128;
+              const int at = i0 + u * LM_EPI_T;
               v[u] = make_int4(0, 0, 0, 0); mx[u] = 0.f;
               if (at < total) {
                 const int g = at % G, bj = at / G;
@@ -543,12 +552,12 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-              const int at = i0 + u * 128;
+              const int at = i0 + u * LM_EPI_T;
               if (at < total) terms2[at] = __int_as_float(v[u].y) * fast_exp2((__int_as_float(v[u].x) - mx[u]) * cT);
             }
           }
           epi_sync();
-          for (int bj = ew; bj < p.B * p.k; bj += 4) {
+          for (int bj = ew; bj < p.B * p.k; bj += LM_EPI) {
             float sv = 0.f;
             for (int g = lane; g < G; g += 32) sv += terms2[bj * G + g];
             sv = warp_sum(sv);
@@ -576,7 +585,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         };
         if (with_targets) {
         sum_rows(false);                                   // target rows t = 0..k-1 of every sequence
-        for (int b = ew; b < p.B; b += 4) {
+        for (int b = ew; b < p.B; b += LM_EPI) {
           const int t = lane;
           const int cv = (t < p.k) ? cand_s[b * p.k + t] : -1;
           const bool in_range = cv >= 0 && cv < p.V;
@@ -612,11 +621,11 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           }
         }
         } else {
-          for (int b = et; b < p.B; b += 128) istar[b] = p.n_accept[b];
+          for (int b = et; b < p.B; b += LM_EPI_T) istar[b] = p.n_accept[b];
         }
         epi_sync();
         if (with_masks && !literal) {                      // point-mass drafts: arg-max of mask row (i*, j+1), P_c = 1
-          for (int bj = et; bj < p.B * p.k; bj += 128) {
+          for (int bj = et; bj < p.B * p.k; bj += LM_EPI_T) {
             const int b = bj / p.k, j = bj - b * p.k;
             p.next_cand[bj] = row_i[mask_row(b, istar[b], j)];
             p.next_cand_prob[bj] = 1.f;
@@ -624,7 +633,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         } else if (with_masks) {
           // candidates sampled from the mask rows of group i*, with their probabilities
           sum_rows(true);
-          for (int bj = ew; bj < p.B * p.k; bj += 4) {
+          for (int bj = ew; bj < p.B * p.k; bj += LM_EPI) {
             const int b = bj / p.k, jj = bj - b * p.k;
             const int row = mask_row(b, istar[b], jj);
             float gz;
@@ -637,7 +646,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         }
       } else {
       // acceptance scan and emitted tokens: one warp per sequence
-      for (int b = ew; b < p.B && with_targets; b += 4) {
+      for (int b = ew; b < p.B && with_targets; b += LM_EPI) {
         const int cv = (lane < p.k) ? cand_s[b * p.k + lane] : -1;
         const bool in_range = cv >= 0 && cv < p.V;
         const unsigned bad = __ballot_sync(0xFFFFFFFFu, lane < p.k && !in_range);
@@ -659,15 +668,15 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           if (p.status && bad) atomicOr(p.status + b, SPACE_ST_BAD_CANDIDATE);
         }
       }
-      if (!with_targets) for (int b = et; b < p.B; b += 128) istar[b] = p.n_accept[b];
+      if (!with_targets) for (int b = et; b < p.B; b += LM_EPI_T) istar[b] = p.n_accept[b];
       epi_sync();
       // sums of the mask rows of group i*: (sequence, mask row, range) triples spread over the threads
       const int total = with_masks ? p.B * p.k * G : 0;
-      for (int i0 = et; i0 < total; i0 += 128 * 8) {
+      for (int i0 = et; i0 < total; i0 += LM_EPI_T * 8) {
         int4 v[8]; float mx[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const int at = i0 + u * 128;
+          const int at = i0 + u * LM_EPI_T;
           v[u] = make_int4(0, 0, 0, 0); mx[u] = 0.f;
           if (at < total) {
             const int g = at % G, bj = at / G;
@@ -679,13 +688,13 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         }
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const int at = i0 + u * 128;
+          const int at = i0 + u * LM_EPI_T;
           if (at < total) terms[at] = __int_as_float(v[u].y) * fast_exp2((__int_as_float(v[u].x) - mx[u]) * LOG2E);
         }
       }
       epi_sync();
       // fixed summation order: the result does not depend on which block came last or on timing
-      for (int bj = ew; bj < p.B * p.k && with_masks; bj += 4) {
+      for (int bj = ew; bj < p.B * p.k && with_masks; bj += LM_EPI) {
         float sv = 0.f;
         for (int g = lane; g < G; g += 32) sv += terms[bj * G + g];
         sv = warp_sum(sv);
