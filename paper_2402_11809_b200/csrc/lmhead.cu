@@ -23,7 +23,7 @@
 // whose box holds only the rows a range's tail can have, so a range reads at
 // most 15 rows of its neighbour.
 //
-// Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2..9 epilogue (two per TMEM
+// Warps: 0 TMA producer, 1 TMEM owner and MMA issuer, 2..17 epilogue (four per TMEM
 // lane quarter).  With at most 128 block rows two accumulators alternate
 // between boxes so that the epilogue of one box runs under the products of the
 // next.  Every wait is bounded; an expired wait sets SPACE_ST_TIMEOUT, the block
@@ -35,7 +35,7 @@
 
 namespace {
 
-constexpr int LM_EPI = 8;                   // epilogue warps: two per TMEM lane quarter
+constexpr int LM_EPI = 16;                  // epilogue warps: four per TMEM lane quarter
 constexpr int LM_EPI_T = 32 * LM_EPI;
 constexpr int LM_THREADS = 64 + LM_EPI_T;
 constexpr int LM_M = 128;                   // block rows per accumulator (MMA M)
@@ -423,11 +423,11 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
     // ================= epilogue ================================================
     const int quarter = warp & 3;                          // TMEM lanes 32*quarter .. +31
     const int ew = warp - 2;
-    // The two warps of a lane quarter: with two accumulators each has one of them; with one accumulator they
-    // take its column groups in turn and meet at the end (a warp alone was what a sampling call waited for).
-    const int half = ew >> 2;
-    const bool split = p.n_mt == 1;
-    const int row = quarter * 32 + lane + (split ? 0 : half * LM_M);   // this thread's block row
+    // The warps of a lane quarter share the accumulators, and take an accumulator's column groups in turn;
+    // they meet at the end (with one warp per quarter its scan was what a call ended on, and what a sampling
+    // call waited for all along).
+    const int mt = (ew >> 2) % p.n_mt, n_parts = LM_EPI / 4 / p.n_mt, part = (ew >> 2) / p.n_mt;
+    const int row = mt * LM_M + quarter * 32 + lane;       // this thread's block row
     // the candidates are an input: fetched now, so that the last block's scan does not wait for them
     for (int t = threadIdx.x - 64; t < p.B * p.k; t += LM_EPI_T) cand_s[t] = p.cand[t];
     float m0 = LM_NEG, s0 = 0.f;
@@ -446,9 +446,9 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       tc_fence_after();
       const int row0 = r0 + box * p.n_box;
       const int n_valid = min(r1 - row0, (r1 - row0 <= p.tail_rows) ? p.tail_rows : p.n_box);
-      const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((split ? buf : half) * LM_MAX_BOX);
+      const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((buf * p.n_mt + mt) * LM_MAX_BOX);
       if (has_rows) {
-        for (int c0 = split ? 16 * half : 0; c0 < n_valid; c0 += split ? 32 : 16) {
+        for (int c0 = 16 * part; c0 < n_valid; c0 += 16 * n_parts) {
           uint32_t v[16];
           tmem_ld16(acc + (uint32_t)c0, v);
           tmem_wait_ld();
@@ -461,31 +461,36 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       __syncwarp();
       if (lane == 0) mbar_arrive(LBAR(B_ACCEMPTY + buf));
     }
-    if (split) {
-      // the second half's columns join the first's (the pipeline stages are idle: every product is done)
-      float* x = reinterpret_cast<float*>(smem_raw) + quarter * 32 + lane;   // [7][LM_M]
-      if (half == 1 && has_rows) {
-        x[0] = m0; x[LM_M] = s0; x[2 * LM_M] = __int_as_float(i0);
-        if (sample) { x[3 * LM_M] = n0.gs; x[4 * LM_M] = n0.gz; x[5 * LM_M] = __int_as_float(n0.gidx); x[6 * LM_M] = n0.zc; }
+    {
+      // the other parts' columns join the first's (the pipeline stages are idle: every product is done)
+      float* x = reinterpret_cast<float*>(smem_raw) + row;   // [n_parts - 1][7][2 LM_M]
+      constexpr int W = 2 * LM_M;
+      if (part > 0 && has_rows) {
+        float* y = x + (part - 1) * 7 * W;
+        y[0] = m0; y[W] = s0; y[2 * W] = __int_as_float(i0);
+        if (sample) { y[3 * W] = n0.gs; y[4 * W] = n0.gz; y[5 * W] = __int_as_float(n0.gidx); y[6 * W] = n0.zc; }
       }
       epi_sync();
-      if (half == 0 && has_rows) {
-        const float m2 = x[0], s2 = x[LM_M], c = sample ? p.c_t : LOG2E;
-        const int i2 = __float_as_int(x[2 * LM_M]);
-        if (m2 > m0 || (m2 == m0 && i2 < i0)) i0 = i2;
-        const float e = fast_exp2(-fabsf(m0 - m2) * c);     // (one of the two exponentials is exp(0))
-        s0 = (m0 >= m2) ? fmaf(s2, e, s0) : fmaf(s0, e, s2);
-        m0 = fmaxf(m0, m2);
-        if (sample) {
-          const float g2 = x[3 * LM_M];
-          const int gi2 = __float_as_int(x[5 * LM_M]);
-          if (g2 > n0.gs || (g2 == n0.gs && gi2 < n0.gidx)) { n0.gs = g2; n0.gz = x[4 * LM_M]; n0.gidx = gi2; }
-          n0.zc = fmaxf(n0.zc, x[6 * LM_M]);
+      if (part == 0 && has_rows) {
+        for (int o = 1; o < n_parts; ++o) {
+          const float* y = x + (o - 1) * 7 * W;
+          const float m2 = y[0], s2 = y[W], c = sample ? p.c_t : LOG2E;
+          const int i2 = __float_as_int(y[2 * W]);
+          if (m2 > m0 || (m2 == m0 && i2 < i0)) i0 = i2;
+          const float e = fast_exp2(-fabsf(m0 - m2) * c);   // (one of the two exponentials is exp(0))
+          s0 = (m0 >= m2) ? fmaf(s2, e, s0) : fmaf(s0, e, s2);
+          m0 = fmaxf(m0, m2);
+          if (sample) {
+            const float g2 = y[3 * W];
+            const int gi2 = __float_as_int(y[5 * W]);
+            if (g2 > n0.gs || (g2 == n0.gs && gi2 < n0.gidx)) { n0.gs = g2; n0.gz = y[4 * W]; n0.gidx = gi2; }
+            n0.zc = fmaxf(n0.zc, y[6 * W]);
+          }
         }
       }
     }
     // publish this block's statistics of every block row
-    if (row < p.n_rows && !(split && half == 1)) {
+    if (row < p.n_rows && part == 0) {
       LmPartial out; out.m = m0; out.s = s0; out.idx = i0; out.pad = 0;
       *reinterpret_cast<int4*>(p.part + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&out);
       atomicMax(p.keys + row, argmax_key(m0, i0));
