@@ -845,20 +845,19 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
 
 }  // namespace
 
-// Which launches a batch takes.  Up to 128 block rows: one launch over all of them, bound by the stream of
-// the output embedding (one pass).  More: the step decides on 2k+1 rows of every sequence only, so the target
-// rows go first and the mask rows of the groups they select second -- two passes over the embedding, each at
-// the pace of the stream, instead of one or more over all (k+1)^2 rows that the product (from 128 rows on)
-// or the noise (a Philox block and eight logarithms per four tokens in every epilogue warp) paces.
-// Greedy calls of 129..256 rows stay with one launch: its 1.5 passes' time beats two (4 x 36 rows of
-// D = 4096, V = 32000: 83 us against 104), and so do calls that ask for every row's maximum.
-// Measured: 16 x 36 rows, V = 128256, sampling 934 -> 396 us; 4 x 49 rows, D = 1088, V = 128256 163 -> 129 us.
+// Which launches a batch takes.  Up to 256 block rows: one launch over all of them, one pass over the output
+// embedding.  More: the step decides on 2k+1 rows of every sequence only, so the target rows go first and the
+// mask rows of the groups they select second -- two passes over the embedding, each near the pace of its
+// stream, instead of one per 256 rows at the pace of the product.  Calls that ask for every row's maximum
+// keep to the full rows.
+// Measured: 16 x 36 rows, V = 128256, D = 4096, sampling: 934 us as three launches over all rows, 363 by phase;
+// 4 x 36 rows, V = 32000, sampling: 111 by phase, 73 as one launch; 16 x 16 rows of V = 50257: 168 and 125.
 int launch_lmhead_verify(space_ctx* ctx, const space_lmhead_args* a, cudaStream_t st) {
   const int n_q = (a->k + 1) * (a->k + 1), k1 = a->k + 1;
   const int rows = a->batch * n_q;
   const int64_t fit = LM_GATHER_ELEMS / ((int64_t)a->k * a->hidden_dim);   // sequences whose mask rows can be gathered
   const int per_phase = fit < LM_M / k1 ? (int)fit : LM_M / k1, per_all = LM_MAX_N / n_q;
-  bool by_phase = per_phase > 0 && !a->row_max && !a->row_argmax && rows > (a->mode == SPACE_MODE_SAMPLE ? LM_M : LM_MAX_N);
+  bool by_phase = per_phase > 0 && !a->row_max && !a->row_argmax && rows > LM_MAX_N;
   // a small embedding (under about 10 us of stream) is paced by launches instead: as few of them as can be
   if (by_phase && (int64_t)a->vocab * a->hidden_dim < (32ll << 20))
     by_phase = 2 * ((a->batch + per_phase - 1) / per_phase) < (a->batch + per_all - 1) / per_all;
