@@ -234,8 +234,17 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
   const int n_quarters = (m_valid + 31) >> 5;              // TMEM lane quarters with live rows
   const int n_soft = 64 * n_quarters;                      // softmax threads that take part
 
+  // the query rows' box holds rows_per_mb block rows; the rows after them in shared memory stay zero
+  const int q_rows = p.rows_per_mb * p.G;
+  const uint32_t q_bytes = (uint32_t)q_rows * DH * 2;
+
   // ---- set-up ------------------------------------------------------------
   pdl_launch_dependents();
+  for (int x = q_rows * 8 + threadIdx.x; x < ROWS * 8; x += THREADS)      // 16-byte pieces of 128-byte rows
+#pragma unroll
+    for (int hf = 0; hf < S::HALVES; ++hf)
+      asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(sm_base + S::Q_OFF + hf * (ROWS * 128) + x * 16), "r"(0u) : "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (threadIdx.x == 0) {
     *abort_flag = (sm_base & 1023u) ? 1 : 0;               // swizzled tiles need a 1024-byte aligned base
     mbar_init(BAR(B_QFULL), 1);
@@ -275,7 +284,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
   if (cl_mine && warp == WARP_K && lane == 0 && !*abort_flag) {
     // the query rows and the first K tile, before any length is read (should the length turn out too short for
     // that tile, or the cut not be taken, the S issuer lets both buffers go unused)
-    mbar_expect_tx(BAR(B_QFULL), S::Q_BYTES);
+    mbar_expect_tx(BAR(B_QFULL), q_bytes);
 #pragma unroll
     for (int hf = 0; hf < S::HALVES; ++hf)
       tma_load_4d(sm_base + S::Q_OFF + hf * (ROWS * 128), &p.tm_q, BAR(B_QFULL), hf * 64, cl_h * p.G, i0, cl_b);
@@ -363,7 +372,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
           if (!pre) {
             if (seg > 0) ok = mbar_wait(BAR(B_QEMPTY), (seg - 1) & 1, abort_flag, p.err, 3);
             if (!ok) break;
-            mbar_expect_tx(BAR(B_QFULL), S::Q_BYTES);
+            mbar_expect_tx(BAR(B_QFULL), q_bytes);
 #pragma unroll
             for (int hf = 0; hf < S::HALVES; ++hf)
               tma_load_4d(sm_base + S::Q_OFF + hf * (ROWS * 128), &p.tm_q, BAR(B_QFULL), hf * 64,
@@ -536,7 +545,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
           // four independent running maxima: one chain over 64 values would cost 64 dependent steps
           float t4[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
 #pragma unroll
-          for (int cidx = 0; cidx < HC; ++cidx) t4[cidx & 3] = fmaxf(t4[cidx & 3], __uint_as_float(sreg[cidx]));
+          for (int cidx = 0; cidx < HC; cidx += 2)
+            t4[(cidx >> 1) & 3] = max3(t4[(cidx >> 1) & 3], __uint_as_float(sreg[cidx]), __uint_as_float(sreg[cidx + 1]));
           tmax = fmaxf(fmaxf(t4[0], t4[1]), fmaxf(t4[2], t4[3]));
         }
         // the row maximum needs the other half's keys; the pair barrier also orders
@@ -570,21 +580,34 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
           }
           tmem_wait_st();
         }
-        const float m_use = (m_ref > -CUDART_INF_F) ? m_ref : 0.f;
+        // (rows past the last one are kept at zero, in Q and in P: under the power cap a product's energy is time,
+        // and zeros cost little of it)
+        const float m_use = !row_valid ? CUDART_INF_F : (m_ref > -CUDART_INF_F) ? m_ref : 0.f;
         // P = P_hi + P_lo, two bf16 terms: bf16 alone (8 significant bits) leaves
         // an output error near 1e-2 of the output RMS.  P_hi occupies columns
         // 0..63 of the S buffer, P_lo columns 64..127 (two keys per column).
         uint32_t lreg[HC / 2];
+        const uint64_t cc = pack2(c, c), mm = pack2(-m_use, -m_use), neg = pack2(-1.f, -1.f);
+        uint64_t sum[2] = {0ull, 0ull};
 #pragma unroll
         for (int x = 0; x < HC / 2; ++x) {
-          const float p0 = fast_exp2(fmaf(__uint_as_float(sreg[2 * x]), c, -m_use));
-          const float p1 = fast_exp2(fmaf(__uint_as_float(sreg[2 * x + 1]), c, -m_use));
-          l_sum += p0 + p1;
+          float e0, e1;
+          unpack2(fma2(pack2(__uint_as_float(sreg[2 * x]), __uint_as_float(sreg[2 * x + 1])), cc, mm), e0, e1);
+          const float p0 = fast_exp2(e0), p1 = fast_exp2(e1);
+          const uint64_t pp = pack2(p0, p1);
+          sum[x & 1] = add2(sum[x & 1], pp);
           const __nv_bfloat162 hi = __floats2bfloat162_rn(p0, p1);   // .x (low half) = even key
           const float2 hf = __bfloat1622float2(hi);
-          const __nv_bfloat162 lw = __floats2bfloat162_rn(p0 - hf.x, p1 - hf.y);
+          float l0, l1;
+          unpack2(fma2(pack2(hf.x, hf.y), neg, pp), l0, l1);         // (exact)
+          const __nv_bfloat162 lw = __floats2bfloat162_rn(l0, l1);
           sreg[x] = *reinterpret_cast<const uint32_t*>(&hi);
           lreg[x] = *reinterpret_cast<const uint32_t*>(&lw);
+        }
+        {
+          float a0, a1;
+          unpack2(add2(sum[0], sum[1]), a0, a1);
+          l_sum += a0 + a1;
         }
         tmem_st32(ts + half * (HC / 2), sreg);
         tmem_st32(ts + TILE_N / 2 + half * (HC / 2), lreg);
@@ -867,7 +890,7 @@ int launch_attn_rows(space_ctx* ctx, const space_attn_args* a, const uint64_t* m
     const cuuint32_t kb[4] = {64, TILE_N, 1, 1};
     const cuuint64_t qd[4] = {(cuuint64_t)DH, (cuuint64_t)p.H_q, (cuuint64_t)p.n_q, (cuuint64_t)a->batch};
     const cuuint64_t qs[3] = {(cuuint64_t)DH * 2, (cuuint64_t)p.H_q * DH * 2, (cuuint64_t)p.n_q * p.H_q * DH * 2};
-    const cuuint32_t qb[4] = {64, (cuuint32_t)p.G, (cuuint32_t)(ROWS / p.G), 1};
+    const cuuint32_t qb[4] = {64, (cuuint32_t)p.G, (cuuint32_t)p.rows_per_mb, 1};
     int rc = make_map((CUtensorMap*)ctx->tm_k, a->k_cache, kd, ks, kb);
     if (rc == SPACE_OK) rc = make_map((CUtensorMap*)ctx->tm_v, a->v_cache, kd, ks, kb);
     if (rc == SPACE_OK) rc = make_map((CUtensorMap*)ctx->tm_q, a->q, qd, qs, qb);
