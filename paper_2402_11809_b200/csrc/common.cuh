@@ -115,19 +115,19 @@ __device__ __forceinline__ void prefetch_chunk(const T* row, int begin, int end)
 }
 
 // Chunks per row and their length.  A sweep of a block is four vectors per thread (8192 bf16 logits); a
-// block costs about 3 us whatever it scans (reduction, fence, arrival), so it should make one sweep while
-// there are fewer of them than about three resident blocks per SM can take at once, and up to four when
-// there are more.  Measured, us per call: one row-chunk per SM's worth of blocks as before / this rule:
-// 5 x 16 rows of 50257 15.2 / 9.9, 2 x 49 rows of 128256 21.3 / 12, one sequence of 36 rows of 32000 6.4 / 6.4,
-// sampling 64 x 5 rows of 128256 67 / 57; one sweep per block there instead of four 71.
+// block costs about 3 us whatever it scans (reduction, fence, arrival).  So: as few sweeps per block as let all
+// blocks be resident at once (three per SM, and a few more), four where they cannot be.  Measured, us per call with
+// 1 / 2 / 3 / 4 sweeps per block: 80 rows of 50257 9.5 / 8.1 / 9.0 / 10.6, 98 rows of 128256 16 / 12 / 11 / 9.9,
+// 576 rows of 32000 22 / 16 / 16 / 15, top-10 lists of 72 and 48 rows of 128256 45 / 37 / 35 / 39 (33 with three
+// and two), sampling 64 x 5 rows of 128256 105 / 71 / 67 / 57.
 static inline int row_chunks(int vocab, int rows, int vec, int sm_count, int max_chunks, int* chunk_out) {
   const int sweep = SPACE_VERIFY_THREADS * vec * 4;
-  const int64_t total = (int64_t)rows * ((vocab + sweep - 1) / sweep);
-  const int64_t slots = 3 * (int64_t)sm_count;
-  int64_t per_block = (total + slots / 2) / slots;
-  if (per_block < 1) per_block = 1;
-  if (per_block > 4) per_block = 4;
-  int64_t nc = (vocab + per_block * sweep - 1) / (per_block * sweep);
+  const int64_t slots = 3 * (int64_t)sm_count * 21 / 20;
+  int64_t nc = 1;
+  for (int per_block = 1; per_block <= 4; ++per_block) {
+    nc = (vocab + (int64_t)per_block * sweep - 1) / ((int64_t)per_block * sweep);
+    if (nc * rows <= slots) break;
+  }
   if (nc > max_chunks) nc = max_chunks;
   int chunk = (int)((vocab + nc - 1) / nc);
   chunk = (chunk + vec - 1) / vec * vec;
