@@ -375,21 +375,13 @@ __device__ Stat block_reduce_plain(Stat st, float c) {
 }
 
 __device__ __forceinline__ void store_partial(VerifyPartial* p, const Stat& st) {
-  VerifyPartial v;
-  v.m = st.m; v.s = st.s; v.gs = st.gs; v.idx = st.idx; v.gidx = st.gidx;
-  v.pad0 = v.pad1 = v.pad2 = 0;
-  *reinterpret_cast<volatile float*>(&p->m) = v.m;
-  *reinterpret_cast<volatile float*>(&p->s) = v.s;
-  *reinterpret_cast<volatile float*>(&p->gs) = v.gs;
-  *reinterpret_cast<volatile int*>(&p->idx) = v.idx;
-  *reinterpret_cast<volatile int*>(&p->gidx) = v.gidx;
+  __stcg(reinterpret_cast<float4*>(p), make_float4(st.m, st.s, st.gs, __int_as_float(st.idx)));
+  __stcg(&p->gidx, st.gidx);
 }
 
 __device__ __forceinline__ Stat load_partial(const VerifyPartial* p) {
-  Stat st;
-  st.m = __ldcg(&p->m); st.s = __ldcg(&p->s); st.gs = __ldcg(&p->gs);
-  st.idx = __ldcg(&p->idx); st.gidx = __ldcg(&p->gidx);
-  return st;
+  const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
+  return Stat{v.x, v.y, __float_as_int(v.w), v.z, __ldcg(&p->gidx)};
 }
 
 // Combine the chunk partials of one row with a warp; result valid in every lane.
@@ -399,18 +391,17 @@ __device__ Stat gather_row(const VerifyPartial* p, int n_chunks, float c) {
   return warp_reduce(st, c);
 }
 
-// Returns true in exactly one block per sequence: the last one to arrive.
+// Returns true in exactly one block per sequence: the last one to arrive.  Thread 0 has stored the block's
+// result; its release-acquire count hands it over, whatever else the other threads still have to store.
 __device__ bool arrive_last(int* counter, int expected) {
   __shared__ int last;
-  __threadfence();
-  __syncthreads();
   if (threadIdx.x == 0) {
-    const int prev = atomicAdd(counter, 1);
+    int prev;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(prev) : "l"(counter) : "memory");
     last = (prev == expected - 1);
     if (last) *counter = 0;            // ready for the next launch
   }
   __syncthreads();
-  if (last) __threadfence();
   return last != 0;
 }
 
@@ -424,7 +415,19 @@ verify_target_kernel(const VerifyParams p) {
   const int begin = ch * p.chunk, end = min(p.V, begin + p.chunk);
   if (!p.mapped) prefetch_chunk<T>(row, begin, end);
   pdl_wait();
+  // what the block that finishes the sequence needs besides the rows' results: fetched by every block, in
+  // flight during the scan (warp tt < k tests candidate c_{tt+1})
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool sample = p.mode == SPACE_MODE_SAMPLE, tests = lane == 0 && warp < p.k;
+  const int my_cand = tests ? p.cand[b * p.k + warp] : -1;
+  const float my_prob = tests && sample ? p.cand_prob[b * p.k + warp] : 0.f;
+  const uint32_t seq = tests && sample && p.seq_id ? p.seq_id[b] : (uint32_t)b;
+  const int L = tests && sample && p.kv_len ? p.kv_len[b] : 0;
   Stat st = scan_chunk<T, ALIGNED, false, STAT_SUM>(row, begin, end, p.c_t, -1, 0, 0, 0, 0, 0);
+  const bool in_range = my_cand >= 0 && my_cand < p.V;
+  float zc = 0.f;
+  if (sample && in_range)
+    zc = load_logit(reinterpret_cast<const T*>(p.logits) + ((int64_t)b * p.n_q + (int64_t)warp * k1) * p.row_stride + my_cand);
   st = block_reduce_plain(st, p.c_t);
   VerifyPartial* part = p.part + ((int64_t)b * (p.k + 2) + t) * p.n_chunks;
   if (threadIdx.x == 0) store_partial(part + ch, st);
@@ -435,7 +438,6 @@ verify_target_kernel(const VerifyParams p) {
   // acceptance test of candidate c_{tt+1}; thread 0 then walks the prefix.
   __shared__ int sh_ok[SPACE_MAX_K + 1];
   __shared__ int sh_bits;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) sh_bits = 0;
   __syncthreads();
   if (warp < k1) {
@@ -446,24 +448,14 @@ verify_target_kernel(const VerifyParams p) {
       p.rows[b * k1 + tt] = vr;
       bool ok = false;
       if (tt < p.k) {                  // row tt scores candidate c_{tt+1}
-        const int c = p.cand[b * p.k + tt];
-        const bool in_range = (c >= 0 && c < p.V);
         if (!in_range) atomicOr(&sh_bits, SPACE_ST_BAD_CANDIDATE);
-        if (p.mode == SPACE_MODE_GREEDY) {
-          ok = in_range && (c == r.idx);
+        if (!sample) {
+          ok = in_range && (my_cand == r.idx);
         } else {
-          const T* base = reinterpret_cast<const T*>(p.logits) + (int64_t)b * p.n_q * p.row_stride;
-          const uint32_t seq = p.seq_id ? p.seq_id[b] : (uint32_t)b;
-          const int L = p.kv_len ? p.kv_len[b] : 0;
-          float q = 0.f;
-          if (in_range) {
-            const float zc = load_logit(base + (int64_t)tt * k1 * p.row_stride + c);
-            q = fast_exp2((zc - r.m) * p.c_t) / r.s;
-          }
+          const float q = in_range ? fast_exp2((zc - r.m) * p.c_t) / r.s : 0.f;
           const Philox4 w = philox4x32_10(0u, PURPOSE_ACCEPT, seq, (uint32_t)(L + tt + 1), p.key0, p.key1);
-          const float pc = p.cand_prob[b * p.k + tt];
-          const float lhs = uniform_open(w.x) * pc;                          // r <= Q/P_c  <=>  r*P_c <= Q
-          ok = in_range && pc > 0.f && lhs <= q;                             // NaN, zero or negative P_c: rejected
+          const float lhs = uniform_open(w.x) * my_prob;                     // r <= Q/P_c  <=>  r*P_c <= Q
+          ok = in_range && my_prob > 0.f && lhs <= q;                        // NaN, zero or negative P_c: rejected
         }
       }
       sh_ok[tt] = ok;
