@@ -28,7 +28,7 @@
 // 24 x 3 rows of 128256 logits and 65 us on ten rows of 32000 with top_k = 32.)
 // Keys are 64-bit words whose unsigned order is "larger logit, then lower token", so exact ties go to
 // the lower token everywhere.  Block lists go to a scratch array, and an arrival counter picks the block
-// that finishes a sequence; it merges the lists of a row with one warp, a list per lane.
+// that finishes a sequence; it merges the lists of a row with one warp.
 #include "common.cuh"
 #include <math_constants.h>
 
@@ -82,13 +82,6 @@ __device__ __forceinline__ unsigned long long shfl_xor64(unsigned long long x, i
   const uint32_t lo = __shfl_xor_sync(0xFFFFFFFFu, (uint32_t)x, o), hi = __shfl_xor_sync(0xFFFFFFFFu, (uint32_t)(x >> 32), o);
   return ((unsigned long long)hi << 32) | lo;
 }
-// Largest key over the warp, in every lane (keys are distinct, or 0 = none).
-__device__ __forceinline__ unsigned long long warp_max64(unsigned long long x) {
-  const uint32_t hi = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(x >> 32));
-  const uint32_t lo = __reduce_max_sync(0xFFFFFFFFu, (uint32_t)(x >> 32) == hi ? (uint32_t)x : 0u);
-  return ((unsigned long long)hi << 32) | lo;
-}
-
 __device__ __forceinline__ float ld_logit(const float* p) { return *p; }
 __device__ __forceinline__ float ld_logit(const __nv_bfloat16* p) { return __bfloat162float(*p); }
 
@@ -108,7 +101,8 @@ struct FiltShared {
   unsigned long long tau;
   int count, last, bits, i_star;
   int ok[SPACE_MAX_K + 1];
-  unsigned long long buf[FILT_BUF];    // collected keys of a segment, later the chunk lists of the rows the last block works on
+  unsigned long long buf[FILT_BUF];    // collected keys of a segment, later those of the rows the last block works on
+  unsigned long long top[FILT_THREADS / 32][FILT_MAX_K];
 };
 static_assert(FILT_BUF >= FILT_MAX_K * FILT_GROUP * FILT_U * 8, "one sweep's keys of the longest list must fit");
 static_assert(FILT_BUF >= (SPACE_MAX_K + 1) * FILT_MAX_CHUNKS * FILT_MAX_K, "the chunk lists of k+1 rows must fit");
@@ -240,19 +234,50 @@ __device__ int chunk_top_k(const T* row, int begin, int end, int K, FiltShared& 
   return cur;
 }
 
-// Sorted top K of a row from its chunks' sorted lists in shared memory (lists[c * 32 + j]), lane j
-// holding the j-th largest: every lane stands for one list, K rounds of a warp-wide maximum.
-__device__ __forceinline__ unsigned long long merge_lists(const unsigned long long* lists, int n_chunks, int K, int lane) {
-  unsigned long long mine = 0ull;
-  int at = 0;
-  unsigned long long head = lane < n_chunks ? lists[lane * FILT_MAX_K] : 0ull;
-  for (int j = 0; j < K; ++j) {
-    const unsigned long long best = warp_max64(head);
-    if (best == 0ull) break;                                // (the same in every lane)
-    if (lane == j) mine = best;
-    if (head == best) { ++at; head = at < K ? lists[lane * FILT_MAX_K + at] : 0ull; }
+__device__ __forceinline__ unsigned long long shfl64(unsigned long long x, int src) {
+  const uint32_t lo = __shfl_sync(0xFFFFFFFFu, (uint32_t)x, src), hi = __shfl_sync(0xFFFFFFFFu, (uint32_t)(x >> 32), src);
+  return ((unsigned long long)hi << 32) | lo;
+}
+// Sorted top K of a row from its chunks' sorted lists in L2 (lists[c * 32 + j]), lane j holding the j-th largest:
+// all lists are fetched at once, a bound that at least K keys reach leaves a few more than K of them (the largest
+// K-th key of a list, or the smallest key at the place that K / n_chunks keys of every list reach), and those are
+// ranked by counting in shared memory (tmp: n_chunks * K keys, out: K keys, the warp's own).  (K rounds of a
+// warp-wide maximum over the lists' heads took 3 us for ten keys, 7 for 23.)
+__device__ unsigned long long merge_lists(const unsigned long long* lists, int n_chunks, int K, int lane,
+                                          unsigned long long* tmp, unsigned long long* out) {
+  unsigned long long v[FILT_MAX_CHUNKS];
+#pragma unroll
+  for (int c = 0; c < FILT_MAX_CHUNKS; ++c)
+    v[c] = c < n_chunks && lane < K ? __ldcg(lists + c * FILT_MAX_K + lane) : 0ull;
+  unsigned long long lo = ~0ull, hi = 0ull;
+#pragma unroll
+  for (int c = 0; c < FILT_MAX_CHUNKS; ++c) {
+    if (c < n_chunks && v[c] < lo) lo = v[c];
+    if (v[c] > hi) hi = v[c];
   }
-  return mine;
+  lo = shfl64(lo, (K + n_chunks - 1) / n_chunks - 1);
+  hi = shfl64(hi, K - 1);
+  const unsigned long long tau = lo > hi ? lo : hi;
+  int n = 0;
+#pragma unroll
+  for (int c = 0; c < FILT_MAX_CHUNKS; ++c) {
+    const bool keep = v[c] != 0ull && v[c] >= tau;
+    const unsigned who = __ballot_sync(0xFFFFFFFFu, keep);
+    if (keep) tmp[n + __popc(who & ((1u << lane) - 1u))] = v[c];
+    n += __popc(who);
+  }
+  out[lane] = 0ull;
+  __syncwarp();
+  for (int i = lane; i < n; i += 64) {                      // two keys per lane and pass
+    const unsigned long long a = tmp[i], b = i + 32 < n ? tmp[i + 32] : 0ull;
+    int ra = 0, rb = 0;
+#pragma unroll 8
+    for (int j = 0; j < n; ++j) { const unsigned long long x = tmp[j]; ra += x > a; rb += x > b; }
+    if (ra < K) out[ra] = a;
+    if (b != 0ull && rb < K) out[rb] = b;
+  }
+  __syncwarp();
+  return out[lane];
 }
 
 template <typename T, bool ALIGNED>
@@ -272,6 +297,12 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
   // target row r, mask row (i*, r+1), or block row r
   const int brow = p.phase == PHASE_TARGETS ? r * k1 : p.phase == PHASE_MASKS ? i_star0 * k1 + r + 1 : r;
   const T* row = reinterpret_cast<const T*>(p.logits) + ((int64_t)b * p.n_q + brow) * p.row_stride;
+  // what the block that finishes the sequence needs besides the lists, in flight during the search (lane j holds
+  // candidate c_{j+1})
+  const int my_cand = lane < p.k ? p.cand[b * p.k + lane] : -1;
+  const float my_prob = lane < p.k ? p.cand_prob[b * p.k + lane] : 0.f;
+  const uint32_t seq = p.seq_id ? p.seq_id[b] : (uint32_t)b;
+  const int L = p.kv_len ? p.kv_len[b] : 0;
   int Lc = 0;
   if (p.do_commit) {                                        // (phase 1: i* is known, every block moves its slice)
     Lc = p.cm.kv_len[b];
@@ -298,20 +329,13 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
 
   const bool with_lists = p.resample == SPACE_RESAMPLE_RESIDUAL_DRAFT;
   const bool literal = p.resample == SPACE_RESAMPLE_PAPER_LITERAL || with_lists;   // candidates are sampled
-  const uint32_t seq = p.seq_id ? p.seq_id[b] : (uint32_t)b;
-  const int L = p.kv_len ? p.kv_len[b] : 0;
   float z = 0.f, q = 0.f; int idx = -1; bool keep = false;
   // ---- filtered distribution of row list_row(w) by warp w < count
   auto build = [&](int count, int first, int step) {
-    for (int i = threadIdx.x; i < count * p.n_chunks * FILT_MAX_K; i += FILT_THREADS) {
-      const int j = i % FILT_MAX_K, c = (i / FILT_MAX_K) % p.n_chunks, w = i / (FILT_MAX_K * p.n_chunks);
-      if (j < K) sh.buf[(w * FILT_MAX_CHUNKS + c) * FILT_MAX_K + j] =
-          __ldcg(part + ((int64_t)(first + w * step) * FILT_MAX_CHUNKS + c) * FILT_MAX_K + j);
-    }
-    __syncthreads();
     z = 0.f; q = 0.f; idx = -1; keep = false;
     if (warp >= count) return;
-    const unsigned long long lst = merge_lists(sh.buf + warp * FILT_MAX_CHUNKS * FILT_MAX_K, p.n_chunks, K, lane);
+    const unsigned long long lst = merge_lists(part + (int64_t)(first + warp * step) * FILT_MAX_CHUNKS * FILT_MAX_K, p.n_chunks, K, lane,
+                                               sh.buf + warp * FILT_MAX_CHUNKS * FILT_MAX_K, sh.top[warp]);
     const bool valid = lst != 0ull;
     if (valid) split_key(lst, z, idx);
     // temperature, then softmax over the top-k, then the shortest prefix that reaches top_p
@@ -342,14 +366,14 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
     build(k1, 0, p.phase == PHASE_BOTH ? k1 : 1);
     // acceptance test of candidate c_{t+1} against the filtered law of target row t (warp t)
     if (warp < p.k) {
-      const int c = p.cand[b * p.k + warp];
+      const int c = __shfl_sync(0xFFFFFFFFu, my_cand, warp);
+      const float pc = __shfl_sync(0xFFFFFFFFu, my_prob, warp);
       const bool in_range = c >= 0 && c < p.V;
       const unsigned hit = __ballot_sync(0xFFFFFFFFu, keep && idx == c);
       const float qc = hit ? __shfl_sync(0xFFFFFFFFu, q, __ffs(hit) - 1) : 0.f;
       if (lane == 0) {
         if (!in_range) atomicOr(&sh.bits, SPACE_ST_BAD_CANDIDATE);
         const Philox4 w = philox4x32_10(0u, PURPOSE_ACCEPT, seq, (uint32_t)(L + warp + 1), p.key0, p.key1);
-        const float pc = p.cand_prob[b * p.k + warp];
         sh.ok[warp] = in_range && pc > 0.f && uniform_open(w.x) * pc <= qc;   // r <= Q'/P_c  <=>  r P_c <= Q'
       }
     }
@@ -358,7 +382,11 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
     if (warp == i_star) {
       // extra token: Gumbel arg-max over the kept tokens of row i*, the rejected point-mass candidate left out
       int exclude = -1;
-      if (!literal && i_star < p.k && p.cand_prob[b * p.k + i_star] == 1.0f) exclude = p.cand[b * p.k + i_star];
+      {
+        const float pc = __shfl_sync(0xFFFFFFFFu, my_prob, min(i_star, p.k - 1));
+        const int c = __shfl_sync(0xFFFFFFFFu, my_cand, min(i_star, p.k - 1));
+        if (!literal && i_star < p.k && pc == 1.0f) exclude = c;
+      }
       float sc = -CUDART_INF_F;
       // compact draft distribution of the rejected candidate: the weight of a kept token is
       // max(0, Q - D); Q itself when nothing was rejected, there are no lists, or nothing is left
@@ -396,7 +424,7 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
       }
       const int bonus = bi;
       const int j = lane;
-      const int tok = (j < i_star) ? p.cand[b * p.k + min(j, p.k - 1)] : (j == i_star ? bonus : -1);
+      const int tok = (j < i_star) ? my_cand : (j == i_star ? bonus : -1);
       const bool is_eos = p.eos_id >= 0 && j <= i_star && tok == p.eos_id;
       const unsigned eos_mask = __ballot_sync(0xFFFFFFFFu, is_eos && j < k1);
       const int n_out = eos_mask ? __ffs(eos_mask) - 1 : i_star + 1;
@@ -413,7 +441,6 @@ __global__ void __launch_bounds__(FILT_THREADS) verify_filter_kernel(const FiltP
   // (one launch: the whole move falls to this block, i* has only just become known)
   if (p.do_commit && p.phase == PHASE_BOTH && commit_fits(p.cm, Lc))
     commit_rows_any(p.cm, b, Lc, i_star, 0, 1, threadIdx.x, FILT_THREADS);
-  __syncthreads();                                          // the list buffer is free again
   if (p.phase == PHASE_BOTH) build(p.k, i_star * k1 + 1, 1);
   else build(p.k, 0, 1);
   // every thread of the sequence's blocks has read the old length by now
