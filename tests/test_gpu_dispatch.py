@@ -43,7 +43,8 @@ def test_verify_rows_off_the_16_byte_grid(B, H, mode, V, dtype):  # noqa: F811
 
 # Several segments per chunk (their lists are merged), chunks in both launches, and rows that defeat the
 # expectation behind the bound: ascending logits (every later segment beats the list) and few distinct values.
-@pytest.mark.parametrize("Bn,k,V,top_k,dtype", [(90, 2, 50003, 32, "bf16"), (2, 4, 20000, 32, "f32"), (1, 2, 8200, 3, "bf16")])
+@pytest.mark.parametrize("Bn,k,V,top_k,dtype", [(90, 2, 50003, 32, "bf16"), (2, 4, 20000, 32, "f32"), (1, 2, 8200, 3, "bf16"),
+                                                (1, 2, 70001, 2, "f32"), (1, 5, 65537, 32, "f32")])
 def test_filtered_sampling_on_sorted_and_tied_rows(B, H, Bn, k, V, top_k, dtype):  # noqa: F811
     cfg = _small_cfg(k, (5, 40), H_q=1, H_kv=1, d=64, Bn=Bn, V=V, dtype=dtype, seed=77)
     x = workloads.make_step_inputs(cfg)
