@@ -2,13 +2,13 @@
 // row orientation: used when the query block of one kv head has more than 64
 // rows (block rows times GQA group), where a full 128-row MMA tile is well
 // filled.  Narrower blocks go to the transposed kernel of attn_tc.cu, which
-// this file mirrors in structure (flat tile partition, split partials, merge).
+// this file mirrors in structure (clustered cut or flat tile list, split partials, merge).
 //
 // Here the query rows are the MMA M extent and the 128 keys of a tile the N
-// extent: S = Q K^T (128 x 128) into one of two TMEM buffers, P overwrites S in
+// extent: S = Q K^T (128 x 128) into one of three TMEM buffers, P overwrites S in
 // TMEM as two bf16 terms, O += (P_hi + P_lo) V with P read back from TMEM.
-// Inside a block (12 warps): warps 0 and 2 stream K and V tiles with TMA, warp
-// 3 loads the query rows, warp 1 issues tcgen05.mma, warps 4-11 are two threads
+// Inside a block (12 warps): warps 0 and 2 stream K (and the query rows) and V tiles
+// with TMA, warps 1 and 3 issue the S and the O products, warps 4-11 are two threads
 // per query row (64 keys of the tile each) with a running row maximum and lazy
 // rescaling of O.  Every wait is bounded; an expired wait sets SPACE_ST_TIMEOUT
 // and the block drains and exits.

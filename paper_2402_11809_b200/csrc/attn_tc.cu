@@ -1,12 +1,14 @@
 // Tensor-core attention of the block rows over cache + block (Eq. 5) for sm_100a.
 //
-// Persistent split-KV flash-decode kernel.  The (sequence, kv head) key ranges
-// are cut into 128-key tiles, the tiles of all sequences form one flat list
-// and every thread-block group takes an equal contiguous share of it, so ragged
-// batches balance without host knowledge of the lengths.  A share that does not
-// cover a whole (sequence, head) leaves an unnormalised partial (reference
-// maximum, sum, accumulator) in scratch memory; attn_merge_kernel combines the
-// partials of every (sequence, head) that was cut.
+// Split-KV flash-decode kernel.  The key ranges of the (sequence, kv head) pairs are cut into 128-key tiles; a
+// share that does not cover a whole pair leaves an unnormalised partial (reference maximum, sum, accumulator).
+// At most one pair per cluster of blocks that fits on the chip (the usual decoding case): a cluster per pair,
+// piece i of n takes tiles i, i + n, ..., so that a block's first tile does not depend on the length and is
+// requested, with the query rows, before the length is read; the partials meet in the cluster's shared memory.
+// More pairs, or very unequal lengths: the tiles of all sequences form one flat list and every thread-block
+// group takes an equal contiguous share of it, so ragged batches balance without host knowledge of the lengths;
+// partials go to scratch memory and attn_merge_kernel combines them (the clustered launch with unequal lengths
+// has no such kernel after it: there the piece that finds all others stored does it).
 //
 // The query block of one kv head is small here (the (k+1)^2 block rows times the GQA
 // group, at most 64 rows; wider blocks go to attn_rows.cu), so the two tile products are taken transposed: the
@@ -29,12 +31,6 @@
 //           across keys once per share.
 // Every wait is bounded; an expired wait sets SPACE_ST_TIMEOUT and the block
 // drains and exits.
-//
-// One sequence (the usual decoding case) takes a partition of its own: every kv head gets the
-// same number of groups, piece i of a head takes tiles i, i + pieces, ... (so a group's first
-// tile does not depend on the length and is requested, with the query rows, before the length
-// is read), and the groups left over take the heads' last tiles, the ones with the block's own
-// keys and the Eq. 5 mask.
 #include "common.cuh"
 #include "tc_common.cuh"
 #include "attn_common.cuh"

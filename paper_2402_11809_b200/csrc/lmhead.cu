@@ -1,4 +1,4 @@
-// Output projection fused with greedy verification (Algorithm 1: the end of the
+// Output projection fused with verification, greedy or sampling (Algorithm 1: the end of the
 // model call P = M(I) and the loop after it).
 //
 // logits[r, x] = <h_r, W_x> for the (k+1)^2 block rows of every sequence and the
@@ -14,8 +14,9 @@
 // finish combines the vocabulary ranges and runs the acceptance scan, the extra
 // token, the <EOS> cut and the next candidates.
 //
-// The output embedding is streamed exactly once (the step's HBM roof); the
-// hidden rows are re-read from L2 by every thread block.
+// The output embedding is streamed exactly once (the step's HBM roof) for up to 256 block rows, by phase beyond
+// (the target rows of every sequence, then the mask rows of its group i*); the hidden rows are re-read from L2
+// by every thread block.
 //
 // Vocabulary ranges: thread block c owns rows [V*c/G, V*(c+1)/G) and covers them
 // with boxes of n_box rows (256, or the longest range rounded up to 16 when that

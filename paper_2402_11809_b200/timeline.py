@@ -3,9 +3,8 @@
 The kernels carry optional %globaltimer stamps (compiled in with -DSPACE_TIMELINE; see csrc/attn_tc.cu and
 csrc/verify.cu).  This module builds a second copy of the library with them, libspace_timeline.so, next to
 the regular one, replays a graph of eight steps of a single-sequence workload and prints, in microseconds
-after the attention kernel's dependency wait of the last step: when the attention blocks pass their stages
-when the merge and verify blocks become resident, when their
-dependency waits return and when they finish.  What a kernel boundary costs and where a launch spends its
+after the attention kernel's dependency wait of the last step: when the attention blocks pass their stages,
+when the merge and verify blocks become resident, when their dependency waits return and when they finish.  What a kernel boundary costs and where a launch spends its
 time cannot be seen from outside the kernels: a profiler serialises the launches.
 
 Usage: python -m paper_2402_11809_b200.timeline [workload]      (default llama7b; needs a B200)
