@@ -69,6 +69,21 @@ struct MergeAcc {
     }
     mx = mn;
   }
+  // four partials at once (a missing one: m = -inf, l = 0, o = 0): one maximum, independent weights, where one
+  // after the other is a chain of two exponentials each (sixteen pieces of two short sequences: step 16.5 -> 16.0 us)
+  __device__ __forceinline__ void add4(const float (&m)[4], const float (&l)[4], const float4 (&o)[4]) {
+    const float mn = fmaxf(fmaxf(fmaxf(mx, m[0]), fmaxf(m[1], m[2])), m[3]);
+    if (mn > -CUDART_INF_F) {
+      const float e = tc::fast_exp2(mx - mn);
+      den *= e; a.x *= e; a.y *= e; a.z *= e; a.w *= e;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float w = tc::fast_exp2(m[j] - mn);
+        den += l[j] * w; a.x += o[j].x * w; a.y += o[j].y * w; a.z += o[j].z * w; a.w += o[j].w * w;
+      }
+    }
+    mx = mn;
+  }
   template <int DH, class P>
   __device__ __forceinline__ void store(const P& p, int b, int h, int i0, int r, int c4) const {
     const float rd = 1.f / den;
@@ -97,6 +112,7 @@ __device__ __forceinline__ void cluster_merge(const P& p, int b, int h, int i0, 
       float4 ov[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
+        ms[j] = -CUDART_INF_F; ls[j] = 0.f; ov[j] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (x0 + j < n) {
           const uint32_t rank = (uint32_t)((x0 + j) * p.n_mblocks + mb);
           ms[j] = ld_cluster(map_cluster(m_at + r * 4, rank));
@@ -104,9 +120,7 @@ __device__ __forceinline__ void cluster_merge(const P& p, int b, int h, int i0, 
           ov[j] = ld_cluster4(map_cluster(o_at + (r * DH + c4 * 4) * 4, rank));
         }
       }
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (x0 + j < n) acc.add(ms[j], ls[j], ov[j]);
+      acc.add4(ms, ls, ov);
     }
     acc.template store<DH>(p, b, h, i0, r, c4);
   }
