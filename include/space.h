@@ -354,8 +354,10 @@ int space_kv_commit(space_ctx* ctx, const space_commit_args* args, void* stream)
  * Needs cfg.host_staging.  Only sequence prefixes in use are copied (with
  * cache_resident: only the block's rows, see the field).  The call stages the
  * small per-sequence arrays in a pinned buffer of the context: one call at a
- * time per context.  Errors: INVALID_ARG (NULL pointer), WORKSPACE (no staging,
- * or sizes beyond cfg), CUDA. */
+ * time per context.  Errors: INVALID_ARG (NULL pointer, or a value that
+ * space_attn_step or space_verify_commit refuses), WORKSPACE (no staging, or sizes
+ * beyond cfg), both before anything is launched; CUDA, after which nothing that the
+ * call launched is still running and the outputs are undefined. */
 int space_step_host(space_ctx* ctx, const space_host_step_args* args, void* stream);
 
 /* Device-resident state of the decoding loop (Algorithm 1 in full): the generated

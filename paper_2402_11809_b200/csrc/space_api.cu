@@ -125,6 +125,27 @@ void build_layout(int k, int variant, space_layout_t* out) {
 // Every entry point that takes a context makes the context's device current.
 bool use_device(const space_ctx* ctx) { return cudaSetDevice(ctx->cfg.device) == cudaSuccess; }
 
+int check_attn_args(const space_ctx* ctx, const space_attn_args* a) {
+  if (a->batch < 0 || a->batch > ctx->cfg.max_batch) return SPACE_E_WORKSPACE;
+  if (a->k < 1 || a->k > ctx->cfg.k_max) return SPACE_E_INVALID_ARG;
+  if (a->batch == 0) return SPACE_OK;
+  if (!a->q || !a->k_cache || !a->v_cache || !a->kv_len || !a->out) return SPACE_E_INVALID_ARG;
+  if (!(a->scale > 0.f)) return SPACE_E_INVALID_ARG;
+  if (a->out_dtype != SPACE_DTYPE_F32 && a->out_dtype != SPACE_DTYPE_BF16) return SPACE_E_INVALID_ARG;
+  if (a->mask_variant != SPACE_MASK_SAME_GROUP && a->mask_variant != SPACE_MASK_EQ5_LITERAL)
+    return SPACE_E_INVALID_ARG;
+  if (!aligned16(a->q) || !aligned16(a->k_cache) || !aligned16(a->v_cache) || !aligned16(a->out))
+    return SPACE_E_ALIGNMENT;
+  if (a->kv_stride_s < ctx->cfg.head_dim || a->kv_stride_b < 1 || a->kv_stride_h < 1) return SPACE_E_INVALID_ARG;
+  if (a->kv_stride_b % 8 || a->kv_stride_h % 8 || a->kv_stride_s % 8) return SPACE_E_ALIGNMENT;
+  if (a->page_table && (a->pages_per_seq < 1 || a->n_pages < 1 ||
+                        (int64_t)a->pages_per_seq * SPACE_PAGE_SIZE > ctx->cfg.s_cap))
+    return SPACE_E_INVALID_ARG;
+  if (a->impl != SPACE_ATTN_SIMT && a->impl != SPACE_ATTN_TENSOR && a->impl != SPACE_ATTN_TENSOR_ROWS)
+    return SPACE_E_INVALID_ARG;
+  return SPACE_OK;
+}
+
 int check_verify_args(const space_ctx* ctx, const space_verify_args* a) {
   if (a->batch < 0 || a->batch > ctx->cfg.max_batch) return SPACE_E_WORKSPACE;
   if (a->k < 1 || a->k > ctx->cfg.k_max) return SPACE_E_INVALID_ARG;
@@ -297,21 +318,8 @@ int space_layout(int k, int mask_variant, space_layout_t* out) {
 
 int space_attn_step(space_ctx* ctx, const space_attn_args* a, void* stream) {
   if (!ctx || !a) return SPACE_E_INVALID_ARG;
-  if (a->batch < 0 || a->batch > ctx->cfg.max_batch) return SPACE_E_WORKSPACE;
-  if (a->k < 1 || a->k > ctx->cfg.k_max) return SPACE_E_INVALID_ARG;
-  if (a->batch == 0) return SPACE_OK;
-  if (!a->q || !a->k_cache || !a->v_cache || !a->kv_len || !a->out) return SPACE_E_INVALID_ARG;
-  if (!(a->scale > 0.f)) return SPACE_E_INVALID_ARG;
-  if (a->out_dtype != SPACE_DTYPE_F32 && a->out_dtype != SPACE_DTYPE_BF16) return SPACE_E_INVALID_ARG;
-  if (a->mask_variant != SPACE_MASK_SAME_GROUP && a->mask_variant != SPACE_MASK_EQ5_LITERAL)
-    return SPACE_E_INVALID_ARG;
-  if (!aligned16(a->q) || !aligned16(a->k_cache) || !aligned16(a->v_cache) || !aligned16(a->out))
-    return SPACE_E_ALIGNMENT;
-  if (a->kv_stride_s < ctx->cfg.head_dim || a->kv_stride_b < 1 || a->kv_stride_h < 1) return SPACE_E_INVALID_ARG;
-  if (a->kv_stride_b % 8 || a->kv_stride_h % 8 || a->kv_stride_s % 8) return SPACE_E_ALIGNMENT;
-  if (a->page_table && (a->pages_per_seq < 1 || a->n_pages < 1 ||
-                        (int64_t)a->pages_per_seq * SPACE_PAGE_SIZE > ctx->cfg.s_cap))
-    return SPACE_E_INVALID_ARG;
+  const int rc = check_attn_args(ctx, a);
+  if (rc != SPACE_OK || a->batch == 0) return rc;
   if (!use_device(ctx)) return SPACE_E_CUDA;
   if (ctx->lay_k != a->k || ctx->lay_variant != a->mask_variant) {   // the layout is rebuilt only when k or the reading changes
     space_layout_t lay;
@@ -321,7 +329,6 @@ int space_attn_step(space_ctx* ctx, const space_attn_args* a, void* stream) {
   }
   cudaStream_t st = (cudaStream_t)stream;
   if (a->impl == SPACE_ATTN_SIMT) return launch_attn_simt(ctx, a, ctx->lay_mask, st);
-  if (a->impl != SPACE_ATTN_TENSOR && a->impl != SPACE_ATTN_TENSOR_ROWS) return SPACE_E_INVALID_ARG;
   return launch_attn_tensor(ctx, a, ctx->lay_mask, st);
 }
 
@@ -457,12 +464,23 @@ int space_step_host(space_ctx* ctx, const space_host_step_args* a, void* stream)
   ve.logits = d_logits; ve.logits_row_stride = a->vocab; ve.cand = d_cand; ve.cand_prob = d_cprob;
   ve.seq_id = nullptr; ve.kv_len = d_kvlen; ve.n_accept = d_nacc; ve.out_tokens = d_tok; ve.n_out = d_nout;
   ve.next_cand = d_ncand; ve.next_cand_prob = d_nprob; ve.finished = d_fin; ve.status = d_status;
+  // whatever the stages refuse is refused here, before anything is launched
   int rc = check_verify_args(ctx, &ve);
+  if (rc == SPACE_OK) rc = check_attn_args(ctx, &at);
   if (rc != SPACE_OK) return rc;
 
   // Two streams beside one another, ordered by events: what the attention needs and the attention on `st`, the
   // logits (and what is made of them) on the second.  The call ends with everything done.
   cudaStream_t sb = ctx->aux_stream;
+  // A call that fails half way has work in flight that reads and writes the caller's buffers, and may leave status
+  // bits of a verification that no download has fetched and cleared: wait for both streams and clear the bits.
+  auto failed = [&](int code) {
+    cudaStreamSynchronize(sb);
+    cudaMemsetAsync(ctx->vstatus, 0, (size_t)c.max_batch * sizeof(int32_t), st);
+    cudaStreamSynchronize(st);
+    cudaGetLastError();
+    return code;
+  };
   void *v_q, *v_k, *v_v, *v_logits, *v_out, *v_small;
   if (a->cache_resident && (v_small = device_view(hsm, 11 * slot)) && (v_q = device_view(a->q, q_bytes)) &&
       (v_k = device_view(a->k_cache, cache_bytes)) && (v_v = device_view(a->v_cache, cache_bytes)) &&
@@ -486,10 +504,10 @@ int space_step_host(space_ctx* ctx, const space_host_step_args* a, void* stream)
     ve.logits = v_logits; ve.status = ctx->vstatus;
     ok = ok && launch_verify(ctx, &ve, nullptr, sb, true) == SPACE_OK;
     ok = ok && cudaEventRecord(ctx->aux_ev[1], sb) == cudaSuccess;
-    if (!ok) { cudaGetLastError(); return SPACE_E_CUDA; }
+    if (!ok) return failed(SPACE_E_CUDA);
     at.out = v_out;
     rc = space_attn_step(ctx, &at, stream);
-    if (rc != SPACE_OK) return rc;
+    if (rc != SPACE_OK) return failed(rc);
     ok = ok && cudaStreamWaitEvent(st, ctx->aux_ev[1], 0) == cudaSuccess;
     // rows L .. L+k (the compacted ones) and the results
     hc.run_vecs = k1 * (d / 8); hc.small_words = (int)(6 * slot / 4);
@@ -519,21 +537,21 @@ int space_step_host(space_ctx* ctx, const space_host_step_args* a, void* stream)
     ok = ok && cudaStreamWaitEvent(sb, ctx->aux_ev[0], 0) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(d_logits, a->logits, logit_bytes, cudaMemcpyHostToDevice, sb) == cudaSuccess;
     ok = ok && cudaEventRecord(ctx->aux_ev[1], sb) == cudaSuccess;          // logits uploaded
-    if (!ok) { cudaGetLastError(); return SPACE_E_CUDA; }
+    if (!ok) return failed(SPACE_E_CUDA);
     rc = space_attn_step(ctx, &at, stream);
-    if (rc != SPACE_OK) return rc;
+    if (rc != SPACE_OK) return failed(rc);
     ok = ok && cudaEventRecord(ctx->aux_ev[2], st) == cudaSuccess;
     ok = ok && cudaStreamWaitEvent(sb, ctx->aux_ev[2], 0) == cudaSuccess;
     ok = ok && cudaMemcpyAsync(a->out, d_out, out_bytes, cudaMemcpyDeviceToHost, sb) == cudaSuccess;
     ok = ok && cudaEventRecord(ctx->aux_ev[3], sb) == cudaSuccess;
     ok = ok && cudaStreamWaitEvent(st, ctx->aux_ev[1], 0) == cudaSuccess;   // verification needs the logits
-    if (!ok) { cudaGetLastError(); return SPACE_E_CUDA; }
+    if (!ok) return failed(SPACE_E_CUDA);
     space_commit_args cm{};
     cm.batch = B; cm.k = k; cm.k_cache = d_k; cm.v_cache = d_v;
     cm.kv_stride_b = at.kv_stride_b; cm.kv_stride_h = at.kv_stride_h; cm.kv_stride_s = at.kv_stride_s;
     cm.n_accept = d_nacc; cm.kv_len = d_kvlen; cm.kv_len_out = d_kvlen_out; cm.status = d_status;
     rc = space_verify_commit(ctx, &ve, &cm, stream);
-    if (rc != SPACE_OK) return rc;
+    if (rc != SPACE_OK) return failed(rc);
     ok = ok && cudaMemcpyAsync(hsm + 3 * slot, d_small + 3 * slot, 8 * slot, cudaMemcpyDeviceToHost, st) == cudaSuccess;
     for (int b = 0; b < B && ok; ++b) {                    // rows L .. L+k: the compacted rows
       if (!fits(b)) continue;
@@ -545,8 +563,8 @@ int space_step_host(space_ctx* ctx, const space_host_step_args* a, void* stream)
     }
     ok = ok && cudaStreamWaitEvent(st, ctx->aux_ev[3], 0) == cudaSuccess;   // ... and the output has arrived
   }
-  if (!ok) { cudaGetLastError(); return SPACE_E_CUDA; }
-  if (cudaStreamSynchronize(st) != cudaSuccess) return SPACE_E_CUDA;
+  if (!ok) return failed(SPACE_E_CUDA);
+  if (cudaStreamSynchronize(st) != cudaSuccess) return failed(SPACE_E_CUDA);
   memcpy(a->n_accept, hsm + 3 * slot, (size_t)B * 4);
   memcpy(a->out_tokens, hsm + 4 * slot, (size_t)B * k1 * 4);
   memcpy(a->n_out, hsm + 5 * slot, (size_t)B * 4);

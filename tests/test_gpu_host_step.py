@@ -27,7 +27,7 @@ def _pinned(arr):
     return torch.from_numpy(arr.view(np.int16) if arr.dtype == np.uint16 else arr).clone().pin_memory()
 
 
-def _run(B, ctx, cfg, x, pin, resident):
+def _run(B, ctx, cfg, x, pin, resident, **over):
     k = cfg["k"]
     n_q = (k + 1) ** 2
     outs = dict(out=torch.full((cfg["B"], n_q, cfg["H_q"], cfg["d"]), float("nan")).pin_memory(),
@@ -39,10 +39,12 @@ def _run(B, ctx, cfg, x, pin, resident):
                 finished=torch.zeros(cfg["B"], dtype=torch.uint8).pin_memory(),
                 status=torch.full((cfg["B"],), -1, dtype=torch.int32).pin_memory())
     h2d, d2h = C.c_int64(0), C.c_int64(0)
-    hs = B.HostStepArgs(batch=cfg["B"], k=k, vocab=cfg["V"],
-                        logits_dtype=B.DTYPE_F32 if cfg["logits_dtype"] == "f32" else B.DTYPE_BF16,
-                        mode=B.MODE_GREEDY, resample=B.RESAMPLE_RESIDUAL_POINTMASS, eos_id=-1,
-                        mask_variant=B.MASK_SAME_GROUP, scale=x["scale"], temperature=1.0, seed=0,
+    args = dict(batch=cfg["B"], k=k, vocab=cfg["V"],
+                logits_dtype=B.DTYPE_F32 if cfg["logits_dtype"] == "f32" else B.DTYPE_BF16,
+                mode=B.MODE_GREEDY, resample=B.RESAMPLE_RESIDUAL_POINTMASS, eos_id=-1,
+                mask_variant=B.MASK_SAME_GROUP, scale=x["scale"], temperature=1.0, seed=0)
+    args.update(over)
+    hs = B.HostStepArgs(**args,
                         **{n: C.c_void_p(t.data_ptr()) for n, t in pin.items()},
                         **{n: C.c_void_p(t.data_ptr()) for n, t in outs.items()},
                         h2d_bytes=C.cast(C.pointer(h2d), C.c_void_p), d2h_bytes=C.cast(C.pointer(d2h), C.c_void_p),
@@ -103,3 +105,29 @@ def test_host_step_matches_oracle_full_and_resident(B, k, L, H_q, H_kv):
     assert torch.equal(outs2["out"], outs["out"])
     block_bytes = cfg["B"] * 2 * n_q * cfg["d"] * 2 * H_kv
     assert h2d_full - h2d_res == kv_bytes - block_bytes
+
+
+# An argument that only the attention refuses: nothing is launched, the host's buffers stay as they are, and the next
+# call reports its own status only (candidate 0 of the refused call is out of range).
+@pytest.mark.parametrize("resident", [False, True])
+def test_host_step_refuses_before_launching(B, resident):
+    import gpu_harness as H
+    k, V = 2, 300
+    cfg = workloads.resolve("tiny", B=2, H_q=2, H_kv=2, d=64, L=(30, 90), k=k, V=V, logits_dtype="bf16", seed=3)
+    x = workloads.make_step_inputs(cfg)
+    ctx = B.Context(max_batch=2, n_q_heads=2, n_kv_heads=2, head_dim=64, k_max=k, vocab=V, host_staging=1, s_cap=x["s_cap"])
+    names = ("q", "k_cache", "v_cache", "logits", "cand", "cand_prob", "kv_len")
+    _run(B, ctx, cfg, x, {n: _pinned(x[n]) for n in names}, False)           # the cache is on the device from here on
+    bad = {n: _pinned(x[n]) for n in names}
+    bad["cand"][:] = V + 1
+    for over in (dict(scale=0.0), dict(scale=float("nan")), dict(mask_variant=9)):
+        n0 = ctx.launch_count
+        with pytest.raises(B.SpaceError) as e:
+            _run(B, ctx, cfg, x, bad, resident, **over)
+        assert e.value.code == B.E_INVALID_ARG and ctx.launch_count == n0
+        assert np.array_equal(bad["kv_len"].numpy(), x["kv_len"])
+    outs, _, _ = _run(B, ctx, cfg, x, {n: _pinned(x[n]) for n in names}, resident)
+    r = verify_step(x["logits"], x["cand"], x["cand_prob"], k, "greedy")
+    assert outs["status"].tolist() == [0, 0] and np.array_equal(outs["n_accept"].numpy(), r["n_accept"])
+    ref, _ = attention_step(x["q"], x["k_cache"], x["v_cache"], x["kv_len"], k, x["scale"])
+    H.check_attention(outs["out"].numpy().astype(np.float64), ref, "after a refused call")
