@@ -2,6 +2,7 @@
 verification, KV commit, copies out) against the fp64 oracle, with the whole
 cache uploaded and with the cache kept on the device between calls."""
 import ctypes as C
+from types import SimpleNamespace
 
 import numpy as np
 import pytest
@@ -11,6 +12,7 @@ from oracle.attention import attention_step
 from oracle.verify import verify_step
 from oracle.commit import commit_step
 from paper_2402_11809_b200 import workloads
+from test_gpu_parity import _check_verify
 
 pytestmark = pytest.mark.gpu
 
@@ -131,3 +133,41 @@ def test_host_step_refuses_before_launching(B, resident):
     assert outs["status"].tolist() == [0, 0] and np.array_equal(outs["n_accept"].numpy(), r["n_accept"])
     ref, _ = attention_step(x["q"], x["k_cache"], x["v_cache"], x["kv_len"], k, x["scale"])
     H.check_attention(outs["out"].numpy().astype(np.float64), ref, "after a refused call")
+
+
+# Sampling from host buffers, both resampling readings: the Gumbel row and the second read of target row i* go over
+# PCIe when the buffers are pinned and the cache is resident, and are copied otherwise.  V = 20003: rows off the
+# 16-byte grid (bf16 and f32), several chunks per row; V = 901: one chunk.
+@pytest.mark.parametrize("resample", ["residual_pointmass", "paper_literal"])
+@pytest.mark.parametrize("V,dtype", [(901, "bf16"), (20003, "bf16"), (20003, "f32")])
+@pytest.mark.parametrize("pinned", [True, False])
+def test_host_step_sampling(B, V, dtype, resample, pinned):
+    import gpu_harness as H
+    k, T, seed = 3, 0.8, 0x123456789
+    cfg = workloads.resolve("sampling64", B=4, H_q=4, H_kv=2, d=64, L=(20, 140), k=k, V=V, logits_dtype=dtype, seed=6)
+    x = workloads.make_step_inputs(cfg)
+    x["cand"][3, 1] = V + 4                                   # out of range: rejected and flagged
+    if resample == "paper_literal":
+        x["cand_prob"] = np.random.default_rng(1).uniform(0.2, 1.0, size=x["cand_prob"].shape).astype(np.float32)
+    x["cand_prob"][0, :] = np.inf                             # Algorithm 1's initial state
+    ctx = B.Context(max_batch=4, n_q_heads=4, n_kv_heads=2, head_dim=64, k_max=k, vocab=V, host_staging=1, s_cap=x["s_cap"])
+    r = verify_step(x["logits"], x["cand"], x["cand_prob"], k, "sample", temperature=T, seed=seed, kv_len=x["kv_len"],
+                    resample=resample)
+    ref, _ = attention_step(x["q"], x["k_cache"], x["v_cache"], x["kv_len"], k, x["scale"])
+    code = {"residual_pointmass": B.RESAMPLE_RESIDUAL_POINTMASS, "paper_literal": B.RESAMPLE_PAPER_LITERAL}[resample]
+    for resident in (False, True, True):
+        pin = {n: _pinned(x[n]) if pinned else _pinned(x[n]).clone() for n in ("q", "k_cache", "v_cache", "logits", "cand", "cand_prob", "kv_len")}
+        assert pin["logits"].is_pinned() == pinned
+        outs, _, _ = _run(B, ctx, cfg, x, pin, resident, mode=B.MODE_SAMPLE, temperature=T, seed=seed, resample=code)
+        excl = _check_verify(SimpleNamespace(**outs), r, k, sample=True)
+        assert not excl.any()                                 # (these inputs have no tie)
+        assert outs["status"].tolist() == [0, 0, 0, B.ST_BAD_CANDIDATE]
+        H.check_attention(outs["out"].numpy().astype(np.float64), ref, resample)
+        Kc, Vc = x["k_cache"].copy(), x["v_cache"].copy()
+        new_len, _, _ = commit_step(Kc, Vc, x["kv_len"], r["n_accept"], k)
+        assert np.array_equal(pin["kv_len"].numpy(), new_len)
+        for name, want in (("k_cache", Kc), ("v_cache", Vc)):
+            got = pin[name].numpy().view(np.uint16)
+            for b in range(4):
+                n = int(new_len[b])
+                assert np.array_equal(got[b, :, :n], want[b, :, :n]), (name, b, resident)
