@@ -416,6 +416,13 @@ def run_ours(args):
         bool(torch.equal(outs["n_accept"], steps_dev[0].n_accept.cpu()))
     if args.top_k and sample:
         res_ok = None
+    # The call's own count names all rows of logits; from pinned buffers verification reads only what it needs over
+    # PCIe: 2k+1 rows, one of them twice in sampling, or all of them in its single launch where the rows it could
+    # skip come to 512 KB at most (csrc/verify.cu: launch_verify).
+    row_bytes = x["logits"].dtype.itemsize * cfg["V"]
+    single = not sample and cfg["B"] * (n_q - 2 * k - 1) * row_bytes <= 512 << 10
+    rows_read = n_q if single else 2 * k + (2 if sample else 1)
+    h2d_res = int(h2d.value) - cfg["B"] * (n_q - rows_read) * row_bytes
 
     if rank != 0:
         replicas.shutdown()
@@ -476,11 +483,12 @@ def run_ours(args):
                      "kernel_us": per_kernel_us},
         "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": h2d_full,
                 "d2h_bytes_per_step": d2h_full, "steps": n_e2e, "matches_device_run": e2e_ok},
-        "e2e_resident_cache": {"value": res_val, "unit": UNIT, "h2d_bytes_per_step": int(h2d.value),
+        "e2e_resident_cache": {"value": res_val, "unit": UNIT, "h2d_bytes_per_step": h2d_res,
                                "d2h_bytes_per_step": int(d2h.value), "steps": n_res,
                                "matches_device_run": res_ok,
-                               "note": "space_step_host with cache_resident=1: only the block's K/V rows, q, "
-                                       "logits and candidates are uploaded; the verified cache stays on the device"},
+                               "note": "space_step_host with cache_resident=1: only the block's K/V rows, q, the "
+                                       "candidates and the rows of logits that verification reads go up; the "
+                                       "verified cache stays on the device"},
         "cpu_baseline": {"value": cpu_sps, "unit": UNIT, "cores": blas_threads(), "kind": "oracle",
                          "sample": f"{cpu_reps} whole step(s) of {cfg['name']} in {cpu_el:.1f} s"},
         "clocks": clocks,
