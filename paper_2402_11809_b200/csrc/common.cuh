@@ -154,7 +154,7 @@ struct space_ctx {
   size_t ws_bytes;
   float* attn_part;        // split partials
   size_t attn_part_slots;
-  int* counters;           // [4][max_batch] self-resetting arrival counters
+  int* counters;           // [3][max_batch] self-resetting arrival counters (two verify launches, commit), then an error word
   int* merge_cnt;          // attention, row kernel: cut descriptors, one per (sequence, kv head, row block), and owners
   int* arrived;            // attention: pieces of a cut that are stored, one per (sequence, kv head, row block)
   VerifyPartial* vpart;    // [max_batch][k_max+2][SPACE_VERIFY_MAX_CHUNKS]

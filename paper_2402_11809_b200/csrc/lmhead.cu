@@ -8,10 +8,10 @@
 // in TMEM: lane = block row, column = token).  An instruction of this kind costs
 // about the same whatever its N, so the tokens go on N: measured with the tokens
 // on M (128 per instruction) the 512 instructions of a thread block took longer
-// than its share of W takes to arrive.  Every epilogue thread owns one block row
-// and folds its accumulator columns into (max, lowest arg-max, sum exp(z - max))
-// in registers, without any exchange between threads.  The last thread block to
-// finish combines the vocabulary ranges and runs the acceptance scan, the extra
+// than its share of W takes to arrive.  Four epilogue threads share one block row
+// (two beyond 128 rows): each folds its part of the accumulator columns into (max,
+// lowest arg-max, sum exp(z - max)) in registers, and they meet once, at the end of the
+// block's range.  The last thread block to finish combines the vocabulary ranges and runs the acceptance scan, the extra
 // token, the <EOS> cut and the next candidates.
 //
 // The output embedding is streamed exactly once (the step's HBM roof) for up to 256 block rows, by phase beyond

@@ -30,10 +30,8 @@ constexpr int64_t SPACE_FUSED_MAX_BYTES = 64ll << 20;
 
 struct VerifyParams {
   int B, k, V, n_q, n_chunks, chunk;
-  int n_chunks_g, chunk_g;   // the row with Gumbel noise is cut finer (several times the work per logit)
   int mode, resample, eos_id;
   float c_t;                 // log2(e) / T   (target rows, sampled rows)
-  float inv_t;               // 1 / T
   uint32_t key0, key1;
   const void* logits;
   int64_t row_stride;
@@ -111,11 +109,11 @@ template <> struct Vec<__nv_bfloat16> {
   }
 };
 
-// One logit (the ragged ends of a chunk and unaligned rows).
 // What a scan keeps of its logits: nothing (the noisy arg-max alone), the maximum with its
 // lowest-index arg-max, or those and the sum of exp((z - max) c).
 enum { STAT_NONE = 0, STAT_MAX = 1, STAT_SUM = 2 };
 
+// One logit (the end of a chunk that is shorter than a vector).
 template <bool GUMBEL, int STATS>
 __device__ __forceinline__ void fold_one(Stat& st, float v, int x, float c, int exclude,
                                          uint32_t key0, uint32_t key1, uint32_t purpose,
@@ -477,25 +475,23 @@ verify_emit_kernel(const VerifyParams p) {
   pdl_wait();
   const int k1 = p.k + 1;
   const bool sample = p.mode == SPACE_MODE_SAMPLE;
-  // One-dimensional grid.  In sampling mode the first B * n_chunks_g blocks are the chunks of the
+  // One-dimensional grid.  In sampling mode the first B * n_chunks blocks are the chunks of the
   // extra-token rows: a logit there costs a Philox block and two logarithms, several times a plain
-  // one, so those rows are cut finer (their work spreads over every SM) and start first (no long
-  // block is left for the tail of the launch).  Then the mask rows: chunk, sequence, slot.
-  const int n_g = sample ? p.B * p.n_chunks_g : 0;
-  int b, ch, slot, chunk_len, n_ch;
+  // one, so those rows start first (no long block is left for the tail of the launch; a finer cut of
+  // them, up to 8x, was no faster).  Then the mask rows: chunk, sequence, slot.
+  const int n_g = sample ? p.B * p.n_chunks : 0;
+  int b, ch, slot;
   if ((int)blockIdx.x < n_g) {
-    slot = p.k; b = blockIdx.x / p.n_chunks_g; ch = blockIdx.x - b * p.n_chunks_g;
-    chunk_len = p.chunk_g; n_ch = p.n_chunks_g;
+    slot = p.k; b = blockIdx.x / p.n_chunks; ch = blockIdx.x - b * p.n_chunks;
   } else {
     int r = blockIdx.x - n_g;
     ch = r % p.n_chunks; r /= p.n_chunks;
     b = r % p.B; slot = r / p.B;
-    chunk_len = p.chunk; n_ch = p.n_chunks;
   }
   const int i_star = p.n_accept[b];
   const bool literal = sample && p.resample == SPACE_RESAMPLE_PAPER_LITERAL;
-  const int blocks_per_seq = p.k * p.n_chunks + (sample ? p.n_chunks_g : 0);
-  const int part_id = (slot == p.k) ? ch : (sample ? p.n_chunks_g : 0) + slot * p.n_chunks + ch;
+  const int blocks_per_seq = (p.k + (sample ? 1 : 0)) * p.n_chunks;
+  const int part_id = slot * p.n_chunks + ch;               // (slot k: the extra-token row)
   const uint32_t seq = p.seq_id ? p.seq_id[b] : (uint32_t)b;
   const int L = p.kv_len ? p.kv_len[b] : 0;
   const T* base = reinterpret_cast<const T*>(p.logits) + (int64_t)b * p.n_q * p.row_stride;
@@ -510,7 +506,7 @@ verify_emit_kernel(const VerifyParams p) {
   // slot o < k: mask row (i*, o+1); slot k: target row i* (extra token, sampling)
   const int brow = (slot < p.k) ? i_star * k1 + slot + 1 : i_star * k1;
   const T* row = base + (int64_t)brow * p.row_stride;
-  const int begin = ch * chunk_len, end = min(p.V, begin + chunk_len);
+  const int begin = ch * p.chunk, end = min(p.V, begin + p.chunk);
   const float c = sample ? p.c_t : 1.4426950408889634f;
   Stat st;
   if (slot == p.k) {
@@ -558,7 +554,7 @@ verify_emit_kernel(const VerifyParams p) {
     }
   } else if (warp == p.k) {
     int bonus;
-    if (sample) bonus = gather_row(pb + (int64_t)p.k * SPACE_VERIFY_MAX_CHUNKS, p.n_chunks_g, c).gidx;
+    if (sample) bonus = gather_row(pb + (int64_t)p.k * SPACE_VERIFY_MAX_CHUNKS, p.n_chunks, c).gidx;
     else bonus = p.rows[b * k1 + i_star].idx;
     if (lane == 0) sh_bonus = bonus;
   }
@@ -729,9 +725,9 @@ void launch_fused(space_ctx* ctx, const VerifyParams& p, cudaStream_t st) {
 }
 
 template <typename T, bool ALIGNED>
-void launch_both(space_ctx* ctx, const VerifyParams& p, int n_slots_b, cudaStream_t st) {
+void launch_both(space_ctx* ctx, const VerifyParams& p, cudaStream_t st) {
   dim3 ga(p.n_chunks, p.k + 1, p.B);
-  const dim3 gb(p.B * (p.k * p.n_chunks + (p.mode == SPACE_MODE_SAMPLE ? p.n_chunks_g : 0)));
+  const dim3 gb(p.B * (p.k + (p.mode == SPACE_MODE_SAMPLE ? 1 : 0)) * p.n_chunks);
   {
     ProfScope ps(ctx, SPACE_K_VERIFY_TARGET, st);
     launch_pdl(verify_target_kernel<T, ALIGNED>, ga, dim3(SPACE_VERIFY_THREADS), 0, st, p);
@@ -786,7 +782,6 @@ int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit
   p.mode = a->mode; p.resample = a->resample; p.eos_id = a->eos_id;
   const float T = (a->mode == SPACE_MODE_SAMPLE) ? a->temperature : 1.0f;
   p.c_t = 1.4426950408889634f / T;
-  p.inv_t = 1.0f / T;
   p.key0 = (uint32_t)(a->seed & 0xFFFFFFFFull); p.key1 = (uint32_t)(a->seed >> 32);
   p.logits = a->logits; p.row_stride = a->logits_row_stride;
   p.cand = a->cand; p.cand_prob = a->cand_prob; p.seq_id = a->seq_id; p.kv_len = a->kv_len;
@@ -804,7 +799,7 @@ int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit
   const int64_t spare_bytes = (int64_t)a->batch * (p.n_q - 2 * a->k - 1) * a->vocab * esz;
   if (verify_is_fused(a) && (!mapped || spare_bytes <= 512 << 10)) {
     int chunk, nc = row_chunks(a->vocab, a->batch * p.n_q, vec, ctx->sm_count, SPACE_FUSED_MAX_CHUNKS, &chunk);
-    p.n_chunks = nc; p.chunk = chunk; p.n_chunks_g = 0; p.chunk_g = 0;
+    p.n_chunks = nc; p.chunk = chunk;
     if (a->logits_dtype == SPACE_DTYPE_F32) {
       if (aligned) launch_fused<float, true>(ctx, p, st); else launch_fused<float, false>(ctx, p, st);
     } else {
@@ -815,14 +810,11 @@ int launch_verify(space_ctx* ctx, const space_verify_args* a, const space_commit
   }
   int chunk, nc = row_chunks(a->vocab, a->batch * (a->k + 1), vec, ctx->sm_count, SPACE_VERIFY_MAX_CHUNKS, &chunk);
   p.n_chunks = nc; p.chunk = chunk;
-  const int n_slots_b = (a->mode == SPACE_MODE_SAMPLE) ? a->k + 1 : a->k;
-  p.n_chunks_g = nc; p.chunk_g = chunk;                     // (measured: a finer cut of the noisy row, up to 8x, is no faster)
-
   if (a->logits_dtype == SPACE_DTYPE_F32) {
-    if (aligned) launch_both<float, true>(ctx, p, n_slots_b, st); else launch_both<float, false>(ctx, p, n_slots_b, st);
+    if (aligned) launch_both<float, true>(ctx, p, st); else launch_both<float, false>(ctx, p, st);
   } else {
-    if (aligned) launch_both<__nv_bfloat16, true>(ctx, p, n_slots_b, st);
-    else launch_both<__nv_bfloat16, false>(ctx, p, n_slots_b, st);
+    if (aligned) launch_both<__nv_bfloat16, true>(ctx, p, st);
+    else launch_both<__nv_bfloat16, false>(ctx, p, st);
   }
   ctx->launches += 2;
   return cuda_ok(cudaGetLastError());
@@ -892,7 +884,7 @@ int launch_verify_noalloc(const space_verify_args* a, cudaStream_t st) {
   VerifyParams p;
   p.B = a->batch; p.k = a->k; p.V = a->vocab; p.n_q = (a->k + 1) * (a->k + 1);
   p.mode = SPACE_MODE_GREEDY; p.resample = SPACE_RESAMPLE_RESIDUAL_POINTMASS; p.eos_id = a->eos_id;
-  p.c_t = 1.4426950408889634f; p.inv_t = 1.0f;
+  p.c_t = 1.4426950408889634f;
   p.key0 = 0; p.key1 = 0;
   p.logits = a->logits; p.row_stride = a->logits_row_stride;
   p.cand = a->cand; p.cand_prob = a->cand_prob; p.seq_id = a->seq_id; p.kv_len = a->kv_len;
