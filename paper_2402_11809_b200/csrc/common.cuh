@@ -102,8 +102,9 @@ __device__ __forceinline__ uint4 shift_pieces(const Piece2& r, const T* row) {
 
 // Asks L2 for a chunk's first sweep of logits, for the time before a kernel's dependency wait: with a programmatic
 // launch the blocks are resident while the kernel before them still runs.  Only a request to the point of
-// coherence: whatever is still being written is what the loads after the wait will see.  (One sequence of 36
-// rows of 32000 behind its attention: step 20.6 -> 19.9 us; eight steps for two sequences 199 -> 192 us.)
+// coherence: whatever is still being written is what the loads after the wait will see.  (Without / with, us:
+// sixteen sequences of 36 rows of 32000 behind a short attention, graph replay, 24.9 / 24.4 a step; eight decoding
+// steps for two sequences, steady loop, 185 / 182; one sequence's step the same either way.)
 template <typename T>
 __device__ __forceinline__ void prefetch_chunk(const T* row, int begin, int end) {
   constexpr int N = 16 / (int)sizeof(T);
@@ -116,10 +117,10 @@ __device__ __forceinline__ void prefetch_chunk(const T* row, int begin, int end)
 
 // Chunks per row and their length.  A sweep of a block is four vectors per thread (8192 bf16 logits); a
 // block costs about 3 us whatever it scans (reduction, fence, arrival).  So: as few sweeps per block as let all
-// blocks be resident at once (three per SM, and a few more), four where they cannot be.  Measured, us per call with
-// 1 / 2 / 3 / 4 sweeps per block: 80 rows of 50257 9.5 / 8.1 / 9.0 / 10.6, 98 rows of 128256 16 / 12 / 11 / 9.9,
-// 576 rows of 32000 22 / 16 / 16 / 15, top-10 lists of 72 and 48 rows of 128256 45 / 37 / 35 / 39 (33 with three
-// and two), sampling 64 x 5 rows of 128256 105 / 71 / 67 / 57.
+// blocks be resident at once (three per SM, and a few more), four where they cannot be.  Measured, us per call
+// (graph replay of space_verify_commit) with 1 / 2 / 3 / 4 sweeps per block: 80 rows of 50257 10.7 / 9.4 / 10.9 /
+// 13.6, 98 rows of 128256 16.6 / 12.5 / 13.1 / 10.5, 576 rows of 32000 22.7 / 16.5 / 16.6 / 15.2, top-10 lists of 72
+// and 48 rows of 128256 39 / 31 / 29 / 32 (27.7 with three and two), sampling 64 x 5 rows of 128256 106 / 71 / 66 / 57.
 static inline int row_chunks(int vocab, int rows, int vec, int sm_count, int max_chunks, int* chunk_out) {
   const int sweep = SPACE_VERIFY_THREADS * vec * 4;
   const int64_t slots = 3 * (int64_t)sm_count * 21 / 20;

@@ -4,9 +4,10 @@
 // What a resident-cache step moves besides the logits and the attention output are many small pieces: the
 // query rows, one run of block rows per kv head of K and of V, a handful of numbers per sequence, and back one
 // run of k+1 rows per kv head and the results.  A copy command costs 6-7 us on its stream whatever it moves
-// (13-20 us alone), a strided one more, and they queue behind one another: five up and three down were half
-// of the step's 141 us on one 7B-shaped sequence.  One kernel each way moves the same bytes with all pieces in
-// flight together.  Bound by PCIe: measured 46 GB/s plus 4 us either way, whatever the number of blocks.
+// (13-20 us alone), a strided one more, and they queue behind one another: with five up and three down, half of
+// the step on one 7B-shaped sequence (141 us in a steady loop, 88 now).  One kernel each way moves the same bytes
+// with all pieces in flight together.  Bound by PCIe: measured 46 GB/s plus 4 us either way, whatever the number
+// of blocks.
 #include "common.cuh"
 
 namespace {

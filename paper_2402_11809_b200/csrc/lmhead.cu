@@ -43,7 +43,7 @@ constexpr int LM_M = 128;                   // block rows per accumulator (MMA M
 constexpr int LM_MAX_BOX = 256;             // vocabulary rows per box (MMA N), at most
 constexpr int LM_KB = 64;                   // hidden elements per slice (128 bytes: one swizzle row)
 constexpr int LM_MAX_STAGES = 10;
-constexpr int LM_L2_AHEAD = 8;              // slices of W a block asks L2 for before its dependency wait (4: half the gain)
+constexpr int LM_L2_AHEAD = 8;              // slices of W a block asks L2 for before its dependency wait (4: two thirds of the gain)
 constexpr float LM_NEG = -3.0e38f;          // "no logit yet": finite, so that differences never give NaN
 constexpr int LM_MAX_N = 256;               // block rows of the whole batch, padded to 16
 // Which block rows a launch projects: all of them, the target rows of every sequence (row b(k+1)+t), or
@@ -327,7 +327,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
   if (warp == 0 && lane == 0) {
     // With a programmatic launch the block is resident before its dependency wait returns: ask L2 for its
     // first slices of W meanwhile (a request to the point of coherence, so whatever the kernel before still
-    // writes is what the loads will see).  57.2 -> 55.8 us per call on V = 32000, D = 4096, 36 rows.
+    // writes is what the loads will see).  V = 32000, D = 4096, 36 rows: 51.3 -> 49.8 us per call in bursts, 53.5 ->
+    // 53.2 in a steady loop, where the power cap sets the pace.
     const int first = (int)(((long long)p.V * blockIdx.x) / gridDim.x) & ~15;
     const uint64_t pol = l2_evict_first_policy();
     for (int kb = 0; kb < min(LM_L2_AHEAD, (p.D + LM_KB - 1) / LM_KB); ++kb)
@@ -749,7 +750,7 @@ int lm_make_map(CUtensorMap* tm, const void* base, int64_t rows, int64_t D, int6
   const cuuint32_t estr[4] = {1, 1, 1, 1};
   const CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B,      // measured against 128 B, 64 B, none: 0.4 us better
+                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B,      // (128 B, 64 B or none: 52.4 us per call instead of 49.8)
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? SPACE_OK : SPACE_E_CUDA;
 }
@@ -795,9 +796,10 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   p.n_box = max_len >= LM_MAX_BOX ? LM_MAX_BOX : (max_len + 15) / 16 * 16;
   p.tail_rows = (((max_len - 1) % p.n_box) + 1 + 15) / 16 * 16;
   // Slices per stage: one (finer hand-over, more W in flight: with 144 block rows of V = 32000 two would leave
-  // two stages, 84 us instead of 69), except where a slice's products take less time than its hand-over, that is
-  // with few tokens per thread block (us for one / two / four: 64 rows of V = 2091 30 / 24 / 22, 25 rows of
-  // V = 5000 26 / 22 / 19, V = 12000 28 / 26 / -).  As many stages as fit, at most LM_MAX_STAGES.
+  // two stages, a fifth slower), except where a slice's products take less time than its hand-over, that is
+  // with few tokens per thread block (us per call, graph replay, for one / two / four: 64 rows of V = 2091
+  // 23.6 / 18.5 / 16.4, 25 rows of V = 5000 25.0 / 20.6 / 18.4, 36 rows of V = 12000 28.2 / 26.9 / 26.9, of
+  // V = 32000 53.2 / 53.5 / -).  As many stages as fit, at most LM_MAX_STAGES.
   const size_t budget = 220 * 1024;
   int stages = 0;
   for (p.kbs = p.n_box <= 128 ? 4 : 1; p.kbs >= 1; p.kbs /= 2) {
@@ -851,8 +853,9 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
 // mask rows of the groups they select second -- two passes over the embedding, each near the pace of its
 // stream, instead of one per 256 rows at the pace of the product.  Calls that ask for every row's maximum
 // keep to the full rows.
-// Measured: 16 x 36 rows, V = 128256, D = 4096, sampling: 934 us as three launches over all rows, 363 by phase;
-// 4 x 36 rows, V = 32000, sampling: 111 by phase, 73 as one launch; 16 x 16 rows of V = 50257: 168 and 125.
+// Measured, us per call, D = 4096, sampling, steady loop (bursts), over all rows / by phase: 16 x 36 rows of
+// V = 128256 832 (722) / 409 (361); 4 x 36 rows of V = 32000 80 (71) / 115 (109); 16 x 16 rows of V = 50257
+// 140 (125) / 182 (169).
 int launch_lmhead_verify(space_ctx* ctx, const space_lmhead_args* a, cudaStream_t st) {
   const int n_q = (a->k + 1) * (a->k + 1), k1 = a->k + 1;
   const int rows = a->batch * n_q;

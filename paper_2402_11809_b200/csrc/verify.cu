@@ -14,13 +14,18 @@
 // results meet in a small scratch array and an arrival counter (reset by the
 // last block) decides who finishes the sequence.
 //
-// Small greedy problems (all (k+1)^2 rows of the batch within 64 MB; measured: at
-// 37 MB one launch still beats two by 6 us) are
+// Small greedy problems (all (k+1)^2 rows of the batch within 64 MB) are
 // latency bound, not bandwidth bound: for them verify_fused_kernel streams
 // every row in one launch and the last block of a sequence picks i* and the
 // mask rows of group i* from the per-row results, which removes the second
 // launch and its dependent round trips at the price of reading rows that the
-// two-launch path skips.
+// two-launch path skips.  Measured, us per step behind a short attention (graph
+// replay), one launch / two: 1 x 36 rows of V = 32000 (2 MB) 15.1 / 22.1, 8 x 36
+// (18 MB) 21.4 / 26.9, 16 x 36 (37 MB) 28.7 / 30.5, 24 x 36 (55 MB) 44.0 / 43.5,
+// 28 x 36 (65 MB) 51.3 / 47.4; 8 x 25 rows of 128256 (51 MB) 27.9 / 28.5.  The two
+// meet near 50 MB, a little below the line; rows off the 16-byte grid, whose reading
+// costs instructions, meet earlier the more of them can be skipped (16 x 9 rows of
+// 50257, 14 MB, 22.7 / 29.1; 40 x 9, 36 MB, 52.0 / 52.5; 4 x 64, 26 MB, 34.4 / 27.3).
 #include "common.cuh"
 #include <math_constants.h>
 

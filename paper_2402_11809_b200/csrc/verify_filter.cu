@@ -23,8 +23,9 @@
 // only about top_k do (128 groups of which top_k hold a larger logit: 10 for top_k = 10, 37 for 32).  Only
 // groups whose maximum reaches tau can hold such a logit, so at most top_k groups' worth are collected
 // whatever the row looks like; their threads read again the vector that has their maximum and, only where the
-// second largest of their vectors reaches tau too, the others (reading all of them again in an unrolled loop: 64 x 4
-// rows of 128256 logits, top-10, 95 -> 72 us with this; 4 x 3 rows of 3000, where it is code size, 13.6 -> 12.5).
+// second largest of their vectors reaches tau too, the others (reading all of them again in an unrolled loop took
+// 95 us per call on 64 x 4 rows of 128256 logits, top-10, and 13.6 on 4 x 3 rows of 3000, where it is code size; this
+// way 72 and 12.6).
 // The collected keys are ranked together with the list of the segments before by counting.
 // (Inserting logit by logit into warp lists, with a ballot and shuffles each, took 47 us per launch on
 // 24 x 3 rows of 128256 logits and 65 us on ten rows of 32000 with top_k = 32.)
@@ -43,8 +44,10 @@ constexpr int FILT_GROUP = 2;                            // threads per group wh
 constexpr int FILT_GROUPS = FILT_THREADS / FILT_GROUP;
 constexpr int FILT_U = 4;                                // vectors per thread and sweep
 constexpr int FILT_BUF = 4096;                           // keys a segment may collect
-// A call with at most this many block rows and bytes of logits takes one launch over all block rows (measured,
-// us, two launches / one: 2 MB 22 / 18, 12 MB 28 / 21, 18 MB 36 / 34, 41 MB 39 / 52).
+// A call with at most this many block rows and bytes of logits takes one launch over all block rows.  Measured, us
+// per call (graph replay, top-10), two launches / one: 4 x 9 rows of 32000 (2 MB) 17.6 / 12.5, 5 x 25 rows of 50257
+// (13 MB) 22.5 / 21.1, 24 x 9 rows of 50257 (22 MB) 27.5 / 25.0, 8 x 9 rows of 128256 (18 MB) 23.2 / 18.2, 16 x 9
+// (37 MB) 25.2 / 27.0: the two meet between 22 and 37 MB, above the line.
 constexpr int FILT_BOTH_ROWS = 256;
 constexpr int64_t FILT_BOTH_BYTES = 16ll << 20;
 enum { PHASE_TARGETS = 0, PHASE_MASKS = 1, PHASE_BOTH = 2 };
@@ -514,8 +517,9 @@ int launch_verify_filtered(space_ctx* ctx, const space_verify_args* a, const spa
   const bool aligned = ((uintptr_t)a->logits % 16 == 0) && ((a->logits_row_stride * esz) % 16 == 0);
   if (cm) fill_commit_params(ctx, cm, &p.cm);
   const bool both = (int64_t)a->batch * p.n_q <= FILT_BOTH_ROWS && (int64_t)a->batch * p.n_q * a->vocab * esz <= FILT_BOTH_BYTES;
-  // the commit rides along, except where one block would have more than 32 KB of rows to move (a launch of
-  // its own, about 2 us, is faster then)
+  // the commit rides along, except where one block would have more than 32 KB of rows to move: a launch of its
+  // own is faster then (two sequences, one launch; us per step, riding / own: 16 KB 22.1 / 23.7, 32 KB 25.8 / 26.1,
+  // 57 KB 29.8 / 28.5)
   const bool carry = cm && !(both && (int64_t)a->k * p.cm.H_kv * p.cm.d * 4 > (32 << 10));
   for (int phase = both ? PHASE_BOTH : PHASE_TARGETS; phase <= (both ? PHASE_BOTH : PHASE_MASKS); ++phase) {
     p.phase = phase;
