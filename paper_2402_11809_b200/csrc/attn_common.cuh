@@ -1,7 +1,8 @@
-// What the two tensor-core attention kernels (attn_tc.cu, attn_rows.cu) share: how partial results of a
-// (sequence, kv head, query-row block) that was cut over several thread blocks are combined, either in the
-// shared memory of a cluster or, from global memory, by the block that stored the last of them.  `P` is a
-// kernel's parameter struct (G, H_q, n_q, n_mblocks, out_dtype, out, lse, part).
+// What the two tensor-core attention kernels (attn_tc.cu, attn_rows.cu) share: page look-ups, the arithmetic of the
+// flat tile list, and how partial results of a (sequence, kv head, query-row block) that was cut over several
+// thread blocks are combined, either in the shared memory of a cluster or, from global memory, by the block that
+// stored the last of them.  `P` is a kernel's parameter struct (G, H_q, n_q, n_mblocks, out_dtype, out, lse, part;
+// page_table, pages_per_seq, n_pages, status).
 #pragma once
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -31,6 +32,30 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t a) {
   float4 v;
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
   return v;
+}
+
+// Page of tile t of sequence b (paged cache).  An entry outside the pool is flagged and answered
+// with a page past the pool's end: the TMA load then fills the tile with zeros.
+// (flag = false: a request made before the length is known, for a tile the sequence may not have.)
+template <class P>
+__device__ __forceinline__ int page_of(const P& p, int b, int t, bool flag = true) {
+  const int pg = t < p.pages_per_seq ? p.page_table[(int64_t)b * p.pages_per_seq + t] : -1;
+  if (pg >= 0 && pg < p.n_pages) return pg;
+  if (flag && p.status) atomicOr(p.status + b, SPACE_ST_BAD_PAGE);
+  return p.n_pages;
+}
+
+// floor(a * b / c) for a*b that may need 64 bits; 32-bit division when it fits
+__device__ __forceinline__ long long muldiv(long long a, long long b, long long c) {
+  const unsigned long long prod = (unsigned long long)a * (unsigned long long)b;
+  if ((prod >> 32) == 0) return (long long)((unsigned)prod / (unsigned)c);
+  return (long long)(prod / (unsigned long long)c);
+}
+// group that owns flat tile f (largest g with floor(W*g/NG) <= f)
+__device__ __forceinline__ int group_of(long long f, long long W, long long NG) {
+  const unsigned long long num = (unsigned long long)(f + 1) * (unsigned long long)NG - 1ull;
+  if ((num >> 32) == 0) return (int)((unsigned)num / (unsigned)W);
+  return (int)(num / (unsigned long long)W);
 }
 
 // Query row r of the row block that starts at block row i0, columns 4 c4 .. of (sequence b, kv head h).

@@ -73,16 +73,6 @@ struct AttnParams {
   uint64_t visq[2][SPACE_MAX_ROWS];
 };
 
-// Page of tile t of sequence b (paged cache).  An entry outside the pool is flagged and answered
-// with a page past the pool's end: the TMA load then fills the tile with zeros.
-// (flag = false: a request made before the length is known, for a tile the sequence may not have.)
-__device__ __forceinline__ int page_of(const AttnParams& p, int b, int t, bool flag = true) {
-  const int pg = t < p.pages_per_seq ? p.page_table[(int64_t)b * p.pages_per_seq + t] : -1;
-  if (pg >= 0 && pg < p.n_pages) return pg;
-  if (flag && p.status) atomicOr(p.status + b, SPACE_ST_BAD_PAGE);
-  return p.n_pages;
-}
-
 // One share: tiles t0, t0 + step, ... (n of them) of the T tiles of (sequence b, kv head h).
 struct Seg {
   int b, h, t0, n, step, T, L, slot, dfirst, dn;   // slot: partial slot; dfirst/dn: cut (aligned mode)
@@ -121,13 +111,6 @@ __device__ __noinline__ void mbar_drain(uint32_t bar, uint32_t parity) { mbar_dr
 // ------------------------------------------------------------ work partition
 // Flat tile index space: sequence-major, then kv head, then tile.  Group g of
 // n_groups owns flat tiles [W*g/n_groups, W*(g+1)/n_groups).
-// floor(a * b / c) for a*b that may need 64 bits; 32-bit division when it fits
-__device__ __forceinline__ long long muldiv(long long a, long long b, long long c) {
-  const unsigned long long prod = (unsigned long long)a * (unsigned long long)b;
-  if ((prod >> 32) == 0) return (long long)((unsigned)prod / (unsigned)c);
-  return (long long)(prod / (unsigned long long)c);
-}
-
 // Piece `piece` of `a` of a (sequence, head) with T tiles: tiles [t0, t1).  When the last tile is a
 // partial one and there are at least `a` full tiles, the full tiles are cut evenly (the first pieces
 // take the remainder) and the partial tile goes to the last piece on top; otherwise all T tiles are
@@ -205,13 +188,6 @@ struct Partition {
     }
   }
 };
-
-// group that owns flat tile f (largest g with floor(W*g/NG) <= f)
-__device__ __forceinline__ int group_of(long long f, long long W, long long NG) {
-  const unsigned long long num = (unsigned long long)(f + 1) * (unsigned long long)NG - 1ull;
-  if ((num >> 32) == 0) return (int)((unsigned)num / (unsigned)W);
-  return (int)(num / (unsigned long long)W);
-}
 
 // Shared-memory plan (up to 64 query rows per thread block).
 template <int DH>
@@ -1168,35 +1144,6 @@ __global__ void __launch_bounds__(128) attn_merge_kernel(const AttnParams p) {
 }
 
 // ------------------------------------------------------------------ host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
-                                  CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                                  CUtensorMapFloatOOBfill);
-
-EncodeTiledFn get_encode() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* ptr = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) != cudaSuccess ||
-        qres != cudaDriverEntryPointSuccess)
-      return nullptr;
-    fn = (EncodeTiledFn)ptr;
-  }
-  return fn;
-}
-
-int make_map(CUtensorMap* tm, const void* base, const cuuint64_t dims[4], const cuuint64_t strides_bytes[3],
-             const cuuint32_t box[4]) {
-  EncodeTiledFn enc = get_encode();
-  if (!enc) return SPACE_E_CUDA;
-  const cuuint32_t estr[4] = {1, 1, 1, 1};
-  const CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides_bytes,
-                         box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                         CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? SPACE_OK : SPACE_E_CUDA;
-}
-
 void plan(const space_config* cfg, int sm_count, int k, AttnPlanHost* pl) {
   const int G = cfg->n_q_heads / cfg->n_kv_heads;
   const int n_q = (k + 1) * (k + 1);
