@@ -35,13 +35,13 @@ from paper_2402_11809_b200 import replicas, workloads  # noqa: E402
 
 L2_BYTES = 126 * 1024 * 1024
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from the ncu captures
-# summarised under profiles/: (bytes, kernel source file, first 12 hex digits of that file's sha256 when
-# the capture was taken).  The figure is reported only while the source still has that hash; once the
-# kernel has changed the bench line carries null until the capture is taken again.
-ATTN_TRAFFIC = {"llama7b": (34528512, "attn_tc.cu", "502073d548d8"),
-                "gqa70b": (289103104, "attn_rows.cu", "f24cb4707758")}
-LMHEAD_TRAFFIC = {"lmhead_llama7b": (262672896, "lmhead.cu", "3b9abf44fb19"),
-                  "lmhead_vocab128k": (1087277568, "lmhead.cu", "3b9abf44fb19")}
+# summarised under profiles/: (bytes, kernel source file, first 12 hex digits of the sha256 of that file and
+# the headers it shares when the capture was taken).  The figure is reported only while the sources still have
+# that hash; once the kernel has changed the bench line carries null until the capture is taken again.
+ATTN_TRAFFIC = {"llama7b": (34530048, "attn_tc.cu", "34c9cecbc38a"),
+                "gqa70b": (288952320, "attn_rows.cu", "44432e1bd57e")}
+LMHEAD_TRAFFIC = {"lmhead_llama7b": (262679040, "lmhead.cu", "891963138291"),
+                  "lmhead_vocab128k": (1087231744, "lmhead.cu", "891963138291")}
 METRIC = "auto-correct steps/sec"
 UNIT = "steps/s"
 
@@ -50,9 +50,8 @@ def source_hash(fname):
     import hashlib
     path = os.path.join(ROOT, "paper_2402_11809_b200", "csrc", fname)
     h = hashlib.sha256()
-    for f in (path, os.path.join(os.path.dirname(path), "tc_common.cuh")):
-        if os.path.exists(f):
-            h.update(open(f, "rb").read())
+    for f in (path, *(os.path.join(os.path.dirname(path), n) for n in ("tc_common.cuh", "attn_common.cuh"))):
+        h.update(open(f, "rb").read())
     return h.hexdigest()[:12]
 
 
