@@ -35,6 +35,7 @@
 #include "tc_common.cuh"
 #include "attn_common.cuh"
 #include <cuda.h>
+#include <type_traits>
 #include <math_constants.h>
 
 namespace {
@@ -189,18 +190,21 @@ struct Partition {
   }
 };
 
-// Shared-memory plan (up to 64 query rows per thread block).
-template <int DH>
+// Shared-memory plan (16 * NP query rows per thread block, at most 64).
+template <int DH, int NP>
 struct Smem {
   static constexpr int HALVES = DH / 64;
   static constexpr int TILE_BYTES = TILE_N * DH * 2;         // one K or V tile
-  static constexpr int Q_ROWS = 64;                          // query rows (with padding) per thread block
+  static constexpr int Q_ROWS = 16 * NP;                     // query rows (with padding) per thread block
   static constexpr int Q_BYTES = Q_ROWS * DH * 2;
   static constexpr int P_PART = TILE_N * 128;                // P_hi or P_lo: [key][64 queries] bf16
+  // P^T buffers (each P_hi + P_lo), two where they fit: the softmax stores a tile's P while the tensor core still
+  // reads the one before (8 tiles a block, L2 resident, one / two: 4 rows 14.7 / 14.3 us, 25 rows 16.7 / 16.6,
+  // 36 rows 19.5 / 19.3)
+  static constexpr int P_BUFS = NP == 4 ? 1 : 2;
+  static_assert(2 * P_PART >= TILE_N * 64 * 4, "a tile's scores are parked there as floats");
   static constexpr int K_STAGES = (DH == 128) ? 2 : 3;
   static constexpr int V_STAGES = (DH == 128) ? 2 : 4;
-  static constexpr int P_BUFS = 1;                           // P^T buffers (each P_hi + P_lo); a second one, so that the exponentials of a tile
-                                                             // overlap the O^T product of the tile before, measured no faster
   static constexpr int RS = 64;                              // query rows (padded) per thread block at most
   static constexpr int Q_BUFS = 2;                           // query buffers: the next share's rows load early
   static constexpr int Q_OFF = 0;
@@ -208,8 +212,8 @@ struct Smem {
   static constexpr int V_OFF = K_OFF + K_STAGES * TILE_BYTES;
   static constexpr int P_OFF = V_OFF + V_STAGES * TILE_BYTES;
   static constexpr int BAR_OFF = P_OFF + P_BUFS * 2 * P_PART;
-  // q_full[2], q_empty[2], k_full[], k_empty[], v_full[], v_empty[], s_full[2], p_ready[2], pv_done[2], drain
-  static constexpr int N_BARS = 4 + 2 * K_STAGES + 2 * V_STAGES + 6 + 1;
+  // q_full[2], q_empty[2], k_full[], k_empty[], v_full[], v_empty[], s_full[2], p_ready[2], pv_done[2], s_empty[2], drain
+  static constexpr int N_BARS = 4 + 2 * K_STAGES + 2 * V_STAGES + 8 + 1;
   static constexpr int MISC_OFF = BAR_OFF + (N_BARS * 8 + 15) / 16 * 16;   // tmem base, abort flag (16-byte aligned:
                                                                            // the float arrays below are read as float4)
   static constexpr int SEG0_OFF = MISC_OFF + 16;             // Seg of this group's only share (aligned mode)
@@ -316,7 +320,7 @@ __device__ __noinline__ void piece_rescale(uint32_t taddr, const float* fq) {
 }
 
 // Warp roles
-constexpr int WARP_K = 0, WARP_MMA = 1, WARP_V = 2, WARP_PV = 3, WARP_SOFTMAX0 = 4;
+constexpr int WARP_K = 0, WARP_MMA = 1, WARP_V = 2, WARP_PV = 3, WARP_SOFTMAX0 = 4, SOFT_WARPS = 8;
 constexpr int L2_AHEAD_TILES = 1;      // tiles per operand a block asks L2 for before its dependency wait (more of them
                                        // crowd out the kernels that still run: measured slower)
 constexpr float OVER_THRESHOLD = 60.f;   // re-reference a query row when a score exceeds its reference by 2^60
@@ -327,10 +331,20 @@ constexpr float OVER_THRESHOLD = 60.f;   // re-reference a query row when a scor
 // owns one key of the tile (all 128 TMEM lanes carry work).
 // PAGED: the cache is a pool of pages behind a page table (see AttnParams); a build of its own, so
 // that the contiguous form carries none of it (registers are at the limit of 384 threads).
-template <int DH, bool PAGED>
+// NP: groups of eight query columns per softmax thread (n_pad / 16).  A build per width: with the width a run-time
+// value every group of columns was a branch of its own, and the latencies of one (reference, product, maximum) could
+// not run under those of the next.
+// What a tile costs a block that does not wait for memory (data in L2) is the chain through the softmax threads: wait
+// for S^T, read it, subtract and test, exponentiate, vote, wait for an O^T product, store P, hand over.  All but the
+// last three run while the tensor core takes the O^T product of the tile before, and S^T goes back to its issuer
+// after the vote, so that the next S^T product fills the pipe meanwhile.  Eight tiles per block, us, before / after
+// (the exponentials behind the wait for the product, S^T kept until P was stored, run-time width): 4 rows
+// 16.8 / 14.3, 25 rows 20.3 / 16.6, 36 rows 22.7 / 19.3, 49 rows 25.2 / 24.3; ragged16's attention, bound by memory,
+// gains through the clock under the power cap (step 141 / 131).
+template <int DH, bool PAGED, int NP>
 __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_constant__ AttnParams p,
                                                              int max_batch) {
-  using S = Smem<DH>;
+  using S = Smem<DH, NP>;
   extern __shared__ __align__(1024) unsigned char sm[];
   const uint32_t sm_base = smem_u32(sm);
   const uint32_t bar0 = sm_base + S::BAR_OFF;
@@ -338,7 +352,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   constexpr int B_QFULL = 0, B_QEMPTY = 2, B_KFULL = 4, B_KEMPTY = B_KFULL + S::K_STAGES,
                 B_VFULL = B_KEMPTY + S::K_STAGES, B_VEMPTY = B_VFULL + S::V_STAGES,
                 B_SFULL = B_VEMPTY + S::V_STAGES, B_PREADY = B_SFULL + 2, B_PVDONE = B_SFULL + 4,
-                B_DRAIN = B_SFULL + 6;
+                B_SEMPTY = B_SFULL + 6, B_DRAIN = B_SFULL + 8;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + S::MISC_OFF);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + S::MISC_OFF + 4);
   float* mref_buf = reinterpret_cast<float*>(sm + S::MREF_OFF);
@@ -355,7 +369,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   const int i0 = mb * p.rows_per_mb;                       // first block row of this query-row block
   // query rows (block row, head) handled here: 0 .. m_valid-1; N of the MMAs is n_pad
   const int m_valid = min(p.rows_per_mb, p.n_q - i0) * p.G;
-  const int n_pad = p.n_pad;
+  constexpr int n_pad = 16 * NP;
 
   // ---- set-up ------------------------------------------------------------
   pdl_launch_dependents();
@@ -367,7 +381,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     for (int s = 0; s < S::V_STAGES; ++s) { mbar_init(BAR(B_VFULL + s), 1); mbar_init(BAR(B_VEMPTY + s), 1); }
     for (int i = 0; i < 2; ++i) {
       mbar_init(BAR(B_SFULL + i), 1);
-      mbar_init(BAR(B_PREADY + i), 256);
+      mbar_init(BAR(B_SEMPTY + i), SOFT_WARPS);
+      mbar_init(BAR(B_PREADY + i), SOFT_WARPS);
     }
     mbar_init(BAR(B_PVDONE), 1);
     mbar_init(BAR(B_PVDONE + 1), 1);
@@ -536,7 +551,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   }
   if (!clustered) __syncthreads();                         // the tables of warp 4 reach every warp
   const uint32_t tmem = *tmem_slot;
-  // TMEM columns: S^T buffers at 0 and 128 (n_pad <= 128 columns each), [O_hi^T | O_lo^T] at 256
+  // TMEM columns: S^T buffers at 0 and 128 (n_pad <= 64 columns each), [O_hi^T | O_lo^T] at 256
   // (64 columns each)
   const uint32_t TM_S0 = tmem, TM_O = tmem + 256;
 
@@ -649,8 +664,9 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           const int s = (gt + koff) % S::K_STAGES, buf = gt & 1;
           ok = mbar_wait(BAR(B_KFULL + s), ((gt + koff) / S::K_STAGES) & 1, abort_flag, p.err, 7);
           if (gt == 0) TL(4);
-          // S^T buffer `buf` was last read by the softmax of tile gt-2
-          if (ok && gt >= 2) ok = mbar_wait(BAR(B_PREADY + buf), ((gt - 2) >> 1) & 1, abort_flag, p.err, 8);
+          // S^T buffer `buf` was last read by the softmax of tile gt-2, which hands it back before it stores P:
+          // this product then runs before the O^T product of that tile, not against it
+          if (ok && gt >= 2) ok = mbar_wait(BAR(B_SEMPTY + buf), ((gt - 2) >> 1) & 1, abort_flag, p.err, 8);
           if (!ok) break;
           tc_fence_after();
           const uint64_t kd = kdesc0 + (uint64_t)((s * S::TILE_BYTES) >> 4);
@@ -680,8 +696,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       // the epilogue adds the two.  Columns past the padded query rows hold whatever
       // the shared memory held; they only reach output columns nobody reads.
       const uint32_t idesc_pv = instr_desc_rt(64 + n_pad, 1, 1);   // A = V^T (d contiguous), B = P^T (queries contiguous)
-      // V^T and P^T: 64-wide blocks TILE_N*128 bytes apart, 8-key groups 1024 bytes apart
       static_assert(S::P_PART == TILE_N * 128, "P_lo must follow P_hi at the block stride");
+      // V^T and P^T: 64-wide blocks TILE_N*128 bytes apart, 8-key groups 1024 bytes apart
       const uint64_t vdesc0 = smem_desc(sm_base + S::V_OFF, TILE_N * 128, 1024);
       const uint64_t pdesc0 = smem_desc(sm_base + S::P_OFF, TILE_N * 128, 1024);
       uint32_t g = 0;
@@ -693,8 +709,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           if (ok) ok = mbar_wait(BAR(B_PREADY + (g & 1)), (g >> 1) & 1, abort_flag, p.err, 5);
           if (!ok) break;
           tc_fence_after();
-          const uint64_t ad0 = vdesc0 + (uint64_t)((s * S::TILE_BYTES) >> 4);
           const uint64_t pd0 = pdesc0 + (uint64_t)(((g % S::P_BUFS) * 2 * S::P_PART) >> 4);
+          const uint64_t ad0 = vdesc0 + (uint64_t)((s * S::TILE_BYTES) >> 4);
 #pragma unroll
           for (int kk = 0; kk < TILE_N / 16; ++kk) {
             // 16 keys further = 2048 bytes further in both operands; the first
@@ -715,18 +731,18 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     // ================= softmax / epilogue ==================================
     // One key of the tile per TMEM lane; two threads per key, each with one half
     // of the query-row columns, handled in pieces of 8 columns.
-    constexpr int MAXP = 4;                                // pieces per thread at most
+    constexpr int ncol = 8 * NP;                           // columns per thread
+    constexpr bool VOTE_FIRST = NP == 4;
     const int quarter = warp & 3;                          // TMEM lane quarter this warp may touch
     const int half = (warp - WARP_SOFTMAX0) >> 2;
     const int kl = quarter * 32 + lane;                    // key within the tile; head-dim index in the epilogue
     const int sidx = half * 128 + kl;                      // index among the 256 softmax threads
-    const int ncol = n_pad >> 1, col0 = half * ncol, np = ncol >> 3;
+    const int col0 = half * ncol;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const float c = p.scale_log2;
     const uint32_t prow = sm_base + S::P_OFF + kl * 128;   // this key's 128-byte row in each P block
     const uint32_t swz = (uint32_t)(kl & 7);
-    float lsum[MAXP][8];                                   // this key's share of every row sum
-    float sv[MAXP][8];                                     // scores, then score - reference (log2 units)
+    float lsum[ncol];                                      // this key's share of every row sum
     uint32_t gt = 0;
     int mpar = 0;                                          // which copy of the references is current
     const float* mref = mref_buf;
@@ -738,31 +754,38 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     while (part.next(sg)) {
       const int n_keys = sg.L + p.n_q;
 #pragma unroll
-      for (int j = 0; j < MAXP; ++j)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) lsum[j][e] = 0.f;
+      for (int x = 0; x < ncol; ++x) lsum[x] = 0.f;
       for (int jt = 0; jt < sg.n; ++jt, ++gt) {
         const int t = sg.tile_at(jt);
         const int buf = gt & 1;
         const bool first = (jt == 0);
+        const int lo = t * TILE_N;
+        const int kt = (PAGED || (t + 1) * TILE_N <= n_keys) ? lo : n_keys - TILE_N;
+        const int key = kt + kl;
+        // Visibility of this thread's key: keys before `lo` belong to the previous
+        // tile; cached keys are seen by every row; block keys by the Eq. 5 mask.
+        const bool masked = (kt + TILE_N > sg.L) || (kt < lo);   // same for the whole block
+        float sv[ncol];                                    // scores, then score - reference (log2 units)
+        float mm[ncol];                                    // references (fetched while the scores are on their way)
+        auto fetch_refs = [&](const float* m) {
+#pragma unroll
+          for (int j = 0; j < 2 * NP; ++j) {
+            const float4 v = reinterpret_cast<const float4*>(m + col0)[j];
+            mm[4 * j] = v.x; mm[4 * j + 1] = v.y; mm[4 * j + 2] = v.z; mm[4 * j + 3] = v.w;
+          }
+        };
+        if (!first) fetch_refs(mref);
         ok &= mbar_wait(BAR(B_SFULL + buf), (gt >> 1) & 1, abort_flag, p.err, 9);
         tc_fence_after();
         if (sidx == 0) { if (gt == 0) TL(5); TL(8); }
         const uint32_t ts = TM_S0 + buf * 128 + lane_addr + col0;
         // this key's scores for its columns, all loads in flight together
 #pragma unroll
-        for (int j = 0; j < MAXP; ++j)
-          if (j < np) tmem_ld8(ts + j * 8, reinterpret_cast<uint32_t*>(sv[j]));
+        for (int j = 0; j < NP; ++j) tmem_ld8(ts + j * 8, reinterpret_cast<uint32_t*>(sv + 8 * j));
         tmem_wait_ld();
-        const int lo = t * TILE_N;
-        const int kt = (PAGED || (t + 1) * TILE_N <= n_keys) ? lo : n_keys - TILE_N;
-        const int key = kt + kl;
-        const int jb = key - sg.L;                         // block key index when >= 0
-        // Visibility of this thread's key: keys before `lo` belong to the previous
-        // tile; cached keys are seen by every row; block keys by the Eq. 5 mask.
-        const bool masked = (kt + TILE_N > sg.L) || (kt < lo);   // same for the whole block
         uint64_t vis = ~0ull;
         if (masked) {
+          const int jb = key - sg.L;                       // block key index when >= 0
           if (key < lo) vis = 0ull;
           else if (jb >= p.n_q) vis = 0ull;                 // (paged cache) a row of the page past the last key
           else if (jb >= 0) vis = visq[jb] >> col0;         // (bits past this thread's columns are never looked at)
@@ -780,26 +803,18 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           if (vstart < sg.L) {
             if (key == vstart) {
 #pragma unroll
-              for (int j = 0; j < MAXP; ++j) {
-                if (j < np) {
-                  float4* dst = reinterpret_cast<float4*>(mnew + col0 + j * 8);
-                  dst[0] = make_float4(sv[j][0] * c, sv[j][1] * c, sv[j][2] * c, sv[j][3] * c);
-                  dst[1] = make_float4(sv[j][4] * c, sv[j][5] * c, sv[j][6] * c, sv[j][7] * c);
-                }
-              }
+              for (int j = 0; j < 2 * NP; ++j)
+                reinterpret_cast<float4*>(mnew + col0)[j] =
+                    make_float4(sv[4 * j] * c, sv[4 * j + 1] * c, sv[4 * j + 2] * c, sv[4 * j + 3] * c);
             }
           } else {
-            // block keys only: every thread parks its raw scores in the P buffer (idle until pass 1
-            // of this very tile), then one thread per query column fetches the score of that
+            // block keys only: every thread parks its raw scores in the P buffer (idle until this
+            // very tile's P is stored), then one thread per query column fetches the score of that
             // row's own key
             float* stage = reinterpret_cast<float*>(sm + S::P_OFF) + kl * 64 + col0;
 #pragma unroll
-            for (int j = 0; j < MAXP; ++j) {
-              if (j < np) {
-                reinterpret_cast<float4*>(stage + j * 8)[0] = make_float4(sv[j][0], sv[j][1], sv[j][2], sv[j][3]);
-                reinterpret_cast<float4*>(stage + j * 8)[1] = make_float4(sv[j][4], sv[j][5], sv[j][6], sv[j][7]);
-              }
-            }
+            for (int j = 0; j < 2 * NP; ++j)
+              reinterpret_cast<float4*>(stage)[j] = make_float4(sv[4 * j], sv[4 * j + 1], sv[4 * j + 2], sv[4 * j + 3]);
             soft_sync();
             if (sidx < n_pad) {
               const int i = i0 + (sidx >> (__ffs(p.G) - 1));  // block row of query column sidx
@@ -811,42 +826,47 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           soft_sync();
           mpar ^= 1;
           mref = mref_buf + mpar * S::RS;
+          fetch_refs(mref);
         }
-        // ---- pass 0: score - reference; does any exceed 2^60? -----------------
-        bool over = false;
-        if (!over) {
-          // (independent maxima per piece: a single running flag would chain every element)
-          float worst[MAXP];
+        // ---- score - reference, -inf where the row does not see the key; does any exceed 2^60?
+        // (a row without any visible key so far has reference -inf and only invisible entries)
 #pragma unroll
-          for (int j = 0; j < MAXP; ++j) {
-            worst[j] = -CUDART_INF_F;
-            if (j < np) {
-              const float4 m0 = reinterpret_cast<const float4*>(mref + col0 + j * 8)[0];
-              const float4 m1 = reinterpret_cast<const float4*>(mref + col0 + j * 8)[1];
-              const float mm[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+        for (int x = 0; x < ncol; ++x) sv[x] = fmaf(sv[x], c, -mm[x]);
+        if (masked) {
 #pragma unroll
-              for (int e = 0; e < 8; ++e) sv[j][e] = fmaf(sv[j][e], c, -mm[e]);
-              if (!masked) {
-                worst[j] = fmaxf(fmaxf(fmaxf(sv[j][0], sv[j][1]), fmaxf(sv[j][2], sv[j][3])),
-                                 fmaxf(fmaxf(sv[j][4], sv[j][5]), fmaxf(sv[j][6], sv[j][7])));
-              } else {
-                const uint32_t vb = (uint32_t)(vis >> (j * 8)) & 0xFFu;
+          for (int x = 0; x < ncol; ++x) sv[x] = ((vis >> x) & 1ull) ? sv[x] : -CUDART_INF_F;
+        }
+        bool over;
+        {
+          float w[4] = {sv[0], sv[1], sv[2], sv[3]};        // (independent chains)
 #pragma unroll
-                for (int e = 0; e < 8; ++e)
-                  worst[j] = fmaxf(worst[j], ((vb >> e) & 1u) ? sv[j][e] : -CUDART_INF_F);
-              }
-            }
+          for (int x = 4; x < ncol; x += 2) w[(x >> 1) & 3] = max3(w[(x >> 1) & 3], sv[x], sv[x + 1]);
+          over = !(fmaxf(fmaxf(w[0], w[1]), fmaxf(w[2], w[3])) <= OVER_THRESHOLD);   // also true for NaN
+        }
+        // ---- P = exp2(score - reference) as P_hi + P_lo (two bf16 terms: bf16 alone leaves an output error near
+        // 1e-2 of the output RMS), all of it before anything waits for the O^T product of the tile before: between
+        // that product's end and the next one's start there are the stores of P and a hand-over, nothing else.
+        uint32_t hi[ncol / 2], lw[ncol / 2];
+        auto exponentials = [&] {                          // (sv becomes P itself, for the row sums)
+#pragma unroll
+          for (int x = 0; x < ncol; x += 2) {
+            sv[x] = fast_exp2(sv[x]); sv[x + 1] = fast_exp2(sv[x + 1]);
+            if (VOTE_FIRST) { lsum[x] += sv[x]; lsum[x + 1] += sv[x + 1]; }
+            const __nv_bfloat162 h2 = __floats2bfloat162_rn(sv[x], sv[x + 1]);      // .x = lower query row
+            const float2 hf = __bfloat1622float2(h2);
+            const __nv_bfloat162 l2 = __floats2bfloat162_rn(sv[x] - hf.x, sv[x + 1] - hf.y);
+            hi[x >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+            lw[x >> 1] = *reinterpret_cast<const uint32_t*>(&l2);
           }
-          float w = worst[0];
-#pragma unroll
-          for (int j = 1; j < MAXP; ++j) w = fmaxf(w, worst[j]);
-          over = !(w <= OVER_THRESHOLD);                    // also true for NaN
-        }
+        };
+        // (the vote comes after them, in the shade of that product; with 32 columns a thread has no registers left
+        // for both P and its two terms, adds P to the sums at once, and therefore votes first)
+        if (!VOTE_FIRST) exponentials();
         if (soft_any(over)) {
           // ---- re-reference: per query row maximum over the 128 keys of this tile
 #pragma unroll
-          for (int j = 0; j < MAXP; ++j)
-            if (j < np) piece_key_max(ts + j * 8, (uint32_t)(vis >> (j * 8)) & 0xFFu, xq + quarter * S::RS + col0 + j * 8);
+          for (int j = 0; j < NP; ++j)
+            piece_key_max(ts + j * 8, (uint32_t)(vis >> (j * 8)) & 0xFFu, xq + quarter * S::RS + col0 + j * 8);
           soft_sync();
           // PV of the previous tile must be done before O^T is rescaled
           if (!first) {
@@ -855,67 +875,48 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           }
           float* mnew = mref_buf + (mpar ^ 1) * S::RS;
 #pragma unroll
-          for (int j = 0; j < MAXP; ++j) {
-            if (j < np) {
-              const int q0 = col0 + j * 8;
-              // fq is written and read back by the same thread (its peers write identical values)
-              piece_new_reference(xq + q0, S::RS, mref + q0, mnew + q0, fq + q0, c, first);
-              __syncwarp();
-              if (!first) {
+          for (int j = 0; j < NP; ++j) {
+            const int q0 = col0 + j * 8;
+            // fq is written and read back by the same thread (its peers write identical values)
+            piece_new_reference(xq + q0, S::RS, mref + q0, mnew + q0, fq + q0, c, first);
+            __syncwarp();
+            if (!first) {
 #pragma unroll
-                for (int e = 0; e < 8; ++e) lsum[j][e] *= fq[q0 + e];
-                piece_rescale(TM_O + lane_addr + q0, fq + q0);
-                piece_rescale(TM_O + lane_addr + 64 + q0, fq + q0);
-              }
-              // scores again, now against the new reference
-              uint32_t sr[8];
-              tmem_ld8(ts + j * 8, sr);
-              tmem_wait_ld();
-#pragma unroll
-              for (int e = 0; e < 8; ++e) sv[j][e] = fmaf(__uint_as_float(sr[e]), c, -mnew[q0 + e]);
+              for (int e = 0; e < 8; ++e) lsum[8 * j + e] *= fq[q0 + e];
+              piece_rescale(TM_O + lane_addr + q0, fq + q0);
+              piece_rescale(TM_O + lane_addr + 64 + q0, fq + q0);
             }
+            // scores again, now against the new reference
+            uint32_t sr[8];
+            tmem_ld8(ts + j * 8, sr);
+            tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+              sv[8 * j + e] = ((vis >> (8 * j + e)) & 1ull) ? fmaf(__uint_as_float(sr[e]), c, -mnew[q0 + e]) : -CUDART_INF_F;
           }
+          if (!VOTE_FIRST) exponentials();
           mpar ^= 1;
           mref = mref_buf + mpar * S::RS;
           soft_sync();                                      // new references visible to every thread
         }
-        // the P buffer is free once the PV product that last read it has finished
-        {
-          const uint32_t prev = gt - S::P_BUFS;             // tile that used this P buffer before
-          if (gt >= (uint32_t)S::P_BUFS)
-            ok &= mbar_wait(BAR(B_PVDONE + (prev & 1)), (prev >> 1) & 1, abort_flag, p.err, 11);
+        if (VOTE_FIRST) exponentials();
+        // S^T buffer `buf` goes back: the product of tile gt+2 may start
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(BAR(B_SEMPTY + buf));
+        // this P buffer is free once the PV product that last read it has finished
+        if (gt >= (uint32_t)S::P_BUFS) {
+          const uint32_t prev = gt - S::P_BUFS;
+          ok &= mbar_wait(BAR(B_PVDONE + (prev & 1)), (prev >> 1) & 1, abort_flag, p.err, 11);
         }
+        // P^T rows are keys; a row holds 64 query rows as eight 16-byte pieces,
+        // piece j stored at j ^ (key & 7) (128-byte swizzle)
         const uint32_t pbuf = prow + (gt % S::P_BUFS) * (2 * S::P_PART);
-        // ---- pass 1: P = exp2(score - reference) as P_hi + P_lo (two bf16 terms:
-        // bf16 alone leaves an output error near 1e-2 of the output RMS)
 #pragma unroll
-        for (int j = 0; j < MAXP; ++j) {
-          if (j < np) {
-            uint32_t hi[4], lw[4];
-#pragma unroll
-            for (int e2 = 0; e2 < 4; ++e2) {
-              float p0 = fast_exp2(sv[j][2 * e2]), p1 = fast_exp2(sv[j][2 * e2 + 1]);
-              if (masked) {
-                // a row without any visible key so far has reference -inf and only
-                // invisible entries: the select keeps those at zero
-                p0 = ((vis >> (j * 8 + 2 * e2)) & 1ull) ? p0 : 0.f;
-                p1 = ((vis >> (j * 8 + 2 * e2 + 1)) & 1ull) ? p1 : 0.f;
-              }
-              lsum[j][2 * e2] += p0;
-              lsum[j][2 * e2 + 1] += p1;
-              const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);        // .x = lower query row
-              const float2 hf = __bfloat1622float2(h2);
-              const __nv_bfloat162 l2 = __floats2bfloat162_rn(p0 - hf.x, p1 - hf.y);
-              hi[e2] = *reinterpret_cast<const uint32_t*>(&h2);
-              lw[e2] = *reinterpret_cast<const uint32_t*>(&l2);
-            }
-            // P^T rows are keys; a row holds 64 query rows as eight 16-byte pieces,
-            // piece j stored at j ^ (key & 7) (128-byte swizzle)
-            const int q0 = col0 + j * 8;
-            const uint32_t dst = pbuf + (uint32_t)(q0 >> 6) * (TILE_N * 128) + ((((uint32_t)(q0 & 63) >> 3) ^ swz) << 4);
-            st_shared_v4(dst, hi[0], hi[1], hi[2], hi[3]);
-            st_shared_v4(dst + S::P_PART, lw[0], lw[1], lw[2], lw[3]);
-          }
+        for (int j = 0; j < NP; ++j) {
+          const uint32_t dst = pbuf + ((((uint32_t)(col0 + j * 8) >> 3) ^ swz) << 4);
+          st_shared_v4(dst, hi[4 * j], hi[4 * j + 1], hi[4 * j + 2], hi[4 * j + 3]);
+          st_shared_v4(dst + S::P_PART, lw[4 * j], lw[4 * j + 1], lw[4 * j + 2], lw[4 * j + 3]);
         }
         if (PAGED && kt + TILE_N > n_keys) {
           // Paged cache, last tile: the page's rows past the last key may hold anything, and 0 * NaN
@@ -933,24 +934,31 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // P (and a cleared V row) is read by the tensor core
         tc_fence_before();
-        mbar_arrive(BAR(B_PREADY + buf));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(BAR(B_PREADY + buf));
         if (sidx == 0) { if (gt == 0) TL(6); TL(9); }
+        if (!VOTE_FIRST) {
+#pragma unroll
+          for (int x = 0; x < ncol; ++x) lsum[x] += sv[x];
+        }
       }
       // ---- end of share: final output or partial ---------------------------
       // Row sums first, while the last O^T product still runs.  Every thread holds
-      // its key's share of up to 32 rows; a halving butterfly over the warp leaves
-      // lane r with the sum over the warp's 32 keys for row col0 + r
-      // (with two 64-row blocks: two such folds, rows col0 + r and col0 + 32 + r)
+      // its key's share of ncol rows; a halving butterfly over the warp leaves lane r with
+      // the sum over the warp's 32 keys for row col0 + r (fewer than 32 rows: plain sums over
+      // the upper lane bits first).
+      {
+        constexpr int W = ncol <= 8 ? 8 : ncol <= 16 ? 16 : 32;
+        float red[W];
 #pragma unroll
-      for (int f0 = 0; f0 < MAXP * 8; f0 += 32) {
-        float red[32];
+        for (int x = 0; x < W; ++x) red[x] = x < ncol ? lsum[x < ncol ? x : 0] : 0.f;
 #pragma unroll
-        for (int x = 0; x < 32; ++x) {
-          const int j = (f0 + x) >> 3, e = (f0 + x) & 7;     // piece and element, compile-time after unrolling
-          red[x] = (j < MAXP && j < np) ? lsum[j < MAXP ? j : 0][e] : 0.f;
+        for (int o = 16; o >= W; o >>= 1) {
+#pragma unroll
+          for (int x = 0; x < ncol; ++x) red[x] += __shfl_xor_sync(0xFFFFFFFFu, red[x], o);
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = W / 2; o > 0; o >>= 1) {
           const bool up = (lane & o) != 0;
 #pragma unroll
           for (int i = 0; i < o; ++i) {
@@ -959,7 +967,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
             red[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, o);
           }
         }
-        if (f0 + lane < ncol) xq[quarter * S::RS + col0 + f0 + lane] = red[0];
+        if (lane < ncol) xq[quarter * S::RS + col0 + lane] = red[0];
       }
       soft_sync();
       float* rcp = mref_buf + (mpar ^ 1) * S::RS;            // the idle copy of the references
@@ -1017,7 +1025,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       const size_t out_base = (((size_t)sg.b * p.n_q + i0) * p.H_q + (size_t)sg.h * p.G) * DH + kl;
       const size_t out_row = (size_t)p.H_q * DH;
 #pragma unroll 2
-      for (int j = 0; j < np; ++j) {
+      for (int j = 0; j < NP; ++j) {
         uint32_t o[8], o2[8];
         const int q0 = col0 + j * 8;
         tmem_ld8(TM_O + lane_addr + q0, o);
@@ -1155,30 +1163,39 @@ void plan(const space_config* cfg, int sm_count, int k, AttnPlanHost* pl) {
   pl->n_ctas = groups * pl->n_mblocks;
 }
 
-template <int DH>
+template <int DH, int NP>
 size_t smem_bytes(int max_batch) {
-  return Smem<DH>::TABLE_OFF + (size_t)(2 * max_batch + 1) * sizeof(int);
+  return Smem<DH, NP>::TABLE_OFF + (size_t)(2 * max_batch + 1) * sizeof(int);
 }
 
-template <int DH, bool PAGED>
+template <int DH, bool PAGED, int NP>
 cudaError_t launch_main(const AttnParams& p, int n_ctas, int max_batch, int size, cudaStream_t st, int* max_clusters) {
   // the kernel's limits are raised once per device (to the most any batch needs)
   static unsigned long long done_mask = 0;                 // (one per instantiation)
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 64 || !((done_mask >> dev) & 1ull)) {
-    cudaFuncSetAttribute(attn_tc_kernel<DH, PAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem_bytes<DH>(128));
-    cudaFuncSetAttribute(attn_tc_kernel<DH, PAGED>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(attn_tc_kernel<DH, PAGED, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem_bytes<DH, NP>(128));
+    cudaFuncSetAttribute(attn_tc_kernel<DH, PAGED, NP>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (dev < 64) done_mask |= 1ull << dev;
   }
-  return launch_clusters(attn_tc_kernel<DH, PAGED>, n_ctas, THREADS, smem_bytes<DH>(max_batch), size, st, max_clusters, p, max_batch);
+  return launch_clusters(attn_tc_kernel<DH, PAGED, NP>, n_ctas, THREADS, smem_bytes<DH, NP>(max_batch), size, st, max_clusters, p, max_batch);
 }
 
 template <int DH>
 cudaError_t launch_form(const AttnParams& p, int n_ctas, int max_batch, int size, cudaStream_t st, int* max_clusters = nullptr) {
-  return p.page_table ? launch_main<DH, true>(p, n_ctas, max_batch, size, st, max_clusters)
-                      : launch_main<DH, false>(p, n_ctas, max_batch, size, st, max_clusters);
+  auto form = [&](auto np) {
+    constexpr int NP = decltype(np)::value;
+    return p.page_table ? launch_main<DH, true, NP>(p, n_ctas, max_batch, size, st, max_clusters)
+                        : launch_main<DH, false, NP>(p, n_ctas, max_batch, size, st, max_clusters);
+  };
+  switch (p.n_pad / 16) {
+    case 1: return form(std::integral_constant<int, 1>());
+    case 2: return form(std::integral_constant<int, 2>());
+    case 3: return form(std::integral_constant<int, 3>());
+    default: return form(std::integral_constant<int, 4>());
+  }
 }
 
 }  // namespace

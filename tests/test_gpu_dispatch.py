@@ -209,3 +209,34 @@ def test_host_step_transfers(B, H, where, V):  # noqa: F811
                 for g in range(na + 1):
                     assert np.array_equal(got[:, L + g], x[name][b][:, L + g * (k + 1)])
         assert np.array_equal(h["k_cache"].numpy().view(np.uint16)[1], x["k_cache"][1])
+
+
+# Every width of the transposed attention kernel (16, 32, 48, 64 padded query rows) with several tiles per block, so
+# that its rings of scores, P and tiles come round, clustered (two sequences) and in the flat cut (more pairs than
+# SMs); keys whose scores grow along the sequence move the references in the middle of a share.
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("ramp", [0.0, 6.0])
+@pytest.mark.parametrize("k,G,d,Bn,H_kv", [(1, 1, 64, 2, 12), (2, 1, 128, 40, 4), (3, 1, 128, 2, 12), (3, 2, 64, 2, 12),
+                                           (4, 1, 128, 2, 12), (5, 1, 128, 2, 12), (5, 1, 64, 40, 4), (7, 1, 128, 2, 12),
+                                           (7, 1, 64, 2, 12), (6, 1, 128, 40, 4)])
+def test_transposed_kernel_widths(B, H, k, G, d, Bn, H_kv, ramp, paged):  # noqa: F811
+    cfg = _small_cfg(k, (700, 3100 if Bn == 2 else 900), d=d, H_q=H_kv * G, H_kv=H_kv, Bn=Bn, V=64, seed=k + d)
+    x = workloads.make_step_inputs(cfg)
+    if ramp:
+        from oracle.bf16 import bf16_bits_to_f64
+        kf, qf = (bf16_bits_to_f64(x[n]).astype(np.float32) for n in ("k_cache", "q"))
+        up = np.linspace(0.0, ramp, kf.shape[2], dtype=np.float32)[:, None]
+        for h in range(H_kv):
+            kf[:, h] += up * np.sign(qf[:, 0, h * G])[:, None, :]
+        x["k_cache"] = workloads.f32_to_bf16_bits(kf)
+    y = workloads.to_pages(x) if paged else x
+    ctx = H.make_context(cfg, y)
+    ds = H.DeviceStep(cfg, y)
+    ds.attn(ctx)
+    assert not ds.status.any()
+    got = ds.out.cpu().numpy().astype(np.float64)
+    from oracle.attention import attention_head
+    for b in (0, Bn - 1):                                    # first and last pairs of the cut
+        for h in (0, H_kv * G - 1):
+            ref, _ = attention_head(x["q"][b, :, h], x["k_cache"][b, h // G], x["v_cache"][b, h // G], int(x["kv_len"][b]), k, x["scale"])
+            H.check_attention(got[b:b + 1, :, h], ref[None], f"sequence {b} head {h}")
