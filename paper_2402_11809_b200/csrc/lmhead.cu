@@ -2,15 +2,16 @@
 // model call P = M(I) and the loop after it).
 //
 // logits[r, x] = <h_r, W_x> for the (k+1)^2 block rows of every sequence and the
-// whole vocabulary, but the logits never reach memory: the product runs on the
-// tensor cores with the block rows on the MMA M extent (A = hidden rows, K-major)
-// and up to 256 tokens on the N extent (B = rows of W, K-major; fp32 accumulators
-// in TMEM: lane = block row, column = token).  An instruction of this kind costs
-// about the same whatever its N, so the tokens go on N: measured with the tokens
-// on M (128 per instruction) the 512 instructions of a thread block took longer
-// than its share of W takes to arrive.  Four epilogue threads share one block row
-// (two beyond 128 rows): each folds its part of the accumulator columns into (max,
-// lowest arg-max, sum exp(z - max)) in registers, and they meet once, at the end of the
+// whole vocabulary, but the logits never reach memory: the products run on the
+// tensor cores into fp32 accumulators in TMEM.  Two orientations, by the number of rows
+// (launch_group has the rule and what was measured):
+//   rows on M    A = hidden rows, B = up to 256 rows of W; lane = block row, column = token.
+//                Four epilogue threads share one block row (two beyond 128 rows).
+//   tokens on M  A = 128 rows of W (two accumulators per box), B = hidden rows; lane = token,
+//                column = block row.  The epilogue turns eight rows of a warp's 32 tokens at
+//                a time through shared memory and folds them with four lanes per row.
+// Either way an epilogue thread folds its tokens of a row into (max, lowest arg-max,
+// sum exp(z - max)) in registers, and a row's threads meet once, at the end of the
 // block's range.  The last thread block to finish combines the vocabulary ranges and runs the acceptance scan, the extra
 // token, the <EOS> cut and the next candidates.
 //
@@ -46,6 +47,8 @@ constexpr int LM_MAX_STAGES = 10;
 constexpr int LM_L2_AHEAD = 8;              // slices of W a block asks L2 for before its dependency wait (4: two thirds of the gain)
 constexpr float LM_NEG = -3.0e38f;          // "no logit yet": finite, so that differences never give NaN
 constexpr int LM_MAX_N = 256;               // block rows of the whole batch, padded to 16
+constexpr int LM_TOK = 128;                 // tokens per accumulator with the tokens on M
+constexpr int LM_XP_PITCH = 36;             // floats per row of a warp's transposing buffer (8 rows of 32 tokens)
 // Which block rows a launch projects: all of them, the target rows of every sequence (row b(k+1)+t), or
 // the mask rows of every sequence's group i* (row bk+o-1; i* is the launch before's result).
 enum { LM_ALL = 0, LM_TARGETS = 1, LM_MASKS = 2 };
@@ -109,7 +112,7 @@ __device__ __forceinline__ uint64_t smem_desc_k128(uint32_t addr) {
   return d;
 }
 // Instruction descriptor: bf16 x bf16 -> f32, M = 128, N = n, both operands K-major.
-__device__ __forceinline__ uint32_t instr_desc(int n) {
+__device__ __forceinline__ uint32_t instr_desc(int n) {                  // (M = 128 either way)
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(LM_M >> 4) << 24);
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
@@ -118,6 +121,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(LM_EPI_T) : "memory"); }
 
@@ -136,30 +144,29 @@ __device__ __forceinline__ void argmax_unkey(unsigned long long key, float& m, i
   idx = (int)(0xFFFFFFFFu - (uint32_t)key);
 }
 
-// Fold 16 consecutive tokens x0 .. x0+15 (the first nv of them valid) into a row's statistics.
-__device__ __forceinline__ void fold16(float& m, float& s, int& idx, const uint32_t* v, int x0, int nv) {
-  float z[16];
-#pragma unroll
-  for (int j = 0; j < 16; ++j) z[j] = (j < nv) ? __uint_as_float(v[j]) : LM_NEG;
+// Fold N consecutive tokens x0 .. x0+N-1 (the first nv of them valid, at least one) into a row's statistics: sums of
+// exp2((z - max) c).
+template <int N>
+__device__ __forceinline__ void fold(float& m, float& s, int& idx, const float (&z)[N], int x0, float c) {
   float cm = z[0];
 #pragma unroll
-  for (int j = 1; j < 16; ++j) cm = fmaxf(cm, z[j]);
+  for (int j = 1; j < N; ++j) cm = fmaxf(cm, z[j]);
   if (cm > m) {                                           // strictly larger: an earlier token keeps a tie
-    int at = 15;
+    int at = N - 1;
 #pragma unroll
-    for (int j = 14; j >= 0; --j) at = (z[j] == cm) ? j : at;
+    for (int j = N - 2; j >= 0; --j) at = (z[j] == cm) ? j : at;
     idx = x0 + at;
-    s *= fast_exp2((m - cm) * LOG2E);
+    s *= fast_exp2((m - cm) * c);
     m = cm;
   }
-  const float ms = -m * LOG2E;
+  const float ms = -m * c;
   float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
-  for (int j = 0; j < 16; j += 4) {
-    a0 += fast_exp2(fmaf(z[j], LOG2E, ms));
-    a1 += fast_exp2(fmaf(z[j + 1], LOG2E, ms));
-    a2 += fast_exp2(fmaf(z[j + 2], LOG2E, ms));
-    a3 += fast_exp2(fmaf(z[j + 3], LOG2E, ms));
+  for (int j = 0; j < N; j += 4) {
+    a0 += fast_exp2(fmaf(z[j], c, ms));
+    a1 += fast_exp2(fmaf(z[j + 1], c, ms));
+    a2 += fast_exp2(fmaf(z[j + 2], c, ms));
+    a3 += fast_exp2(fmaf(z[j + 3], c, ms));
   }
   s += (a0 + a1) + (a2 + a3);
 }
@@ -174,43 +181,19 @@ struct RowNoisy {
   bool noisy;                 // this row draws a token at all
 };
 
-// Sampling-mode fold of 16 consecutive tokens x0 .. x0+15 (x0 a multiple of 16, the first nv valid):
-// (max, lowest arg-max, sum of exp2((z - max) c)), the candidate's own logit when it lies here, and
-// the best Gumbel-perturbed score z c + noise(token) -- the noise of token x is lane x & 3 of the
-// Philox block with counter word x >> 2, as in the verification kernels.
-__device__ __forceinline__ void fold16_noisy(float& m, float& s, int& idx, RowNoisy& r, const uint32_t* v, int x0,
-                                             int nv, float c, uint32_t key0, uint32_t key1) {
-  float z[16];
+// What sampling keeps of N consecutive tokens x0 .. x0+N-1 (x0 a multiple of 4, the first nv valid) besides: the
+// candidate's own logit when it lies here, and the best Gumbel-perturbed score z c + noise(token) -- the noise of
+// token x is lane x & 3 of the Philox block with counter word x >> 2, as in the verification kernels.
+template <int N>
+__device__ __forceinline__ void fold_noisy(RowNoisy& r, const float (&z)[N], int x0, int nv, float c, uint32_t key0,
+                                           uint32_t key1) {
+  if ((unsigned)(r.cand_tok - x0) < (unsigned)N) {
 #pragma unroll
-  for (int j = 0; j < 16; ++j) z[j] = (j < nv) ? __uint_as_float(v[j]) : LM_NEG;
-  float cm = z[0];
-#pragma unroll
-  for (int j = 1; j < 16; ++j) cm = fmaxf(cm, z[j]);
-  if (cm > m) {
-    int at = 15;
-#pragma unroll
-    for (int j = 14; j >= 0; --j) at = (z[j] == cm) ? j : at;
-    idx = x0 + at;
-    s *= fast_exp2((m - cm) * c);
-    m = cm;
-  }
-  const float ms = -m * c;
-  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll
-  for (int j = 0; j < 16; j += 4) {
-    a0 += fast_exp2(fmaf(z[j], c, ms));
-    a1 += fast_exp2(fmaf(z[j + 1], c, ms));
-    a2 += fast_exp2(fmaf(z[j + 2], c, ms));
-    a3 += fast_exp2(fmaf(z[j + 3], c, ms));
-  }
-  s += (a0 + a1) + (a2 + a3);
-  if ((unsigned)(r.cand_tok - x0) < 16u) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) if (x0 + j == r.cand_tok) r.zc = z[j];
+    for (int j = 0; j < N; ++j) if (x0 + j == r.cand_tok) r.zc = z[j];
   }
   if (r.noisy) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < N / 4; ++i) {
       const Philox4 ph = philox4x32_10((uint32_t)((x0 >> 2) + i), r.purpose, r.seq, r.pos, key0, key1);
       const uint32_t w[4] = {ph.x, ph.y, ph.z, ph.w};
 #pragma unroll
@@ -268,21 +251,26 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // Shared-memory plan (dynamic, 1024-byte aligned base):
 //   [stages]{ [kbs] hidden tiles of n_pad*128 bytes, [kbs] W tiles of n_box*128 bytes } | pad |
+//   (tokens on M: the epilogue warps' transposing buffers, the rows' constants) |
 //   barriers | row results [n_pad] x 2 | candidates | misc
-// A product reads 128 rows from a hidden tile's address whatever n_pad is: the rows past the
-// tile are whatever follows in shared memory (the stage's W tiles, then `pad`) and only reach
+// A product reads 128 rows of its first operand whatever the tile holds: the rows past the
+// tile are whatever follows in shared memory (other tiles, then `pad`) and only reach
 // accumulator lanes nobody reads.  `pad` keeps that read inside the allocation.
+struct RowConst { int cand_tok, exclude; uint32_t purpose, seq, pos; int noisy, pad[2]; };   // (see RowNoisy)
 struct LmSmem {
-  uint32_t a_bytes, b_bytes, b_in_stage, stage_bytes, bar_off, row_off, cand_off, misc_off, total;
-  __host__ __device__ LmSmem(int n_pad, int n_box, int stages, int kbs) {
+  uint32_t a_bytes, b_bytes, b_in_stage, stage_bytes, xp_off, rowc_off, bar_off, row_off, cand_off, misc_off, total;
+  __host__ __device__ LmSmem(bool tokens_on_m, int n_pad, int n_box, int stages, int kbs) {
     a_bytes = (uint32_t)n_pad * LM_KB * 2;
     b_bytes = (uint32_t)n_box * LM_KB * 2;
     b_in_stage = (uint32_t)kbs * a_bytes;
     stage_bytes = b_in_stage + (uint32_t)kbs * b_bytes;
-    const uint32_t reach = 16384u * (n_pad > LM_M ? 2u : 1u);            // bytes a product reads from a hidden tile
-    const uint32_t have = a_bytes + (uint32_t)kbs * b_bytes;             // bytes that follow the last hidden tile's start
+    // bytes the products read from the last tile of their first operand, and bytes that follow its start
+    const uint32_t reach = 16384u * (tokens_on_m ? (n_box > LM_TOK ? 2u : 1u) : (n_pad > LM_M ? 2u : 1u));
+    const uint32_t have = tokens_on_m ? b_bytes : a_bytes + (uint32_t)kbs * b_bytes;
     const uint32_t pad = reach > have ? (reach - have + 1023u) / 1024u * 1024u : 0u;
-    bar_off = (uint32_t)stages * stage_bytes + pad;
+    xp_off = (uint32_t)stages * stage_bytes + pad;
+    rowc_off = xp_off + (tokens_on_m ? LM_EPI * 8u * LM_XP_PITCH * 4u : 0u);
+    bar_off = rowc_off + (tokens_on_m ? (uint32_t)n_pad * (uint32_t)sizeof(RowConst) : 0u);
     row_off = bar_off + 8u * (2 * LM_MAX_STAGES + 4);
     cand_off = row_off + 2u * 4u * (uint32_t)n_pad;                      // candidates of the batch: fewer than n_pad
     misc_off = cand_off + 4u * (uint32_t)n_pad;
@@ -290,10 +278,13 @@ struct LmSmem {
   }
 };
 
+// TM: tokens on the M extent, block rows on N (see the file header and launch_group's rule).
+template <bool TM, bool SAMPLE>
 __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __grid_constant__ LmParams p) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t sm_base = smem_u32(smem_raw);
-  const LmSmem L(p.n_pad, p.n_box, p.stages, p.kbs);
+  const LmSmem L(TM, p.n_pad, p.n_box, p.stages, p.kbs);
+  constexpr bool sample = SAMPLE;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int S = p.stages;
   const uint32_t bar0 = sm_base + L.bar_off;
@@ -350,6 +341,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
   const int KB = (p.D + LM_KB - 1) / LM_KB;
   const int kbs = p.kbs;
   const int n_bufs = p.n_mt == 1 ? 2 : 1;                  // accumulator buffers of n_mt x 256 columns
+  const int acc_cols = TM ? p.n_mt * LM_TOK : 0;           // (tokens on M: columns of one of a buffer's two accumulators)
 
   if (warp == 0) {
     // ================= producer ==============================================
@@ -392,7 +384,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       bool ok = !*abort_flag;
       for (int box = 0; box < nb && ok; ++box) {
         const int row0 = r0 + box * p.n_box;
-        const uint32_t idesc = instr_desc((r1 - row0 <= p.tail_rows) ? p.tail_rows : p.n_box);
+        const uint32_t idesc = instr_desc(TM ? p.n_pad : (r1 - row0 <= p.tail_rows) ? p.tail_rows : p.n_box);
+        const int n_tt = (min(r1 - row0, p.n_box) + LM_TOK - 1) / LM_TOK;   // (tokens on M: accumulators of this box)
         // (the buffer's user before this one: box - n_bufs)
         if (box >= n_bufs) ok = mbar_wait(LBAR(B_ACCEMPTY + buf), (n_bufs == 2 ? (box >> 1) - 1 : box - 1) & 1, abort_flag, p.err, 2);
         if (!ok) break;
@@ -405,7 +398,15 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           const uint32_t st_off = s * L.stage_bytes;
           for (int j = 0; j < nk; ++j) {
             const uint64_t wd = desc0 + (uint64_t)((st_off + L.b_in_stage + (uint32_t)j * L.b_bytes) >> 4);
-            for (int mt = 0; mt < p.n_mt; ++mt) {
+            if (TM) {
+              const uint64_t hd = desc0 + (uint64_t)((st_off + (uint32_t)j * L.a_bytes) >> 4);
+              for (int tt = 0; tt < n_tt; ++tt) {
+                const uint32_t acc = tmem + (uint32_t)((buf * 2 + tt) * acc_cols);
+#pragma unroll
+                for (int kk = 0; kk < LM_KB / 16; ++kk)
+                  mma_ss(acc, wd + (uint64_t)(tt * (16384 >> 4) + kk * 2), hd + (uint64_t)(kk * 2), idesc, (kb0 | j | kk) ? 1u : 0u);
+              }
+            } else for (int mt = 0; mt < p.n_mt; ++mt) {
               // block rows 128*mt .. of the hidden tile (8-row groups are contiguous: 16 KB further on)
               const uint64_t hd = desc0 + (uint64_t)((st_off + (uint32_t)j * L.a_bytes + (uint32_t)mt * 16384u) >> 4);
               const uint32_t acc = tmem + (uint32_t)((buf * p.n_mt + mt) * LM_MAX_BOX);
@@ -425,81 +426,221 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
     // ================= epilogue ================================================
     const int quarter = warp & 3;                          // TMEM lanes 32*quarter .. +31
     const int ew = warp - 2;
-    // The warps of a lane quarter share the accumulators, and take an accumulator's column groups in turn;
-    // they meet at the end (with one warp per quarter its scan was what a call ended on, and what a sampling
-    // call waited for all along).
-    const int mt = (ew >> 2) % p.n_mt, n_parts = LM_EPI / 4 / p.n_mt, part = (ew >> 2) / p.n_mt;
-    const int row = mt * LM_M + quarter * 32 + lane;       // this thread's block row
     // the candidates are an input: fetched now, so that the last block's scan does not wait for them
     for (int t = threadIdx.x - 64; t < p.B * p.k; t += LM_EPI_T) cand_s[t] = p.cand[t];
-    float m0 = LM_NEG, s0 = 0.f;
-    int i0 = 0x7FFFFFFF;
-    const bool sample = p.mode == SPACE_MODE_SAMPLE;
-    RowNoisy n0;
-    if (sample) row_noisy_init(n0, p, row);
-    // a warp whose 32 lanes hold no block row only takes part in the hand-shakes
-    const bool has_rows = row - lane < p.n_rows;
-    bool ok = true;
-    for (int box = 0; box < nb; ++box) {
-      const int buf = n_bufs == 2 ? box & 1 : 0;
-      ok = ok && mbar_wait(LBAR(B_ACCFULL + buf), (n_bufs == 2 ? box >> 1 : box) & 1, abort_flag, p.err, 4, true);
-      ok = __all_sync(0xFFFFFFFFu, ok);
-      if (!ok) break;
-      tc_fence_after();
-      const int row0 = r0 + box * p.n_box;
-      const int n_valid = min(r1 - row0, (r1 - row0 <= p.tail_rows) ? p.tail_rows : p.n_box);
-      const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((buf * p.n_mt + mt) * LM_MAX_BOX);
-      if (has_rows) {
-        for (int c0 = 16 * part; c0 < n_valid; c0 += 16 * n_parts) {
-          uint32_t v[16];
-          tmem_ld16(acc + (uint32_t)c0, v);
-          tmem_wait_ld();
-          if (sample) fold16_noisy(m0, s0, i0, n0, v, row0 + c0, n_valid - c0, p.c_t, p.key0, p.key1);
-          else fold16(m0, s0, i0, v, row0 + c0, n_valid - c0);
+    if (TM) {
+      // ---- tokens on M: lane = token, column = block row.  A warp reads 8 rows of its 32 tokens, turns them through
+      // its shared-memory buffer and folds them with four lanes per row, eight tokens each.  The four warps of a lane
+      // quarter take the groups of eight rows in turn, both accumulators of a box one after the other; what a lane
+      // keeps of its up to eight rows stays in registers until the end of the range.
+      constexpr int GP = LM_MAX_N / 8 / 4;
+      const int part = ew >> 2, n_grp = p.n_pad >> 3;
+      const int rl = lane & 7, tl = (lane >> 3) * 8;         // this lane's row of a group, its first token of the 32
+      float* xp = reinterpret_cast<float*>(smem_raw + L.xp_off) + ew * (8 * LM_XP_PITCH);
+      RowConst* rowc = reinterpret_cast<RowConst*>(smem_raw + L.rowc_off);
+      if (sample) {
+        const int row = threadIdx.x - 64;
+        if (row < p.n_pad) {
+          RowNoisy r;
+          row_noisy_init(r, p, row);
+          rowc[row] = RowConst{r.cand_tok, r.exclude, r.purpose, r.seq, r.pos, r.noisy ? 1 : 0, {0, 0}};
         }
+        epi_sync();
       }
-      // this accumulator buffer may be overwritten by the products of the next box that uses it
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(LBAR(B_ACCEMPTY + buf));
-    }
-    {
-      // the other parts' columns join the first's (the pipeline stages are idle: every product is done)
-      float* x = reinterpret_cast<float*>(smem_raw) + row;   // [n_parts - 1][7][2 LM_M]
-      constexpr int W = 2 * LM_M;
-      if (part > 0 && has_rows) {
-        float* y = x + (part - 1) * 7 * W;
-        y[0] = m0; y[W] = s0; y[2 * W] = __int_as_float(i0);
-        if (sample) { y[3 * W] = n0.gs; y[4 * W] = n0.gz; y[5 * W] = __int_as_float(n0.gidx); y[6 * W] = n0.zc; }
+      float m[GP], sm[GP], gs[GP], gz[GP], zc[GP];
+      int id[GP], gi[GP];
+#pragma unroll
+      for (int i = 0; i < GP; ++i) {
+        m[i] = LM_NEG; sm[i] = 0.f; id[i] = 0x7FFFFFFF;
+        gs[i] = -CUDART_INF_F; gz[i] = 0.f; gi[i] = 0x7FFFFFFF; zc[i] = LM_NEG;
       }
-      epi_sync();
-      if (part == 0 && has_rows) {
-        for (int o = 1; o < n_parts; ++o) {
-          const float* y = x + (o - 1) * 7 * W;
-          const float m2 = y[0], s2 = y[W], c = sample ? p.c_t : LOG2E;
-          const int i2 = __float_as_int(y[2 * W]);
-          if (m2 > m0 || (m2 == m0 && i2 < i0)) i0 = i2;
-          const float e = fast_exp2(-fabsf(m0 - m2) * c);   // (one of the two exponentials is exp(0))
-          s0 = (m0 >= m2) ? fmaf(s2, e, s0) : fmaf(s0, e, s2);
-          m0 = fmaxf(m0, m2);
-          if (sample) {
-            const float g2 = y[3 * W];
-            const int gi2 = __float_as_int(y[5 * W]);
-            if (g2 > n0.gs || (g2 == n0.gs && gi2 < n0.gidx)) { n0.gs = g2; n0.gz = y[4 * W]; n0.gidx = gi2; }
-            n0.zc = fmaxf(n0.zc, y[6 * W]);
+      bool ok = true;
+      for (int box = 0; box < nb; ++box) {
+        const int buf = n_bufs == 2 ? box & 1 : 0;
+        ok = ok && mbar_wait(LBAR(B_ACCFULL + buf), (n_bufs == 2 ? box >> 1 : box) & 1, abort_flag, p.err, 4, true);
+        ok = __all_sync(0xFFFFFFFFu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        const int row0 = r0 + box * p.n_box, n_valid = min(r1 - row0, p.n_box);
+        const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * 2 * acc_cols);
+#pragma unroll
+        for (int i = 0; i < GP; ++i) {
+          const int g = part + 4 * i;
+          if (g < n_grp) {
+            uint32_t v[2][8];                                // (a second accumulator that the box does not use: never read on)
+            tmem_ld8(acc + (uint32_t)(g * 8), v[0]);
+            tmem_ld8(acc + (uint32_t)(acc_cols + g * 8), v[1]);
+            tmem_wait_ld();
+#pragma unroll
+            for (int tt = 0; tt < 2; ++tt) {
+              const int tok = tt * LM_TOK + quarter * 32;    // first token of this warp's lanes within the box
+              if (tok >= n_valid) break;
+#pragma unroll
+              for (int j = 0; j < 8; ++j) xp[j * LM_XP_PITCH + lane] = __uint_as_float(v[tt][j]);
+              __syncwarp();
+              float z[8];
+              *reinterpret_cast<float4*>(z) = *reinterpret_cast<const float4*>(xp + rl * LM_XP_PITCH + tl);
+              *reinterpret_cast<float4*>(z + 4) = *reinterpret_cast<const float4*>(xp + rl * LM_XP_PITCH + tl + 4);
+              __syncwarp();
+              const int nv = n_valid - tok - tl, x0 = row0 + tok + tl;
+              if (nv > 0) {
+#pragma unroll
+                for (int j = 1; j < 8; ++j) z[j] = (j < nv) ? z[j] : LM_NEG;
+                fold(m[i], sm[i], id[i], z, x0, p.c_t);
+                if (sample) {
+                  const RowConst rc = rowc[g * 8 + rl];
+                  RowNoisy r{gs[i], gz[i], gi[i], zc[i], rc.cand_tok, rc.exclude, rc.purpose, rc.seq, rc.pos, rc.noisy != 0};
+                  fold_noisy(r, z, x0, nv, p.c_t, p.key0, p.key1);
+                  gs[i] = r.gs; gz[i] = r.gz; gi[i] = r.gidx; zc[i] = r.zc;
+                }
+              }
+            }
+          }
+        }
+        // this accumulator buffer may be overwritten by the products of the next box that uses it
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(LBAR(B_ACCEMPTY + buf));
+      }
+      // ---- the four lanes of a row meet, then (through the idle stages: every product is done) the four quarters
+      float* x = reinterpret_cast<float*>(smem_raw);         // [4][7][LM_MAX_N]
+      auto join = [&](float& m0, float& s0, int& i0, float& g0, float& z0, int& k0, float& c0, float m2, float s2, int i2,
+                      float g2, float z2, int k2, float c2) {
+        if (m2 > m0 || (m2 == m0 && i2 < i0)) i0 = i2;
+        const float e = fast_exp2(-fabsf(m0 - m2) * p.c_t);  // (one of the two exponentials is exp(0))
+        s0 = (m0 >= m2) ? fmaf(s2, e, s0) : fmaf(s0, e, s2);
+        m0 = fmaxf(m0, m2);
+        if (sample) {
+          if (g2 > g0 || (g2 == g0 && k2 < k0)) { g0 = g2; z0 = z2; k0 = k2; }
+          c0 = fmaxf(c0, c2);
+        }
+      };
+#pragma unroll
+      for (int i = 0; i < GP; ++i) {
+        const int g = part + 4 * i;
+        if (g < n_grp) {
+#pragma unroll
+          for (int o = 8; o <= 16; o <<= 1) {
+            const float m2 = __shfl_xor_sync(0xFFFFFFFFu, m[i], o), s2 = __shfl_xor_sync(0xFFFFFFFFu, sm[i], o);
+            const int i2 = __shfl_xor_sync(0xFFFFFFFFu, id[i], o);
+            float g2 = 0.f, z2 = 0.f, c2 = 0.f;
+            int k2 = 0;
+            if (sample) {
+              g2 = __shfl_xor_sync(0xFFFFFFFFu, gs[i], o); z2 = __shfl_xor_sync(0xFFFFFFFFu, gz[i], o);
+              k2 = __shfl_xor_sync(0xFFFFFFFFu, gi[i], o); c2 = __shfl_xor_sync(0xFFFFFFFFu, zc[i], o);
+            }
+            join(m[i], sm[i], id[i], gs[i], gz[i], gi[i], zc[i], m2, s2, i2, g2, z2, k2, c2);
+          }
+          if (lane < 8) {
+            float* y = x + quarter * 7 * LM_MAX_N + g * 8 + lane;
+            y[0] = m[i]; y[LM_MAX_N] = sm[i]; y[2 * LM_MAX_N] = __int_as_float(id[i]);
+            if (sample) {
+              y[3 * LM_MAX_N] = gs[i]; y[4 * LM_MAX_N] = gz[i]; y[5 * LM_MAX_N] = __int_as_float(gi[i]); y[6 * LM_MAX_N] = zc[i];
+            }
           }
         }
       }
-    }
-    // publish this block's statistics of every block row
-    if (row < p.n_rows && part == 0) {
-      LmPartial out; out.m = m0; out.s = s0; out.idx = i0; out.pad = 0;
-      *reinterpret_cast<int4*>(p.part + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&out);
-      atomicMax(p.keys + row, argmax_key(m0, i0));
-      if (sample) {
-        LmNoisy g; g.gs = n0.gs; g.gz = n0.gz; g.gidx = n0.gidx; g.pad = 0;
-        *reinterpret_cast<int4*>(p.gpart + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&g);
-        if ((unsigned)(n0.cand_tok - r0) < (unsigned)(r1 - r0)) p.zc[row] = n0.zc;   // this block owns the candidate's token
+      epi_sync();
+      // publish this block's statistics of every block row
+      const int row = threadIdx.x - 64;
+      if (row < p.n_rows) {
+        float v[4][7];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int f = 0; f < (SAMPLE ? 7 : 3); ++f) v[q][f] = x[(q * 7 + f) * LM_MAX_N + row];
+        int i0 = __float_as_int(v[0][2]), k0 = sample ? __float_as_int(v[0][5]) : 0;
+#pragma unroll
+        for (int q = 1; q < 4; ++q)
+          join(v[0][0], v[0][1], i0, v[0][3], v[0][4], k0, v[0][6], v[q][0], v[q][1], __float_as_int(v[q][2]),
+               v[q][3], v[q][4], sample ? __float_as_int(v[q][5]) : 0, v[q][6]);
+        LmPartial out; out.m = v[0][0]; out.s = v[0][1]; out.idx = i0; out.pad = 0;
+        *reinterpret_cast<int4*>(p.part + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&out);
+        atomicMax(p.keys + row, argmax_key(v[0][0], i0));
+        if (sample) {
+          LmNoisy gn; gn.gs = v[0][3]; gn.gz = v[0][4]; gn.gidx = k0; gn.pad = 0;
+          *reinterpret_cast<int4*>(p.gpart + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&gn);
+          if ((unsigned)(rowc[row].cand_tok - r0) < (unsigned)(r1 - r0)) p.zc[row] = v[0][6];   // this block owns the candidate's token
+        }
+      }
+    } else {
+      // The warps of a lane quarter share the accumulators, and take an accumulator's column groups in turn;
+      // they meet at the end (with one warp per quarter its scan was what a call ended on, and what a sampling
+      // call waited for all along).
+      const int mt = (ew >> 2) % p.n_mt, n_parts = LM_EPI / 4 / p.n_mt, part = (ew >> 2) / p.n_mt;
+      const int row = mt * LM_M + quarter * 32 + lane;       // this thread's block row
+      float m0 = LM_NEG, s0 = 0.f;
+      int i0 = 0x7FFFFFFF;
+      RowNoisy n0;
+      if (sample) row_noisy_init(n0, p, row);
+      // a warp whose 32 lanes hold no block row only takes part in the hand-shakes
+      const bool has_rows = row - lane < p.n_rows;
+      bool ok = true;
+      for (int box = 0; box < nb; ++box) {
+        const int buf = n_bufs == 2 ? box & 1 : 0;
+        ok = ok && mbar_wait(LBAR(B_ACCFULL + buf), (n_bufs == 2 ? box >> 1 : box) & 1, abort_flag, p.err, 4, true);
+        ok = __all_sync(0xFFFFFFFFu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        const int row0 = r0 + box * p.n_box;
+        const int n_valid = min(r1 - row0, (r1 - row0 <= p.tail_rows) ? p.tail_rows : p.n_box);
+        const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((buf * p.n_mt + mt) * LM_MAX_BOX);
+        if (has_rows) {
+          for (int c0 = 16 * part; c0 < n_valid; c0 += 16 * n_parts) {
+            uint32_t v[16];
+            tmem_ld16(acc + (uint32_t)c0, v);
+            tmem_wait_ld();
+            const int nv = n_valid - c0;
+            float z[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) z[j] = (j < nv) ? __uint_as_float(v[j]) : LM_NEG;
+            fold(m0, s0, i0, z, row0 + c0, p.c_t);
+            if (sample) fold_noisy(n0, z, row0 + c0, nv, p.c_t, p.key0, p.key1);
+          }
+        }
+        // this accumulator buffer may be overwritten by the products of the next box that uses it
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(LBAR(B_ACCEMPTY + buf));
+      }
+      {
+        // the other parts' columns join the first's (the pipeline stages are idle: every product is done)
+        float* x = reinterpret_cast<float*>(smem_raw) + row;   // [n_parts - 1][7][2 LM_M]
+        constexpr int W = 2 * LM_M;
+        if (part > 0 && has_rows) {
+          float* y = x + (part - 1) * 7 * W;
+          y[0] = m0; y[W] = s0; y[2 * W] = __int_as_float(i0);
+          if (sample) { y[3 * W] = n0.gs; y[4 * W] = n0.gz; y[5 * W] = __int_as_float(n0.gidx); y[6 * W] = n0.zc; }
+        }
+        epi_sync();
+        if (part == 0 && has_rows) {
+          for (int o = 1; o < n_parts; ++o) {
+            const float* y = x + (o - 1) * 7 * W;
+            const float m2 = y[0], s2 = y[W], c = p.c_t;
+            const int i2 = __float_as_int(y[2 * W]);
+            if (m2 > m0 || (m2 == m0 && i2 < i0)) i0 = i2;
+            const float e = fast_exp2(-fabsf(m0 - m2) * c);   // (one of the two exponentials is exp(0))
+            s0 = (m0 >= m2) ? fmaf(s2, e, s0) : fmaf(s0, e, s2);
+            m0 = fmaxf(m0, m2);
+            if (sample) {
+              const float g2 = y[3 * W];
+              const int gi2 = __float_as_int(y[5 * W]);
+              if (g2 > n0.gs || (g2 == n0.gs && gi2 < n0.gidx)) { n0.gs = g2; n0.gz = y[4 * W]; n0.gidx = gi2; }
+              n0.zc = fmaxf(n0.zc, y[6 * W]);
+            }
+          }
+        }
+      }
+      // publish this block's statistics of every block row
+      if (row < p.n_rows && part == 0) {
+        LmPartial out; out.m = m0; out.s = s0; out.idx = i0; out.pad = 0;
+        *reinterpret_cast<int4*>(p.part + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&out);
+        atomicMax(p.keys + row, argmax_key(m0, i0));
+        if (sample) {
+          LmNoisy g; g.gs = n0.gs; g.gz = n0.gz; g.gidx = n0.gidx; g.pad = 0;
+          *reinterpret_cast<int4*>(p.gpart + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&g);
+          if ((unsigned)(n0.cand_tok - r0) < (unsigned)(r1 - r0)) p.zc[row] = n0.zc;   // this block owns the candidate's token
+        }
       }
     }
     epi_sync();
@@ -764,7 +905,7 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   p.n_rows = p.B * (phase == LM_ALL ? p.n_q : phase == LM_TARGETS ? a->k + 1 : a->k);
   p.n_pad = (p.n_rows + 15) / 16 * 16;
   if (p.n_pad > LM_MAX_N) return SPACE_E_UNSUPPORTED;
-  p.n_mt = p.n_pad > LM_M ? 2 : 1;
+  p.n_mt = p.n_pad > LM_M ? 2 : 1;                         // (tokens on M: accumulators of 256 columns instead of 128)
   int grid = ctx->sm_count;
   const int max_useful = (a->vocab + 31) / 32;             // at least 32 tokens per thread block
   if (grid > max_useful) grid = max_useful;
@@ -777,16 +918,30 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   // with few tokens per thread block (us per call, graph replay, for one / two / four: 64 rows of V = 2091
   // 23.6 / 18.5 / 16.4, 25 rows of V = 5000 25.0 / 20.6 / 18.4, 36 rows of V = 12000 28.2 / 26.9 / 26.9, of
   // V = 32000 53.2 / 53.5 / -).  As many stages as fit, at most LM_MAX_STAGES.
+  const bool sampling = a->mode == SPACE_MODE_SAMPLE;
+  // Which operand is the block rows'.  Rows on M: an instruction of 128 rows and N tokens takes 43 + N/2 cycles (one per
+  // 128 rows), however few of the 128 are real, and their energy with it, which under the power cap is time.  Tokens
+  // on M: 43 + rows/2 for 128 tokens.  So tokens on M for few rows (energy) and where the rows would take two
+  // instructions for little more than one's worth, as long as the 128-token accumulators are filled; up to about 80
+  // rows and from 200 the time of the products is even, in between it is the other's.  Measured with D = 4096,
+  // us per call in a steady loop (bursts), rows on M / tokens on M: greedy, V = 32000: 9 rows 53.2 (48.3) / 48.5 (48.1),
+  // 36 rows 54.1 (48.8) / 51.1 (49.5), 49 rows 54.7 (49.6) / 52.7 (50.3), 72 rows 55.4 (50.4) / 55.6 (52.6), 108 rows
+  // 57.9 (52.7) / 59.4 (54.1), 144 rows 72.9 (61.2) / 63.0 (56.4), 176 rows 75.8 (62.5) / 72.3 (62.0), 192 rows 75.8 (62.7) /
+  // 74.0 (63.4), 252 rows 79.5 (67.9) / 84.9 (72.6); V = 128256: 36 rows 191 (167) / 171 (161); accumulators half empty,
+  // V = 20000, D = 2048, 36 rows 22.3 (21.4) / 23.1 (23.9).  Sampling, whose epilogue is long either way: V = 32000, 36 rows
+  // 60.7 (56.9) / 58.6 (59.5), 64 rows 61.6 (57.5) / 62.0 (61.2), 144 rows 81.8 (70.5) / 75.4 (70.7), 176 rows 84.1 (72.7) /
+  // 81.9 (75.5).
+  const bool tokens_on_m = p.n_box > 192 && (p.n_pad <= (sampling ? 48 : 64) || (p.n_pad > LM_M && p.n_pad <= 176));
   const size_t budget = 220 * 1024;
   int stages = 0;
   for (p.kbs = p.n_box <= 128 ? 4 : 1; p.kbs >= 1; p.kbs /= 2) {
     stages = LM_MAX_STAGES;
-    while (stages > 1 && LmSmem(p.n_pad, p.n_box, stages, p.kbs).total + 1024 > budget) --stages;
+    while (stages > 1 && LmSmem(tokens_on_m, p.n_pad, p.n_box, stages, p.kbs).total + 1024 > budget) --stages;
     if (stages >= (p.kbs > 1 ? 3 : 2)) break;
   }
   if (stages < 2) return SPACE_E_UNSUPPORTED;
   p.stages = stages;
-  const LmSmem L(p.n_pad, p.n_box, stages, p.kbs);
+  const LmSmem L(tokens_on_m, p.n_pad, p.n_box, stages, p.kbs);
   if (L.total + 1024 > 227 * 1024) return SPACE_E_UNSUPPORTED;
   p.eos_id = a->eos_id;
   p.mode = a->mode; p.resample = a->resample;
@@ -814,10 +969,12 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
                                          a->hidden_row_stride * (phase == LM_TARGETS ? a->k + 1 : 1), p.n_pad);
   if (rc != SPACE_OK) return rc;
   const size_t sm = L.total + 1024;
-  cudaFuncSetAttribute(lmhead_verify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  auto kernel = tokens_on_m ? (sampling ? lmhead_verify_kernel<true, true> : lmhead_verify_kernel<true, false>)
+                            : (sampling ? lmhead_verify_kernel<false, true> : lmhead_verify_kernel<false, false>);
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   {
     ProfScope ps(ctx, SPACE_K_LMHEAD, st);
-    launch_pdl(lmhead_verify_kernel, dim3(grid), dim3(LM_THREADS), sm, st, p);
+    launch_pdl(kernel, dim3(grid), dim3(LM_THREADS), sm, st, p);
   }
   ctx->launches += 1;
   return cuda_ok(cudaGetLastError());

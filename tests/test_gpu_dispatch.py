@@ -240,3 +240,45 @@ def test_transposed_kernel_widths(B, H, k, G, d, Bn, H_kv, ramp, paged):  # noqa
         for h in (0, H_kv * G - 1):
             ref, _ = attention_head(x["q"][b, :, h], x["k_cache"][b, h // G], x["v_cache"][b, h // G], int(x["kv_len"][b]), k, x["scale"])
             H.check_attention(got[b:b + 1, :, h], ref[None], f"sequence {b} head {h}")
+
+
+# Projection with the tokens on the M extent: few rows and 129..176 padded ones, ranges of one box and of two, a last
+# box of one accumulator, D off the slices, odd vocabularies; next to widths that keep the rows on M.  Sampling: noise
+# from the table and past its end (many noisy rows), sequence ids and positions per row.
+@pytest.mark.parametrize("mode", ["greedy", "residual_pointmass", "paper_literal"])
+@pytest.mark.parametrize("V,D,k,Bn", [(30011, 72, 2, 1), (29000, 136, 5, 1), (40003, 64, 7, 1), (38001, 200, 5, 4), (50257, 64, 3, 11),
+                                      (57003, 72, 1, 40), (32000, 64, 3, 15), (60001, 64, 1, 25), (400, 64, 5, 2)])
+def test_lmhead_orientations(B, H, mode, V, D, k, Bn):  # noqa: F811
+    cfg = workloads.resolve_lmhead("lmhead_tiny", V=V, D=D, k=k, B=Bn, p_accept=(0.5, 1.0))
+    x = workloads.make_lmhead_inputs(cfg)
+    rng = np.random.default_rng(V)
+    sample = mode != "greedy"
+    if mode == "paper_literal":
+        x["cand_prob"] = rng.uniform(0.05, 1.0, size=x["cand_prob"].shape).astype(np.float32)
+    kv_len = rng.integers(0, 3000, size=Bn).astype(np.int32)
+    ctx = B.Context(max_batch=Bn, n_q_heads=8, n_kv_heads=8, head_dim=64, k_max=k, vocab=V, s_cap=256)
+    i32 = lambda *s: torch.full(s, -7, dtype=torch.int32, device="cuda")  # noqa: E731
+    got = dict(n_accept=i32(Bn), out_tokens=i32(Bn, k + 1), n_out=i32(Bn), next_cand=i32(Bn, k),
+               next_cand_prob=torch.full((Bn, k), float("nan"), device="cuda"),
+               finished=torch.full((Bn,), 9, dtype=torch.uint8, device="cuda"))
+    keep = [H.to_dev(x[n]) for n in ("hidden", "weight", "cand", "cand_prob")] + [H.to_dev(kv_len)]
+    a = ctx.lmhead_args(keep[0], keep[1], keep[2], k=k, eos_id=-1, seed=7, temperature=0.9,
+                        mode=B.MODE_SAMPLE if sample else B.MODE_GREEDY, cand_prob=keep[3], kv_len=keep[4],
+                        resample=B.RESAMPLE_PAPER_LITERAL if mode == "paper_literal" else B.RESAMPLE_RESIDUAL_POINTMASS, **got)
+    kw = dict(mode="sample", temperature=0.9, seed=7, kv_len=kv_len, resample=mode) if sample else {}
+    r = lmhead_verify_step(x["hidden"], x["weight"], x["cand"], x["cand_prob"], k, eos_id=-1, **kw)
+    excl = np.zeros(Bn, bool)                                # decisions inside the tie bands of the by-phase test
+    for b in range(Bn):
+        i = int(r["n_accept"][b])
+        used = [] if sample else [t * (k + 1) for t in range(k + 1)]
+        used += [] if mode == "paper_literal" else [i * (k + 1) + o for o in range(1, k + 1)]
+        excl[b] = bool(used) and r["row_gap"][b, used].min() <= 1e-3
+    if sample:
+        excl |= (r["accept_margin"] <= 1e-3).any(1) | (r["bonus_gap"] <= 1e-3) | (r["draft_gap"] <= 1e-3).any(1)
+    assert excl.sum() <= max(1, Bn // 8)
+    for again in range(2):
+        ctx.space_lmhead_verify(a)
+        h = {n: t.cpu().numpy() for n, t in got.items()}
+        for n in ("n_accept", "out_tokens", "n_out", "next_cand", "finished"):
+            assert np.array_equal(h[n][~excl], r[n][~excl]), (n, again)
+        np.testing.assert_allclose(h["next_cand_prob"][~excl], r["next_cand_prob"][~excl], rtol=1e-3)
