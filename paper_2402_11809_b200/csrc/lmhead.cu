@@ -48,6 +48,7 @@ constexpr int LM_L2_AHEAD = 8;              // slices of W a block asks L2 for b
 constexpr float LM_NEG = -3.0e38f;          // "no logit yet": finite, so that differences never give NaN
 constexpr int LM_MAX_N = 256;               // block rows of the whole batch, padded to 16
 constexpr int LM_TOK = 128;                 // tokens per accumulator with the tokens on M
+constexpr int LM_NOISE_BYTES = 24 * 1024;   // noise table of a box (sampling), at most
 constexpr int LM_XP_PITCH = 36;             // floats per row of a warp's transposing buffer (8 rows of 32 tokens)
 // Which block rows a launch projects: all of them, the target rows of every sequence (row b(k+1)+t), or
 // the mask rows of every sequence's group i* (row bk+o-1; i* is the launch before's result).
@@ -70,6 +71,7 @@ struct LmParams {
   int n_box;                  // rows of the first tensor map's box (N of its products)
   int tail_rows;              // rows of the second tensor map's box
   int kbs;                    // 64-element slices of the hidden dimension per stage
+  int n_noisy, noise_tok;     // sampling: rows that draw a token, tokens of a box whose noise is tabulated (a multiple of 16)
   int eos_id;
   int mode, resample;         // SPACE_MODE_*, SPACE_RESAMPLE_*
   float c_t;                  // log2(e) / T: exponent scale of the sums and of the noisy scores (sampling)
@@ -171,36 +173,49 @@ __device__ __forceinline__ void fold(float& m, float& s, int& idx, const float (
   s += (a0 + a1) + (a2 + a3);
 }
 
-// What an epilogue thread keeps of one block row in sampling mode.
+// What an epilogue thread keeps of one block row in sampling mode, and what it has to know of the row.
 struct RowNoisy {
   float gs, gz; int gidx;     // best noisy score so far, the logit that has it, its token
   float zc;                   // logit of the candidate this (target) row scores
+};
+struct RowConst {
   int cand_tok;               // that candidate, or -1
   int exclude;                // token left out of the draw (the rejected point-mass candidate), or -1
   uint32_t purpose, seq, pos; // Philox counter words of this row's noise
-  bool noisy;                 // this row draws a token at all
+  int noisy;                  // this row's place among the rows that draw a token at all, or -1
+  int pad[2];
 };
 
+// Noise of the four tokens of Philox block `block`: that of token x is lane x & 3 of the block with counter word
+// x >> 2, as in the verification kernels.
+__device__ __forceinline__ float4 noise4(uint32_t block, const RowConst& rc, uint32_t key0, uint32_t key1) {
+  const Philox4 ph = philox4x32_10(block, rc.purpose, rc.seq, rc.pos, key0, key1);
+  return make_float4(gumbel2_from_uniform(uniform_open(ph.x)), gumbel2_from_uniform(uniform_open(ph.y)),
+                     gumbel2_from_uniform(uniform_open(ph.z)), gumbel2_from_uniform(uniform_open(ph.w)));
+}
+
 // What sampling keeps of N consecutive tokens x0 .. x0+N-1 (x0 a multiple of 4, the first nv valid) besides: the
-// candidate's own logit when it lies here, and the best Gumbel-perturbed score z c + noise(token) -- the noise of
-// token x is lane x & 3 of the Philox block with counter word x >> 2, as in the verification kernels.
+// candidate's own logit when it lies here, and the best Gumbel-perturbed score z c + noise(token), with the noise of
+// the first in_table tokens (a multiple of 4, or not positive) from `table`.
 template <int N>
-__device__ __forceinline__ void fold_noisy(RowNoisy& r, const float (&z)[N], int x0, int nv, float c, uint32_t key0,
-                                           uint32_t key1) {
-  if ((unsigned)(r.cand_tok - x0) < (unsigned)N) {
+__device__ __forceinline__ void fold_noisy(RowNoisy& r, const RowConst& rc, const float (&z)[N], int x0, int nv, float c,
+                                           uint32_t key0, uint32_t key1, const float* table, int in_table) {
+  if ((unsigned)(rc.cand_tok - x0) < (unsigned)N) {
 #pragma unroll
-    for (int j = 0; j < N; ++j) if (x0 + j == r.cand_tok) r.zc = z[j];
+    for (int j = 0; j < N; ++j) if (x0 + j == rc.cand_tok) r.zc = z[j];
   }
-  if (r.noisy) {
+  if (rc.noisy >= 0) {
 #pragma unroll
     for (int i = 0; i < N / 4; ++i) {
-      const Philox4 ph = philox4x32_10((uint32_t)((x0 >> 2) + i), r.purpose, r.seq, r.pos, key0, key1);
-      const uint32_t w[4] = {ph.x, ph.y, ph.z, ph.w};
+      float4 g;
+      if (4 * i < in_table) g = reinterpret_cast<const float4*>(table)[i];
+      else g = noise4((uint32_t)((x0 >> 2) + i), rc, key0, key1);
+      const float gg[4] = {g.x, g.y, g.z, g.w};
 #pragma unroll
       for (int l = 0; l < 4; ++l) {
         const int j = 4 * i + l;
-        const float sc = fmaf(z[j], c, gumbel2_from_uniform(uniform_open(w[l])));
-        if (j < nv && x0 + j != r.exclude && sc > r.gs) { r.gs = sc; r.gidx = x0 + j; r.gz = z[j]; }
+        const float sc = fmaf(z[j], c, gg[l]);
+        if (j < nv && x0 + j != rc.exclude && sc > r.gs) { r.gs = sc; r.gidx = x0 + j; r.gz = z[j]; }
       }
     }
   }
@@ -224,23 +239,25 @@ __device__ __forceinline__ bool row_place(const LmParams& p, int row, int& b, in
 // Per-row constants of the sampling mode; target rows score candidate c_{t+1} and draw the extra token of the
 // case i* = t at position L+t+1; mask rows (t, o) draw candidate o of that case at position
 // L+t+1+o when candidates are sampled (Algorithm 1 as printed).
-__device__ __forceinline__ void row_noisy_init(RowNoisy& r, const LmParams& p, int row) {
-  r.gs = -CUDART_INF_F; r.gz = 0.f; r.gidx = 0x7FFFFFFF; r.zc = LM_NEG;
-  r.cand_tok = -1; r.exclude = -1; r.purpose = 0; r.seq = 0; r.pos = 0; r.noisy = false;
+__device__ __forceinline__ RowConst row_const(const LmParams& p, int row) {
+  RowConst r{-1, -1, 0u, 0u, 0u, -1, {0, 0}};
   int b, t, o;
-  if (!row_place(p, row, b, t, o)) return;
+  if (!row_place(p, row, b, t, o)) return r;
   const bool literal = p.resample == SPACE_RESAMPLE_PAPER_LITERAL;
   r.seq = p.seq_id ? p.seq_id[b] : p.seq_base + (uint32_t)b;
   const int L = p.kv_len ? p.kv_len[b] : 0;
   if (o == 0) {
-    r.noisy = true; r.purpose = PURPOSE_TOKEN; r.pos = (uint32_t)(L + t + 1);
+    r.purpose = PURPOSE_TOKEN; r.pos = (uint32_t)(L + t + 1);
+    r.noisy = (literal || p.phase != LM_ALL) ? row : b * (p.k + 1) + t;
     if (t < p.k) {
       r.cand_tok = p.cand[b * p.k + t];
       if (!literal && p.cand_prob[b * p.k + t] == 1.0f) r.exclude = r.cand_tok;   // residual of a point mass
     }
   } else if (literal) {
-    r.noisy = true; r.purpose = PURPOSE_DRAFT; r.pos = (uint32_t)(L + t + 1 + o);
+    r.purpose = PURPOSE_DRAFT; r.pos = (uint32_t)(L + t + 1 + o);
+    r.noisy = row;
   }
+  return r;
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
@@ -251,15 +268,14 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 // Shared-memory plan (dynamic, 1024-byte aligned base):
 //   [stages]{ [kbs] hidden tiles of n_pad*128 bytes, [kbs] W tiles of n_box*128 bytes } | pad |
-//   (tokens on M: the epilogue warps' transposing buffers, the rows' constants) |
+//   (tokens on M: the epilogue warps' transposing buffers) | (sampling: the rows' constants, the noise table) |
 //   barriers | row results [n_pad] x 2 | candidates | misc
 // A product reads 128 rows of its first operand whatever the tile holds: the rows past the
 // tile are whatever follows in shared memory (other tiles, then `pad`) and only reach
 // accumulator lanes nobody reads.  `pad` keeps that read inside the allocation.
-struct RowConst { int cand_tok, exclude; uint32_t purpose, seq, pos; int noisy, pad[2]; };   // (see RowNoisy)
 struct LmSmem {
-  uint32_t a_bytes, b_bytes, b_in_stage, stage_bytes, xp_off, rowc_off, bar_off, row_off, cand_off, misc_off, total;
-  __host__ __device__ LmSmem(bool tokens_on_m, int n_pad, int n_box, int stages, int kbs) {
+  uint32_t a_bytes, b_bytes, b_in_stage, stage_bytes, xp_off, rowc_off, noise_off, bar_off, row_off, cand_off, misc_off, total;
+  __host__ __device__ LmSmem(bool tokens_on_m, bool sample, int n_noisy, int noise_tok, int n_pad, int n_box, int stages, int kbs) {
     a_bytes = (uint32_t)n_pad * LM_KB * 2;
     b_bytes = (uint32_t)n_box * LM_KB * 2;
     b_in_stage = (uint32_t)kbs * a_bytes;
@@ -270,7 +286,8 @@ struct LmSmem {
     const uint32_t pad = reach > have ? (reach - have + 1023u) / 1024u * 1024u : 0u;
     xp_off = (uint32_t)stages * stage_bytes + pad;
     rowc_off = xp_off + (tokens_on_m ? LM_EPI * 8u * LM_XP_PITCH * 4u : 0u);
-    bar_off = rowc_off + (tokens_on_m ? (uint32_t)n_pad * (uint32_t)sizeof(RowConst) : 0u);
+    noise_off = rowc_off + (sample ? (uint32_t)n_pad * (uint32_t)sizeof(RowConst) : 0u);
+    bar_off = noise_off + (sample && noise_tok ? (uint32_t)n_noisy * (uint32_t)(noise_tok + 4) * 4u : 0u);
     row_off = bar_off + 8u * (2 * LM_MAX_STAGES + 4);
     cand_off = row_off + 2u * 4u * (uint32_t)n_pad;                      // candidates of the batch: fewer than n_pad
     misc_off = cand_off + 4u * (uint32_t)n_pad;
@@ -278,12 +295,13 @@ struct LmSmem {
   }
 };
 
-// TM: tokens on the M extent, block rows on N (see the file header and launch_group's rule).
+// TM: tokens on the M extent, block rows on N, greedy calls only (see the file header and launch_group's rule).
 template <bool TM, bool SAMPLE>
 __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __grid_constant__ LmParams p) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const uint32_t sm_base = smem_u32(smem_raw);
-  const LmSmem L(TM, p.n_pad, p.n_box, p.stages, p.kbs);
+  const LmSmem L(TM, SAMPLE, p.n_noisy, p.noise_tok, p.n_pad, p.n_box, p.stages, p.kbs);
+  static_assert(!TM || !SAMPLE, "sampling keeps the rows on M");
   constexpr bool sample = SAMPLE;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int S = p.stages;
@@ -428,6 +446,32 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
     const int ew = warp - 2;
     // the candidates are an input: fetched now, so that the last block's scan does not wait for them
     for (int t = threadIdx.x - 64; t < p.B * p.k; t += LM_EPI_T) cand_s[t] = p.cand[t];
+    // Sampling: the noise does not depend on the logits, and while the products run the epilogue warps have nothing
+    // else to do.  So they work it out for a box before they wait for its accumulators, spread over all threads,
+    // where the folds would do it for 32 rows in step although only every (k+1)-th of them draws a token, after
+    // the last product, with the whole chip waiting.  D = 4096, bursts, in the folds / tabulated: one sequence of 36 rows,
+    // V = 32000, 56.9 / 52.9 us, V = 128256 (D = 2048) 92.7 / 87.3, 144 rows of V = 32000 69.9 / 66.2, of V = 20000 (D = 2048)
+    // 37.7 / 33.2, 16 x 36 rows of V = 128256 (96 noisy rows: a quarter of a box fits) 351 / 348.
+    RowConst* rowc = reinterpret_cast<RowConst*>(smem_raw + L.rowc_off);
+    float* noise = reinterpret_cast<float*>(smem_raw + L.noise_off);       // [n_noisy][noise_tok + 4]
+    const int noise_pitch = p.noise_tok + 4;
+    if (sample) {
+      for (int row = threadIdx.x - 64; row < p.n_pad; row += LM_EPI_T) rowc[row] = row_const(p, row);
+      epi_sync();
+    }
+    auto fill_noise = [&](int row0, int n_valid) {
+      if (p.noise_tok == 0) return;
+      epi_sync();                                            // (the table of the box before has been read)
+      const int n4 = min(p.noise_tok, (n_valid + 15) & ~15) >> 2;
+      for (int at = threadIdx.x - 64; at < p.n_noisy * n4; at += LM_EPI_T) {
+        const int y = at / n4, q = at - y * n4;
+        // row of the y-th noisy one (row_const says which those are)
+        const int k1 = p.k + 1;
+        const int row = (p.phase != LM_ALL || p.resample == SPACE_RESAMPLE_PAPER_LITERAL) ? y : y / k1 * p.n_q + y % k1 * k1;
+        reinterpret_cast<float4*>(noise + y * noise_pitch)[q] = noise4((uint32_t)(row0 >> 2) + q, rowc[row], p.key0, p.key1);
+      }
+      epi_sync();
+    };
     if (TM) {
       // ---- tokens on M: lane = token, column = block row.  A warp reads 8 rows of its 32 tokens, turns them through
       // its shared-memory buffer and folds them with four lanes per row, eight tokens each.  The four warps of a lane
@@ -437,23 +481,10 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       const int part = ew >> 2, n_grp = p.n_pad >> 3;
       const int rl = lane & 7, tl = (lane >> 3) * 8;         // this lane's row of a group, its first token of the 32
       float* xp = reinterpret_cast<float*>(smem_raw + L.xp_off) + ew * (8 * LM_XP_PITCH);
-      RowConst* rowc = reinterpret_cast<RowConst*>(smem_raw + L.rowc_off);
-      if (sample) {
-        const int row = threadIdx.x - 64;
-        if (row < p.n_pad) {
-          RowNoisy r;
-          row_noisy_init(r, p, row);
-          rowc[row] = RowConst{r.cand_tok, r.exclude, r.purpose, r.seq, r.pos, r.noisy ? 1 : 0, {0, 0}};
-        }
-        epi_sync();
-      }
-      float m[GP], sm[GP], gs[GP], gz[GP], zc[GP];
-      int id[GP], gi[GP];
+      float m[GP], sm[GP];
+      int id[GP];
 #pragma unroll
-      for (int i = 0; i < GP; ++i) {
-        m[i] = LM_NEG; sm[i] = 0.f; id[i] = 0x7FFFFFFF;
-        gs[i] = -CUDART_INF_F; gz[i] = 0.f; gi[i] = 0x7FFFFFFF; zc[i] = LM_NEG;
-      }
+      for (int i = 0; i < GP; ++i) { m[i] = LM_NEG; sm[i] = 0.f; id[i] = 0x7FFFFFFF; }
       bool ok = true;
       for (int box = 0; box < nb; ++box) {
         const int buf = n_bufs == 2 ? box & 1 : 0;
@@ -487,12 +518,6 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
 #pragma unroll
                 for (int j = 1; j < 8; ++j) z[j] = (j < nv) ? z[j] : LM_NEG;
                 fold(m[i], sm[i], id[i], z, x0, p.c_t);
-                if (sample) {
-                  const RowConst rc = rowc[g * 8 + rl];
-                  RowNoisy r{gs[i], gz[i], gi[i], zc[i], rc.cand_tok, rc.exclude, rc.purpose, rc.seq, rc.pos, rc.noisy != 0};
-                  fold_noisy(r, z, x0, nv, p.c_t, p.key0, p.key1);
-                  gs[i] = r.gs; gz[i] = r.gz; gi[i] = r.gidx; zc[i] = r.zc;
-                }
               }
             }
           }
@@ -503,40 +528,24 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         if (lane == 0) mbar_arrive(LBAR(B_ACCEMPTY + buf));
       }
       // ---- the four lanes of a row meet, then (through the idle stages: every product is done) the four quarters
-      float* x = reinterpret_cast<float*>(smem_raw);         // [4][7][LM_MAX_N]
-      auto join = [&](float& m0, float& s0, int& i0, float& g0, float& z0, int& k0, float& c0, float m2, float s2, int i2,
-                      float g2, float z2, int k2, float c2) {
+      float* x = reinterpret_cast<float*>(smem_raw);         // [4][3][LM_MAX_N]
+      auto join = [&](float& m0, float& s0, int& i0, float m2, float s2, int i2) {
         if (m2 > m0 || (m2 == m0 && i2 < i0)) i0 = i2;
         const float e = fast_exp2(-fabsf(m0 - m2) * p.c_t);  // (one of the two exponentials is exp(0))
         s0 = (m0 >= m2) ? fmaf(s2, e, s0) : fmaf(s0, e, s2);
         m0 = fmaxf(m0, m2);
-        if (sample) {
-          if (g2 > g0 || (g2 == g0 && k2 < k0)) { g0 = g2; z0 = z2; k0 = k2; }
-          c0 = fmaxf(c0, c2);
-        }
       };
 #pragma unroll
       for (int i = 0; i < GP; ++i) {
         const int g = part + 4 * i;
         if (g < n_grp) {
 #pragma unroll
-          for (int o = 8; o <= 16; o <<= 1) {
-            const float m2 = __shfl_xor_sync(0xFFFFFFFFu, m[i], o), s2 = __shfl_xor_sync(0xFFFFFFFFu, sm[i], o);
-            const int i2 = __shfl_xor_sync(0xFFFFFFFFu, id[i], o);
-            float g2 = 0.f, z2 = 0.f, c2 = 0.f;
-            int k2 = 0;
-            if (sample) {
-              g2 = __shfl_xor_sync(0xFFFFFFFFu, gs[i], o); z2 = __shfl_xor_sync(0xFFFFFFFFu, gz[i], o);
-              k2 = __shfl_xor_sync(0xFFFFFFFFu, gi[i], o); c2 = __shfl_xor_sync(0xFFFFFFFFu, zc[i], o);
-            }
-            join(m[i], sm[i], id[i], gs[i], gz[i], gi[i], zc[i], m2, s2, i2, g2, z2, k2, c2);
-          }
+          for (int o = 8; o <= 16; o <<= 1)
+            join(m[i], sm[i], id[i], __shfl_xor_sync(0xFFFFFFFFu, m[i], o), __shfl_xor_sync(0xFFFFFFFFu, sm[i], o),
+                 __shfl_xor_sync(0xFFFFFFFFu, id[i], o));
           if (lane < 8) {
-            float* y = x + quarter * 7 * LM_MAX_N + g * 8 + lane;
+            float* y = x + quarter * 3 * LM_MAX_N + g * 8 + lane;
             y[0] = m[i]; y[LM_MAX_N] = sm[i]; y[2 * LM_MAX_N] = __int_as_float(id[i]);
-            if (sample) {
-              y[3 * LM_MAX_N] = gs[i]; y[4 * LM_MAX_N] = gz[i]; y[5 * LM_MAX_N] = __int_as_float(gi[i]); y[6 * LM_MAX_N] = zc[i];
-            }
           }
         }
       }
@@ -544,24 +553,17 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       // publish this block's statistics of every block row
       const int row = threadIdx.x - 64;
       if (row < p.n_rows) {
-        float v[4][7];
+        float v[4][3];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
 #pragma unroll
-          for (int f = 0; f < (SAMPLE ? 7 : 3); ++f) v[q][f] = x[(q * 7 + f) * LM_MAX_N + row];
-        int i0 = __float_as_int(v[0][2]), k0 = sample ? __float_as_int(v[0][5]) : 0;
+          for (int f = 0; f < 3; ++f) v[q][f] = x[(q * 3 + f) * LM_MAX_N + row];
+        int i0 = __float_as_int(v[0][2]);
 #pragma unroll
-        for (int q = 1; q < 4; ++q)
-          join(v[0][0], v[0][1], i0, v[0][3], v[0][4], k0, v[0][6], v[q][0], v[q][1], __float_as_int(v[q][2]),
-               v[q][3], v[q][4], sample ? __float_as_int(v[q][5]) : 0, v[q][6]);
+        for (int q = 1; q < 4; ++q) join(v[0][0], v[0][1], i0, v[q][0], v[q][1], __float_as_int(v[q][2]));
         LmPartial out; out.m = v[0][0]; out.s = v[0][1]; out.idx = i0; out.pad = 0;
         *reinterpret_cast<int4*>(p.part + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&out);
         atomicMax(p.keys + row, argmax_key(v[0][0], i0));
-        if (sample) {
-          LmNoisy gn; gn.gs = v[0][3]; gn.gz = v[0][4]; gn.gidx = k0; gn.pad = 0;
-          *reinterpret_cast<int4*>(p.gpart + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&gn);
-          if ((unsigned)(rowc[row].cand_tok - r0) < (unsigned)(r1 - r0)) p.zc[row] = v[0][6];   // this block owns the candidate's token
-        }
       }
     } else {
       // The warps of a lane quarter share the accumulators, and take an accumulator's column groups in turn;
@@ -571,19 +573,20 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       const int row = mt * LM_M + quarter * 32 + lane;       // this thread's block row
       float m0 = LM_NEG, s0 = 0.f;
       int i0 = 0x7FFFFFFF;
-      RowNoisy n0;
-      if (sample) row_noisy_init(n0, p, row);
+      RowNoisy n0{-CUDART_INF_F, 0.f, 0x7FFFFFFF, LM_NEG};
+      RowConst rc{-1, -1, 0u, 0u, 0u, -1, {0, 0}};
+      if (sample && row < p.n_pad) rc = rowc[row];
       // a warp whose 32 lanes hold no block row only takes part in the hand-shakes
       const bool has_rows = row - lane < p.n_rows;
       bool ok = true;
       for (int box = 0; box < nb; ++box) {
         const int buf = n_bufs == 2 ? box & 1 : 0;
+        if (sample) fill_noise(r0 + box * p.n_box, min(r1 - r0 - box * p.n_box, p.n_box));
         ok = ok && mbar_wait(LBAR(B_ACCFULL + buf), (n_bufs == 2 ? box >> 1 : box) & 1, abort_flag, p.err, 4, true);
         ok = __all_sync(0xFFFFFFFFu, ok);
-        if (!ok) break;
         tc_fence_after();
         const int row0 = r0 + box * p.n_box;
-        const int n_valid = min(r1 - row0, (r1 - row0 <= p.tail_rows) ? p.tail_rows : p.n_box);
+        const int n_valid = ok ? min(r1 - row0, (r1 - row0 <= p.tail_rows) ? p.tail_rows : p.n_box) : 0;
         const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)((buf * p.n_mt + mt) * LM_MAX_BOX);
         if (has_rows) {
           for (int c0 = 16 * part; c0 < n_valid; c0 += 16 * n_parts) {
@@ -595,7 +598,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
 #pragma unroll
             for (int j = 0; j < 16; ++j) z[j] = (j < nv) ? __uint_as_float(v[j]) : LM_NEG;
             fold(m0, s0, i0, z, row0 + c0, p.c_t);
-            if (sample) fold_noisy(n0, z, row0 + c0, nv, p.c_t, p.key0, p.key1);
+            if (sample)
+              fold_noisy(n0, rc, z, row0 + c0, nv, p.c_t, p.key0, p.key1, noise + rc.noisy * noise_pitch + c0, p.noise_tok - c0);
           }
         }
         // this accumulator buffer may be overwritten by the products of the next box that uses it
@@ -639,7 +643,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         if (sample) {
           LmNoisy g; g.gs = n0.gs; g.gz = n0.gz; g.gidx = n0.gidx; g.pad = 0;
           *reinterpret_cast<int4*>(p.gpart + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&g);
-          if ((unsigned)(n0.cand_tok - r0) < (unsigned)(r1 - r0)) p.zc[row] = n0.zc;   // this block owns the candidate's token
+          if ((unsigned)(rc.cand_tok - r0) < (unsigned)(r1 - r0)) p.zc[row] = n0.zc;   // this block owns the candidate's token
         }
       }
     }
@@ -928,20 +932,29 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   // 36 rows 54.1 (48.8) / 51.1 (49.5), 49 rows 54.7 (49.6) / 52.7 (50.3), 72 rows 55.4 (50.4) / 55.6 (52.6), 108 rows
   // 57.9 (52.7) / 59.4 (54.1), 144 rows 72.9 (61.2) / 63.0 (56.4), 176 rows 75.8 (62.5) / 72.3 (62.0), 192 rows 75.8 (62.7) /
   // 74.0 (63.4), 252 rows 79.5 (67.9) / 84.9 (72.6); V = 128256: 36 rows 191 (167) / 171 (161); accumulators half empty,
-  // V = 20000, D = 2048, 36 rows 22.3 (21.4) / 23.1 (23.9).  Sampling, whose epilogue is long either way: V = 32000, 36 rows
-  // 60.7 (56.9) / 58.6 (59.5), 64 rows 61.6 (57.5) / 62.0 (61.2), 144 rows 81.8 (70.5) / 75.4 (70.7), 176 rows 84.1 (72.7) /
-  // 81.9 (75.5).
-  const bool tokens_on_m = p.n_box > 192 && (p.n_pad <= (sampling ? 48 : 64) || (p.n_pad > LM_M && p.n_pad <= 176));
+  // V = 20000, D = 2048, 36 rows 22.3 (21.4) / 23.1 (23.9).  Sampling keeps the rows on M: with seven values per row the
+  // epilogue of the other form is the longer one (measured when both had it, V = 32000: 36 rows 55.7 (52.9) / 56.8 (57.3),
+  // 144 rows 77.2 (66.1) / 75.6 (73.1), 176 rows 82.2 (71.3) / 87.4 (85.7)).
+  const bool tokens_on_m = !sampling && p.n_box > 192 && (p.n_pad <= 64 || (p.n_pad > LM_M && p.n_pad <= 176));
+  if (sampling) {
+    // rows that draw a token (row_const), and as many tokens' noise as the table has room for
+    p.n_noisy = phase == LM_ALL ? (a->resample == SPACE_RESAMPLE_PAPER_LITERAL ? p.n_rows : p.B * (a->k + 1))
+                : (phase == LM_TARGETS || a->resample == SPACE_RESAMPLE_PAPER_LITERAL) ? p.n_rows : 0;
+    if (p.n_noisy) {
+      const int room = LM_NOISE_BYTES / 4 / p.n_noisy - 4;
+      p.noise_tok = (room < p.n_box ? room : p.n_box) & ~15;
+    }
+  }
   const size_t budget = 220 * 1024;
   int stages = 0;
   for (p.kbs = p.n_box <= 128 ? 4 : 1; p.kbs >= 1; p.kbs /= 2) {
     stages = LM_MAX_STAGES;
-    while (stages > 1 && LmSmem(tokens_on_m, p.n_pad, p.n_box, stages, p.kbs).total + 1024 > budget) --stages;
+    while (stages > 1 && LmSmem(tokens_on_m, sampling, p.n_noisy, p.noise_tok, p.n_pad, p.n_box, stages, p.kbs).total + 1024 > budget) --stages;
     if (stages >= (p.kbs > 1 ? 3 : 2)) break;
   }
   if (stages < 2) return SPACE_E_UNSUPPORTED;
   p.stages = stages;
-  const LmSmem L(tokens_on_m, p.n_pad, p.n_box, stages, p.kbs);
+  const LmSmem L(tokens_on_m, sampling, p.n_noisy, p.noise_tok, p.n_pad, p.n_box, stages, p.kbs);
   if (L.total + 1024 > 227 * 1024) return SPACE_E_UNSUPPORTED;
   p.eos_id = a->eos_id;
   p.mode = a->mode; p.resample = a->resample;
@@ -969,8 +982,7 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
                                          a->hidden_row_stride * (phase == LM_TARGETS ? a->k + 1 : 1), p.n_pad);
   if (rc != SPACE_OK) return rc;
   const size_t sm = L.total + 1024;
-  auto kernel = tokens_on_m ? (sampling ? lmhead_verify_kernel<true, true> : lmhead_verify_kernel<true, false>)
-                            : (sampling ? lmhead_verify_kernel<false, true> : lmhead_verify_kernel<false, false>);
+  auto kernel = tokens_on_m ? lmhead_verify_kernel<true, false> : sampling ? lmhead_verify_kernel<false, true> : lmhead_verify_kernel<false, false>;
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   {
     ProfScope ps(ctx, SPACE_K_LMHEAD, st);
