@@ -217,14 +217,38 @@ __device__ __forceinline__ bool commit_fits(const CommitParams& p, int L) {
   return L >= 0 && (int64_t)L + (int64_t)(p.k + 1) * (p.k + 1) <= p.s_cap;
 }
 
+// 16-byte pieces in the move of n rows of a sequence, and piece t of it: its bytes and where they go (nullptr: a bad page).
+__device__ __forceinline__ int commit_pieces(const CommitParams& p, int n) { return n * p.H_kv * 2 * (p.d / 8); }
+template <bool PAGED>
+__device__ __forceinline__ uint4* commit_piece(const CommitParams& p, int b, int L, int t, uint4& val) {
+  const int k1 = p.k + 1, vec_per_row = p.d / 8;
+  int r = t;
+  const int v = r % vec_per_row; r /= vec_per_row;
+  const int which = r % 2;       r /= 2;
+  const int h = r % p.H_kv;      r /= p.H_kv;
+  const int g = r + 1;                                // candidate g
+  __nv_bfloat16* base = which ? p.vc : p.kc;
+  if (!PAGED) {
+    base += (int64_t)b * p.sb + (int64_t)h * p.sh;
+    val = *(reinterpret_cast<const uint4*>(base + (int64_t)(L + g * k1) * p.ss) + v);
+    return reinterpret_cast<uint4*>(base + (int64_t)(L + g) * p.ss) + v;
+  }
+  const int64_t so = kv_row_offset(p.page_table, p.pages_per_seq, p.n_pages, p.sb, p.sh, p.ss, b, h, L + g * k1);
+  const int64_t dof = kv_row_offset(p.page_table, p.pages_per_seq, p.n_pages, p.sb, p.sh, p.ss, b, h, L + g);
+  if (so >= 0 && dof >= 0) {
+    val = *(reinterpret_cast<const uint4*>(base + so) + v);
+    return reinterpret_cast<uint4*>(base + dof) + v;
+  }
+  if (p.status && v == 0 && which == 0 && h == 0) atomicOr(p.status + b, SPACE_ST_BAD_PAGE);   // the row stays where it is
+  return nullptr;
+}
+
 // Slice `part` of `nparts` of sequence b's move, by `nthreads` threads (this one is `tid`).
 // All loads of a batch are issued before its stores.
 template <bool PAGED>
 __device__ __forceinline__ void commit_rows_impl(const CommitParams& p, int b, int L, int i_star, int part, int nparts,
                                                  int tid, int nthreads) {
-  const int k1 = p.k + 1;
-  const int vec_per_row = p.d / 8;                      // 16-byte pieces per row
-  const int total = i_star * p.H_kv * 2 * vec_per_row;
+  const int total = commit_pieces(p, i_star);
   const int stride = nparts * nthreads;
   constexpr int U = 8;
   for (int t0 = part * nthreads + tid; t0 < total; t0 += U * stride) {
@@ -235,26 +259,7 @@ __device__ __forceinline__ void commit_rows_impl(const CommitParams& p, int b, i
       const int t = t0 + u * stride;
       dd[u] = nullptr;
       if (t < total) {
-        int r = t;
-        const int v = r % vec_per_row; r /= vec_per_row;
-        const int which = r % 2;       r /= 2;
-        const int h = r % p.H_kv;      r /= p.H_kv;
-        const int g = r + 1;                            // accepted candidate g = 1..i*
-        if (!PAGED) {
-          __nv_bfloat16* base = (which ? p.vc : p.kc) + (int64_t)b * p.sb + (int64_t)h * p.sh;
-          val[u] = *(reinterpret_cast<const uint4*>(base + (int64_t)(L + g * k1) * p.ss) + v);
-          dd[u] = reinterpret_cast<uint4*>(base + (int64_t)(L + g) * p.ss) + v;
-        } else {
-          __nv_bfloat16* base = which ? p.vc : p.kc;
-          const int64_t so = kv_row_offset(p.page_table, p.pages_per_seq, p.n_pages, p.sb, p.sh, p.ss, b, h, L + g * k1);
-          const int64_t dof = kv_row_offset(p.page_table, p.pages_per_seq, p.n_pages, p.sb, p.sh, p.ss, b, h, L + g);
-          if (so >= 0 && dof >= 0) {
-            val[u] = *(reinterpret_cast<const uint4*>(base + so) + v);
-            dd[u] = reinterpret_cast<uint4*>(base + dof) + v;
-          } else if (p.status && v == 0 && which == 0 && h == 0) {
-            atomicOr(p.status + b, SPACE_ST_BAD_PAGE);        // the row stays where it is
-          }
-        }
+        dd[u] = commit_piece<PAGED>(p, b, L, t, val[u]);
       }
     }
 #pragma unroll

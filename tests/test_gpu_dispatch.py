@@ -282,3 +282,33 @@ def test_lmhead_orientations(B, H, mode, V, D, k, Bn):  # noqa: F811
         for n in ("n_accept", "out_tokens", "n_out", "next_cand", "finished"):
             assert np.array_equal(h[n][~excl], r[n][~excl]), (n, again)
         np.testing.assert_allclose(h["next_cand_prob"][~excl], r["next_cand_prob"][~excl], rtol=1e-3)
+
+
+# The single-launch greedy verify moves its slice of the rows to commit while it scans, one 16-byte piece per thread,
+# where that covers them all (not for k = 1 with many heads and a short vocabulary), and after the scan otherwise
+# (also with rows off the 16-byte grid).
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("k,H_kv,d,V,Bn", [(1, 32, 128, 704, 3), (1, 32, 128, 20000, 2), (7, 1, 64, 48, 3), (5, 8, 64, 9000, 2), (5, 8, 64, 9001, 2)])
+def test_commit_under_the_scan(B, H, k, H_kv, d, V, Bn, paged):  # noqa: F811
+    from oracle.commit import commit_step
+    cfg = _small_cfg(k, (100, 400), d=d, H_q=H_kv, H_kv=H_kv, Bn=Bn, V=V, seed=V)
+    x = workloads.make_step_inputs(cfg)
+    for i in range(k):                                       # the first sequence accepts every candidate
+        x["logits"][0, i * (k + 1), x["cand"][0, i]] = workloads.f32_to_bf16_bits(np.float32([40.0]))[0]
+    y = workloads.to_pages(x) if paged else x
+    ctx = H.make_context(cfg, y)
+    ds = H.DeviceStep(cfg, y)
+    ds.verify_commit(ctx)
+    r = verify_step(x["logits"], x["cand"], x["cand_prob"], k, "greedy")
+    assert not _check_verify(ds, r, k).any() and r["n_accept"][0] == k
+    new_len, _, _ = commit_step(x["k_cache"], x["v_cache"], x["kv_len"], r["n_accept"], k)      # (in place)
+    assert np.array_equal(ds.kv_len_out.cpu().numpy(), new_len)
+    for name, dev in (("k_cache", ds.k_cache), ("v_cache", ds.v_cache)):
+        got = H.bf16_to_bits(dev)
+        for b in range(Bn):
+            n = int(new_len[b])
+            if paged:
+                rows = np.concatenate([got[pg] for pg in y["page_table"][b][: -(-n // 128)]], axis=1)
+            else:
+                rows = got[b]
+            assert np.array_equal(rows[:, :n], x[name][b][:, :n]), (name, b)
