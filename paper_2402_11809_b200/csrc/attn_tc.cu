@@ -943,6 +943,25 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
         }
       }
       // ---- end of share: final output or partial ---------------------------
+      const bool whole = sg.n == sg.T;
+      const int item = sg.b * p.H_kv + sg.h;
+      // (Worked out here, and the row sums below, while the last O^T product still runs.)
+      // How this (sequence, head) was cut, {first partial slot, number of partials}: read by the merge kernel
+      // (every piece writes the same pair)
+      int2 cut_d = make_int2(sg.slot, 1);
+      if (sidx == 0 && ok) {
+        if (sg.dfirst >= 0) {
+          cut_d = make_int2(sg.dfirst, sg.dn);
+        } else if (!whole) {
+          const long long W = prefix[p.B];
+          const long long NG = W < p.n_groups ? W : p.n_groups;
+          const long long f0 = (long long)prefix[sg.b] + (long long)sg.h * (sg.T + SHARE_COST) + SHARE_COST;
+          const int g0 = group_of(f0, W, NG);               // group of the first tile
+          cut_d = make_int2(item + g0, group_of(f0 + sg.T - 1, W, NG) - g0 + 1);
+        }
+        if (!p.pieces) p.desc[(size_t)item * p.n_mblocks + mb] = cut_d;
+        if (!whole && sg.tile_at(sg.n - 1) == sg.T - 1) own = item;   // the piece with the pair's last tile; at most one per block
+      }
       // Row sums first, while the last O^T product still runs.  Every thread holds
       // its key's share of ncol rows; a halving butterfly over the warp leaves lane r with
       // the sum over the warp's 32 keys for row col0 + r (fewer than 32 rows: plain sums over
@@ -980,25 +999,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       tc_fence_after();
       soft_sync();
       if (sidx == 0) TL(10);
-      const bool whole = sg.n == sg.T;
-      const int item = sg.b * p.H_kv + sg.h;
       float* pslot = p.part + ((size_t)sg.slot * p.n_mblocks + mb) * (ROWS * (DH + 2));
-      // How this (sequence, head) was cut, {first partial slot, number of partials}: read by the merge kernel
-      // (every piece writes the same pair)
-      int2 cut_d = make_int2(sg.slot, 1);
-      if (sidx == 0 && ok) {
-        if (sg.dfirst >= 0) {
-          cut_d = make_int2(sg.dfirst, sg.dn);
-        } else if (!whole) {
-          const long long W = prefix[p.B];
-          const long long NG = W < p.n_groups ? W : p.n_groups;
-          const long long f0 = (long long)prefix[sg.b] + (long long)sg.h * (sg.T + SHARE_COST) + SHARE_COST;
-          const int g0 = group_of(f0, W, NG);               // group of the first tile
-          cut_d = make_int2(item + g0, group_of(f0 + sg.T - 1, W, NG) - g0 + 1);
-        }
-        if (!p.pieces) p.desc[(size_t)item * p.n_mblocks + mb] = cut_d;
-        if (!whole && sg.tile_at(sg.n - 1) == sg.T - 1) own = item;   // the piece with the pair's last tile; at most one per block
-      }
       // Where a piece's partial goes: shared memory of the cluster (the P buffer is idle now), or its slot
       // in global memory.
       const bool to_smem = clustered && !whole;
@@ -1024,6 +1025,21 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       // element (block row i0, head h*G, dim kl) of this sequence; one block row further = H_q*DH
       const size_t out_base = (((size_t)sg.b * p.n_q + i0) * p.H_q + (size_t)sg.h * p.G) * DH + kl;
       const size_t out_row = (size_t)p.H_q * DH;
+      if (to_smem) {
+        // (a call ends on this: all reads of TMEM in flight together.  As the rule for the other two destinations it
+        // gained nothing, a store to global memory takes the registers)
+        uint32_t o[NP][8], o2[NP][8];
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+          tmem_ld8(TM_O + lane_addr + col0 + j * 8, o[j]);
+          tmem_ld8(TM_O + lane_addr + 64 + col0 + j * 8, o2[j]);
+        }
+        tmem_wait_ld();
+        float* dst = reinterpret_cast<float*>(sm + S::P_OFF) + col0 * DH + kl;
+#pragma unroll
+        for (int x = 0; x < ncol; ++x)
+          if (col0 + x < m_valid && d_ok) dst[x * DH] = __uint_as_float(o[x >> 3][x & 7]) + __uint_as_float(o2[x >> 3][x & 7]);
+      } else {
 #pragma unroll 2
       for (int j = 0; j < NP; ++j) {
         uint32_t o[8], o2[8];
@@ -1053,17 +1069,13 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
               if (q0 + e < m_valid && d_ok)
                 reinterpret_cast<__nv_bfloat16*>(p.out)[off[e]] = __float2bfloat16_rn(__uint_as_float(o[e]) * rr[e]);
           }
-        } else if (to_smem) {
-          float* dst = reinterpret_cast<float*>(sm + S::P_OFF) + q0 * DH + kl;
-#pragma unroll
-          for (int e = 0; e < 8; ++e)
-            if (q0 + e < m_valid && d_ok) dst[e * DH] = __uint_as_float(o[e]);
         } else {
           float* dst = pslot + (size_t)q0 * DH + kl;
 #pragma unroll
           for (int e = 0; e < 8; ++e)
             if (q0 + e < m_valid && d_ok) dst[e * DH] = __uint_as_float(o[e]);
         }
+      }
       }
       tc_fence_before();
       soft_sync();                                          // scratch, fq and mref are reused by the next share
