@@ -48,7 +48,6 @@ constexpr int LM_L2_AHEAD = 8;              // slices of W a block asks L2 for b
 constexpr float LM_NEG = -3.0e38f;          // "no logit yet": finite, so that differences never give NaN
 constexpr int LM_MAX_N = 256;               // block rows of the whole batch, padded to 16
 constexpr int LM_TOK = 128;                 // tokens per accumulator with the tokens on M
-constexpr int LM_NOISE_BYTES = 24 * 1024;   // noise table of a box (sampling), at most
 constexpr int LM_XP_PITCH = 36;             // floats per row of a warp's transposing buffer (8 rows of 32 tokens)
 // Which block rows a launch projects: all of them, the target rows of every sequence (row b(k+1)+t), or
 // the mask rows of every sequence's group i* (row bk+o-1; i* is the launch before's result).
@@ -936,16 +935,23 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   // epilogue of the other form is the longer one (measured when both had it, V = 32000: 36 rows 55.7 (52.9) / 56.8 (57.3),
   // 144 rows 77.2 (66.1) / 75.6 (73.1), 176 rows 82.2 (71.3) / 87.4 (85.7)).
   const bool tokens_on_m = !sampling && p.n_box > 192 && (p.n_pad <= 64 || (p.n_pad > LM_M && p.n_pad <= 176));
+  const size_t budget = 220 * 1024;
   if (sampling) {
     // rows that draw a token (row_const), and as many tokens' noise as the table has room for
     p.n_noisy = phase == LM_ALL ? (a->resample == SPACE_RESAMPLE_PAPER_LITERAL ? p.n_rows : p.B * (a->k + 1))
                 : (phase == LM_TARGETS || a->resample == SPACE_RESAMPLE_PAPER_LITERAL) ? p.n_rows : 0;
     if (p.n_noisy) {
-      const int room = LM_NOISE_BYTES / 4 / p.n_noisy - 4;
-      p.noise_tok = (room < p.n_box ? room : p.n_box) & ~15;
+      // The table may take what a pipeline of four stages leaves, of three where the rows need two accumulators and a
+      // stage is large (24 KB / this, us per call in bursts, D = 2048, V = 128256, 160 rows 146.7 / 134.9; D = 4096, V = 32000,
+      // 160 rows 71.1 / 68.0, 208 rows 74.1 / 71.0; with two stages 208 rows 88.4, with three 16 x 36 rows, 96 and 80 of them
+      // at a time, 363 against 358).
+      const int keep = p.n_pad > LM_M ? 3 : 4;
+      int64_t rest = (int64_t)budget - 1024 - LmSmem(false, true, 0, 0, p.n_pad, p.n_box, keep, 1).total;
+      if (p.n_box <= 128 && rest > 24 * 1024) rest = 24 * 1024;        // (stages of several slices, see below)
+      const int64_t room = rest / 4 / p.n_noisy - 4;
+      p.noise_tok = room < 16 ? 0 : (int)(room < p.n_box ? room : p.n_box) & ~15;
     }
   }
-  const size_t budget = 220 * 1024;
   int stages = 0;
   for (p.kbs = p.n_box <= 128 ? 4 : 1; p.kbs >= 1; p.kbs /= 2) {
     stages = LM_MAX_STAGES;
