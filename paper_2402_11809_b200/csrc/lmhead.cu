@@ -935,17 +935,21 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   // epilogue of the other form is the longer one (measured when both had it, V = 32000: 36 rows 55.7 (52.9) / 56.8 (57.3),
   // 144 rows 77.2 (66.1) / 75.6 (73.1), 176 rows 82.2 (71.3) / 87.4 (85.7)).
   const bool tokens_on_m = !sampling && p.n_box > 192 && (p.n_pad <= 64 || (p.n_pad > LM_M && p.n_pad <= 176));
-  const size_t budget = 220 * 1024;
+  // (all that a block may have: with 96 rows it holds five stages, with 220 KB four; 16 x 36 rows of V = 128256, greedy,
+  // 350 -> 343 us in bursts, 112 rows of V = 32000 52.8 -> 51.4, 144 sampling 66.7 -> 64.3, 72 of V = 5000 17.8 -> 16.8)
+  const size_t budget = 227 * 1024;
   if (sampling) {
     // rows that draw a token (row_const), and as many tokens' noise as the table has room for
     p.n_noisy = phase == LM_ALL ? (a->resample == SPACE_RESAMPLE_PAPER_LITERAL ? p.n_rows : p.B * (a->k + 1))
                 : (phase == LM_TARGETS || a->resample == SPACE_RESAMPLE_PAPER_LITERAL) ? p.n_rows : 0;
     if (p.n_noisy) {
-      // The table may take what a pipeline of four stages leaves, of three where the rows need two accumulators and a
-      // stage is large (24 KB / this, us per call in bursts, D = 2048, V = 128256, 160 rows 146.7 / 134.9; D = 4096, V = 32000,
-      // 160 rows 71.1 / 68.0, 208 rows 74.1 / 71.0; with two stages 208 rows 88.4, with three 16 x 36 rows, 96 and 80 of them
-      // at a time, 363 against 358).
-      const int keep = p.n_pad > LM_M ? 3 : 4;
+      // The table may take what a pipeline of a few stages leaves: five where they fit with it or every row draws a token
+      // (the folds then work the noise out without waste), four up to 128 rows, three where the rows need two
+      // accumulators and a stage is large.  24 KB / this, us per call in bursts: D = 2048, V = 128256, 160 rows 146.7 / 134.9;
+      // D = 4096, V = 32000, 160 rows 71.1 / 68.0, 208 rows 74.1 / 71.0.  Other numbers of stages: 208 rows, two 88.4; 80
+      // rows of V = 128256 (D = 2048), four / five 94.5 / 92.5; 16 x 36 rows, 96 and 80 of them at a time, three / four /
+      // five 363 / 357 / 353; 108 rows of V = 32000, four / five 56.5 / 58.7.
+      const int keep = p.n_pad > LM_M ? 3 : (p.n_pad <= 80 || (p.n_pad <= 96 && phase != LM_ALL)) ? 5 : 4;
       int64_t rest = (int64_t)budget - 1024 - LmSmem(false, true, 0, 0, p.n_pad, p.n_box, keep, 1).total;
       if (p.n_box <= 128 && rest > 24 * 1024) rest = 24 * 1024;        // (stages of several slices, see below)
       const int64_t room = rest / 4 / p.n_noisy - 4;
