@@ -44,12 +44,16 @@ constexpr int FILT_GROUP = 2;                            // threads per group wh
 constexpr int FILT_GROUPS = FILT_THREADS / FILT_GROUP;
 constexpr int FILT_U = 4;                                // vectors per thread and sweep
 constexpr int FILT_BUF = 4096;                           // keys a segment may collect
-// A call with at most this many block rows and bytes of logits takes one launch over all block rows.  Measured, us
-// per call (graph replay, top-10), two launches / one: 4 x 9 rows of 32000 (2 MB) 17.6 / 12.5, 5 x 25 rows of 50257
-// (13 MB) 22.5 / 21.1, 24 x 9 rows of 50257 (22 MB) 27.5 / 25.0, 8 x 9 rows of 128256 (18 MB) 23.2 / 18.2, 16 x 9
-// (37 MB) 25.2 / 27.0: the two meet between 22 and 37 MB, above the line.
-constexpr int FILT_BOTH_ROWS = 256;
-constexpr int64_t FILT_BOTH_BYTES = 16ll << 20;
+// Which calls take one launch over all block rows: what it saves is a launch and a second search in a chain, what it
+// costs is reading the rows that two launches skip, and more blocks than fit at once.  So: few bytes of logits, or few
+// rows and not many bytes.  Measured, us per call (graph replay, other input every call), two launches / one, with 2 heads
+// of 64 to commit (32 of 128): few rows: 2 x 25 of 128256 f32 (26 MB, top-30) 29.5 / 23.4 (29.1 / 25.4), 4 x 16 of 128256 bf16
+// (16 MB, top-20) 26.6 / 19.1 (27.0 / 21.5), 8 x 9 (18 MB) 23.7 / 18.4 (23.8 / 20.8), 3 x 36 (28 MB) 23.9 / 21.5 (24.4 / 23.8);
+// past them: 2 x 64 (33 MB) 24.0 / 27.5, 16 x 9 (37 MB) 25.7 / 27.2, 10 x 16 of 37201 f32 (24 MB) 26.0 / 34.2, 6 x 36 of 50257
+// (22 MB) 24.8 / 26.2, but 24 x 9 of 50257 (22 MB) 28.2 / 25.2; few bytes: 4 x 9 of 32000 (2 MB) 17.6 / 12.5, 28 x 9 (16 MB)
+// 20.7 / 18.7, 5 x 49 (16 MB) 19.4 / 19.5, 10 x 16 of 50257 (16 MB, top-25) 27.3 / 28.5.
+constexpr int FILT_BOTH_ROWS = 256, FILT_FEW_ROWS = 110;
+constexpr int64_t FILT_BOTH_BYTES = 16ll << 20, FILT_FEW_ROWS_BYTES = 30ll << 20;
 enum { PHASE_TARGETS = 0, PHASE_MASKS = 1, PHASE_BOTH = 2 };
 
 struct FiltParams {
@@ -516,7 +520,9 @@ int launch_verify_filtered(space_ctx* ctx, const space_verify_args* a, const spa
   const int esz = a->logits_dtype == SPACE_DTYPE_F32 ? 4 : 2;
   const bool aligned = ((uintptr_t)a->logits % 16 == 0) && ((a->logits_row_stride * esz) % 16 == 0);
   if (cm) fill_commit_params(ctx, cm, &p.cm);
-  const bool both = (int64_t)a->batch * p.n_q <= FILT_BOTH_ROWS && (int64_t)a->batch * p.n_q * a->vocab * esz <= FILT_BOTH_BYTES;
+  const int64_t block_rows = (int64_t)a->batch * p.n_q;
+  const bool both = block_rows <= FILT_BOTH_ROWS &&
+                    block_rows * a->vocab * esz <= (block_rows <= FILT_FEW_ROWS ? FILT_FEW_ROWS_BYTES : FILT_BOTH_BYTES);
   // the commit rides along, except where one block would have more than 32 KB of rows to move: a launch of its
   // own is faster then (two sequences, one launch; us per step, riding / own: 16 KB 22.1 / 23.7, 32 KB 25.8 / 26.1,
   // 57 KB 29.8 / 28.5)

@@ -312,3 +312,27 @@ def test_commit_under_the_scan(B, H, k, H_kv, d, V, Bn, paged):  # noqa: F811
             else:
                 rows = got[b]
             assert np.array_equal(rows[:, :n], x[name][b][:, :n]), (name, b)
+
+
+# Filtered sampling on both sides of the line between one launch over all block rows and two (few rows: 30 MB of
+# logits, 110 rows; more rows: 16 MB), with the commit on board: the same decisions and cache either way.
+@pytest.mark.parametrize("Bn,k,V,dtype,launches", [(3, 5, 128256, "bf16", 1), (2, 4, 128256, "f32", 1), (4, 5, 64064, "bf16", 2),
+                                                  (3, 5, 146000, "bf16", 2), (7, 3, 70001, "bf16", 1)])
+def test_filtered_one_launch_or_two(B, H, Bn, k, V, dtype, launches):  # noqa: F811
+    from oracle.commit import commit_step
+    cfg = workloads.resolve("sampling64", B=Bn, H_q=2, H_kv=2, d=64, L=(5, 200), k=k, V=V, logits_dtype=dtype, seed=V % 89)
+    x = workloads.make_step_inputs(cfg)
+    ctx = H.make_context(cfg, x)
+    ds = H.DeviceStep(cfg, x)
+    v = ctx.verify_args(ds.logits, ds.cand, ds.cand_prob, ds.kv_len, ds.n_accept, ds.out_tokens, ds.n_out, ds.next_cand,
+                        ds.next_cand_prob, ds.finished, k, mode=B.MODE_SAMPLE, temperature=0.9, seed=3, seq_id=ds.seq_id,
+                        status=ds.status, top_k=10, top_p=0.95)
+    n0 = ctx.launch_count
+    ctx.space_verify_commit(v, ctx.commit_args(ds.k_cache, ds.v_cache, ds.n_accept, ds.kv_len, k, kv_len_out=ds.kv_len_out))
+    assert ctx.launch_count - n0 == launches
+    r = verify_step(x["logits"], x["cand"], x["cand_prob"], k, "sample", temperature=0.9, seed=3, seq_id=x["seq_id"],
+                    kv_len=x["kv_len"], top_k=10, top_p=0.95)
+    assert not _check_verify(ds, r, k, sample=True).any()
+    new_len, _, _ = commit_step(x["k_cache"], x["v_cache"], x["kv_len"], r["n_accept"], k)       # (in place)
+    assert np.array_equal(ds.kv_len_out.cpu().numpy(), new_len)
+    assert np.array_equal(H.bf16_to_bits(ds.k_cache), x["k_cache"]) and np.array_equal(H.bf16_to_bits(ds.v_cache), x["v_cache"])
