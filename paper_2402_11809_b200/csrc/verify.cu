@@ -617,8 +617,10 @@ __device__ unsigned long long g_timeline_verify[4096 * 8];
 
 // PAGED: the commit on board goes through a page table (a build of its own: the table look-ups are
 // not compiled into the contiguous form, whose addressing sits in the critical path).
-template <typename T, bool ALIGNED, bool PAGED = false>
-__global__ void __launch_bounds__(SPACE_VERIFY_THREADS)
+// EARLY: the rows to commit are fetched under the scan.  It costs registers, that is the third block per SM, so only
+// calls whose blocks need no third one take it (see launch_fused).
+template <typename T, bool ALIGNED, bool PAGED = false, bool EARLY = false>
+__global__ void __launch_bounds__(SPACE_VERIFY_THREADS, EARLY ? 2 : 3)
 verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
   TLV(0);
   pdl_launch_dependents();
@@ -634,17 +636,15 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
   if (p.do_commit) Lc = p.cm.kv_len[b];                     // in flight during the scan
   // (the candidates too: the block that finishes the sequence must not start a memory round trip for them)
   const int my_cand = threadIdx.x < p.k ? p.cand[b * p.k + threadIdx.x] : 0;
-  // The block's slice of the rows to commit (below), where one 16-byte piece per thread covers it: fetched under the
-  // scan, so that only stores are left when the block is counted in (one 7B-shaped sequence's step 19.3 -> 18.95 us;
-  // rows off the 16-byte grid, whose scan has no registers to spare, lost 7 % by it).
-  const int cm_at = (row_i * p.n_chunks + ch) * (SPACE_VERIFY_THREADS - 32) + (int)threadIdx.x - 32;
-  const int cm_total = p.do_commit ? commit_pieces(p.cm, p.k) : 0;
-  const bool cm_early = ALIGNED && cm_total <= p.n_q * p.n_chunks * (SPACE_VERIFY_THREADS - 32);
+  // EARLY: the block's slice of the rows to commit (below), one 16-byte piece per thread, fetched under the scan, so that
+  // only stores are left when the block is counted in (one 7B-shaped sequence's step 19.3 -> 18.95 us; rows off the
+  // 16-byte grid, whose scan has no registers to spare, lost 7 % by it).
   uint4 cm_val = make_uint4(0u, 0u, 0u, 0u);
   uint4* cm_dst = nullptr;
   Stat st = scan_chunk<T, ALIGNED, false, STAT_SUM>(row, begin, end, C1, -1, 0, 0, 0, 0, 0, [&] {
-    if (cm_early && threadIdx.x >= 32 && cm_at < cm_total && commit_fits(p.cm, Lc))
-      cm_dst = commit_piece<PAGED>(p.cm, b, Lc, cm_at, cm_val);
+    const int at = (row_i * p.n_chunks + ch) * (SPACE_VERIFY_THREADS - 32) + (int)threadIdx.x - 32;
+    if (EARLY && threadIdx.x >= 32 && at < commit_pieces(p.cm, p.k) && commit_fits(p.cm, Lc))
+      cm_dst = commit_piece<PAGED>(p.cm, b, Lc, at, cm_val);
   });
 #ifdef SPACE_TIMELINE
   if (st.m != 12345.f) TLV(2);                              // (a use of the result: the stamp follows the loads)
@@ -681,9 +681,9 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
       if (last) p.counter_a[b] = 0;                         // ready for the next launch
       sh_last = last;
     }
-  } else if (cm_early) {
+  } else if (EARLY) {
     if (cm_dst) *cm_dst = cm_val;
-  } else if (commit_fits(p.cm, Lc)) {
+  } else if (p.do_commit && commit_fits(p.cm, Lc)) {
     // KV commit on board: which candidates are accepted is known only to the last block, at the very
     // end, so every block moves its slice of ALL k candidate rows (warp 0 has the arrival to make, whose
     // release would wait for its stores).  Rows L+1 .. L+i* end up exactly as the plain commit leaves
@@ -753,10 +753,16 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
 template <typename T, bool ALIGNED>
 void launch_fused(space_ctx* ctx, const VerifyParams& p, cudaStream_t st) {
   ProfScope ps(ctx, SPACE_K_VERIFY_TARGET, st);
-  if (p.do_commit && p.cm.page_table)
-    launch_pdl(verify_fused_kernel<T, ALIGNED, true>, dim3(p.n_chunks, p.n_q, p.B), dim3(SPACE_VERIFY_THREADS), 0, st, p, ctx->vfused);
-  else
-  launch_pdl(verify_fused_kernel<T, ALIGNED>, dim3(p.n_chunks, p.n_q, p.B), dim3(SPACE_VERIFY_THREADS), 0, st, p, ctx->vfused);
+  const dim3 grid(p.n_chunks, p.n_q, p.B), block(SPACE_VERIFY_THREADS);
+  const int per_seq = p.n_q * p.n_chunks;
+  // EARLY where two blocks per SM hold the launch and a piece per thread all rows to commit.  (With the registers it
+  // takes and no such limit, 24 x 36 rows of 32000 took 20.6 us a call instead of 18.0, 8 x 49 14.0 instead of 10.6.)
+  const bool early = ALIGNED && p.do_commit && per_seq * p.B <= 2 * ctx->sm_count &&
+                     p.k * p.cm.H_kv * 2 * (p.cm.d / 8) <= per_seq * (SPACE_VERIFY_THREADS - 32);
+  const bool paged = p.do_commit && p.cm.page_table;
+  auto kernel = early ? (paged ? verify_fused_kernel<T, ALIGNED, true, ALIGNED> : verify_fused_kernel<T, ALIGNED, false, ALIGNED>)
+                      : (paged ? verify_fused_kernel<T, ALIGNED, true> : verify_fused_kernel<T, ALIGNED>);
+  launch_pdl(kernel, grid, block, 0, st, p, ctx->vfused);
 }
 
 template <typename T, bool ALIGNED>
