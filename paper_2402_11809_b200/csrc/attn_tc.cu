@@ -1303,8 +1303,8 @@ int launch_attn_tensor(space_ctx* ctx, const space_attn_args* a, const uint64_t*
   memcpy(&p.tm_k, ctx->tm_k, sizeof(CUtensorMap));
   memcpy(&p.tm_v, ctx->tm_v, sizeof(CUtensorMap));
 
-  // Clustered cut when every (sequence, kv head) gets a cluster of its own.  The grid fills the chip
-  // all the same: the kernel falls back to a cut over all of it when the lengths are too unequal.
+  // Clustered cut when every (sequence, kv head) gets a cluster of its own.  The grid fills the chip all the same where
+  // the kernel may have to fall back to a cut over all of it, for lengths too unequal (see plan_clusters).
   int n_ctas = pl.n_ctas, size = 1, n_clusters = 0;
   auto ask = [&](int sz, int* fit) {
     const int n = ctx->sm_count / sz * sz;
