@@ -70,6 +70,7 @@ struct LmParams {
   int n_box;                  // rows of the first tensor map's box (N of its products)
   int tail_rows;              // rows of the second tensor map's box
   int kbs;                    // 64-element slices of the hidden dimension per stage
+  int backwards;              // a box's stages are taken from the hidden dimension's end (see launch_group)
   int n_noisy, noise_tok;     // sampling: rows that draw a token, tokens of a box whose noise is tabulated (a multiple of 16)
   int eos_id;
   int mode, resample;         // SPACE_MODE_*, SPACE_RESAMPLE_*
@@ -337,9 +338,10 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
     // first slices of W meanwhile (a request to the point of coherence, so whatever the kernel before still
     // writes is what the loads will see).  V = 32000, D = 4096, 36 rows: 51.3 -> 49.8 us per call in bursts, 53.5 ->
     // 53.2 in a steady loop, where the power cap sets the pace.
+    // (Backwards, the launch before has just read the first slices.)
     const int first = (int)(((long long)p.V * blockIdx.x) / gridDim.x) & ~15;
     const uint64_t pol = l2_evict_first_policy();
-    for (int kb = 0; kb < min(LM_L2_AHEAD, (p.D + LM_KB - 1) / LM_KB); ++kb)
+    for (int kb = 0; !p.backwards && kb < min(LM_L2_AHEAD, (p.D + LM_KB - 1) / LM_KB); ++kb)
       tma_prefetch_l2_4d(&p.tm_w, kb * LM_KB, first, 0, 0, pol);
   }
   tc_fence_before();
@@ -357,6 +359,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
   const int nb = (r1 - r0 + p.n_box - 1) / p.n_box;
   const int KB = (p.D + LM_KB - 1) / LM_KB;
   const int kbs = p.kbs;
+  const int KI = (KB + kbs - 1) / kbs;                     // stages per box
+  auto first_slice = [&](int ki) { return (p.backwards ? KI - 1 - ki : ki) * kbs; };   // of a box's ki-th stage
   const int n_bufs = p.n_mt == 1 ? 2 : 1;                  // accumulator buffers of n_mt x 256 columns
   const int acc_cols = TM ? p.n_mt * LM_TOK : 0;           // (tokens on M: columns of one of a buffer's two accumulators)
 
@@ -372,7 +376,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         const bool tail = r1 - row0 <= p.tail_rows;          // the remaining rows fit the small box
         const CUtensorMap* tm = tail ? &p.tm_wt : &p.tm_w;
         const uint32_t slice_bytes = (uint32_t)(tail ? p.tail_rows : p.n_box) * LM_KB * 2 + L.a_bytes;
-        for (int kb0 = 0; kb0 < KB; kb0 += kbs, ++it) {
+        for (int ki = 0; ki < KI; ++ki, ++it) {
+          const int kb0 = first_slice(ki);
           // stage `it`: the W tiles and the hidden tiles of its slices
           if (it >= (uint32_t)S) ok = mbar_wait(LBAR(B_EMPTY + s), empty_phase, abort_flag, p.err, 1);
           if (!ok) break;
@@ -407,7 +412,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         if (box >= n_bufs) ok = mbar_wait(LBAR(B_ACCEMPTY + buf), (n_bufs == 2 ? (box >> 1) - 1 : box - 1) & 1, abort_flag, p.err, 2);
         if (!ok) break;
         tc_fence_after();
-        for (int kb0 = 0; kb0 < KB; kb0 += kbs) {
+        for (int ki = 0; ki < KI; ++ki) {
+          const int kb0 = first_slice(ki);
           const int nk = min(kbs, KB - kb0);
           ok = mbar_wait(LBAR(B_FULL + s), full_phase, abort_flag, p.err, 3);
           if (!ok) break;
@@ -421,7 +427,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
                 const uint32_t acc = tmem + (uint32_t)((buf * 2 + tt) * acc_cols);
 #pragma unroll
                 for (int kk = 0; kk < LM_KB / 16; ++kk)
-                  mma_ss(acc, wd + (uint64_t)(tt * (16384 >> 4) + kk * 2), hd + (uint64_t)(kk * 2), idesc, (kb0 | j | kk) ? 1u : 0u);
+                  mma_ss(acc, wd + (uint64_t)(tt * (16384 >> 4) + kk * 2), hd + (uint64_t)(kk * 2), idesc, (ki | j | kk) ? 1u : 0u);
               }
             } else for (int mt = 0; mt < p.n_mt; ++mt) {
               // block rows 128*mt .. of the hidden tile (8-row groups are contiguous: 16 KB further on)
@@ -429,7 +435,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
               const uint32_t acc = tmem + (uint32_t)((buf * p.n_mt + mt) * LM_MAX_BOX);
 #pragma unroll
               for (int kk = 0; kk < LM_KB / 16; ++kk)      // 32 bytes per 16 elements inside the swizzled row
-                mma_ss(acc, hd + (uint64_t)(kk * 2), wd + (uint64_t)(kk * 2), idesc, (kb0 | j | kk) ? 1u : 0u);
+                mma_ss(acc, hd + (uint64_t)(kk * 2), wd + (uint64_t)(kk * 2), idesc, (ki | j | kk) ? 1u : 0u);
             }
           }
           tc_commit(LBAR(B_EMPTY + s));
@@ -956,6 +962,12 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
       p.noise_tok = room < 16 ? 0 : (int)(room < p.n_box ? room : p.n_box) & ~15;
     }
   }
+  // Where a range is one box, the mask rows' pass takes the slices from the end: those of the target rows' pass that are
+  // still in L2 (us per call in bursts (steady loop), forwards / backwards: 16 x 36 rows, V = 32000, D = 4096 107.8 (116.8) /
+  // 104.9 (112.7), D = 2048, sampling, 76.2 (77.5) / 72.9 (73.0)).  With more boxes the stream itself is slower that way
+  // (V = 128256, D = 4096 359 / 375), and the last box alone first gains nothing that lasts (359 / 360; V = 64000 186.5 / 184.3,
+  // V = 80000, D = 2048 130.3 / 132.7).
+  p.backwards = phase == LM_MASKS && max_len <= p.n_box;
   int stages = 0;
   for (p.kbs = p.n_box <= 128 ? 4 : 1; p.kbs >= 1; p.kbs /= 2) {
     stages = LM_MAX_STAGES;

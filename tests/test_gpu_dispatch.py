@@ -66,10 +66,11 @@ def test_filtered_sampling_on_sorted_and_tied_rows(B, H, Bn, k, V, top_k, dtype)
 
 
 # Wide batches by phase (target rows, then the mask rows of group i*): eight rows per sequence at k = 7, one mask
-# row at k = 1, several groups of sequences, D and V off every tile, and the last sequence's mask rows at the end
-# of the hidden states.
+# row at k = 1, several groups of sequences, D and V off every tile, one box per range and several, a last stage of fewer
+# slices taken first, and the last sequence's mask rows at the end of the hidden states.
 @pytest.mark.parametrize("mode", ["greedy", "residual_pointmass", "paper_literal"])
-@pytest.mark.parametrize("V,D,k,Bn", [(3001, 200, 7, 16), (131075, 264, 1, 67), (20000, 128, 5, 16), (129, 64, 5, 21), (40003, 136, 6, 18)])
+@pytest.mark.parametrize("V,D,k,Bn", [(3001, 200, 7, 16), (131075, 264, 1, 67), (20000, 128, 5, 16), (129, 64, 5, 21), (40003, 136, 6, 18),
+                                       (9001, 328, 7, 16)])
 def test_lmhead_by_phase(B, H, mode, V, D, k, Bn):  # noqa: F811
     cfg = workloads.resolve_lmhead("lmhead_tiny", V=V, D=D, k=k, B=Bn, p_accept=(0.5, 1.0))
     x = workloads.make_lmhead_inputs(cfg)
