@@ -977,7 +977,7 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   if (stages < 2) return SPACE_E_UNSUPPORTED;
   p.stages = stages;
   const LmSmem L(tokens_on_m, sampling, p.n_noisy, p.noise_tok, p.n_pad, p.n_box, stages, p.kbs);
-  if (L.total + 1024 > 227 * 1024) return SPACE_E_UNSUPPORTED;
+  if (L.total + 1024 > budget) return SPACE_E_UNSUPPORTED;
   p.eos_id = a->eos_id;
   p.mode = a->mode; p.resample = a->resample;
   p.c_t = LOG2E / (a->mode == SPACE_MODE_SAMPLE ? a->temperature : 1.0f);
@@ -1005,7 +1005,9 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   if (rc != SPACE_OK) return rc;
   const size_t sm = L.total + 1024;
   auto kernel = tokens_on_m ? lmhead_verify_kernel<true, false> : sampling ? lmhead_verify_kernel<false, true> : lmhead_verify_kernel<false, false>;
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  // (all that a block may have, whatever this call needs: the limit is the kernel's, and a thread with a context of its
+  // own must not find it lowered between this and its launch)
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget);
   {
     ProfScope ps(ctx, SPACE_K_LMHEAD, st);
     launch_pdl(kernel, dim3(grid), dim3(LM_THREADS), sm, st, p);
