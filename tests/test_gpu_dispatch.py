@@ -4,7 +4,8 @@ import numpy as np
 import pytest
 import torch
 
-from oracle.attention import attention_step
+from oracle.attention import attention_head, attention_step
+from oracle.bf16 import bf16_bits_to_f64
 from oracle.lmhead import lmhead_verify_step
 from oracle.verify import verify_step
 from paper_2402_11809_b200 import workloads
@@ -212,35 +213,56 @@ def test_host_step_transfers(B, H, where, V):  # noqa: F811
         assert np.array_equal(h["k_cache"].numpy().view(np.uint16)[1], x["k_cache"][1])
 
 
+def _growing_keys(x, G, per_tile):
+    """Adds t * (a multiple of the signs of block row 0's query) to the keys of tile t of every kv head, so that the scores
+    of that row grow by per_tile binary orders of magnitude from tile to tile.  Returns the least amount by which a tile
+    exceeds the first key of one at least two tiles before it."""
+    kf, qf = (bf16_bits_to_f64(x[n]).astype(np.float32) for n in ("k_cache", "q"))
+    tile = np.arange(kf.shape[2]) // 128
+    log2e, least = float(np.log2(np.e)), np.inf
+    for b in range(kf.shape[0]):
+        for h in range(kf.shape[1]):
+            q = qf[b, 0, h * G]
+            kf[b, h] += tile[:, None] * np.sign(q) * np.float32(per_tile / (log2e * x["scale"] * np.abs(q).sum()))
+    x["k_cache"] = workloads.f32_to_bf16_bits(kf)
+    kf = bf16_bits_to_f64(x["k_cache"])
+    for b in range(kf.shape[0]):
+        L = int(x["kv_len"][b])                              # (cached keys: every row sees them)
+        for h in range(kf.shape[1]):
+            s = kf[b, h, :L] @ qf[b, 0, h * G].astype(np.float64) * (x["scale"] * log2e)
+            top = [s[t:t + 128].max() for t in range(0, L, 128)]
+            least = min([least] + [top[t] - s[u * 128] for t in range(2, len(top)) for u in range(t - 1)])
+    return least
+
+
 # Every width of the transposed attention kernel (16, 32, 48, 64 padded query rows) with several tiles per block, so
 # that its rings of scores, P and tiles come round, clustered (two sequences) and in the flat cut (more pairs than
-# SMs); keys whose scores grow along the sequence move the references in the middle of a share.
+# SMs).  With keys whose scores grow along the sequence every share has a tile that exceeds its reference by more than
+# 2^60, and the references move in its middle (the rows kernel takes the same inputs).
 @pytest.mark.parametrize("paged", [False, True])
-@pytest.mark.parametrize("ramp", [0.0, 6.0])
+@pytest.mark.parametrize("per_tile", [0, 40])
 @pytest.mark.parametrize("k,G,d,Bn,H_kv", [(1, 1, 64, 2, 12), (2, 1, 128, 40, 4), (3, 1, 128, 2, 12), (3, 2, 64, 2, 12),
                                            (4, 1, 128, 2, 12), (5, 1, 128, 2, 12), (5, 1, 64, 40, 4), (7, 1, 128, 2, 12),
                                            (7, 1, 64, 2, 12), (6, 1, 128, 40, 4)])
-def test_transposed_kernel_widths(B, H, k, G, d, Bn, H_kv, ramp, paged):  # noqa: F811
+def test_transposed_kernel_widths(B, H, k, G, d, Bn, H_kv, per_tile, paged):  # noqa: F811
     cfg = _small_cfg(k, (700, 3100 if Bn == 2 else 900), d=d, H_q=H_kv * G, H_kv=H_kv, Bn=Bn, V=64, seed=k + d)
     x = workloads.make_step_inputs(cfg)
-    if ramp:
-        from oracle.bf16 import bf16_bits_to_f64
-        kf, qf = (bf16_bits_to_f64(x[n]).astype(np.float32) for n in ("k_cache", "q"))
-        up = np.linspace(0.0, ramp, kf.shape[2], dtype=np.float32)[:, None]
-        for h in range(H_kv):
-            kf[:, h] += up * np.sign(qf[:, 0, h * G])[:, None, :]
-        x["k_cache"] = workloads.f32_to_bf16_bits(kf)
+    if per_tile:
+        assert _growing_keys(x, G, per_tile) > 60
+        # two sequences: at most 148 // 24 = 6 pieces per pair, taking every sixth tile; otherwise a block's share is
+        # longer than a pair
+        assert x["kv_len"].max() // 128 > (7 if Bn == 2 else 5)
     y = workloads.to_pages(x) if paged else x
     ctx = H.make_context(cfg, y)
-    ds = H.DeviceStep(cfg, y)
-    ds.attn(ctx)
-    assert not ds.status.any()
-    got = ds.out.cpu().numpy().astype(np.float64)
-    from oracle.attention import attention_head
-    for b in (0, Bn - 1):                                    # first and last pairs of the cut
-        for h in (0, H_kv * G - 1):
-            ref, _ = attention_head(x["q"][b, :, h], x["k_cache"][b, h // G], x["v_cache"][b, h // G], int(x["kv_len"][b]), k, x["scale"])
-            H.check_attention(got[b:b + 1, :, h], ref[None], f"sequence {b} head {h}")
+    for impl in (B.ATTN_TENSOR, B.ATTN_TENSOR_ROWS)[:2 if per_tile else 1]:
+        ds = H.DeviceStep(cfg, y)
+        ds.attn(ctx, impl=impl)
+        assert not ds.status.any()
+        got = ds.out.cpu().numpy().astype(np.float64)
+        for b in (0, Bn - 1):                                # first and last pairs of the cut
+            for h in (0, H_kv * G - 1):
+                ref, _ = attention_head(x["q"][b, :, h], x["k_cache"][b, h // G], x["v_cache"][b, h // G], int(x["kv_len"][b]), k, x["scale"])
+                H.check_attention(got[b:b + 1, :, h], ref[None], f"sequence {b} head {h}")
 
 
 # Projection with the tokens on the M extent: few rows and 129..176 padded ones, ranges of one box and of two, a last
