@@ -280,10 +280,9 @@ def test_lmhead_orientations(B, H, mode, V, D, k, Bn):  # noqa: F811
         x["cand_prob"] = rng.uniform(0.05, 1.0, size=x["cand_prob"].shape).astype(np.float32)
     kv_len = rng.integers(0, 3000, size=Bn).astype(np.int32)
     ctx = B.Context(max_batch=Bn, n_q_heads=8, n_kv_heads=8, head_dim=64, k_max=k, vocab=V, s_cap=256)
-    i32 = lambda *s: torch.full(s, -7, dtype=torch.int32, device="cuda")  # noqa: E731
+    i32 = lambda *s: torch.empty(s, dtype=torch.int32, device="cuda")  # noqa: E731
     got = dict(n_accept=i32(Bn), out_tokens=i32(Bn, k + 1), n_out=i32(Bn), next_cand=i32(Bn, k),
-               next_cand_prob=torch.full((Bn, k), float("nan"), device="cuda"),
-               finished=torch.full((Bn,), 9, dtype=torch.uint8, device="cuda"))
+               next_cand_prob=torch.empty((Bn, k), device="cuda"), finished=torch.empty((Bn,), dtype=torch.uint8, device="cuda"))
     keep = [H.to_dev(x[n]) for n in ("hidden", "weight", "cand", "cand_prob")] + [H.to_dev(kv_len)]
     a = ctx.lmhead_args(keep[0], keep[1], keep[2], k=k, eos_id=-1, seed=7, temperature=0.9,
                         mode=B.MODE_SAMPLE if sample else B.MODE_GREEDY, cand_prob=keep[3], kv_len=keep[4],
@@ -298,8 +297,10 @@ def test_lmhead_orientations(B, H, mode, V, D, k, Bn):  # noqa: F811
         excl[b] = bool(used) and r["row_gap"][b, used].min() <= 1e-3
     if sample:
         excl |= (r["accept_margin"] <= 1e-3).any(1) | (r["bonus_gap"] <= 1e-3) | (r["draft_gap"] <= 1e-3).any(1)
-    assert excl.sum() <= max(1, Bn // 8)
+    assert excl.sum() <= Bn // 8                             # (none of a few: something is left to compare)
     for again in range(2):
+        for n, t in got.items():                             # (a call that wrote nothing does not pass)
+            t.fill_({"next_cand_prob": float("nan"), "finished": 9}.get(n, -7))
         ctx.space_lmhead_verify(a)
         h = {n: t.cpu().numpy() for n, t in got.items()}
         for n in ("n_accept", "out_tokens", "n_out", "next_cand", "finished"):
