@@ -22,6 +22,7 @@ With N > 1 (torchrun) every rank runs an independent replica on its own GPU.
 import argparse
 import json
 import os
+import re
 import sys
 import threading
 import time
@@ -36,7 +37,7 @@ from paper_2402_11809_b200 import replicas, workloads  # noqa: E402
 L2_BYTES = 126 * 1024 * 1024
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel, from the ncu captures
 # summarised under profiles/: (bytes, kernel source file, first 12 hex digits of the sha256 of that file and
-# the headers it shares when the capture was taken).  The figure is reported only while the sources still have
+# the headers it includes when the capture was taken).  The figure is reported only while the sources still have
 # that hash; once the kernel has changed the bench line carries null until the capture is taken again.
 ATTN_TRAFFIC = {"llama7b": (34523904, "attn_tc.cu", "27f910bb1083"),
                 "gqa70b": (288936960, "attn_rows.cu", "f0630685f11d")}
@@ -45,12 +46,19 @@ METRIC = "auto-correct steps/sec"
 UNIT = "steps/s"
 
 
-def source_hash(fname):
+def source_hash(fname, root=ROOT):
+    """First 12 hex digits of the sha256 of a kernel source and of every file that it includes by a quoted name,
+    directly or through another."""
     import hashlib
-    path = os.path.join(ROOT, "paper_2402_11809_b200", "csrc", fname)
+    files, todo = [], [os.path.join(root, "paper_2402_11809_b200", "csrc", fname)]
+    while todo:
+        path = os.path.normpath(todo.pop(0))
+        if path not in files:
+            files.append(path)
+            todo += [os.path.join(os.path.dirname(path), n) for n in re.findall(r'^#include "([^"]+)"', open(path).read(), re.M)]
     h = hashlib.sha256()
-    for f in (path, *(os.path.join(os.path.dirname(path), n) for n in ("tc_common.cuh", "attn_common.cuh"))):
-        h.update(open(f, "rb").read())
+    for path in files:
+        h.update(open(path, "rb").read())
     return h.hexdigest()[:12]
 
 
