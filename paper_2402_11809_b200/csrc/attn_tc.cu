@@ -340,7 +340,8 @@ constexpr float OVER_THRESHOLD = 60.f;   // re-reference a query row when a scor
 // after the vote, so that the next S^T product fills the pipe meanwhile.  Eight tiles per block, us, before / after
 // (the exponentials behind the wait for the product, S^T kept until P was stored, run-time width): 4 rows
 // 16.8 / 14.3, 25 rows 20.3 / 16.6, 36 rows 22.7 / 19.3, 49 rows 25.2 / 24.3; ragged16's attention, bound by memory,
-// gains through the clock under the power cap (step 141 / 131).
+// gains through the clock under the power cap (step 141 / 131 in one loop, 148.6 / 138.5 in another, where the runs of
+// one side differed by up to 12 %).
 template <int DH, bool PAGED, int NP>
 __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_constant__ AttnParams p,
                                                              int max_batch) {

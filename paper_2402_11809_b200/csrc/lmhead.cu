@@ -461,7 +461,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
     // where the folds would do it for 32 rows in step although only every (k+1)-th of them draws a token, after
     // the last product, with the whole chip waiting.  D = 4096, bursts, in the folds / tabulated: one sequence of 36 rows,
     // V = 32000, 56.9 / 52.9 us, V = 128256 (D = 2048) 92.7 / 87.3, 144 rows of V = 32000 69.9 / 66.2, of V = 20000 (D = 2048)
-    // 37.7 / 33.2, 16 x 36 rows of V = 128256 (96 noisy rows: a quarter of a box fits) 351 / 348.
+    // 37.7 / 33.2.  (Where the stages leave no room for 16 tokens' noise of every such row, as for the 96 target rows of a
+    // wide batch with five stages, there is no table and the folds work all of it out.)
     RowConst* rowc = reinterpret_cast<RowConst*>(smem_raw + L.rowc_off);
     float* noise = reinterpret_cast<float*>(smem_raw + L.noise_off);       // [n_noisy][noise_tok + 4]
     const int noise_pitch = p.noise_tok + 4;
