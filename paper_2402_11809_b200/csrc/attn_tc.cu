@@ -1042,41 +1042,41 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           if (col0 + x < m_valid && d_ok) dst[x * DH] = __uint_as_float(o[x >> 3][x & 7]) + __uint_as_float(o2[x >> 3][x & 7]);
       } else {
 #pragma unroll 2
-      for (int j = 0; j < NP; ++j) {
-        uint32_t o[8], o2[8];
-        const int q0 = col0 + j * 8;
-        tmem_ld8(TM_O + lane_addr + q0, o);
-        tmem_ld8(TM_O + lane_addr + 64 + q0, o2);
-        tmem_wait_ld();
+        for (int j = 0; j < NP; ++j) {
+          uint32_t o[8], o2[8];
+          const int q0 = col0 + j * 8;
+          tmem_ld8(TM_O + lane_addr + q0, o);
+          tmem_ld8(TM_O + lane_addr + 64 + q0, o2);
+          tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) + __uint_as_float(o2[e]));
-        if (whole) {
-          // query row q of the block is head q mod G of block row q / G (G is a power of two)
-          const float4 r0 = reinterpret_cast<const float4*>(rcp + q0)[0], r1 = reinterpret_cast<const float4*>(rcp + q0)[1];
-          const float rr[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-          size_t off[8];
+          for (int e = 0; e < 8; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) + __uint_as_float(o2[e]));
+          if (whole) {
+            // query row q of the block is head q mod G of block row q / G (G is a power of two)
+            const float4 r0 = reinterpret_cast<const float4*>(rcp + q0)[0], r1 = reinterpret_cast<const float4*>(rcp + q0)[1];
+            const float rr[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+            size_t off[8];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int q = q0 + e;
-            off[e] = out_base + (size_t)(q >> gsh) * out_row + (size_t)(q & (p.G - 1)) * DH;
-          }
-          if (out_f32) {
+            for (int e = 0; e < 8; ++e) {
+              const int q = q0 + e;
+              off[e] = out_base + (size_t)(q >> gsh) * out_row + (size_t)(q & (p.G - 1)) * DH;
+            }
+            if (out_f32) {
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-              if (q0 + e < m_valid && d_ok) reinterpret_cast<float*>(p.out)[off[e]] = __uint_as_float(o[e]) * rr[e];
+              for (int e = 0; e < 8; ++e)
+                if (q0 + e < m_valid && d_ok) reinterpret_cast<float*>(p.out)[off[e]] = __uint_as_float(o[e]) * rr[e];
+            } else {
+#pragma unroll
+              for (int e = 0; e < 8; ++e)
+                if (q0 + e < m_valid && d_ok)
+                  reinterpret_cast<__nv_bfloat16*>(p.out)[off[e]] = __float2bfloat16_rn(__uint_as_float(o[e]) * rr[e]);
+            }
           } else {
+            float* dst = pslot + (size_t)q0 * DH + kl;
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-              if (q0 + e < m_valid && d_ok)
-                reinterpret_cast<__nv_bfloat16*>(p.out)[off[e]] = __float2bfloat16_rn(__uint_as_float(o[e]) * rr[e]);
+              if (q0 + e < m_valid && d_ok) dst[e * DH] = __uint_as_float(o[e]);
           }
-        } else {
-          float* dst = pslot + (size_t)q0 * DH + kl;
-#pragma unroll
-          for (int e = 0; e < 8; ++e)
-            if (q0 + e < m_valid && d_ok) dst[e * DH] = __uint_as_float(o[e]);
         }
-      }
       }
       tc_fence_before();
       soft_sync();                                          // scratch, fq and mref are reused by the next share

@@ -434,13 +434,15 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
                 for (int kk = 0; kk < LM_KB / 16; ++kk)
                   mma_ss(acc, wd + (uint64_t)(tt * (16384 >> 4) + kk * 2), hd + (uint64_t)(kk * 2), idesc, (ki | j | kk) ? 1u : 0u);
               }
-            } else for (int mt = 0; mt < p.n_mt; ++mt) {
-              // block rows 128*mt .. of the hidden tile (8-row groups are contiguous: 16 KB further on)
-              const uint64_t hd = desc0 + (uint64_t)((st_off + (uint32_t)j * L.a_bytes + (uint32_t)mt * 16384u) >> 4);
-              const uint32_t acc = tmem + (uint32_t)((buf * p.n_mt + mt) * LM_MAX_BOX);
+            } else {
+              for (int mt = 0; mt < p.n_mt; ++mt) {
+                // block rows 128*mt .. of the hidden tile (8-row groups are contiguous: 16 KB further on)
+                const uint64_t hd = desc0 + (uint64_t)((st_off + (uint32_t)j * L.a_bytes + (uint32_t)mt * 16384u) >> 4);
+                const uint32_t acc = tmem + (uint32_t)((buf * p.n_mt + mt) * LM_MAX_BOX);
 #pragma unroll
-              for (int kk = 0; kk < LM_KB / 16; ++kk)      // 32 bytes per 16 elements inside the swizzled row
-                mma_ss(acc, hd + (uint64_t)(kk * 2), wd + (uint64_t)(kk * 2), idesc, (ki | j | kk) ? 1u : 0u);
+                for (int kk = 0; kk < LM_KB / 16; ++kk)    // 32 bytes per 16 elements inside the swizzled row
+                  mma_ss(acc, hd + (uint64_t)(kk * 2), wd + (uint64_t)(kk * 2), idesc, (ki | j | kk) ? 1u : 0u);
+              }
             }
           }
           tc_commit(LBAR(B_EMPTY + s));
@@ -482,6 +484,13 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         reinterpret_cast<float4*>(noise + y * noise_pitch)[q] = noise4((uint32_t)(row0 >> 2) + q, rowc[row], p.key0, p.key1);
       }
       epi_sync();
+    };
+    // statistics of other tokens of a row join (m0, s0, i0)
+    auto join = [&](float& m0, float& s0, int& i0, float m2, float s2, int i2) {
+      if (m2 > m0 || (m2 == m0 && i2 < i0)) i0 = i2;
+      const float e = fast_exp2(-fabsf(m0 - m2) * p.c_t);    // (one of the two exponentials is exp(0))
+      s0 = (m0 >= m2) ? fmaf(s2, e, s0) : fmaf(s0, e, s2);
+      m0 = fmaxf(m0, m2);
     };
     if (TM) {
       // ---- tokens on M: lane = token, column = block row.  A warp reads 8 rows of its 32 tokens, turns them through
@@ -540,12 +549,6 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       }
       // ---- the four lanes of a row meet, then (through the idle stages: every product is done) the four quarters
       float* x = reinterpret_cast<float*>(smem_raw);         // [4][3][LM_MAX_N]
-      auto join = [&](float& m0, float& s0, int& i0, float m2, float s2, int i2) {
-        if (m2 > m0 || (m2 == m0 && i2 < i0)) i0 = i2;
-        const float e = fast_exp2(-fabsf(m0 - m2) * p.c_t);  // (one of the two exponentials is exp(0))
-        s0 = (m0 >= m2) ? fmaf(s2, e, s0) : fmaf(s0, e, s2);
-        m0 = fmaxf(m0, m2);
-      };
 #pragma unroll
       for (int i = 0; i < GP; ++i) {
         const int g = part + 4 * i;
@@ -632,12 +635,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         if (part == 0 && has_rows) {
           for (int o = 1; o < n_parts; ++o) {
             const float* y = x + (o - 1) * 7 * W;
-            const float m2 = y[0], s2 = y[W], c = p.c_t;
-            const int i2 = __float_as_int(y[2 * W]);
-            if (m2 > m0 || (m2 == m0 && i2 < i0)) i0 = i2;
-            const float e = fast_exp2(-fabsf(m0 - m2) * c);   // (one of the two exponentials is exp(0))
-            s0 = (m0 >= m2) ? fmaf(s2, e, s0) : fmaf(s0, e, s2);
-            m0 = fmaxf(m0, m2);
+            join(m0, s0, i0, y[0], y[W], __float_as_int(y[2 * W]));
             if (sample) {
               const float g2 = y[3 * W];
               const int gi2 = __float_as_int(y[5 * W]);
