@@ -115,15 +115,17 @@ __device__ __forceinline__ void prefetch_chunk(const T* row, int begin, int end)
   }
 }
 
+// Blocks that a launch over rows and chunks may have to be resident at once: three per SM, and a few more.
+static inline int64_t row_chunk_slots(int sm_count) { return 3 * (int64_t)sm_count * 21 / 20; }
 // Chunks per row and their length.  A sweep of a block is four vectors per thread (8192 bf16 logits); a
 // block costs about 3 us whatever it scans (reduction, fence, arrival).  So: as few sweeps per block as let all
-// blocks be resident at once (three per SM, and a few more), four where they cannot be.  Measured, us per call
+// blocks be resident at once, four where they cannot be.  Measured, us per call
 // (graph replay of space_verify_commit) with 1 / 2 / 3 / 4 sweeps per block: 80 rows of 50257 10.7 / 9.4 / 10.9 /
 // 13.6, 98 rows of 128256 16.6 / 12.5 / 13.1 / 10.5, 576 rows of 32000 22.7 / 16.5 / 16.6 / 15.2, top-10 lists of 72
 // and 48 rows of 128256 39 / 31 / 29 / 32 (27.7 with three and two), sampling 64 x 5 rows of 128256 106 / 71 / 66 / 57.
 static inline int row_chunks(int vocab, int rows, int vec, int sm_count, int max_chunks, int* chunk_out) {
   const int sweep = SPACE_VERIFY_THREADS * vec * 4;
-  const int64_t slots = 3 * (int64_t)sm_count * 21 / 20;
+  const int64_t slots = row_chunk_slots(sm_count);
   int64_t nc = 1;
   for (int per_block = 1; per_block <= 4; ++per_block) {
     nc = (vocab + (int64_t)per_block * sweep - 1) / ((int64_t)per_block * sweep);
