@@ -945,7 +945,16 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   // V = 20000, D = 2048, 36 rows 22.3 (21.4) / 23.1 (23.9).  Sampling keeps the rows on M: with seven values per row the
   // epilogue of the other form is the longer one (measured when both had it, V = 32000: 36 rows 55.7 (52.9) / 56.8 (57.3),
   // 144 rows 77.2 (66.1) / 75.6 (73.1), 176 rows 82.2 (71.3) / 87.4 (85.7)).
-  const bool tokens_on_m = !sampling && p.n_box > 192 && (p.n_pad <= 64 || (p.n_pad > LM_M && p.n_pad <= 176));
+  // (At 1965 MHz that is 1.4 % given away at 36 to 49 rows of V = 32000, D = 4096, for 5 % under the cap.)  Accumulators
+  // less than three quarters full are the exception: a range of 257 to 288 tokens takes a third one for a few of them.
+  // V = 37800 (271 tokens), bursts (loop), rows on M / tokens on M: 36 rows, D = 512 16.3 (16.0) / 16.5 (16.2), 64 rows
+  // 16.6 (16.3) / 16.9 (16.7), D = 2048 39.6 (39.6) / 40.1 (39.9), 175 rows 53.8 (53.8) / 55.5 (54.9), D = 4096 87.5 (94.0) /
+  // 91.5 (93.0); but 9 rows, D = 4096 69.0 (70.3) / 67.2 (66.8), 36 rows 69.1 (71.5) / 69.3 (69.0), 64 rows 69.8 (71.3) / 68.6
+  // (68.4), 144 rows, D = 512 25.3 (24.7) / 23.3 (22.9), D = 4096 87.2 (93.4) / 83.1 (84.3).
+  const int in_acc = (max_len + LM_TOK - 1) / LM_TOK * LM_TOK;            // tokens that a range's accumulators have room for
+  const bool filled = 4 * max_len > 3 * in_acc;
+  const bool tokens_on_m = !sampling && p.n_box > 192 && (p.n_pad <= (filled || p.D > 3072 ? 64 : 16) ||
+                                                          (p.n_pad > LM_M && p.n_pad <= (filled ? 176 : 144)));
   // (all that a block may have: with 96 rows it holds five stages, with 220 KB four; 16 x 36 rows of V = 128256, greedy,
   // 350 -> 343 us in bursts, 112 rows of V = 32000 52.8 -> 51.4, 144 sampling 66.7 -> 64.3, 72 of V = 5000 17.8 -> 16.8)
   const size_t budget = 227 * 1024;
