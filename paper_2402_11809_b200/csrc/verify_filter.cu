@@ -53,13 +53,15 @@ constexpr int FILT_BUF = 4096;                           // keys a segment may c
 // (22 MB) 24.8 / 26.2, but 24 x 9 of 50257 (22 MB) 28.2 / 25.2; few bytes: 4 x 9 of 32000 (2 MB) 17.6 / 12.5, 28 x 9 (16 MB)
 // 20.7 / 18.7, 5 x 49 (16 MB) 19.4 / 19.5, 10 x 16 of 50257 (16 MB, top-25) 27.3 / 28.5.
 // Not, among the few rows, where one launch has more blocks than fit at once (2 x 36 of 100000 f32, 504 blocks, 24.6 /
-// 25.7; 3 x 25, 525 blocks, 23.7 / 25.6; at 448 blocks, 1 x 64, 23.4 / 23.5), nor where rows off the 16-byte grid, which
-// every vector is put together for, make more than 10 MB of rows that two launches skip (2 x 49 of 50257 f32 (14 MB of
-// them) 22.9 / 25.4, 3 x 36 (15 MB) 22.7 / 25.4, 2 x 49 of 100001 bf16 (14 MB) 24.1 / 25.9, 6 x 16 of 50257 f32 (11 MB)
-// 24.1 / 24.4, but 12 x 9 (9.6 MB) 27.3 / 24.8; on the grid, of 128256 bf16, 2 x 49 (18 MB) 22.2 / 21.1, 3 x 36 (19 MB)
-// 23.3 / 21.1).
+// 25.7; 3 x 25, 525 blocks, 23.7 / 25.6; at 448 blocks, 1 x 64, 23.4 / 23.5).  Rows off the 16-byte grid, whose every
+// vector is put together from two, have no room for more than three blocks per SM (1 x 64 of 80001 f32, 448 blocks, 25.0 /
+// 30.1; 3 x 25 of 70001, 450, 25.9 / 28.8; 1 x 49 of 100001, 441, 25.9 / 24.5), and two sweeps more than both launches take
+// together cost more than the launch: two more, 2 x 49 of 50257 f32 22.9 / 25.4, of 128257 bf16 25.6 / 28.6, 3 x 36 of 50257
+// f32 22.7 / 25.4, 4 x 25 23.7 / 25.0, 6 x 16 24.1 / 24.4, of 100001 bf16 25.1 / 25.0; one more, 12 x 9 of 50257 f32 27.3 /
+// 24.8, of 128257 bf16 29.9 / 27.6; as many, 2 x 25 of 128257 f32 31.0 / 29.1.  On the grid two more gain: 2 x 49 of 128256
+// bf16 22.2 / 21.1, of 52000 f32 20.1 / 19.4, 6 x 16 of 50256 f32 21.2 / 18.3.
 constexpr int FILT_BOTH_ROWS = 256, FILT_FEW_ROWS = 110;
-constexpr int64_t FILT_BOTH_BYTES = 16ll << 20, FILT_FEW_ROWS_BYTES = 30ll << 20, FILT_UNALIGNED_EXTRA = 10ll << 20;
+constexpr int64_t FILT_BOTH_BYTES = 16ll << 20, FILT_FEW_ROWS_BYTES = 30ll << 20;
 enum { PHASE_TARGETS = 0, PHASE_MASKS = 1, PHASE_BOTH = 2 };
 
 struct FiltParams {
@@ -530,10 +532,16 @@ int launch_verify_filtered(space_ctx* ctx, const space_verify_args* a, const spa
   const int64_t row_bytes = (int64_t)a->vocab * esz;
   bool both = block_rows <= FILT_BOTH_ROWS && block_rows * row_bytes <= FILT_BOTH_BYTES;
   if (!both && block_rows <= FILT_FEW_ROWS && block_rows * row_bytes <= FILT_FEW_ROWS_BYTES) {
-    int chunk;
-    const int blocks = row_chunks(a->vocab, (int)block_rows, 16 / esz, ctx->sm_count, FILT_MAX_CHUNKS, &chunk) * (int)block_rows;
-    both = blocks <= row_chunk_slots(ctx->sm_count) &&
-           (aligned || a->batch * (int64_t)(p.n_q - 2 * a->k - 1) * row_bytes <= FILT_UNALIGNED_EXTRA);
+    const int vec = 16 / esz;
+    auto sweeps = [&](int64_t rows, int64_t* blocks) {     // that a block takes over its chunk in a launch of so many rows
+      int chunk;
+      *blocks = rows * row_chunks(a->vocab, (int)rows, vec, ctx->sm_count, FILT_MAX_CHUNKS, &chunk);
+      return (chunk + FILT_THREADS * vec * FILT_U - 1) / (FILT_THREADS * vec * FILT_U);
+    };
+    int64_t blocks, unused;
+    const int one = sweeps(block_rows, &blocks);
+    const int two = sweeps((int64_t)a->batch * (a->k + 1), &unused) + sweeps((int64_t)a->batch * a->k, &unused);
+    both = aligned ? blocks <= row_chunk_slots(ctx->sm_count) : blocks <= 3 * (int64_t)ctx->sm_count && one <= two + 1;
   }
   // the commit rides along, except where one block would have more than 32 KB of rows to move: a launch of its
   // own is faster then (two sequences, one launch; us per step, riding / own: 16 KB 22.1 / 23.7, 32 KB 25.8 / 26.1,

@@ -342,7 +342,8 @@ def test_commit_under_the_scan(B, H, k, H_kv, d, V, Bn, paged):  # noqa: F811
 # logits, 110 rows; more rows: 16 MB; rows off the 16-byte grid; blocks that do not fit at once), with the commit on board: the same decisions and cache either way.
 @pytest.mark.parametrize("Bn,k,V,dtype,launches", [(3, 5, 128256, "bf16", 1), (2, 4, 128256, "f32", 1), (4, 5, 64064, "bf16", 2),
                                                   (3, 5, 146000, "bf16", 2), (7, 3, 70001, "bf16", 1),
-                                                  (2, 6, 50257, "f32", 2), (12, 2, 50257, "f32", 1), (3, 4, 100000, "f32", 2)])
+                                                  (2, 6, 50257, "f32", 2), (12, 2, 50257, "f32", 1), (3, 4, 100000, "f32", 2),
+                                                  (1, 7, 80001, "f32", 2), (2, 4, 128257, "f32", 1)])
 def test_filtered_one_launch_or_two(B, H, Bn, k, V, dtype, launches):  # noqa: F811
     from oracle.commit import commit_step
     cfg = workloads.resolve("sampling64", B=Bn, H_q=2, H_kv=2, d=64, L=(5, 200), k=k, V=V, logits_dtype=dtype, seed=V % 89)
