@@ -947,14 +947,16 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   // 144 rows 77.2 (66.1) / 75.6 (73.1), 176 rows 82.2 (71.3) / 87.4 (85.7)).
   // (At 1965 MHz that is 1.4 % given away at 36 to 49 rows of V = 32000, D = 4096, for 5 % under the cap.)  Accumulators
   // less than three quarters full are the exception: a range of 257 to 288 tokens takes a third one for a few of them.
-  // V = 37800 (271 tokens), bursts (loop), rows on M / tokens on M: 36 rows, D = 512 16.3 (16.0) / 16.5 (16.2), 64 rows
-  // 16.6 (16.3) / 16.9 (16.7), D = 2048 39.6 (39.6) / 40.1 (39.9), 175 rows 53.8 (53.8) / 55.5 (54.9), D = 4096 87.5 (94.0) /
-  // 91.5 (93.0); but 9 rows, D = 4096 69.0 (70.3) / 67.2 (66.8), 36 rows 69.1 (71.5) / 69.3 (69.0), 64 rows 69.8 (71.3) / 68.6
-  // (68.4), 144 rows, D = 512 25.3 (24.7) / 23.3 (22.9), D = 4096 87.2 (93.4) / 83.1 (84.3).
+  // Bursts (loop), rows on M / tokens on M: V = 37800 (271 tokens), D = 1024 25 rows 22.2 (21.9) / 23.4 (23.2), 64 rows
+  // 22.9 (22.5) / 24.1 (23.6), 160 rows 34.1 (33.6) / 35.7 (35.2), 175 rows 34.3 (33.6) / 36.7 (36.3); D = 2048 64 rows 38.2
+  // (39.0) / 39.8 (39.6), 175 rows 51.7 (53.2) / 55.5 (54.9); D = 3072 25 rows 51.7 (53.5) / 53.1 (52.7), 160 rows 68.6 (73.7) /
+  // 71.7 (71.4), 175 rows 71.0 (73.1) / 74.4 (74.8); V = 40000 (286 tokens), D = 1024 25 rows 22.9 (22.8) / 24.1 (23.6), D = 2048
+  // 37.6 (39.8) / 38.2 (37.9).  So rows on M there for short products, and from 161 rows for all; 144 rows keep the tokens
+  // there (V = 37800, D = 512 25.3 (24.7) before this form / 23.3 (22.9) with it, D = 4096 87.2 (93.4) / 83.1 (84.3)).
   const int in_acc = (max_len + LM_TOK - 1) / LM_TOK * LM_TOK;            // tokens that a range's accumulators have room for
   const bool filled = 4 * max_len > 3 * in_acc;
-  const bool tokens_on_m = !sampling && p.n_box > 192 && (p.n_pad <= (filled || p.D > 3072 ? 64 : 16) ||
-                                                          (p.n_pad > LM_M && p.n_pad <= (filled ? 176 : 144)));
+  const bool tokens_on_m = !sampling && p.n_box > 192 && (p.n_pad <= (filled || p.D > 1536 ? 64 : 16) ||
+                                                          (p.n_pad > LM_M && p.n_pad <= (filled ? 176 : p.D > 1536 ? 160 : 144)));
   // (all that a block may have: with 96 rows it holds five stages, with 220 KB four; 16 x 36 rows of V = 128256, greedy,
   // 350 -> 343 us in bursts, 112 rows of V = 32000 52.8 -> 51.4, 144 sampling 66.7 -> 64.3, 72 of V = 5000 17.8 -> 16.8)
   const size_t budget = 227 * 1024;
