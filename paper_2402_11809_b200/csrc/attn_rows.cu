@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
         // an output error near 1e-2 of the output RMS.  P_hi occupies columns
         // 0..63 of the S buffer, P_lo columns 64..127 (two keys per column).
         uint32_t lreg[HC / 2];
-        const uint64_t cc = pack2(c, c), mm = pack2(-m_use, -m_use), neg = pack2(-1.f, -1.f);
+        const uint64_t cc = pack2(c, c), mm = pack2(-m_use, -m_use);
         uint64_t sum[2] = {0ull, 0ull};
 #pragma unroll
         for (int x = 0; x < HC / 2; ++x) {
@@ -573,11 +573,10 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
           const uint64_t pp = pack2(p0, p1);
           sum[x & 1] = add2(sum[x & 1], pp);
           const __nv_bfloat162 hi = __floats2bfloat162_rn(p0, p1);   // .x (low half) = even key
-          const float2 hf = __bfloat1622float2(hi);
-          float l0, l1;
-          unpack2(fma2(pack2(hf.x, hf.y), neg, pp), l0, l1);         // (exact)
-          const __nv_bfloat162 lw = __floats2bfloat162_rn(l0, l1);
           sreg[x] = *reinterpret_cast<const uint32_t*>(&hi);
+          float l0, l1;
+          low_terms(sreg[x], p0, p1, l0, l1);
+          const __nv_bfloat162 lw = __floats2bfloat162_rn(l0, l1);
           lreg[x] = *reinterpret_cast<const uint32_t*>(&lw);
         }
         {

@@ -854,9 +854,10 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
             sv[x] = fast_exp2(sv[x]); sv[x + 1] = fast_exp2(sv[x + 1]);
             if (VOTE_FIRST) { lsum[x] += sv[x]; lsum[x + 1] += sv[x + 1]; }
             const __nv_bfloat162 h2 = __floats2bfloat162_rn(sv[x], sv[x + 1]);      // .x = lower query row
-            const float2 hf = __bfloat1622float2(h2);
-            const __nv_bfloat162 l2 = __floats2bfloat162_rn(sv[x] - hf.x, sv[x + 1] - hf.y);
             hi[x >> 1] = *reinterpret_cast<const uint32_t*>(&h2);
+            float l0, l1;
+            low_terms(hi[x >> 1], sv[x], sv[x + 1], l0, l1);
+            const __nv_bfloat162 l2 = __floats2bfloat162_rn(l0, l1);
             lw[x >> 1] = *reinterpret_cast<const uint32_t*>(&l2);
           }
         };
