@@ -27,7 +27,9 @@
 // costs instructions, meet earlier the more of them can be skipped (16 x 9 rows of
 // 50257, 14 MB, 22.7 / 29.1; 40 x 9, 36 MB, 52.0 / 52.5; 4 x 64, 26 MB, 34.4 / 27.3).
 #include "common.cuh"
+#include "tc_common.cuh"
 #include <math_constants.h>
+#include <type_traits>
 
 namespace {
 
@@ -112,6 +114,16 @@ template <> struct Vec<__nv_bfloat16> {
       v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
     }
   }
+  // (two logits per instruction, before any is widened)
+  static __device__ __forceinline__ uint32_t max2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+  }
+  static __device__ __forceinline__ float maximum(const uint4& x) {
+    const uint32_t m = max2(max2(x.x, x.y), max2(x.z, x.w));
+    return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xFFFF0000u));
+  }
 };
 
 // What a scan keeps of its logits: nothing (the noisy arg-max alone), the maximum with its
@@ -142,24 +154,36 @@ __device__ __forceinline__ void fold_one(Stat& st, float v, int x, float c, int 
   }
 }
 
-// (max, lowest arg-max, sum of exp2((z - max) c)) of U vectors of N logits, the
+// (max, lowest arg-max, sum of exp2((z - max) c)) of U vectors of N logits (v: their values, unless PACKED), the
 // first at index x0, the u-th `stride` further: one maximum and one rescale per
 // call, then independent exponentials and tree sums.  -inf entries (slots past the
 // end of the chunk) change neither the maximum nor the sum.  st.idx is left at the first
 // index of the vector that holds the maximum (see scan_chunk).
-template <int U, int N, bool SUMS>
-__device__ __forceinline__ void fold_stats(Stat& st, const float (&v)[U][N], int x0, int stride, float c) {
+// PACKED (bf16 rows on the 16-byte grid): the maximum is taken of the vectors as they were loaded, two logits per
+// instruction, and for the sums one vector at a time is widened, with two logits per multiply-add and addition: fewer
+// instructions and 16 registers less.  The sums are added in the same order either way.  Measured, us per step behind a
+// short attention (steady loop), without / with: 16 x 36 rows of 32000 20.9 / 20.5, 8 x 49 18.8 / 18.2, sampling
+// 64 x 5 of 128256 77.3 / 73.7, two launches 64 x 6 greedy 85.3 / 80.6.  Not where it cost: f32 (3 x 25 rows of 128256
+// 18.1 / 18.6), rows off the grid (5 x 16 of 50257 13.7 / 14.4).
+template <int U, typename T, bool SUMS, bool PACKED>
+__device__ __forceinline__ void fold_stats(Stat& st, const uint4 (&raw)[U], float (&v)[PACKED ? 1 : U][Vec<T>::N], int x0,
+                                           int stride, float c) {
+  constexpr int N = Vec<T>::N;
   float vm[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    float a[N];
+    if constexpr (PACKED) {
+      vm[u] = Vec<T>::maximum(raw[u]);
+    } else {
+      float a[N];
 #pragma unroll
-    for (int i = 0; i < N; ++i) a[i] = v[u][i];
+      for (int i = 0; i < N; ++i) a[i] = v[u][i];
 #pragma unroll
-    for (int w = N / 2; w > 0; w >>= 1)
+      for (int w = N / 2; w > 0; w >>= 1)
 #pragma unroll
-      for (int i = 0; i < w; ++i) a[i] = fmaxf(a[i], a[i + w]);
-    vm[u] = a[0];
+        for (int i = 0; i < w; ++i) a[i] = fmaxf(a[i], a[i + w]);
+      vm[u] = a[0];
+    }
   }
   float vmax = vm[0];
 #pragma unroll
@@ -179,14 +203,33 @@ __device__ __forceinline__ void fold_stats(Stat& st, const float (&v)[U][N], int
     float su[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      float e[N];
+      if constexpr (PACKED) {
+        const uint64_t cc = tc::pack2(c, c), nn = tc::pack2(nmc, nmc);
+        Vec<T>::convert(raw[u], v[0]);
+        uint64_t e[N / 2];
 #pragma unroll
-      for (int i = 0; i < N; ++i) e[i] = fast_exp2(fmaf(v[u][i], c, nmc));
+        for (int i = 0; i < N / 2; ++i) {
+          float a, b;
+          tc::unpack2(tc::fma2(tc::pack2(v[0][2 * i], v[0][2 * i + 1]), cc, nn), a, b);
+          e[i] = tc::pack2(fast_exp2(a), fast_exp2(b));
+        }
 #pragma unroll
-      for (int w = N / 2; w > 0; w >>= 1)
+        for (int w = N / 4; w > 0; w >>= 1)
 #pragma unroll
-        for (int i = 0; i < w; ++i) e[i] += e[i + w];
-      su[u] = e[0];
+          for (int i = 0; i < w; ++i) e[i] = tc::add2(e[i], e[i + w]);
+        float a, b;
+        tc::unpack2(e[0], a, b);
+        su[u] = a + b;
+      } else {
+        float e[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) e[i] = fast_exp2(fmaf(v[u][i], c, nmc));
+#pragma unroll
+        for (int w = N / 2; w > 0; w >>= 1)
+#pragma unroll
+          for (int i = 0; i < w; ++i) e[i] += e[i + w];
+        su[u] = e[0];
+      }
     }
     float tot = su[0];
 #pragma unroll
@@ -236,19 +279,24 @@ __device__ Stat scan_chunk(const T* row, int begin, int end, float c, int exclud
   int x = begin + threadIdx.x * N;
   // one sweep of U vectors, the first at x; slots past the end read as -inf
   auto fold = [&](const uint4 (&cur)[U], int x) {
-    float v[U][N];
+    constexpr bool PACKED = ALIGNED && sizeof(T) == 2;
+    float v[PACKED ? 1 : U][N];                             // (packed: one vector at a time)
+    if (!PACKED) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) Vec<T>::convert(cur[u], v[u]);
-    if (STATS) fold_stats<U, N, STATS == STAT_SUM>(st, v, x, stride, c);
+      for (int u = 0; u < (PACKED ? 1 : U); ++u) Vec<T>::convert(cur[u], v[u]);
+    }
+    if (STATS) fold_stats<U, T, STATS == STAT_SUM, PACKED>(st, cur, v, x, stride, c);
     if (GUMBEL) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int xu = x + u * stride;
+        float (&vu)[N] = v[PACKED ? 0 : u];
+        if (PACKED) Vec<T>::convert(cur[u], vu);
         if ((unsigned)(exclude - xu) < (unsigned)N) {       // the one token left out of the draw
 #pragma unroll
-          for (int i = 0; i < N; ++i) if (xu + i == exclude) v[u][i] = -CUDART_INF_F;
+          for (int i = 0; i < N; ++i) if (xu + i == exclude) vu[i] = -CUDART_INF_F;
         }
-        if (xu < full_end) fold_gumbel<N>(st, v[u], xu, c, key0, key1, purpose, seq, pos);
+        if (xu < full_end) fold_gumbel<N>(st, vu, xu, c, key0, key1, purpose, seq, pos);
       }
     }
   };
@@ -617,11 +665,12 @@ __device__ unsigned long long g_timeline_verify[4096 * 8];
 
 // PAGED: the commit on board goes through a page table (a build of its own: the table look-ups are
 // not compiled into the contiguous form, whose addressing sits in the critical path).
-// EARLY: the rows to commit are fetched under the scan.  It costs registers, that is the third block per SM, so only
-// calls whose blocks need no third one take it (see launch_fused).
-template <typename T, bool ALIGNED, bool PAGED = false, bool EARLY = false>
-__global__ void __launch_bounds__(SPACE_VERIFY_THREADS, EARLY ? 2 : 3)
+// BLOCKS: how many per SM the build leaves registers for (launch_fused has the rule).  With two the rows to commit are
+// fetched under the scan (EARLY).
+template <typename T, bool ALIGNED, bool PAGED = false, int BLOCKS = 3>
+__global__ void __launch_bounds__(SPACE_VERIFY_THREADS, BLOCKS)
 verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
+  constexpr bool EARLY = ALIGNED && BLOCKS == 2;
   TLV(0);
   pdl_launch_dependents();
   const int b = blockIdx.z, row_i = blockIdx.y, ch = blockIdx.x;
@@ -760,8 +809,18 @@ void launch_fused(space_ctx* ctx, const VerifyParams& p, cudaStream_t st) {
   const bool early = ALIGNED && p.do_commit && per_seq * p.B <= 2 * ctx->sm_count &&
                      p.k * p.cm.H_kv * 2 * (p.cm.d / 8) <= per_seq * (SPACE_VERIFY_THREADS - 32);
   const bool paged = p.do_commit && p.cm.page_table;
-  auto kernel = early ? (paged ? verify_fused_kernel<T, ALIGNED, true, ALIGNED> : verify_fused_kernel<T, ALIGNED, false, ALIGNED>)
-                      : (paged ? verify_fused_kernel<T, ALIGNED, true> : verify_fused_kernel<T, ALIGNED>);
+  // Four blocks per SM where three would not hold the launch: its last wave would be nearly empty.  Measured, us per step
+  // behind a short attention, three / four: 16 x 36 rows of 32000 (576 blocks) 20.5 / 20.0, 8 x 25 of 128256 (800) 23.5 / 22.8,
+  // 4 x 64 of 50257 (512, off the 16-byte grid) 23.7 / 21.3; where three hold it the fourth only takes registers: 8 x 49 rows
+  // (392 blocks) 18.2 / 20.2, 12 x 16 (384) 13.8 / 14.5.
+  const bool four = (int64_t)per_seq * p.B > 3 * ctx->sm_count;
+  auto form = [&](auto pg) {
+    constexpr bool PG = decltype(pg)::value;
+    return early && ALIGNED ? verify_fused_kernel<T, ALIGNED, PG, ALIGNED ? 2 : 3>
+           : four           ? verify_fused_kernel<T, ALIGNED, PG, 4>
+                            : verify_fused_kernel<T, ALIGNED, PG, 3>;
+  };
+  auto kernel = paged ? form(std::true_type()) : form(std::false_type());
   launch_pdl(kernel, grid, block, 0, st, p, ctx->vfused);
 }
 
