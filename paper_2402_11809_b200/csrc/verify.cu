@@ -114,16 +114,6 @@ template <> struct Vec<__nv_bfloat16> {
       v[2 * i + 1] = __uint_as_float(w[i] & 0xFFFF0000u);
     }
   }
-  // (two logits per instruction, before any is widened)
-  static __device__ __forceinline__ uint32_t max2(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-  }
-  static __device__ __forceinline__ float maximum(const uint4& x) {
-    const uint32_t m = max2(max2(x.x, x.y), max2(x.z, x.w));
-    return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xFFFF0000u));
-  }
 };
 
 // What a scan keeps of its logits: nothing (the noisy arg-max alone), the maximum with its
@@ -173,7 +163,7 @@ __device__ __forceinline__ void fold_stats(Stat& st, const uint4 (&raw)[U], floa
 #pragma unroll
   for (int u = 0; u < U; ++u) {
     if constexpr (PACKED) {
-      vm[u] = Vec<T>::maximum(raw[u]);
+      vm[u] = max_bf16x8(raw[u]);
     } else {
       float a[N];
 #pragma unroll
@@ -265,7 +255,8 @@ __device__ __forceinline__ void fold_gumbel(Stat& st, const float* v, int x0, fl
 // arg-max and sum; GUMBEL: the best noisy score (token `exclude` left out).  ALIGNED: the row is 16-byte
 // aligned; otherwise every vector is put together from two aligned pieces (see load_pieces).
 // `meanwhile` runs once, when the first sweep's loads are on their way (aligned rows only).
-template <typename T, bool ALIGNED, bool GUMBEL, int STATS, class F>
+// SHORT: for launches of a sweep or two per block, whose time is the way to the first logits.
+template <typename T, bool ALIGNED, bool GUMBEL, int STATS, bool SHORT, class F>
 __device__ Stat scan_chunk(const T* row, int begin, int end, float c, int exclude,
                            uint32_t key0, uint32_t key1, uint32_t purpose, uint32_t seq,
                            uint32_t pos, F meanwhile) {
@@ -274,7 +265,9 @@ __device__ Stat scan_chunk(const T* row, int begin, int end, float c, int exclud
   constexpr int U = 4;                                      // independent vectors in flight per thread
   // the tail shorter than N is handled one by one
   const int full_end = begin + ((end - begin) / N) * N;
-  const int stride = blockDim.x * N;
+  // (As a constant in SHORT scans of bf16 it took the compiler to 80 registers, 94 without, and the loads closer to their
+  // use: one 7B-shaped sequence's step 18.06 -> 18.43 us.  f32, 12.30 -> 12.16, and the others are better off with it.)
+  const int stride = SHORT && sizeof(T) == 2 ? (int)blockDim.x * N : SPACE_VERIFY_THREADS * N;
   const uint4 ninf = make_uint4(Vec<T>::NEG_INF, Vec<T>::NEG_INF, Vec<T>::NEG_INF, Vec<T>::NEG_INF);
   int x = begin + threadIdx.x * N;
   // one sweep of U vectors, the first at x; slots past the end read as -inf
@@ -301,22 +294,49 @@ __device__ Stat scan_chunk(const T* row, int begin, int end, float c, int exclud
     }
   };
   if (ALIGNED) {
-    // The U loads of the next sweep are issued before the current one is folded,
-    // so a thread always has loads in flight.
-    uint4 cur[U], nxt[U];
+    // The U loads of the next sweep are issued before the current one is folded, so a thread always has loads in
+    // flight.  Sweeps that lie in the chunk as a whole load without a test (us per step behind a short attention, a test
+    // per vector / without: 16 x 36 rows of 32000 20.0 / 19.6, 8 x 25 of 128256 23.0 / 22.4, 3 x 25 of them in f32
+    // 17.4 / 16.7; SHORT, where the first address came later for it: 2 x 36 rows of 32000 13.0 / 13.6).
+    const uint4* src = reinterpret_cast<const uint4*>(row + begin) + threadIdx.x;
+    const int nv = (end - begin) / N, full = nv / (U * SPACE_VERIFY_THREADS), ns = (nv + U * SPACE_VERIFY_THREADS - 1) / (U * SPACE_VERIFY_THREADS);
+    auto load = [&](uint4 (&d)[U], int sweep) {
+      const uint4* at = src + sweep * (U * SPACE_VERIFY_THREADS);
+      if (sweep < full) {
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      cur[u] = (x + u * stride < full_end) ? __ldg(reinterpret_cast<const uint4*>(row + x + u * stride)) : ninf;
-    meanwhile();
-    while (x < full_end) {
-      const int xn = x + U * stride;
+        for (int u = 0; u < U; ++u) d[u] = __ldg(at + u * SPACE_VERIFY_THREADS);
+      } else {
+        const int left = nv - sweep * (U * SPACE_VERIFY_THREADS) - (int)threadIdx.x;   // (no more than 0 past the last sweep)
+#pragma unroll
+        for (int u = 0; u < U; ++u) d[u] = u * SPACE_VERIFY_THREADS < left ? __ldg(at + u * SPACE_VERIFY_THREADS) : ninf;
+      }
+    };
+    uint4 cur[U], nxt[U];
+    if constexpr (SHORT) {
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        nxt[u] = (xn + u * stride < full_end) ? __ldg(reinterpret_cast<const uint4*>(row + xn + u * stride)) : ninf;
+        cur[u] = (x + u * stride < full_end) ? __ldg(reinterpret_cast<const uint4*>(row + x + u * stride)) : ninf;
+      meanwhile();
+      while (x < full_end) {
+        const int xn = x + U * stride;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          nxt[u] = (xn + u * stride < full_end) ? __ldg(reinterpret_cast<const uint4*>(row + xn + u * stride)) : ninf;
+        fold(cur, x);
+#pragma unroll
+        for (int u = 0; u < U; ++u) cur[u] = nxt[u];
+        x = xn;
+      }
+    } else {
+    load(cur, 0);
+    meanwhile();
+    for (int sweep = 0; sweep < ns; ++sweep) {
+      load(nxt, sweep + 1);
       fold(cur, x);
 #pragma unroll
       for (int u = 0; u < U; ++u) cur[u] = nxt[u];
-      x = xn;
+      x += U * stride;
+    }
     }
   } else {
     // (two loads per vector are in flight here; holding the next sweep's as well would cost 32 registers)
@@ -352,7 +372,7 @@ __device__ Stat scan_chunk(const T* row, int begin, int end, float c, int exclud
 template <typename T, bool ALIGNED, bool GUMBEL, int STATS>
 __device__ __forceinline__ Stat scan_chunk(const T* row, int begin, int end, float c, int exclude, uint32_t key0, uint32_t key1,
                                            uint32_t purpose, uint32_t seq, uint32_t pos) {
-  return scan_chunk<T, ALIGNED, GUMBEL, STATS>(row, begin, end, c, exclude, key0, key1, purpose, seq, pos, [] {});
+  return scan_chunk<T, ALIGNED, GUMBEL, STATS, false>(row, begin, end, c, exclude, key0, key1, purpose, seq, pos, [] {});
 }
 
 __device__ __forceinline__ Stat warp_reduce(Stat st, float c) {
@@ -690,7 +710,7 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
   // 16-byte grid, whose scan has no registers to spare, lost 7 % by it).
   uint4 cm_val = make_uint4(0u, 0u, 0u, 0u);
   uint4* cm_dst = nullptr;
-  Stat st = scan_chunk<T, ALIGNED, false, STAT_SUM>(row, begin, end, C1, -1, 0, 0, 0, 0, 0, [&] {
+  Stat st = scan_chunk<T, ALIGNED, false, STAT_SUM, EARLY>(row, begin, end, C1, -1, 0, 0, 0, 0, 0, [&] {
     const int at = (row_i * p.n_chunks + ch) * (SPACE_VERIFY_THREADS - 32) + (int)threadIdx.x - 32;
     if (EARLY && threadIdx.x >= 32 && at < commit_pieces(p.cm, p.k) && commit_fits(p.cm, Lc))
       cm_dst = commit_piece<PAGED>(p.cm, b, Lc, at, cm_val);
