@@ -65,7 +65,8 @@ struct AttnParams {
   float* part;                         // [slots][ROWS*(DH+2)]
   int* err;                            // one word: first timeout site
   int2* desc;                          // [B*H_kv*n_mblocks] {first partial slot, number of partials} of each cut (read by the merge kernel)
-  int* owner;                          // [grid] (sequence, kv head) whose last piece this thread block computed, or -1
+  int4* owner;                         // [grid] the cut whose last piece this thread block computed: {(sequence, kv head) or -1,
+                                       // its descriptor}
   int merge_by_owner;                  // the merge grid is indexed by attention thread block, not by (sequence, head)
   int* arrived;                        // [B*H_kv*n_mblocks] pieces of a cut whose partial is stored (self-resetting)
   // Eq. 5 per (query column, block key), worked out by the host once per call: bit q of
@@ -751,7 +752,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
     // same control flow so that the block-wide barriers below always match up;
     // once the abort flag is set all later waits return at once and the block drains.
     bool ok = true;
-    int own = -1;                                          // item whose last piece of a cut this block holds
+    int4 own = make_int4(-1, 0, 0, 0);                     // the cut whose last piece this block holds
     while (part.next(sg)) {
       const int n_keys = sg.L + p.n_q;
 #pragma unroll
@@ -961,8 +962,9 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
           const int g0 = group_of(f0, W, NG);               // group of the first tile
           cut_d = make_int2(item + g0, group_of(f0 + sg.T - 1, W, NG) - g0 + 1);
         }
-        if (!p.pieces) p.desc[(size_t)item * p.n_mblocks + mb] = cut_d;
-        if (!whole && sg.tile_at(sg.n - 1) == sg.T - 1) own = item;   // the piece with the pair's last tile; at most one per block
+        if (!p.pieces && !p.merge_by_owner) p.desc[(size_t)item * p.n_mblocks + mb] = cut_d;
+        // the piece with the pair's last tile; at most one per block
+        if (!whole && sg.tile_at(sg.n - 1) == sg.T - 1) own = make_int4(item, cut_d.x, cut_d.y, 0);
       }
       // Row sums first, while the last O^T product still runs.  Every thread holds
       // its key's share of ncol rows; a halving butterfly over the warp leaves lane r with
@@ -1086,7 +1088,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
         merge_if_last<DH>(p, sg.b, sg.h, i0, m_valid, mb, cut_d, p.arrived + (size_t)item * p.n_mblocks + mb,
                           reinterpret_cast<float*>(sm + S::P_OFF), 2 * S::P_PART / 4, sidx, 256, [] { soft_sync(); });
     }
-    if (!p.pieces && sidx == 0) p.owner[blockIdx.x] = own;
+    if (p.merge_by_owner && sidx == 0) p.owner[blockIdx.x] = own;
   }
   if (clustered && cl_n > 1)
     cluster_merge<DH>(p, cl_b, cl_h, i0, m_valid, cl_piece, p.pieces, cl_n, mb, sm_base + S::P_OFF, sm_base + S::XQ_OFF,
@@ -1119,18 +1121,24 @@ __global__ void __launch_bounds__(128) attn_merge_kernel(const AttnParams p) {
   constexpr int C4 = DH / 4;
   // Large batches: one grid column per attention thread block (each holds the last
   // piece of at most one cut); small ones: one per (sequence, head, row block).
-  int item = blockIdx.x / p.n_mblocks;
+  int item = blockIdx.x / p.n_mblocks, b, h, n;
   const int mb = blockIdx.x % p.n_mblocks;
+  int2 d;
   if (p.merge_by_owner) {
-    item = p.owner[blockIdx.x];
-    if (item < 0) return;
+    // (one round trip to the partials' place; with the block's cut looked up by number in the descriptors it was two:
+    // sixteen ragged sequences 130.2 -> 129.2, 24 short paged ones 89.4 -> 89.1 us a step)
+    const int4 o = __ldcg(p.owner + blockIdx.x);
+    if (o.x < 0) return;
+    item = o.x; b = item / p.H_kv; h = item % p.H_kv; d = make_int2(o.y, o.z);
+    n = d.y;
+  } else {
+    b = item / p.H_kv; h = item % p.H_kv;
+    // both loads are issued before either is tested: one round trip, not two
+    const int L = __ldcg(p.kv_len + b);
+    d = __ldcg(p.desc + (size_t)item * p.n_mblocks + mb);
+    if (L < 0 || (int64_t)L + p.n_q > p.s_cap) return;
+    n = d.y;
   }
-  const int b = item / p.H_kv, h = item % p.H_kv;
-  // both loads are issued before either is tested: one round trip, not two
-  const int L = __ldcg(p.kv_len + b);
-  const int2 d = __ldcg(p.desc + (size_t)item * p.n_mblocks + mb);
-  if (L < 0 || (int64_t)L + p.n_q > p.s_cap) return;
-  const int n = d.y;
   TLM(2);
   if (n <= 1) return;                                       // written directly by the main kernel
   const int i0 = mb * p.rows_per_mb;
@@ -1263,7 +1271,7 @@ int launch_attn_tensor(space_ctx* ctx, const space_attn_args* a, const uint64_t*
   p.part = ctx->attn_part; p.err = ctx->counters + 3 * cfg.max_batch;
   p.arrived = ctx->arrived;
   p.desc = reinterpret_cast<int2*>(ctx->merge_cnt);
-  p.owner = ctx->merge_cnt + (size_t)cfg.max_batch * cfg.n_kv_heads * 8 * 2;
+  p.owner = reinterpret_cast<int4*>(ctx->merge_cnt + (size_t)cfg.max_batch * cfg.n_kv_heads * 8 * 2);
   p.merge_by_owner = (a->batch * p.H_kv * p.n_mblocks > pl.n_ctas) ? 1 : 0;
   if (p.n_mblocks > 2) return SPACE_E_UNSUPPORTED;         // (cannot happen: at most 64 block rows, at least 32 per block)
   if (ctx->visq_k != a->k || ctx->visq_variant != a->mask_variant) {

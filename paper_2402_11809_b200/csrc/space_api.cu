@@ -42,8 +42,8 @@ Carve carve(const space_config* c, int sm_count) {
   off += align_up(attn_tensor_partial_floats(c, sm_count, &v.part_slots) * sizeof(float), 256);
   v.counters = off; off += align_up((size_t)(3 * c->max_batch + 4) * sizeof(int), 256);
   v.merge_cnt = off;
-  // up to 8 row blocks, one {first, count} pair each; then one word per thread block of the attention grid
-  off += align_up((size_t)c->max_batch * c->n_kv_heads * 8 * sizeof(int2) + (size_t)(sm_count + 8) * sizeof(int), 256);
+  // up to 8 row blocks, one {first, count} pair each; then four words per thread block of the attention grid
+  off += align_up((size_t)c->max_batch * c->n_kv_heads * 8 * sizeof(int2) + (size_t)(sm_count + 8) * sizeof(int4), 256);
   // pieces of a cut that are stored, per (sequence, kv head, row block)
   v.arrived = off; off += align_up((size_t)c->max_batch * c->n_kv_heads * 8 * sizeof(int), 256);
   v.vtopk = off; off += align_up(verify_filter_scratch_bytes(c->max_batch, c->k_max), 256);
