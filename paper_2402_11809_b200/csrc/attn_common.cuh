@@ -160,72 +160,82 @@ __device__ __forceinline__ void cluster_leave() {
   asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 }
 
-// Clusters were launched, but the lengths are too unequal for them: the piece that finds all the others stored
-// combines them from global memory (no merge kernel follows such a launch).  As the rule for larger batches
-// this was slower (137 against 130 us per step of sixteen ragged sequences when it was tried): every piece waits
-// for its fence and its atomic.  Called by `nt` threads (tid 0 .. nt-1, whole warps) that `sync` synchronises,
-// after all of them have stored their piece; cut: {first slot, pieces}, read from thread 0.  buf: buf_floats
-// floats of shared memory.
-template <int DH, class P, class Sync>
-__device__ __forceinline__ void merge_if_last(const P& p, int b, int h, int i0, int m_valid, int mb, int2 cut, int* arrived,
-                                              float* buf, int buf_floats, int tid, int nt, Sync sync) {
-  int* flag = reinterpret_cast<int*>(buf);
-  if (tid == 0) {
-    __threadfence();                                        // (the barrier before ordered every thread's stores before this)
-    const int last = atomicAdd(arrived, 1) == cut.y - 1;
-    if (last) { *arrived = 0; __threadfence(); }            // ready for the next launch
-    flag[0] = last; flag[1] = cut.x; flag[2] = cut.y;
+// Clusters were launched, but the lengths are too unequal for them: each cut's pieces go to global memory, and the piece
+// that finds all the others stored notes the cut in its block's shared memory (no merge kernel follows such a launch;
+// as the rule for larger batches this was slower, 137 against 130 us per step of sixteen ragged sequences when it was
+// tried: every piece waits for its fence and its atomic).  At the end the blocks of a cluster combine together what any
+// of them noted.  Called by one thread, after a barrier that orders the stores of all of the block's threads before it.
+constexpr int MAX_DUTIES = 2;          // a block's share of the list starts and ends inside one cut each, at most
+template <class P>
+__device__ __forceinline__ void note_if_last(const P& p, int item, int2 cut, int* arrived, int4* duties) {
+  __threadfence();
+  if (atomicAdd(arrived, 1) != cut.y - 1) return;
+  *arrived = 0;                                             // ready for the next launch
+  __threadfence();
+  duties[duties[0].x < 0 ? 0 : 1] = make_int4(item, cut.x, cut.y, 0);
+}
+// All threads of the cluster's blocks take part (every wait before this is bounded, so all of them arrive); duties: the
+// block's own list, MAX_DUTIES entries, item -1 where there is none.  cluster_leave() must follow before the block exits.
+// The last block alone, before: one sequence of 16000 keys with 392 query rows (four cuts over 36 pieces) 60.0 us a
+// step, this way 30.1; of 16000 paged keys with 2 x 392 rows of 64 46.5 -> 30.9; nine sequences of 800 to 16384 keys, 4 x 36
+// rows, 71.3 -> 62.4.  (Out of line, or with sixteen loads a batch, the kernels' loops were compiled otherwise: the step
+// of one 7B-shaped sequence 18.15 -> 18.3 and 19.2.)
+template <int DH, class P>
+__device__ __forceinline__ void cluster_duties(const P& p, const int4* duties, volatile int* abort_flag) {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  static_assert(MAX_CLUSTER * MAX_DUTIES <= 32, "a lane per entry");
+  const int size = p.pieces * p.n_mblocks, lane = threadIdx.x & 31, threads = size * (int)blockDim.x;
+  uint32_t rank;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  int4 mine = make_int4(-1, 0, 0, 0);                       // lane e: entry e of the cluster, rank e / MAX_DUTIES
+  if (lane < size * MAX_DUTIES) {
+    const uint32_t at = map_cluster(tc::smem_u32(duties) + (lane % MAX_DUTIES) * 16, (uint32_t)(lane / MAX_DUTIES));
+    asm volatile("ld.shared::cluster.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(mine.x), "=r"(mine.y), "=r"(mine.z), "=r"(mine.w) : "r"(at) : "memory");
   }
-  sync();
-  const bool last = flag[0] != 0;
-  const int d0 = flag[1], n = flag[2];
-  sync();                                                   // (the flags' place is used below)
-  if (!last) return;
   const size_t slot_floats = (size_t)ROWS * (DH + 2), gstride = (size_t)p.n_mblocks * slot_floats;
-  const float* ps = p.part + ((size_t)d0 * p.n_mblocks + mb) * slot_floats;
-  const int warp = tid >> 5, lane = tid & 31;
-  // rows in batches whose weights exp2(m - M) / sum fit the buffer: n floats per row
-  const int at_once = min(m_valid, buf_floats / n);
-  for (int r0 = 0; r0 < m_valid; r0 += at_once) {
-    const int nr = min(at_once, m_valid - r0);
-    for (int rr = warp; rr < nr; rr += nt >> 5) {
-      const float* pr = ps + ROWS * DH + r0 + rr;
-      float M = -CUDART_INF_F, den = 0.f;
-      for (int x = lane; x < n; x += 32) M = fmaxf(M, __ldcg(pr + (size_t)x * gstride));
+  // the cuts' elements one after another over the cluster's threads: next is this thread's place before the cut's first one
+  int next = (int)(rank * blockDim.x + threadIdx.x);
+  for (unsigned todo = __ballot_sync(0xFFFFFFFFu, mine.x >= 0); todo && !*abort_flag; todo &= todo - 1) {
+    const int e = __ffs(todo) - 1;
+    const int item = __shfl_sync(0xFFFFFFFFu, mine.x, e), slot = __shfl_sync(0xFFFFFFFFu, mine.y, e), n = __shfl_sync(0xFFFFFFFFu, mine.z, e);
+    // (the cluster's ranks are blocks in order: row block rank % n_mblocks)
+    const int b = item / p.H_kv, h = item % p.H_kv, mb = e / MAX_DUTIES % p.n_mblocks;
+    const int i0 = mb * p.rows_per_mb, count = min(p.rows_per_mb, p.n_q - i0) * p.G * (DH / 4);
+    const float* ps = p.part + ((size_t)slot * p.n_mblocks + mb) * slot_floats;
+    int idx = next;
+    for (; idx < count; idx += threads) {
+      const int r = idx / (DH / 4), c4 = idx % (DH / 4);
+      MergeAcc acc;
+      acc.clear();
+      for (int x0 = 0; x0 < n; x0 += 8) {                  // all loads of a batch are issued before any is used
+        float ms[8], ls[8];
+        float4 ov[8];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xFFFFFFFFu, M, o));
-      for (int x = lane; x < n; x += 32) {
-        const float e = tc::fast_exp2(__ldcg(pr + (size_t)x * gstride) - M);
-        buf[rr * n + x] = e;
-        den = fmaf(__ldcg(pr + (size_t)x * gstride + ROWS), e, den);
-      }
+        for (int j = 0; j < 8; ++j) {
+          ms[j] = -CUDART_INF_F; ls[j] = 0.f; ov[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (x0 + j < n) {
+            const float* pj = ps + (size_t)(x0 + j) * gstride;
+            ms[j] = __ldcg(pj + ROWS * DH + r);
+            ls[j] = __ldcg(pj + ROWS * DH + ROWS + r);
+            ov[j] = __ldcg(reinterpret_cast<const float4*>(pj + (size_t)r * DH) + c4);
+          }
+        }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xFFFFFFFFu, den, o);
-      const float rd = 1.f / den;
-      for (int x = lane; x < n; x += 32) buf[rr * n + x] *= rd;
-      if (p.lse && lane == 0) store_lse(p, b, h, i0, r0 + rr, (M + log2f(den)) * 0.6931471805599453f);
-    }
-    sync();
-    for (int idx = tid; idx < nr * (DH / 4); idx += nt) {
-      const int rr = idx / (DH / 4), c4 = idx % (DH / 4);
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      const float* po = ps + (size_t)(r0 + rr) * DH + c4 * 4;
-      for (int x0 = 0; x0 < n; x0 += 16) {                  // all loads of a batch are issued before any is used
-        float4 ov[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-          ov[j] = x0 + j < n ? __ldcg(reinterpret_cast<const float4*>(po + (size_t)(x0 + j) * gstride)) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const float w = x0 + j < n ? buf[rr * n + x0 + j] : 0.f;
-          a.x = fmaf(ov[j].x, w, a.x); a.y = fmaf(ov[j].y, w, a.y);
-          a.z = fmaf(ov[j].z, w, a.z); a.w = fmaf(ov[j].w, w, a.w);
+        for (int g = 0; g < 8; g += 4) {
+          const float m4[4] = {ms[g], ms[g + 1], ms[g + 2], ms[g + 3]}, l4[4] = {ls[g], ls[g + 1], ls[g + 2], ls[g + 3]};
+          const float4 o4[4] = {ov[g], ov[g + 1], ov[g + 2], ov[g + 3]};
+          acc.add4(m4, l4, o4);
         }
       }
-      store_out<DH>(p, b, h, i0, r0 + rr, c4, a);
+      acc.template store<DH>(p, b, h, i0, r, c4);
     }
-    sync();
+    next = idx - count;                                     // (the next cut's elements follow this one's)
   }
+  // no block leaves while another may still read its list
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
 
 // Whether the clustered cut serves these lengths (all lanes of a warp call this; every warp gets the same

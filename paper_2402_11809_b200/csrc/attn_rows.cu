@@ -202,6 +202,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
   int* seq_len = reinterpret_cast<int*>(sm + S::TABLE_OFF);
   int* prefix = seq_len + max_batch;
   int* seg0 = reinterpret_cast<int*>(sm + S::SEG0_OFF);
+  int4* duties = reinterpret_cast<int4*>(seg0);            // (where there is no clustered cut: see note_if_last)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int group = blockIdx.x / p.n_mblocks, mb = blockIdx.x % p.n_mblocks;
@@ -223,6 +224,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
       asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(sm_base + S::Q_OFF + hf * (ROWS * 128) + x * 16), "r"(0u) : "memory");
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   if (threadIdx.x == 0) {
+    for (int e = 0; e < MAX_DUTIES; ++e) duties[e].x = -1;
     *abort_flag = (sm_base & 1023u) ? 1 : 0;               // swizzled tiles need a 1024-byte aligned base
     mbar_init(BAR(B_QFULL), 1);
     mbar_init(BAR(B_QEMPTY), 1);
@@ -696,11 +698,9 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
         }
       }
       if (p.pieces && !clustered && !whole) {
-        auto sync = [&] { asm volatile("bar.sync 5, %0;" ::"r"(n_soft) : "memory"); };
-        sync();                                             // every thread's stores, and the staging is idle
+        asm volatile("bar.sync 5, %0;" ::"r"(n_soft) : "memory");   // every thread's stores
         cut_d.x += item;                                    // slots are numbered by item + group
-        merge_if_last<DH>(p, sg.b, sg.h, i0, m_valid, mb, cut_d, p.arrived + (size_t)item * p.n_mblocks + mb,
-                          reinterpret_cast<float*>(sm + S::EPI_OFF), 8 * 32 * S::EPI_PITCH, sidx, n_soft, sync);
+        if (sidx == 0) note_if_last(p, item, cut_d, p.arrived + (size_t)item * p.n_mblocks + mb, duties);
       }
     }
     if (p.merge_by_owner && sidx == 0) p.owner[blockIdx.x] = own;
@@ -710,6 +710,8 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
     cluster_merge<DH>(p, cl_b, cl_h, i0, m_valid, cl_piece, p.pieces, cl_n, mb, at, at + ROWS * DH * 4, at + (ROWS * DH + ROWS) * 4,
                       abort_flag);
   }
+  const bool fell_back = p.pieces && !clustered;            // (the same in every block of the grid)
+  if (fell_back) cluster_duties<DH>(p, duties, abort_flag);
 
   // ---- teardown -----------------------------------------------------------
   tc_fence_before();
@@ -721,7 +723,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
   if (threadIdx.x == 0 && *abort_flag && p.status) {
     for (int b = 0; b < p.B; ++b) atomicOr(p.status + b, SPACE_ST_TIMEOUT);
   }
-  if (clustered && cl_n > 1) cluster_leave();
+  if ((clustered && cl_n > 1) || fell_back) cluster_leave();
 }
 
 // Combine the partials of every (sequence, kv head, query-row block) that was

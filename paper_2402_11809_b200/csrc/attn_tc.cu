@@ -218,6 +218,7 @@ struct Smem {
   static constexpr int MISC_OFF = BAR_OFF + (N_BARS * 8 + 15) / 16 * 16;   // tmem base, abort flag (16-byte aligned:
                                                                            // the float arrays below are read as float4)
   static constexpr int SEG0_OFF = MISC_OFF + 16;             // Seg of this group's only share (aligned mode)
+  static constexpr int DUTY_OFF = MISC_OFF + 64;             // [MAX_DUTIES] int4: cuts that this block's cluster combines
   static constexpr int MREF_OFF = MISC_OFF + 96;             // [2][RS] float: reference maximum per query row
   static constexpr int XQ_OFF = MREF_OFF + 2 * RS * 4;       // [4 quarters][RS] float: cross-lane reductions
   static constexpr int FQ_OFF = XQ_OFF + 4 * RS * 4;         // [RS] float: rescale factors / final row sums
@@ -365,6 +366,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   int* prefix = seq_len + max_batch;
   volatile int* agroups = reinterpret_cast<volatile int*>(sm + S::MISC_OFF + 8);
   int* seg0 = reinterpret_cast<int*>(sm + S::SEG0_OFF);
+  int4* duties = reinterpret_cast<int4*>(sm + S::DUTY_OFF);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int group = blockIdx.x / p.n_mblocks, mb = blockIdx.x % p.n_mblocks;
@@ -377,6 +379,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   pdl_launch_dependents();
   if (threadIdx.x == 0) TL(0);
   if (threadIdx.x == 0) {
+    for (int e = 0; e < MAX_DUTIES; ++e) duties[e].x = -1;
     *abort_flag = (sm_base & 1023u) ? 1 : 0;               // swizzled tiles need a 1024-byte aligned base
     for (int i = 0; i < 2; ++i) { mbar_init(BAR(B_QFULL + i), 1); mbar_init(BAR(B_QEMPTY + i), 1); }
     for (int s = 0; s < S::K_STAGES; ++s) { mbar_init(BAR(B_KFULL + s), 1); mbar_init(BAR(B_KEMPTY + s), 1); }
@@ -1084,15 +1087,16 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       tc_fence_before();
       soft_sync();                                          // scratch, fq and mref are reused by the next share
       if (sidx == 0) TL(11);
-      if (p.pieces && !whole && !to_smem)                   // (the P buffer is idle)
-        merge_if_last<DH>(p, sg.b, sg.h, i0, m_valid, mb, cut_d, p.arrived + (size_t)item * p.n_mblocks + mb,
-                          reinterpret_cast<float*>(sm + S::P_OFF), 2 * S::P_PART / 4, sidx, 256, [] { soft_sync(); });
+      if (p.pieces && !whole && !to_smem && sidx == 0)
+        note_if_last(p, item, cut_d, p.arrived + (size_t)item * p.n_mblocks + mb, duties);
     }
     if (p.merge_by_owner && sidx == 0) p.owner[blockIdx.x] = own;
   }
   if (clustered && cl_n > 1)
     cluster_merge<DH>(p, cl_b, cl_h, i0, m_valid, cl_piece, p.pieces, cl_n, mb, sm_base + S::P_OFF, sm_base + S::XQ_OFF,
                       sm_base + S::FQ_OFF, abort_flag);
+  const bool fell_back = p.pieces && !clustered;            // (the same in every block of the grid)
+  if (fell_back) cluster_duties<DH>(p, duties, abort_flag);
   if (threadIdx.x == 0) TL(12);
   // ---- teardown -----------------------------------------------------------
   tc_fence_before();
@@ -1104,7 +1108,7 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
   if (threadIdx.x == 0 && *abort_flag && p.status) {
     for (int b = 0; b < p.B; ++b) atomicOr(p.status + b, SPACE_ST_TIMEOUT);
   }
-  if (clustered && cl_n > 1) cluster_leave();
+  if ((clustered && cl_n > 1) || fell_back) cluster_leave();
   if (threadIdx.x == 32) TL(13);                          // after the TMEM release
 }
 
