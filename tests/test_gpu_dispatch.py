@@ -362,3 +362,65 @@ def test_filtered_one_launch_or_two(B, H, Bn, k, V, dtype, launches):  # noqa: F
     new_len, _, _ = commit_step(x["k_cache"], x["v_cache"], x["kv_len"], r["n_accept"], k)       # (in place)
     assert np.array_equal(ds.kv_len_out.cpu().numpy(), new_len)
     assert np.array_equal(H.bf16_to_bits(ds.k_cache), x["k_cache"]) and np.array_equal(H.bf16_to_bits(ds.v_cache), x["v_cache"])
+
+
+# Clusters launched for lengths that are too unequal (or too long for the pieces a cluster can hold) for them: every cut of
+# the list over the grid is combined by the whole cluster of the block that finds its last piece.  Four row blocks of one
+# pair over all blocks, two pairs of a smaller head, one long sequence among short ones.  Twice: the counters are back
+# where they were, and the pieces are added in a fixed order.
+@pytest.mark.parametrize("k,d,H_q,H_kv,lens,paged", [(6, 128, 8, 1, (9000,), False), (6, 64, 16, 2, (9001,), True),
+                                                     (5, 64, 4, 4, (16000, 800, 127, 640, 0), False),
+                                                     (7, 128, 2, 1, (9000, 300), True)])
+def test_attention_cuts_combined_by_the_cluster(B, H, k, d, H_q, H_kv, lens, paged):  # noqa: F811
+    cfg = _small_cfg(k, (0, max(lens)), d=d, H_q=H_q, H_kv=H_kv, Bn=len(lens), V=64, seed=k + d + len(lens))
+    x = workloads.make_step_inputs(cfg)
+    x["kv_len"][:] = lens
+    y = workloads.to_pages(x) if paged else x
+    ctx = H.make_context(cfg, y)
+    ds = H.DeviceStep(cfg, y)
+    n0 = ctx.launch_count
+    ds.attn(ctx)
+    assert ctx.launch_count - n0 == 1 and not ds.status.any()    # (no merge kernel)
+    got = ds.out.clone()
+    ds.out.fill_(float("nan"))
+    ds.attn(ctx)
+    assert torch.equal(got, ds.out)
+    got = got.cpu().numpy().astype(np.float64)
+    for b, L in enumerate(lens):
+        for h in (0, H_q - 1):
+            G = H_q // H_kv
+            ref, _ = attention_head(x["q"][b, :, h], x["k_cache"][b, h // G], x["v_cache"][b, h // G], L, k, x["scale"])
+            H.check_attention(got[b:b + 1, :, h], ref[None], f"sequence {b} head {h}")
+
+
+# Sweeps of a block that lie in its chunk as a whole and the one that does not, at the edges (a sweep is 8192 bf16 or 4096
+# f32 logits), in launches of more blocks than three per SM hold (576 and 640 of one chunk), with the commit on board; and
+# the two launches of sampling.
+@pytest.mark.parametrize("V,dtype", [(296, "bf16"), (8192, "bf16"), (8200, "bf16"), (16380, "bf16"), (24584, "bf16"),
+                                     (4096, "f32"), (4100, "f32"), (12284, "f32")])
+@pytest.mark.parametrize("mode,Bn,k,paged", [("greedy", 16, 5, False), ("greedy", 40, 3, True), ("sample", 3, 4, False)])
+def test_verify_sweeps_and_many_blocks(B, H, mode, Bn, k, paged, V, dtype):  # noqa: F811
+    from oracle.commit import commit_step
+    cfg = _small_cfg(k, (5, 150), H_q=2, H_kv=2, d=64, Bn=Bn, V=V, dtype=dtype, seed=V % 97 + Bn)
+    x = workloads.make_step_inputs(cfg)
+    y = workloads.to_pages(x) if paged else x
+    ctx = H.make_context(cfg, y)
+    ds = H.DeviceStep(cfg, y)
+    if mode == "sample":
+        v = ctx.verify_args(ds.logits, ds.cand, ds.cand_prob, ds.kv_len, ds.n_accept, ds.out_tokens, ds.n_out, ds.next_cand,
+                            ds.next_cand_prob, ds.finished, k, mode=B.MODE_SAMPLE, temperature=0.9, seed=5, seq_id=ds.seq_id,
+                            status=ds.status)
+        ctx.space_verify(v)
+        r = verify_step(x["logits"], x["cand"], x["cand_prob"], k, "sample", temperature=0.9, seed=5, seq_id=x["seq_id"],
+                        kv_len=x["kv_len"])
+        assert _check_verify(ds, r, k, sample=True).sum() <= 1
+        return
+    ds.verify_commit(ctx)
+    r = verify_step(x["logits"], x["cand"], x["cand_prob"], k, "greedy")
+    assert not _check_verify(ds, r, k).any()
+    new_len, _, _ = commit_step(x["k_cache"], x["v_cache"], x["kv_len"], r["n_accept"], k)       # (in place)
+    assert np.array_equal(ds.kv_len_out.cpu().numpy(), new_len)
+    got = H.bf16_to_bits(ds.k_cache)
+    for b in range(Bn):
+        rows = np.concatenate([got[pg] for pg in y["page_table"][b][: -(-int(new_len[b]) // 128)]], axis=1) if paged else got[b]
+        assert np.array_equal(rows[:, :int(new_len[b])], x["k_cache"][b][:, :int(new_len[b])]), b
