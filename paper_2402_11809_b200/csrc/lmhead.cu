@@ -50,7 +50,9 @@ constexpr int LM_MAX_N = 256;               // block rows of the whole batch, pa
 constexpr int LM_TOK = 128;                 // tokens per accumulator with the tokens on M
 constexpr int LM_XP_PITCH = 36;             // floats per row of a warp's transposing buffer (8 rows of 32 tokens)
 // Which block rows a launch projects: all of them, the target rows of every sequence (row b(k+1)+t), or
-// the mask rows of every sequence's group i* (row bk+o-1; i* is the launch before's result).
+// the mask rows of every sequence's group i* (row bk+o-1; i* is the launch before's result) and, in sampling mode, target
+// row i* of every sequence once more (row Bk+b): the extra token is drawn there, so that only one target row per
+// sequence needs noise, not every one that could turn out to be row i*.
 enum { LM_ALL = 0, LM_TARGETS = 1, LM_MASKS = 2 };
 constexpr int64_t LM_GATHER_ELEMS = 128 * 8192;   // mask rows gathered for the second phase
 constexpr uint64_t LM_WAIT_NS = 1000000000ull;
@@ -71,6 +73,7 @@ struct LmParams {
   int tail_rows;              // rows of the second tensor map's box
   int kbs;                    // 64-element slices of the hidden dimension per stage
   int backwards;              // a box's stages are taken from the hidden dimension's end (see launch_group)
+  int sums;                   // whether any row's sum of exponentials is asked for
   int n_noisy, noise_tok;     // sampling: rows that draw a token, tokens of a box whose noise is tabulated (a multiple of 16)
   int eos_id;
   int mode, resample;         // SPACE_MODE_*, SPACE_RESAMPLE_*
@@ -173,6 +176,20 @@ __device__ __forceinline__ void fold(float& m, float& s, int& idx, const float (
   s += (a0 + a1) + (a2 + a3);
 }
 
+template <int N>
+__device__ __forceinline__ void fold_max(float& m, int& idx, const float (&z)[N], int x0) {
+  float cm = z[0];
+#pragma unroll
+  for (int j = 1; j < N; ++j) cm = fmaxf(cm, z[j]);
+  if (cm > m) {
+    int at = N - 1;
+#pragma unroll
+    for (int j = N - 2; j >= 0; --j) at = (z[j] == cm) ? j : at;
+    idx = x0 + at;
+    m = cm;
+  }
+}
+
 // What an epilogue thread keeps of one block row in sampling mode, and what it has to know of the row.
 struct RowNoisy {
   float gs, gz; int gidx;     // best noisy score so far, the logit that has it, its token
@@ -237,7 +254,9 @@ __device__ __forceinline__ bool row_place(const LmParams& p, int row, int& b, in
     return true;
   }
   if (p.phase == LM_TARGETS) { b = row / k1; t = row - b * k1; o = 0; return true; }
-  b = row / p.k; o = row - b * p.k + 1; t = p.n_accept[b];
+  if (row < p.B * p.k) { b = row / p.k; o = row - b * p.k + 1; }
+  else { b = row - p.B * p.k; o = 0; }
+  t = max(0, min(p.n_accept[b], p.k));                      // (a first pass that gave up has left it as it was)
   return true;
 }
 
@@ -253,10 +272,11 @@ __device__ __forceinline__ RowConst row_const(const LmParams& p, int row) {
   const int L = p.kv_len ? p.kv_len[b] : 0;
   if (o == 0) {
     r.purpose = PURPOSE_TOKEN; r.pos = (uint32_t)(L + t + 1);
-    r.noisy = (literal || p.phase != LM_ALL) ? row : b * (p.k + 1) + t;
+    if (p.phase != LM_TARGETS) r.noisy = literal ? row : p.phase == LM_MASKS ? b : b * (p.k + 1) + t;
     if (t < p.k) {
-      r.cand_tok = p.cand[b * p.k + t];
-      if (!literal && p.cand_prob[b * p.k + t] == 1.0f) r.exclude = r.cand_tok;   // residual of a point mass
+      const int tok = p.cand[b * p.k + t];
+      if (p.phase != LM_MASKS) r.cand_tok = tok;
+      if (!literal && p.cand_prob[b * p.k + t] == 1.0f) r.exclude = tok;          // residual of a point mass
     }
   } else if (literal) {
     r.purpose = PURPOSE_DRAFT; r.pos = (uint32_t)(L + t + 1 + o);
@@ -480,7 +500,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         const int y = at / n4, q = at - y * n4;
         // row of the y-th noisy one (row_const says which those are)
         const int k1 = p.k + 1;
-        const int row = (p.phase != LM_ALL || p.resample == SPACE_RESAMPLE_PAPER_LITERAL) ? y : y / k1 * p.n_q + y % k1 * k1;
+        const int row = p.resample == SPACE_RESAMPLE_PAPER_LITERAL ? y : p.phase == LM_MASKS ? p.B * p.k + y : y / k1 * p.n_q + y % k1 * k1;
         reinterpret_cast<float4*>(noise + y * noise_pitch)[q] = noise4((uint32_t)(row0 >> 2) + q, rowc[row], p.key0, p.key1);
       }
       epi_sync();
@@ -611,7 +631,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
             float z[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) z[j] = (j < nv) ? __uint_as_float(v[j]) : LM_NEG;
-            fold(m0, s0, i0, z, row0 + c0, p.c_t);
+            if (!sample || p.sums) fold(m0, s0, i0, z, row0 + c0, p.c_t);
+            else fold_max(m0, i0, z, row0 + c0);
             if (sample)
               fold_noisy(n0, rc, z, row0 + c0, nv, p.c_t, p.key0, p.key1,
                          c0 < p.noise_tok ? noise + rc.noisy * noise_pitch + c0 : nullptr);   // (both multiples of 16)
@@ -745,6 +766,19 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           gz_out = gz;
           return gi;
         };
+        // emitted tokens of a sequence (one warp): the candidates before i*, then the draw of row i*
+        auto emit = [&](int b, int i_star, int cv) {
+          float gz_unused;
+          const int bonus = best_noisy(p.phase == LM_ALL ? target_row(b, i_star) : p.B * p.k + b, gz_unused);
+          const int j = lane;
+          const int c_j = __shfl_sync(0xFFFFFFFFu, cv, min(j, p.k - 1));
+          const int tok = (j < i_star) ? c_j : (j == i_star ? bonus : -1);
+          const bool is_eos = p.eos_id >= 0 && j <= i_star && tok == p.eos_id;
+          const unsigned eos_mask = __ballot_sync(0xFFFFFFFFu, is_eos && j < k1);
+          const int n_out = eos_mask ? __ffs(eos_mask) - 1 : i_star + 1;
+          if (j < k1) p.out_tokens[b * k1 + j] = (j < n_out) ? tok : -1;
+          if (j == 0) { p.n_out[b] = n_out; p.finished[b] = (uint8_t)(eos_mask != 0); }
+        };
         if (with_targets) {
         sum_rows(false);                                   // target rows t = 0..k-1 of every sequence
         for (int b = ew; b < p.B; b += LM_EPI) {
@@ -765,25 +799,16 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           }
           const unsigned acc_mask = __ballot_sync(0xFFFFFFFFu, okc);
           const int i_star = __ffs(~acc_mask) - 1;          // first candidate that is not accepted (k when all are)
-          float gz_unused;
-          const int bonus = best_noisy(target_row(b, i_star), gz_unused);   // a: the draw of the case i* (row i*)
-          const int j = lane;
-          const int c_j = __shfl_sync(0xFFFFFFFFu, cv, min(j, p.k - 1));
-          const int tok = (j < i_star) ? c_j : (j == i_star ? bonus : -1);
-          const bool is_eos = p.eos_id >= 0 && j <= i_star && tok == p.eos_id;
-          const unsigned eos_mask = __ballot_sync(0xFFFFFFFFu, is_eos && j < k1);
-          const int n_out = eos_mask ? __ffs(eos_mask) - 1 : i_star + 1;
-          if (j < k1) p.out_tokens[b * k1 + j] = (j < n_out) ? tok : -1;
-          if (j == 0) {
+          if (p.phase == LM_ALL) emit(b, i_star, cv);
+          if (lane == 0) {
             istar[b] = i_star;
             p.n_accept[b] = i_star;
-            p.n_out[b] = n_out;
-            p.finished[b] = (uint8_t)(eos_mask != 0);
             if (p.status && bad) atomicOr(p.status + b, SPACE_ST_BAD_CANDIDATE);
           }
         }
         } else {
-          for (int b = et; b < p.B; b += LM_EPI_T) istar[b] = p.n_accept[b];
+          for (int b = et; b < p.B; b += LM_EPI_T) istar[b] = max(0, min(p.n_accept[b], p.k));
+          for (int b = ew; b < p.B; b += LM_EPI) emit(b, max(0, min(p.n_accept[b], p.k)), lane < p.k ? cand_s[b * p.k + lane] : -1);
         }
         epi_sync();
         if (with_masks && !literal) {                      // point-mass drafts: arg-max of mask row (i*, j+1), P_c = 1
@@ -830,7 +855,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
           if (p.status && bad) atomicOr(p.status + b, SPACE_ST_BAD_CANDIDATE);
         }
       }
-      if (!with_targets) for (int b = et; b < p.B; b += LM_EPI_T) istar[b] = p.n_accept[b];
+      if (!with_targets) for (int b = et; b < p.B; b += LM_EPI_T) istar[b] = max(0, min(p.n_accept[b], p.k));
       epi_sync();
       // sums of the mask rows of group i*: (sequence, mask row, range) triples spread over the threads
       const int total = with_masks ? p.B * p.k * G : 0;
@@ -896,15 +921,15 @@ size_t lmhead_partial_bytes(int sm_count) {
 
 namespace {
 
-// Mask rows (i*, 1..k) of every sequence, one thread block per row, next to one another for the second phase's
-// box.  (Fetching them by a box per sequence instead, eight rows of 128 bytes each, paced the whole phase:
+// Mask rows (i*, 1..k) of every sequence, then target row i* of every one where the grid asks for it, one thread block per
+// row, next to one another for the second phase's box.  (Fetching them by a box per sequence instead, eight rows of 128 bytes each, paced the whole phase:
 // 406 us under ncu for 16 sequences, D = 4096, V = 128256.)
-__global__ void __launch_bounds__(256) lm_gather_kernel(const uint4* hidden, int64_t row_stride, int n_q, int k, int vecs,
+__global__ void __launch_bounds__(256) lm_gather_kernel(const uint4* hidden, int64_t row_stride, int n_q, int k, int n_masks, int vecs,
                                                         const int32_t* n_accept, uint4* dst) {
   pdl_launch_dependents();
   pdl_wait();
-  const int b = blockIdx.x / k, o = blockIdx.x - b * k + 1;
-  const uint4* src = hidden + ((int64_t)b * n_q + n_accept[b] * (k + 1) + o) * row_stride;
+  const int r = blockIdx.x, b = r < n_masks ? r / k : r - n_masks, o = r < n_masks ? r - b * k + 1 : 0;
+  const uint4* src = hidden + ((int64_t)b * n_q + max(0, min(n_accept[b], k)) * (k + 1) + o) * row_stride;
   for (int i = threadIdx.x; i < vecs; i += blockDim.x) dst[(int64_t)blockIdx.x * vecs + i] = src[i];
 }
 
@@ -916,7 +941,9 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   p.B = a->batch; p.k = a->k; p.V = a->vocab; p.D = a->hidden_dim;
   p.n_q = (a->k + 1) * (a->k + 1);
   p.phase = phase;
-  p.n_rows = p.B * (phase == LM_ALL ? p.n_q : phase == LM_TARGETS ? a->k + 1 : a->k);
+  const bool sampling = a->mode == SPACE_MODE_SAMPLE, literal = a->resample == SPACE_RESAMPLE_PAPER_LITERAL;
+  p.n_rows = p.B * (phase == LM_ALL ? p.n_q : (phase == LM_TARGETS || sampling) ? a->k + 1 : a->k);
+  p.sums = !(sampling && phase == LM_MASKS && !literal);    // (point-mass drafts: arg-maxes and the draw alone)
   p.n_pad = (p.n_rows + 15) / 16 * 16;
   if (p.n_pad > LM_MAX_N) return SPACE_E_UNSUPPORTED;
   p.n_mt = p.n_pad > LM_M ? 2 : 1;                         // (tokens on M: accumulators of 256 columns instead of 128)
@@ -932,7 +959,6 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   // with few tokens per thread block (us per call, graph replay, for one / two / four: 64 rows of V = 2091
   // 23.6 / 18.5 / 16.4, 25 rows of V = 5000 25.0 / 20.6 / 18.4, 36 rows of V = 12000 28.2 / 26.9 / 26.9, of
   // V = 32000 53.2 / 53.5 / -).  As many stages as fit, at most LM_MAX_STAGES.
-  const bool sampling = a->mode == SPACE_MODE_SAMPLE;
   // Which operand is the block rows'.  Rows on M: an instruction of 128 rows and N tokens takes 43 + N/2 cycles (one per
   // 128 rows), however few of the 128 are real, and their energy with it, which under the power cap is time.  Tokens
   // on M: 43 + rows/2 for 128 tokens.  So tokens on M for few rows (energy) and where the rows would take two
@@ -962,15 +988,14 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   const size_t budget = 227 * 1024;
   if (sampling) {
     // rows that draw a token (row_const), and as many tokens' noise as the table has room for
-    p.n_noisy = phase == LM_ALL ? (a->resample == SPACE_RESAMPLE_PAPER_LITERAL ? p.n_rows : p.B * (a->k + 1))
-                : (phase == LM_TARGETS || a->resample == SPACE_RESAMPLE_PAPER_LITERAL) ? p.n_rows : 0;
+    p.n_noisy = phase == LM_TARGETS ? 0 : literal ? p.n_rows : p.B * (phase == LM_ALL ? a->k + 1 : 1);
     if (p.n_noisy) {
       // The table may take what a pipeline of a few stages leaves: five where they fit with it or every row draws a token
       // (the folds then work the noise out without waste), four up to 128 rows, three where the rows need two
       // accumulators and a stage is large.  24 KB / this, us per call in bursts: D = 2048, V = 128256, 160 rows 146.7 / 134.9;
       // D = 4096, V = 32000, 160 rows 71.1 / 68.0, 208 rows 74.1 / 71.0.  Other numbers of stages: 208 rows, two 88.4; 80
-      // rows of V = 128256 (D = 2048), four / five 94.5 / 92.5; 16 x 36 rows, 96 and 80 of them at a time, three / four /
-      // five 363 / 357 / 353; 108 rows of V = 32000, four / five 56.5 / 58.7.
+      // rows of V = 128256 (D = 2048), four / five 94.5 / 92.5; 16 x 36 rows, 96 of them at a time, four / five
+      // 343.6 / 340.8; 108 rows of V = 32000, four / five 56.5 / 58.7.
       const int keep = p.n_pad > LM_M ? 3 : (p.n_pad <= 80 || (p.n_pad <= 96 && phase != LM_ALL)) ? 5 : 4;
       int64_t rest = (int64_t)budget - 1024 - LmSmem(false, true, 0, 0, p.n_pad, p.n_box, keep, 1).total;
       if (p.n_box <= 128 && rest > 24 * 1024) rest = 24 * 1024;        // (stages of several slices, see below)
@@ -1036,16 +1061,19 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
 
 // Which launches a batch takes.  Up to 256 block rows: one launch over all of them, one pass over the output
 // embedding.  More: the step decides on 2k+1 rows of every sequence only, so the target rows go first and the
-// mask rows of the groups they select second -- two passes over the embedding, each near the pace of its
+// mask rows of the groups they select second (sampling: with target row i* once more, which draws the extra token; the
+// noise of every target row, of which k in k+1 was for nothing, before: 16 x 36 rows of V = 128256 376 -> 370 us in a loop, of
+// V = 32000 119.0 -> 115.1, 16 x 64 rows of V = 60000, D = 1024 76.6 -> 72.7, drafts sampled 16 x 36 of V = 32000 88.3 -> 85.5) -- two passes over the embedding, each near the pace of its
 // stream, instead of one per 256 rows at the pace of the product.  Calls that ask for every row's maximum
 // keep to the full rows.
 // Measured, us per call, D = 4096, sampling, steady loop (bursts), over all rows / by phase: 16 x 36 rows of
-// V = 128256 832 (722) / 409 (361); 4 x 36 rows of V = 32000 80 (71) / 115 (109); 16 x 16 rows of V = 50257
+// V = 128256 832 (722) / 370 (341); 4 x 36 rows of V = 32000 80 (71) / 115 (109); 16 x 16 rows of V = 50257
 // 140 (125) / 182 (169).
 int launch_lmhead_verify(space_ctx* ctx, const space_lmhead_args* a, cudaStream_t st) {
   const int n_q = (a->k + 1) * (a->k + 1), k1 = a->k + 1;
   const int rows = a->batch * n_q;
-  const int64_t fit = LM_GATHER_ELEMS / ((int64_t)a->k * a->hidden_dim);   // sequences whose mask rows can be gathered
+  const int second = a->mode == SPACE_MODE_SAMPLE ? k1 : a->k;             // rows of a sequence in the second phase
+  const int64_t fit = LM_GATHER_ELEMS / ((int64_t)second * a->hidden_dim);  // sequences whose rows can be gathered
   const int per_phase = fit < LM_M / k1 ? (int)fit : LM_M / k1, per_all = LM_MAX_N / n_q;
   bool by_phase = per_phase > 0 && !a->row_max && !a->row_argmax && rows > LM_MAX_N;
   // a small embedding (under about 10 us of stream) is paced by launches instead: as few of them as can be
@@ -1069,8 +1097,8 @@ int launch_lmhead_verify(space_ctx* ctx, const space_lmhead_args* a, cudaStream_
     if (a->row_argmax) g.row_argmax = a->row_argmax + (int64_t)b0 * n_q;
     int rc = launch_group(ctx, &g, (uint32_t)b0, by_phase ? LM_TARGETS : LM_ALL, st);
     if (rc == SPACE_OK && by_phase) {
-      launch_pdl(lm_gather_kernel, dim3(g.batch * a->k), dim3(256), 0, st, static_cast<const uint4*>(g.hidden),
-                 a->hidden_row_stride / 8, n_q, a->k, a->hidden_dim / 8, (const int32_t*)g.n_accept, (uint4*)ctx->lm_gather);
+      launch_pdl(lm_gather_kernel, dim3(g.batch * second), dim3(256), 0, st, static_cast<const uint4*>(g.hidden),
+                 a->hidden_row_stride / 8, n_q, a->k, g.batch * a->k, a->hidden_dim / 8, (const int32_t*)g.n_accept, (uint4*)ctx->lm_gather);
       ctx->launches += 1;
       rc = launch_group(ctx, &g, (uint32_t)b0, LM_MASKS, st);
     }

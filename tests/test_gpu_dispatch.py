@@ -424,3 +424,11 @@ def test_verify_sweeps_and_many_blocks(B, H, mode, Bn, k, paged, V, dtype):  # n
     for b in range(Bn):
         rows = np.concatenate([got[pg] for pg in y["page_table"][b][: -(-int(new_len[b]) // 128)]], axis=1) if paged else got[b]
         assert np.array_equal(rows[:, :int(new_len[b])], x["k_cache"][b][:, :int(new_len[b])]), b
+
+
+# Sampling by phase: target row i* is projected once more beside the mask rows and draws the extra token there.  As many
+# rows as an accumulator holds, groups of sequences with a small last one, a range of two boxes.
+@pytest.mark.parametrize("mode", ["residual_pointmass", "paper_literal"])
+@pytest.mark.parametrize("V,D,k,Bn", [(9001, 64, 7, 17), (9000, 72, 4, 50), (40009, 64, 5, 42)])
+def test_lmhead_extra_token_in_the_second_pass(B, H, mode, V, D, k, Bn):  # noqa: F811
+    test_lmhead_orientations(B, H, mode, V, D, k, Bn)
