@@ -19,13 +19,14 @@
 // every row in one launch and the last block of a sequence picks i* and the
 // mask rows of group i* from the per-row results, which removes the second
 // launch and its dependent round trips at the price of reading rows that the
-// two-launch path skips.  Measured, us per step behind a short attention (graph
-// replay), one launch / two: 1 x 36 rows of V = 32000 (2 MB) 15.1 / 22.1, 8 x 36
-// (18 MB) 21.4 / 26.9, 16 x 36 (37 MB) 28.7 / 30.5, 24 x 36 (55 MB) 44.0 / 43.5,
-// 28 x 36 (65 MB) 51.3 / 47.4; 8 x 25 rows of 128256 (51 MB) 27.9 / 28.5.  The two
-// meet near 50 MB, a little below the line; rows off the 16-byte grid, whose reading
+// two-launch path skips.  Measured, us per step behind a short attention (steady
+// loop), one launch / two: 1 x 36 rows of V = 32000 (2 MB) 13.2 / 20.2, 8 x 36
+// (18 MB) 16.0 / 24.4, 16 x 36 (37 MB) 19.9 / 23.6, 24 x 36 (55 MB) 32.2 / 31.8,
+// 28 x 36 (65 MB) 34.3 / 32.3; 8 x 25 rows of 128256 (51 MB) 22.3 / 26.7.  The two
+// meet near 55 MB, a little below the line; rows off the 16-byte grid, whose reading
 // costs instructions, meet earlier the more of them can be skipped (16 x 9 rows of
-// 50257, 14 MB, 22.7 / 29.1; 40 x 9, 36 MB, 52.0 / 52.5; 4 x 64, 26 MB, 34.4 / 27.3).
+// 50257, 14 MB, 16.5 / 22.8; 40 x 9, 36 MB, 34.6 / 36.7; 4 x 64, 26 MB, 21.4 / 26.4; 10 x 64,
+// 64 MB, 43.1 / 29.2).
 #include "common.cuh"
 #include "tc_common.cuh"
 #include <math_constants.h>
@@ -266,8 +267,9 @@ __device__ Stat scan_chunk(const T* row, int begin, int end, float c, int exclud
   // the tail shorter than N is handled one by one
   const int full_end = begin + ((end - begin) / N) * N;
   // (As a constant in SHORT scans of bf16 it took the compiler to 80 registers, 94 without, and the loads closer to their
-  // use: one 7B-shaped sequence's step 18.06 -> 18.43 us.  f32, 12.30 -> 12.16, and the others are better off with it.)
-  const int stride = SHORT && sizeof(T) == 2 ? (int)blockDim.x * N : SPACE_VERIFY_THREADS * N;
+  // use: one 7B-shaped sequence's step 18.06 -> 18.43 us; off the 16-byte grid 5 x 16 rows of 50257 17.42 -> 17.57.  f32,
+  // 12.30 -> 12.16, and the long scans are better off with it.)
+  const int stride = (SHORT ? sizeof(T) == 4 : ALIGNED) ? SPACE_VERIFY_THREADS * N : (int)blockDim.x * N;
   const uint4 ninf = make_uint4(Vec<T>::NEG_INF, Vec<T>::NEG_INF, Vec<T>::NEG_INF, Vec<T>::NEG_INF);
   int x = begin + threadIdx.x * N;
   // one sweep of U vectors, the first at x; slots past the end read as -inf
