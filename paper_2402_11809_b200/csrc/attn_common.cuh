@@ -46,16 +46,25 @@ __device__ __forceinline__ int page_of(const P& p, int b, int t, bool flag = tru
 }
 
 // floor(a * b / c) for a*b that may need 64 bits; 32-bit division when it fits
-__device__ __forceinline__ long long muldiv(long long a, long long b, long long c) {
+__host__ __device__ __forceinline__ long long muldiv(long long a, long long b, long long c) {
   const unsigned long long prod = (unsigned long long)a * (unsigned long long)b;
   if ((prod >> 32) == 0) return (long long)((unsigned)prod / (unsigned)c);
   return (long long)(prod / (unsigned long long)c);
 }
 // group that owns flat tile f (largest g with floor(W*g/NG) <= f)
-__device__ __forceinline__ int group_of(long long f, long long W, long long NG) {
+__host__ __device__ __forceinline__ int group_of(long long f, long long W, long long NG) {
   const unsigned long long num = (unsigned long long)(f + 1) * (unsigned long long)NG - 1ull;
   if ((num >> 32) == 0) return (int)((unsigned)num / (unsigned)W);
   return (int)(num / (unsigned long long)W);
+}
+// {first group, number of groups} that the list gives the T tiles of (sequence b, kv head h) to.  The lengths alone say
+// it, so every piece of a cut comes to the same answer, one whose waits ran out as well: the pieces are counted by it.
+__host__ __device__ __forceinline__ int2 list_cut(const int* prefix, int B, int n_groups, int share_cost, int b, int h, int T) {
+  const long long W = prefix[B];
+  const long long NG = W < n_groups ? W : n_groups;
+  const long long f0 = (long long)prefix[b] + (long long)h * (T + share_cost) + share_cost;   // its first tile
+  const int g0 = group_of(f0, W, NG);
+  return make_int2(g0, group_of(f0 + T - 1, W, NG) - g0 + 1);
 }
 
 // Query row r of the row block that starts at block row i0, columns 4 c4 .. of (sequence b, kv head h).
@@ -164,7 +173,9 @@ __device__ __forceinline__ void cluster_leave() {
 // that finds all the others stored notes the cut in its block's shared memory (no merge kernel follows such a launch;
 // as the rule for larger batches this was slower, 137 against 130 us per step of sixteen ragged sequences when it was
 // tried: every piece waits for its fence and its atomic).  At the end the blocks of a cluster combine together what any
-// of them noted.  Called by one thread, after a barrier that orders the stores of all of the block's threads before it.
+// of them noted.  Called by one thread, after a barrier that orders the stores of all of the block's threads before it,
+// for every piece of the cut and with the same cut, also where a wait ran out and nothing was stored: a piece that did
+// not count, or counted to another number, would leave the counter off for every later call.
 constexpr int MAX_DUTIES = 2;          // a block's share of the list starts and ends inside one cut each, at most
 template <class P>
 __device__ __forceinline__ void note_if_last(const P& p, int item, int2 cut, int* arrived, int4* duties) {

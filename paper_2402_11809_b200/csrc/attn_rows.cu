@@ -55,6 +55,10 @@ struct AttnParams {
 
 // One share: tiles t0, t0 + step, ... (n of them) of the T tiles of (sequence b, kv head h).
 struct Seg { int b, h, t0, n, step, T, L; };
+// How a share's (sequence, head) was cut: {first group, number of groups}.
+__host__ __device__ __forceinline__ int2 share_cut(const int* prefix, int B, int n_groups, const Seg& sg, int group) {
+  return sg.n == sg.T ? make_int2(group, 1) : attn::list_cut(prefix, B, n_groups, SHARE_COST, sg.b, sg.h, sg.T);
+}
 
 // PTX helpers: tc_common.cuh.  Every wait of this kernel is bounded by WAIT_NS.
 using namespace tc;
@@ -108,7 +112,7 @@ struct Partition {
   __device__ void init_one(const int* share) { one = share; cur = 0; end = share[3] > 0 ? 1 : 0; }
   // Only min(n_groups, W) groups take part, so every taking-part group owns at
   // least one tile and the groups of one (sequence, head) are consecutive.
-  __device__ void init(const int* sl, const int* pf, int B_, int H, int nq, int group, int n_groups) {
+  __host__ __device__ void init(const int* sl, const int* pf, int B_, int H, int nq, int group, int n_groups) {
     seq_len = sl; prefix = pf; B = B_; H_kv = H; n_q = nq; b = 0; one = nullptr;
     const long long W = pf[B_];
     const long long NG = W < n_groups ? W : n_groups;
@@ -116,7 +120,7 @@ struct Partition {
     cur = muldiv(W, group, NG);
     end = muldiv(W, group + 1, NG);
   }
-  __device__ bool next(Seg& s) {
+  __host__ __device__ bool next(Seg& s) {
     if (one) {
       if (cur >= end) return false;
       ++cur;
@@ -630,17 +634,10 @@ __global__ void __launch_bounds__(THREADS, 1) attn_rows_kernel(const __grid_cons
       float* pslot = to_smem ? reinterpret_cast<float*>(sm + S::PART_OFF)
                              : p.part + ((size_t)(item + group) * p.n_mblocks + mb) * (ROWS * (DH + 2));
       const float inv = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
-      // how this (sequence, head) was cut, {first group, number of groups}: read by attn_rows_merge_kernel (every
-      // group of the cut writes the same pair)
-      int2 cut_d = make_int2(group, 1);
-      if (sidx == 0 && ok && !clustered) {
-        if (!whole) {
-          const long long W = prefix[p.B];
-          const long long NG = W < p.n_groups ? W : p.n_groups;
-          const long long f0 = (long long)prefix[sg.b] + (long long)sg.h * (sg.T + SHARE_COST) + SHARE_COST;
-          cut_d.x = group_of(f0, W, NG);                    // group of the first tile
-          cut_d.y = group_of(f0 + sg.T - 1, W, NG) - cut_d.x + 1;
-        }
+      // how this (sequence, head) was cut is read by attn_rows_merge_kernel (every group of the cut writes the same pair)
+      int2 cut_d = make_int2(0, 0);
+      if (sidx == 0 && !clustered) {
+        cut_d = share_cut(prefix, p.B, p.n_groups, sg, group);
         if (!p.pieces && !p.merge_by_owner) p.desc[(size_t)item * p.n_mblocks + mb] = cut_d;
         // at most one per block: only its first share can start late
         if (sg.t0 > 0 && sg.t0 + sg.n == sg.T) own = make_int4(item, cut_d.x, cut_d.y, 0);

@@ -80,6 +80,13 @@ struct Seg {
   int b, h, t0, n, step, T, L, slot, dfirst, dn;   // slot: partial slot; dfirst/dn: cut (aligned mode)
   __device__ __forceinline__ int tile_at(int j) const { return t0 + j * step; }
 };
+// How a share's (sequence, head) was cut: {first partial slot, number of partials}.
+__host__ __device__ __forceinline__ int2 share_cut(const int* prefix, int B, int H_kv, int n_groups, const Seg& sg) {
+  if (sg.dfirst >= 0) return make_int2(sg.dfirst, sg.dn);
+  if (sg.n == sg.T) return make_int2(sg.slot, 1);
+  const int2 g = attn::list_cut(prefix, B, n_groups, SHARE_COST, sg.b, sg.h, sg.T);
+  return make_int2(sg.b * H_kv + sg.h + g.x, g.y);
+}
 
 // Optional per-block timeline (compiled in with -DSPACE_TIMELINE): one %globaltimer stamp
 // per named point and thread block, read back with space_debug_timeline_read.
@@ -142,7 +149,7 @@ struct Partition {
   // of groups and is cut evenly among them, so no group straddles two of them and
   // pays the per-share set-up and epilogue twice.
   // agroups: groups that have a share in aligned mode, or < 0 for flat mode
-  __device__ void init(const int* sl, const int* pf, int agroups, const int* seg0_, int B_, int H, int nq,
+  __host__ __device__ void init(const int* sl, const int* pf, int agroups, const int* seg0_, int B_, int H, int nq,
                        int group_, int n_groups) {
     seq_len = sl; prefix = pf; seg0 = seg0_; B = B_; H_kv = H; n_q = nq; b = 0;
     group = group_; ngroups = n_groups;
@@ -157,7 +164,7 @@ struct Partition {
     cur = muldiv(W, group_, NG);
     end = muldiv(W, group_ + 1, NG);
   }
-  __device__ bool next(Seg& s) {
+  __host__ __device__ bool next(Seg& s) {
     if (aligned) {
       // the share was worked out once per thread block during the set-up
       if (cur >= end) return false;
@@ -952,19 +959,10 @@ __global__ void __launch_bounds__(THREADS, 1) attn_tc_kernel(const __grid_consta
       const bool whole = sg.n == sg.T;
       const int item = sg.b * p.H_kv + sg.h;
       // (Worked out here, and the row sums below, while the last O^T product still runs.)
-      // How this (sequence, head) was cut, {first partial slot, number of partials}: read by the merge kernel
-      // (every piece writes the same pair)
-      int2 cut_d = make_int2(sg.slot, 1);
-      if (sidx == 0 && ok) {
-        if (sg.dfirst >= 0) {
-          cut_d = make_int2(sg.dfirst, sg.dn);
-        } else if (!whole) {
-          const long long W = prefix[p.B];
-          const long long NG = W < p.n_groups ? W : p.n_groups;
-          const long long f0 = (long long)prefix[sg.b] + (long long)sg.h * (sg.T + SHARE_COST) + SHARE_COST;
-          const int g0 = group_of(f0, W, NG);               // group of the first tile
-          cut_d = make_int2(item + g0, group_of(f0 + sg.T - 1, W, NG) - g0 + 1);
-        }
+      // How this (sequence, head) was cut is read by the merge kernel (every piece writes the same pair)
+      int2 cut_d = make_int2(0, 0);
+      if (sidx == 0) {
+        cut_d = share_cut(prefix, p.B, p.H_kv, p.n_groups, sg);
         if (!p.pieces && !p.merge_by_owner) p.desc[(size_t)item * p.n_mblocks + mb] = cut_d;
         // the piece with the pair's last tile; at most one per block
         if (!whole && sg.tile_at(sg.n - 1) == sg.T - 1) own = make_int4(item, cut_d.x, cut_d.y, 0);
