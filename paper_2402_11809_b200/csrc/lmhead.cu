@@ -54,7 +54,10 @@ constexpr int LM_XP_PITCH = 36;             // floats per row of a warp's transp
 // row i* of every sequence once more (row Bk+b): the extra token is drawn there, so that only one target row per
 // sequence needs noise, not every one that could turn out to be row i*.
 enum { LM_ALL = 0, LM_TARGETS = 1, LM_MASKS = 2 };
-constexpr int64_t LM_GATHER_ELEMS = 128 * 8192;   // mask rows gathered for the second phase
+// rows gathered for the second phase: all that an accumulator holds, up to D = 16384 (fewer sequences at a time beyond).
+// Of half the size it cut sampling batches beyond D = 8192 into more groups, two passes over the embedding each, with k + 1
+// rows of a sequence than with k (12 sequences, k = 5, D = 16384, V = 16000: 368 us in bursts in two groups, 200 in one).
+constexpr int64_t LM_GATHER_ELEMS = 128 * 16384;
 constexpr uint64_t LM_WAIT_NS = 1000000000ull;
 constexpr float LOG2E = 1.4426950408889634f;
 

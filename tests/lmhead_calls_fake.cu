@@ -8,13 +8,14 @@ namespace {
 const space_lmhead_args* other_args;
 int other_rc;
 
-int call(const space_lmhead_args* a) {
+int call(const space_lmhead_args* a, int* launches = nullptr) {
   static char scratch[64];                        // (never read or written: nothing runs)
   space_ctx* c = new space_ctx();
   c->sm_count = 148;
   c->lm_part = c->lm_gather = scratch;
   c->lm_counter = reinterpret_cast<int*>(scratch);
   const int rc = launch_lmhead_verify(c, a, nullptr);
+  if (launches) *launches = (int)c->launches;
   delete c;
   return rc;
 }
@@ -29,4 +30,11 @@ extern "C" void fake_lmhead_two(const space_lmhead_args* a, const space_lmhead_a
   rc[0] = call(a);
   rc[1] = other_rc;
   *smem = fake_largest_launch();
+}
+
+// Launches that a call of `a` takes.
+extern "C" int fake_lmhead_launches(const space_lmhead_args* a) {
+  int n = 0;
+  fake_limits_reset(0, nullptr);
+  return call(a, &n) == SPACE_OK ? n : -1;
 }

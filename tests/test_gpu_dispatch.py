@@ -432,3 +432,10 @@ def test_verify_sweeps_and_many_blocks(B, H, mode, Bn, k, paged, V, dtype):  # n
 @pytest.mark.parametrize("V,D,k,Bn", [(9001, 64, 7, 17), (9000, 72, 4, 50), (40009, 64, 5, 42)])
 def test_lmhead_extra_token_in_the_second_pass(B, H, mode, V, D, k, Bn):  # noqa: F811
     test_lmhead_orientations(B, H, mode, V, D, k, Bn)
+
+
+# Hidden rows as wide as the gathered rows' buffer takes for a full accumulator, and wider.
+@pytest.mark.parametrize("mode", ["greedy", "residual_pointmass"])
+@pytest.mark.parametrize("V,D,k,Bn", [(2101, 16384, 5, 12), (1501, 24008, 1, 65)])
+def test_lmhead_by_phase_wide_hidden_rows(B, H, mode, V, D, k, Bn):  # noqa: F811
+    test_lmhead_by_phase(B, H, mode, V, D, k, Bn)

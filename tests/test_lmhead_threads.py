@@ -30,6 +30,7 @@ def lib(B, tmp_path_factory):
     assert res.returncode == 0, res.stderr[-2000:]
     lib = C.CDLL(str(so))
     lib.fake_lmhead_two.argtypes = [C.POINTER(B.LmHeadArgs)] * 2 + [C.c_int, C.POINTER(C.c_int), C.POINTER(C.c_size_t)]
+    lib.fake_lmhead_launches.argtypes = [C.POINTER(B.LmHeadArgs)]
     return lib
 
 
@@ -56,3 +57,13 @@ def test_another_threads_call_before_a_launch(B, lib, big, small, sample, at):
         lib.fake_lmhead_two(C.byref(x), C.byref(y), at, rc, C.byref(smem))
         assert list(rc) == [B.OK, B.OK]
         assert smem.value <= 227 * 1024
+
+
+# Beyond 256 block rows a group of sequences takes three launches (targets, gather, masks), each group two passes over the
+# embedding.  As many sequences as an accumulator of 128 rows holds, up to D = 16384; beyond it the gathered rows' buffer
+# (128 * 16384 elements) decides, never on fewer than 128 * 8192 // (k D), greedy or sampling.
+@pytest.mark.parametrize("sample", [False, True])
+@pytest.mark.parametrize("batch,k,D,groups", [(12, 5, 16384, 1), (17, 5, 12288, 1), (21, 5, 16384, 1), (22, 5, 16384, 2),
+                                              (9, 7, 16384, 1), (128, 1, 16384, 2), (42, 2, 8192, 1), (65, 1, 24008, 2)])
+def test_groups_of_wide_hidden_rows(B, lib, batch, k, D, groups, sample):
+    assert lib.fake_lmhead_launches(C.byref(_args(B, batch, k, 32000, D, sample))) == 3 * groups
