@@ -49,7 +49,8 @@ constexpr float LM_NEG = -3.0e38f;          // "no logit yet": finite, so that d
 constexpr int LM_MAX_N = 256;               // block rows of the whole batch, padded to 16
 constexpr int LM_TOK = 128;                 // tokens per accumulator with the tokens on M
 constexpr int LM_XP_PITCH = 36;             // floats per row of a warp's transposing buffer (8 rows of 32 tokens)
-// Which block rows a launch projects: all of them, the target rows of every sequence (row b(k+1)+t), or
+// Which block rows a launch projects: all of them, the target rows of every sequence that decide on its candidates (row
+// b n + t: n = k+1 greedy, whose extra token is row i*'s arg-max; n = k in sampling mode, where nothing asks for row k), or
 // the mask rows of every sequence's group i* (row bk+o-1; i* is the launch before's result) and, in sampling mode, target
 // row i* of every sequence once more (row Bk+b): the extra token is drawn there, so that only one target row per
 // sequence needs noise, not every one that could turn out to be row i*.
@@ -76,6 +77,8 @@ struct LmParams {
   int tail_rows;              // rows of the second tensor map's box
   int kbs;                    // 64-element slices of the hidden dimension per stage
   int backwards;              // a box's stages are taken from the hidden dimension's end (see launch_group)
+  int targets;                // rows of a sequence in a launch over the target rows
+  int h_bytes;                // of the hidden rows' box per 64-element slice
   int sums;                   // whether any row's sum of exponentials is asked for
   int n_noisy, noise_tok;     // sampling: rows that draw a token, tokens of a box whose noise is tabulated (a multiple of 16)
   int eos_id;
@@ -256,7 +259,7 @@ __device__ __forceinline__ bool row_place(const LmParams& p, int row, int& b, in
     t = i / k1; o = i - t * k1;
     return true;
   }
-  if (p.phase == LM_TARGETS) { b = row / k1; t = row - b * k1; o = 0; return true; }
+  if (p.phase == LM_TARGETS) { b = row / p.targets; t = row - b * p.targets; o = 0; return true; }
   if (row < p.B * p.k) { b = row / p.k; o = row - b * p.k + 1; }
   else { b = row - p.B * p.k; o = 0; }
   t = max(0, min(p.n_accept[b], p.k));                      // (a first pass that gave up has left it as it was)
@@ -403,7 +406,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         const int row0 = r0 + box * p.n_box;
         const bool tail = r1 - row0 <= p.tail_rows;          // the remaining rows fit the small box
         const CUtensorMap* tm = tail ? &p.tm_wt : &p.tm_w;
-        const uint32_t slice_bytes = (uint32_t)(tail ? p.tail_rows : p.n_box) * LM_KB * 2 + L.a_bytes;
+        const uint32_t slice_bytes = (uint32_t)(tail ? p.tail_rows : p.n_box) * LM_KB * 2 + (uint32_t)p.h_bytes;
         for (int ki = 0; ki < KI; ++ki, ++it) {
           const int kb0 = first_slice(ki);
           // stage `it`: the W tiles and the hidden tiles of its slices
@@ -675,8 +678,10 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
         *reinterpret_cast<int4*>(p.part + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&out);
         atomicMax(p.keys + row, argmax_key(m0, i0));
         if (sample) {
-          LmNoisy g; g.gs = n0.gs; g.gz = n0.gz; g.gidx = n0.gidx; g.pad = 0;
-          *reinterpret_cast<int4*>(p.gpart + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&g);
+          if (p.n_noisy) {
+            LmNoisy g; g.gs = n0.gs; g.gz = n0.gz; g.gidx = n0.gidx; g.pad = 0;
+            *reinterpret_cast<int4*>(p.gpart + (size_t)row * G + c) = *reinterpret_cast<const int4*>(&g);
+          }
           if ((unsigned)(rc.cand_tok - r0) < (unsigned)(r1 - r0)) p.zc[row] = n0.zc;   // this block owns the candidate's token
         }
       }
@@ -698,7 +703,7 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
       const int k1 = p.k + 1;
       // the launch's rows of target t and of mask row (i*, j+1) of sequence b
       const bool with_targets = p.phase != LM_MASKS, with_masks = p.phase != LM_TARGETS;
-      auto target_row = [&](int b, int t) { return p.phase == LM_ALL ? b * p.n_q + t * k1 : b * k1 + t; };
+      auto target_row = [&](int b, int t) { return p.phase == LM_ALL ? b * p.n_q + t * k1 : b * p.targets + t; };
       auto mask_row = [&](int b, int i_star, int j) { return p.phase == LM_ALL ? b * p.n_q + i_star * k1 + j + 1 : b * p.k + j; };
       float* row_m = row_s;                                // [n_rows] maxima (row_s is reused: sums come later)
       int* istar = reinterpret_cast<int*>(smem_raw);       // [B] (the pipeline stages are idle now)
@@ -945,7 +950,12 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   p.n_q = (a->k + 1) * (a->k + 1);
   p.phase = phase;
   const bool sampling = a->mode == SPACE_MODE_SAMPLE, literal = a->resample == SPACE_RESAMPLE_PAPER_LITERAL;
-  p.n_rows = p.B * (phase == LM_ALL ? p.n_q : (phase == LM_TARGETS || sampling) ? a->k + 1 : a->k);
+  // Sampling: target row k scores no candidate and draws nothing in the first pass, and row i* comes once more in the
+  // second.  k+1 rows / k rows, us per call in a loop, V = 32000, D = 4096 (the draws all in the first pass, before the second
+  // had row i*, in brackets): k = 1, 128 sequences 253.5 / 243.9 (247.6), 70 229.4 / 225.1 (228.1), k = 2, 32 121.7 / 118.7
+  // (121.9), k = 3, 20 120.0 / 115.7 (120.8); 16 x 36 rows of V = 128256 394.7 / 392.3 (399.8).
+  p.targets = sampling ? a->k : a->k + 1;
+  p.n_rows = p.B * (phase == LM_ALL ? p.n_q : phase == LM_TARGETS ? p.targets : sampling ? a->k + 1 : a->k);
   p.sums = !(sampling && phase == LM_MASKS && !literal);    // (point-mass drafts: arg-maxes and the draw alone)
   p.n_pad = (p.n_rows + 15) / 16 * 16;
   if (p.n_pad > LM_MAX_N) return SPACE_E_UNSUPPORTED;
@@ -1041,11 +1051,21 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
   int rc = lm_make_map(&p.tm_w, a->weight, a->vocab, a->hidden_dim, a->weight_row_stride, p.n_box);
   if (rc == SPACE_OK) rc = lm_make_map(&p.tm_wt, a->weight, a->vocab, a->hidden_dim, a->weight_row_stride, p.tail_rows);
   // hidden rows in one box: all of them, every (k+1)-th (the target rows lie k+1 rows apart, across
-  // sequences too), or the gathered mask rows
-  if (rc == SPACE_OK)
+  // sequences too), the first k of those of every sequence (sampling; no rows of zeros up to n_pad follow them: what lies
+  // there only reaches accumulator lanes nobody reads), or the gathered rows
+  const bool first_k = sampling && phase == LM_TARGETS;
+  p.h_bytes = (first_k ? p.n_rows : p.n_pad) * LM_KB * 2;
+  if (rc == SPACE_OK && first_k) {
+    const cuuint64_t ld = (cuuint64_t)a->hidden_row_stride * 2;
+    const cuuint64_t dims[4] = {(cuuint64_t)p.D, (cuuint64_t)p.k, (cuuint64_t)p.B, 1};
+    const cuuint64_t strides[3] = {ld * (p.k + 1), ld * p.n_q, ld * p.n_q * p.B};
+    const cuuint32_t box[4] = {(cuuint32_t)LM_KB, (cuuint32_t)p.k, (cuuint32_t)p.B, 1};
+    rc = make_map(&p.tm_h, a->hidden, dims, strides, box);
+  } else if (rc == SPACE_OK) {
     rc = phase == LM_MASKS ? lm_make_map(&p.tm_h, ctx->lm_gather, p.n_rows, a->hidden_dim, a->hidden_dim, p.n_pad)
                            : lm_make_map(&p.tm_h, a->hidden, p.n_rows, a->hidden_dim,
                                          a->hidden_row_stride * (phase == LM_TARGETS ? a->k + 1 : 1), p.n_pad);
+  }
   if (rc != SPACE_OK) return rc;
   const size_t sm = L.total + 1024;
   auto kernel = tokens_on_m ? lmhead_verify_kernel<true, false> : sampling ? lmhead_verify_kernel<false, true> : lmhead_verify_kernel<false, false>;
