@@ -257,13 +257,12 @@ __device__ __forceinline__ uint4* commit_piece(const CommitParams& p, int b, int
 }
 
 // Slice `part` of `nparts` of sequence b's move, by `nthreads` threads (this one is `tid`).
-// All loads of a batch are issued before its stores.
-template <bool PAGED>
+// All loads of a batch of U pieces are issued before its stores.
+template <bool PAGED, int U = 8>
 __device__ __forceinline__ void commit_rows_impl(const CommitParams& p, int b, int L, int i_star, int part, int nparts,
                                                  int tid, int nthreads) {
   const int total = commit_pieces(p, i_star);
   const int stride = nparts * nthreads;
-  constexpr int U = 8;
   for (int t0 = part * nthreads + tid; t0 < total; t0 += U * stride) {
     uint4 val[U];
     uint4* dd[U];

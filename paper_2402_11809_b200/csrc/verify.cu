@@ -760,7 +760,9 @@ verify_fused_kernel(const VerifyParams p, VerifyPartial* fpart) {
     // release would wait for its stores).  Rows L+1 .. L+i* end up exactly as the plain commit leaves
     // them; rows L+i*+1 .. L+k, which lie beyond the new length and held mask-token rows nobody reads
     // again, receive the rejected candidates' rows instead.
-    commit_rows_impl<PAGED>(p.cm, b, Lc, p.k, row_i * p.n_chunks + ch, p.n_q * p.n_chunks, threadIdx.x - 32, SPACE_VERIFY_THREADS - 32);
+    // (Four pieces a batch where eight with the look-ups of a page table do not fit four blocks' registers: with 88 to 92
+    // bytes spilled, paged 22 x 25 rows of 16000 28.8 -> 28.4 us a step, 8 x 25 of 64128 in f32 22.0 -> 21.5.)
+    commit_rows_impl<PAGED, PAGED && BLOCKS == 4 ? 4 : 8>(p.cm, b, Lc, p.k, row_i * p.n_chunks + ch, p.n_q * p.n_chunks, threadIdx.x - 32, SPACE_VERIFY_THREADS - 32);
   }
   __syncthreads();
   TLV(3);
@@ -831,10 +833,13 @@ void launch_fused(space_ctx* ctx, const VerifyParams& p, cudaStream_t st) {
   const bool early = ALIGNED && p.do_commit && per_seq * p.B <= 2 * ctx->sm_count &&
                      p.k * p.cm.H_kv * 2 * (p.cm.d / 8) <= per_seq * (SPACE_VERIFY_THREADS - 32);
   const bool paged = p.do_commit && p.cm.page_table;
-  // Four blocks per SM where three would not hold the launch: its last wave would be nearly empty.  Measured, us per step
-  // behind a short attention, three / four: 16 x 36 rows of 32000 (576 blocks) 20.5 / 20.0, 8 x 25 of 128256 (800) 23.5 / 22.8,
-  // 4 x 64 of 50257 (512, off the 16-byte grid) 23.7 / 21.3; where three hold it the fourth only takes registers: 8 x 49 rows
-  // (392 blocks) 18.2 / 20.2, 12 x 16 (384) 13.8 / 14.5.
+  // Four blocks per SM where three do not hold the launch.  Measured, us per step behind a short attention (loop), three /
+  // four: bf16 16 x 36 rows of 32000 (576 blocks) 20.4 / 19.9, 8 x 25 of 128256 (800) 23.5 / 22.3, 36 x 25 of 28000 (900) 32.6 /
+  // 31.1, 50 x 25 of 24000 (1250) 38.5 / 37.3, 64 x 64 of 1000 (4096) 56.8 / 52.8; f32 16 x 36 of 16000 (576) 19.8 / 17.6,
+  // 36 x 25 of 14000 31.7 / 29.3, 8 x 25 of 64128 (800: two waves either way) 21.6 / 21.8; paged 16 x 36 of 32000 20.2 / 19.9,
+  // 22 x 25 of 16000 (880) 29.9 / 28.4, f32 28.6 / 27.2; off the 16-byte grid 4 x 64 of 50257 (512) 24.4 / 21.9, 40 x 16 of
+  // 16001 28.2 / 27.9.  Where three hold it the fourth only takes registers: 8 x 49 rows (392 blocks) 18.2 / 20.2, 12 x 16
+  // (384) 13.8 / 14.5.
   const bool four = (int64_t)per_seq * p.B > 3 * ctx->sm_count;
   auto form = [&](auto pg) {
     constexpr bool PG = decltype(pg)::value;
