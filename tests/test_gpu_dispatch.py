@@ -366,12 +366,20 @@ def test_filtered_one_launch_or_two(B, H, Bn, k, V, dtype, launches):  # noqa: F
 
 # Clusters launched for lengths that are too unequal (or too long for the pieces a cluster can hold) for them: every cut of
 # the list over the grid is combined by the whole cluster of the block that finds its last piece.  Four row blocks of one
-# pair over all blocks, two pairs of a smaller head, one long sequence among short ones.  Twice: the counters are back
-# where they were, and the pieces are added in a fixed order.
-@pytest.mark.parametrize("k,d,H_q,H_kv,lens,paged", [(6, 128, 8, 1, (9000,), False), (6, 64, 16, 2, (9001,), True),
-                                                     (5, 64, 4, 4, (16000, 800, 127, 640, 0), False),
-                                                     (7, 128, 2, 1, (9000, 300), True)])
-def test_attention_cuts_combined_by_the_cluster(B, H, k, d, H_q, H_kv, lens, paged):  # noqa: F811
+# pair over all blocks, two pairs of a smaller head, one long sequence among short ones, two row blocks of the transposed
+# kernel.  Twice: the counters are back where they were, and the pieces are added in a fixed order.
+@pytest.mark.parametrize("k,d,H_q,H_kv,lens,paged,row_blocks", [(6, 128, 8, 1, (9000,), False, 4), (6, 64, 16, 2, (9001,), True, 4),
+                                                                (5, 64, 4, 4, (16000, 800, 127, 640, 0), False, 1),
+                                                                (7, 128, 2, 1, (16000, 300), True, 2)])
+def test_attention_cuts_combined_by_the_cluster(B, H, k, d, H_q, H_kv, lens, paged, row_blocks):  # noqa: F811
+    # These lengths do not get the clustered cut, whatever number of pieces is launched: its longest piece has more than ten
+    # tiles over an even share (plan_clusters, cluster_fits; up to two clusters fewer than the SMs would hold may fit).
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tiles, pairs = [-(-(L + (k + 1) ** 2) // 128) for L in lens], len(lens) * H_kv
+    launched = [c for c in range(1, 16 // row_blocks + 1) if pairs * c * row_blocks <= sms]
+    for c in launched:
+        groups = max(pairs, sms // (c * row_blocks) - 2) * c
+        assert -(-max(tiles) // c) > -(-sum(tiles) * H_kv // groups) + 10, c
     cfg = _small_cfg(k, (0, max(lens)), d=d, H_q=H_q, H_kv=H_kv, Bn=len(lens), V=64, seed=k + d + len(lens))
     x = workloads.make_step_inputs(cfg)
     x["kv_len"][:] = lens
@@ -381,16 +389,18 @@ def test_attention_cuts_combined_by_the_cluster(B, H, k, d, H_q, H_kv, lens, pag
     n0 = ctx.launch_count
     ds.attn(ctx)
     assert ctx.launch_count - n0 == 1 and not ds.status.any()    # (no merge kernel)
-    got = ds.out.clone()
+    got, got_lse = ds.out.clone(), ds.lse.clone()
     ds.out.fill_(float("nan"))
+    ds.lse.fill_(float("nan"))
     ds.attn(ctx)
-    assert torch.equal(got, ds.out)
-    got = got.cpu().numpy().astype(np.float64)
+    assert torch.equal(got, ds.out) and torch.equal(got_lse, ds.lse)
+    got, got_lse = got.cpu().numpy().astype(np.float64), got_lse.cpu().numpy()
     for b, L in enumerate(lens):
         for h in (0, H_q - 1):
             G = H_q // H_kv
-            ref, _ = attention_head(x["q"][b, :, h], x["k_cache"][b, h // G], x["v_cache"][b, h // G], L, k, x["scale"])
+            ref, lse = attention_head(x["q"][b, :, h], x["k_cache"][b, h // G], x["v_cache"][b, h // G], L, k, x["scale"])
             H.check_attention(got[b:b + 1, :, h], ref[None], f"sequence {b} head {h}")
+            np.testing.assert_allclose(got_lse[b, h], lse, rtol=0, atol=2e-3)
 
 
 # Sweeps of a block that lie in its chunk as a whole and the one that does not, at the edges (a sweep is 8192 bf16 or 4096
