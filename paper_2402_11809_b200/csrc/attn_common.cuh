@@ -1,7 +1,7 @@
 // What the two tensor-core attention kernels (attn_tc.cu, attn_rows.cu) share: page look-ups, the arithmetic of the
 // flat tile list, and how partial results of a (sequence, kv head, query-row block) that was cut over several
-// thread blocks are combined, either in the shared memory of a cluster or, from global memory, by the block that
-// stored the last of them.  `P` is a kernel's parameter struct (G, H_q, n_q, n_mblocks, out_dtype, out, lse, part;
+// thread blocks are combined: in the shared memory of a cluster, or from global memory by the cluster of the block that
+// stored the last of them (by a merge kernel of its own where no clusters are launched).  `P` is a kernel's parameter struct (G, H_q, n_q, n_mblocks, out_dtype, out, lse, part;
 // page_table, pages_per_seq, n_pages, status).
 #pragma once
 #include "common.cuh"

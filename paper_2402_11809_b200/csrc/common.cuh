@@ -100,17 +100,6 @@ __device__ __forceinline__ uint4 shift_pieces(const Piece2& r, const T* row) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Largest of eight bf16 logits as they were loaded: two per instruction, before any is widened (a NaN never wins).
-__device__ __forceinline__ float max_bf16x8(const uint4& x) {
-  auto max2 = [](uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-  };
-  const uint32_t m = max2(max2(x.x, x.y), max2(x.z, x.w));
-  return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xFFFF0000u));
-}
-
 // Asks L2 for a chunk's first sweep of logits, for the time before a kernel's dependency wait: with a programmatic
 // launch the blocks are resident while the kernel before them still runs.  Only a request to the point of
 // coherence: whatever is still being written is what the loads after the wait will see.  (Without / with, us:

@@ -267,7 +267,7 @@ __device__ __forceinline__ bool row_place(const LmParams& p, int row, int& b, in
 }
 
 // Per-row constants of the sampling mode; target rows score candidate c_{t+1} and draw the extra token of the
-// case i* = t at position L+t+1; mask rows (t, o) draw candidate o of that case at position
+// case i* = t at position L+t+1 (by phase, the first pass scores and the second draws, from row i* alone); mask rows (t, o) draw candidate o of that case at position
 // L+t+1+o when candidates are sampled (Algorithm 1 as printed).
 __device__ __forceinline__ RowConst row_const(const LmParams& p, int row) {
   RowConst r{-1, -1, 0u, 0u, 0u, -1, {0, 0}};
@@ -489,8 +489,8 @@ __global__ void __launch_bounds__(LM_THREADS, 1) lmhead_verify_kernel(const __gr
     // where the folds would do it for 32 rows in step although only every (k+1)-th of them draws a token, after
     // the last product, with the whole chip waiting.  D = 4096, bursts, in the folds / tabulated: one sequence of 36 rows,
     // V = 32000, 56.9 / 52.9 us, V = 128256 (D = 2048) 92.7 / 87.3, 144 rows of V = 32000 69.9 / 66.2, of V = 20000 (D = 2048)
-    // 37.7 / 33.2.  (Where the stages leave no room for 16 tokens' noise of every such row, as for the 96 target rows of a
-    // wide batch with five stages, there is no table and the folds work all of it out.)
+    // 37.7 / 33.2.  (A launch whose rows draw nothing, as the first of two by phase, has no table; what the stages leave no
+    // room for, up to all of it, the folds work out.)
     RowConst* rowc = reinterpret_cast<RowConst*>(smem_raw + L.rowc_off);
     float* noise = reinterpret_cast<float*>(smem_raw + L.noise_off);       // [n_noisy][noise_tok + 4]
     const int noise_pitch = p.noise_tok + 4;
@@ -1003,8 +1003,8 @@ int launch_group(space_ctx* ctx, const space_lmhead_args* a, uint32_t seq_base, 
     // rows that draw a token (row_const), and as many tokens' noise as the table has room for
     p.n_noisy = phase == LM_TARGETS ? 0 : literal ? p.n_rows : p.B * (phase == LM_ALL ? a->k + 1 : 1);
     if (p.n_noisy) {
-      // The table may take what a pipeline of a few stages leaves: five where they fit with it or every row draws a token
-      // (the folds then work the noise out without waste), four up to 128 rows, three where the rows need two
+      // The table may take what a pipeline of a few stages leaves: five up to 80 rows (96 by phase, where only every
+      // (k+1)-th draws a token unless drafts are sampled too), four up to 128 rows, three where the rows need two
       // accumulators and a stage is large.  24 KB / this, us per call in bursts: D = 2048, V = 128256, 160 rows 146.7 / 134.9;
       // D = 4096, V = 32000, 160 rows 71.1 / 68.0, 208 rows 74.1 / 71.0.  Other numbers of stages: 208 rows, two 88.4; 80
       // rows of V = 128256 (D = 2048), four / five 94.5 / 92.5; 16 x 36 rows, 96 of them at a time, four / five

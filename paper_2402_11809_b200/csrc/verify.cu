@@ -145,6 +145,17 @@ __device__ __forceinline__ void fold_one(Stat& st, float v, int x, float c, int 
   }
 }
 
+// Largest of eight bf16 logits as they were loaded: two per instruction, before any is widened (a NaN never wins).
+__device__ __forceinline__ float max_bf16x8(const uint4& x) {
+  auto max2 = [](uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+  };
+  const uint32_t m = max2(max2(x.x, x.y), max2(x.z, x.w));
+  return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xFFFF0000u));
+}
+
 // (max, lowest arg-max, sum of exp2((z - max) c)) of U vectors of N logits (v: their values, unless PACKED), the
 // first at index x0, the u-th `stride` further: one maximum and one rescale per
 // call, then independent exponentials and tree sums.  -inf entries (slots past the
@@ -330,15 +341,15 @@ __device__ Stat scan_chunk(const T* row, int begin, int end, float c, int exclud
         x = xn;
       }
     } else {
-    load(cur, 0);
-    meanwhile();
-    for (int sweep = 0; sweep < ns; ++sweep) {
-      load(nxt, sweep + 1);
-      fold(cur, x);
+      load(cur, 0);
+      meanwhile();
+      for (int sweep = 0; sweep < ns; ++sweep) {
+        load(nxt, sweep + 1);
+        fold(cur, x);
 #pragma unroll
-      for (int u = 0; u < U; ++u) cur[u] = nxt[u];
-      x += U * stride;
-    }
+        for (int u = 0; u < U; ++u) cur[u] = nxt[u];
+        x += U * stride;
+      }
     }
   } else {
     // (two loads per vector are in flight here; holding the next sweep's as well would cost 32 registers)
